@@ -48,14 +48,13 @@ GRID_CELL_LARGE_M = 50.0
 # parameters (a multiply each; the differences to the box faces are shared
 # per viewpoint and box), their min/max, and the running max of entries and
 # min of exits, then one compare: 6 FMUL + 12 FMNMX + 1 compare = 19 FP32
-# operations in 3D, 13 in 2D.  Every test the tile kernel counts (row tests
-# of the sweep, corner tests of the one-box checks) decides one
-# segment/box pair.  The separable sweep itself issues only ~6 lane
-# operations per row test (two selects, two fused w-margins, their max and a
-# compare), sharing the u and n parts across a column's rows; those are
-# reported beside the fraction.
+# operations in 3D, 13 in 2D.  The units counted are the tests the tile kernel
+# executes: the corner tests of the one-box checks, each a segment/box pair,
+# and the sweep's interval tests, each a patch column against a box, which
+# decides all of the column's rows (up to 32 segments) but counts once.  The
+# lane operations issued for either are reported beside the fraction.
 OPS_PER_SLAB_TEST = {3: 19, 2: 13}
-ISSUED_OPS_PER_ROW_TEST = 6
+ISSUED_OPS_PER_INTERVAL_TEST = 36
 ISSUED_OPS_PER_CORNER_TEST = 15
 L2_FLUSH_BYTES = 512 << 20
 # kernels of ours that one step launches: k_prologue, k_tiles (two passes:
@@ -373,13 +372,14 @@ def alu_roofline(stats, dims, kern_ms, sm_count, profile=None):
     kern_s = float(np.mean(kern_ms)) / 1e3
     units = stats["slab_tests"] + stats["corner_tests"]
     achieved = units * OPS_PER_SLAB_TEST[dims] / kern_s
-    issued = (stats["slab_tests"] * ISSUED_OPS_PER_ROW_TEST + stats["corner_tests"] * ISSUED_OPS_PER_CORNER_TEST) / kern_s
+    issued = (stats["slab_tests"] * ISSUED_OPS_PER_INTERVAL_TEST +
+              stats["corner_tests"] * ISSUED_OPS_PER_CORNER_TEST) / kern_s
     return {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "Tops/s",
             "frac": achieved / peak, "traffic": profiled_traffic(profile) if profile else None,
-            "kernel": "k_tiles (both passes)", "work_unit": "segment/box slab test",
+            "kernel": "k_tiles (both passes)", "work_unit": "segment/box or column/box slab test",
             "ops_per_unit": OPS_PER_SLAB_TEST[dims],
             "issued_slab_ops": {"value": issued / 1e12, "frac": issued / peak,
-                                "ops_per_row_test": ISSUED_OPS_PER_ROW_TEST,
+                                "ops_per_interval_test": ISSUED_OPS_PER_INTERVAL_TEST,
                                 "ops_per_corner_test": ISSUED_OPS_PER_CORNER_TEST},
             "units_per_launch": units, "kernel_ms": float(np.mean(kern_ms)),
             "peak_basis": "%d SMs x 128 lane-instr/clk x %.0f MHz (issue limit; derived, "

@@ -177,7 +177,8 @@ typedef struct {
     uint32_t vmax_bits;                /* largest v (float bits), accumulated on device */
     uint32_t edge_cells;               /* viewpoints within 1e-5 (relative) of a color bin edge */
     uint32_t error;                    /* VCM_DEVERR_*: nonzero if a device-side check failed */
-    unsigned long long slab_tests;     /* lane-level slab tests executed in the row sweep */
+    unsigned long long slab_tests;     /* slab tests executed in the sweep: a patch column against a box
+                                          (VCM_VIEWER: a segment against a box) */
     unsigned long long rechecked;      /* segment-box pairs re-decided by the exact float64 predicate */
     unsigned long long segments;       /* viewpoint-patch pairs decided (= viewpoints x patches) */
     unsigned long long boxes_listed;   /* sum over tiles of culled candidate-list lengths */
@@ -221,7 +222,8 @@ enum { VCM_FORM_PERSISTENT = 0, VCM_FORM_ONE_TILE = 1, VCM_FORM_RECOLOR = 2 };
 /* Autotuned launch shape for one class of request (see vcm_autotune). */
 typedef struct {
     uint32_t tile_x, tile_y;   /* viewpoints per tile (a tile is one block's work item) */
-    uint32_t patch_k;          /* patch rows per lane held in registers per pass (0 = auto; at most 8) */
+    uint32_t patch_k;          /* patch rows per lane and pass asked for (0 = auto; at most 8); results do
+                                  not depend on it, and the sweep holds up to 32 rows whatever it says */
     uint32_t box_cap;          /* candidate boxes staged in shared memory per tile */
 } vcm_tune;
 

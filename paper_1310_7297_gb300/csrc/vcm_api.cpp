@@ -105,6 +105,7 @@ struct Canon {
     int au = 0, an = 1, aw = 2, perm = 0;
     float sn = 1.f, p_n = 0.f;
     int nu = 1, nw = 1, P = 1, words = 1;
+    float row_step = 1.f, row_dev = 0.f;   // rows along w: mean step, and how far a row is off an even step
     float measure = 0.f;
     int nx = 1, ny = 1, nl = 1;
     std::vector<float> u_coord, w_coord, x_coord, y_coord, z_coord;
@@ -268,6 +269,15 @@ vcm_status canonicalise(const vcm_request *r, Canon &c)
             c.w_coord[iw] = units_to_float(v);
         }
     }
+    if (c.nw > 1) {
+        const double w0 = c.w_coord.front(), step = ((double)c.w_coord.back() - w0) / (c.nw - 1);
+        double dev = 0.0;
+        for (int iw = 0; iw < c.nw; ++iw)
+            dev = std::max(dev, std::fabs(c.w_coord[iw] - (w0 + iw * step)));
+        // rows that all round to one height have no row numbers: the sweep tests them one by one
+        c.row_step = step != 0.0 ? (float)step : 1.f;
+        c.row_dev = step != 0.0 ? (float)dev : 1e30f;
+    }
     c.p_n = units_to_float(cu[c.an]);
     c.u_min = *std::min_element(c.u_coord.begin(), c.u_coord.end());
     c.u_max = *std::max_element(c.u_coord.begin(), c.u_coord.end());
@@ -333,20 +343,28 @@ vcm_status canonicalise_grid(const vcm_request *r, Canon &c)
     return VCM_OK;
 }
 
+// Patch rows per lane and pass that a launch shape asks for, as vcm_get_tune
+// reports them.  The sweep holds up to 32 rows of a lane as one bit mask
+// whatever this says: results never depended on it.
+int rows_per_pass(const Canon &c, const vcm_tune &t)
+{
+    if (c.cone || (c.flags & VCM_TWO_SIDED))
+        return 8;
+    const int groups = 32 / std::min(c.nu, 32);
+    int k = pow2_at_least(std::min((c.nw + groups - 1) / groups, 8));
+    if (t.patch_k > 0)
+        k = std::min(k, pow2_at_least(std::min<int>(t.patch_k, 8)));
+    return k;
+}
+
 // lane mapping and tiling of a canonical request under a launch shape
 void fill_shape(const Canon &c, const vcm_tune &t, DevRequest &d)
 {
     d.nuc = std::min(c.nu, 32);
     d.groups = 32 / d.nuc;
     d.col_passes = (c.nu + d.nuc - 1) / d.nuc;
-    const int rows_per_lane = (c.nw + d.groups - 1) / d.groups;
-    int k = pow2_at_least(std::min(rows_per_lane, 8));
-    if (t.patch_k > 0)
-        k = std::min(k, pow2_at_least(std::min<int>(t.patch_k, 8)));
-    if (c.cone || (c.flags & VCM_TWO_SIDED))
-        k = 8;   // the tile kernel sweeps these requests with its 8-row variant
-    d.k_rows = k;
-    d.row_passes = (c.nw + d.groups * k - 1) / (d.groups * k);
+    d.inv_row = 1.f / ((float)d.groups * c.row_step);
+    d.row_dev = c.row_dev;
     // Work sharing: chunks of 32 open viewpoints, published from a tile
     // with at least 8 open.  Smaller chunks for requests with many patches
     // (about the same work per chunk) were slower: each chunk stages its
@@ -878,7 +896,6 @@ struct Prepared {
     int blocks = 0;
     size_t n = 0;
     bool extra = false;   // a request is two-sided or has a field-of-view cone
-    bool any_bits = false;   // a request emits occlusion bits
     bool tile_check = false;   // every request has many patches: whole-tile check
 };
 
@@ -901,11 +918,10 @@ vcm_status prepare_launch(vcm_ctx *ctx, Slot &s, const std::vector<const Canon *
     P.box_cap = launch_box_cap(shapes);
     P.blocks = grid_blocks_for(ctx, P.box_cap, P.L.total_tiles);
     P.n = cs.size();
-    P.extra = P.any_bits = false;
+    P.extra = false;
     P.tile_check = !cs.empty();
     for (const Canon *c : cs) {
         P.extra = P.extra || needs_extra(*c);
-        P.any_bits = P.any_bits || (c->flags & VCM_EMIT_BITS);
         P.tile_check = P.tile_check && c->P >= kTileCheckMinPatches;
     }
     vcm_status st = ensure_slot(ctx, s, P.L.bytes, cs.size(), P.blocks, sync_stream);
@@ -936,7 +952,7 @@ vcm_status record_launch(vcm_ctx *ctx, Slot &s, const Prepared &P, vcm_stats *st
     const int *d_tiles = reinterpret_cast<const int *>(s.d_desc + P.L.off_tiles);
     const long long *d_vps = reinterpret_cast<const long long *>(s.d_desc + P.L.off_vps);
     (void)stats;   // the descriptors point into it; the prologue clears it
-    CUDA_TRY(launch_prologue(d_reqs, (int)P.n, s.d_work, P.any_bits, stream));
+    CUDA_TRY(launch_prologue(d_reqs, (int)P.n, s.d_work, stream));
     if (P.tile_check && P.L.blocker_ints > 0)   // no blocker recorded yet (-1)
         CUDA_TRY(cudaMemsetAsync(s.d_work + kWorkHeader + kBlockerOff, 0xFF, (size_t)P.L.blocker_ints * sizeof(int),
                                  stream));
@@ -1000,8 +1016,8 @@ vcm_status enqueue_graph(vcm_ctx *ctx, Slot &s, const std::vector<const Canon *>
     const std::vector<unsigned long long> key = {
         ctx->scene_gen, P.L.off_reqs, P.L.off_tiles, P.L.off_vps, P.L.off_coords, P.L.bytes,
         (unsigned long long)P.L.total_tiles, (unsigned long long)P.L.total_vp, (unsigned long long)P.box_cap,
-        (unsigned long long)P.blocks, P.n, (unsigned long long)P.extra, (unsigned long long)P.any_bits,
-        (unsigned long long)P.tile_check, ptr(s.d_desc), ptr(s.h_desc), ptr(s.d_work), ptr(s.d_spill),
+        (unsigned long long)P.blocks, P.n, (unsigned long long)P.extra, (unsigned long long)P.tile_check,
+        ptr(s.d_desc), ptr(s.h_desc), ptr(s.d_work), ptr(s.d_spill),
         ptr(s.d_spill_busy), ptr(stats)};
     direct_only = direct_only || after != nullptr;   // a graph holds no wait on another stream's event
     s.chained = false;
@@ -2424,9 +2440,7 @@ vcm_status vcm_get_tune(vcm_ctx *ctx, const vcm_request *req, vcm_tune *out)
     std::vector<vcm_tune> shapes{shape_for(ctx, c)};
     shrink_small_launch(ctx, {&c}, shapes);
     *out = shapes[0];
-    DevRequest d{};
-    fill_shape(c, *out, d);
-    out->patch_k = (uint32_t)d.k_rows;
+    out->patch_k = (uint32_t)rows_per_pass(c, *out);
     return VCM_OK;
 }
 
@@ -2630,7 +2644,7 @@ vcm_status vcm_compute_static(const float *lo, const float *hi, uint32_t n_boxes
         CUDA_TRY(cudaGetDevice(&dev));
         CUDA_TRY(cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev));
         const int blocks = std::max(1, std::min(lay.total_tiles, tiles_blocks_per_sm((int)t.box_cap) * sm_count));
-        CUDA_TRY(launch_prologue(d_reqs, 1, s_work, (c.flags & VCM_EMIT_BITS) != 0, sm));
+        CUDA_TRY(launch_prologue(d_reqs, 1, s_work, sm));
         CUDA_TRY(launch_tiles(sc, d_reqs, d_tiles, 1, lay.total_tiles, s_work, s_spill, blocks, (int)t.box_cap,
                               needs_extra(c), c.P >= kTileCheckMinPatches, sm));
         CUDA_TRY(launch_quantise(d_reqs, d_vps, 1, lay.total_vp, sm));
@@ -2688,10 +2702,7 @@ vcm_status vcm_autotune(vcm_ctx *ctx, const vcm_request *samples, uint32_t n, vc
         CUDA_TRY(cudaEventCreate(&e1));
         const uint32_t tiles[][2] = {{8, 4}, {8, 8}, {16, 8}, {32, 8}, {16, 16}};
         const uint32_t caps[] = {256, 448, 768};
-        // Rows per pass stay automatic: a batch whose classes used different
-        // row counts would keep several sweep variants hot at once, a cost
-        // that timing one class at a time does not see (the kernel is
-        // sensitive to its instruction footprint).
+        // Rows per pass are left out: the sweep has one form.
         double best_ms[kTuneClasses];
         vcm_tune best[kTuneClasses];
         bool seen[kTuneClasses] = {false};

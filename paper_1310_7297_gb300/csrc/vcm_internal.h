@@ -21,11 +21,6 @@ constexpr int kTileCheckMinPatches = 512;
 constexpr int kMaxPlanes = 32;            // separating planes kept per tile hull
 constexpr float kBand = 1e-6f;            // FP32 slab margin re-decided in FP64
 constexpr int kMaxBoxCap = 5000;          // candidate boxes a tile stages in shared memory
-// Candidate lists longer than this get the per-pass pyramid filter.  At 6-7
-// blocks per SM the filter pays from short lists on (100,000-box step:
-// 3.68 ms with 64, 3.55 with 16, 3.49 with 8, 3.52 with 0; the 256-request
-// batch 102 ms with 0, 87-88 with 8 or more).
-constexpr int kPyramidMinCount = 8;
 constexpr int kMaxTileViewpoints = 1024;  // viewpoints in one tile (tile_x * tile_y)
 constexpr int kClaimRounds = 4096;        // bounded retries of a spill-region claim (2 us pauses)
 
@@ -101,7 +96,8 @@ struct DevRequest {
     float measure;             // patch area (3D) or length (2D), metres
     int nx, ny, nl;            // viewpoint grid
     int tile_x, tile_y, tiles_x, tiles_y, n_tiles;
-    int nuc, groups, col_passes, row_passes, k_rows;   // lane mapping
+    int nuc, groups, col_passes;   // lane mapping
+    float inv_row, row_dev;    // 1 / w step between a lane's rows; how far a row is off an even step
     int chunk_vp, min_publish;   // work sharing: viewpoints per chunk, open viewpoints to publish
     int blk_base;                // offset of its tile positions in the blocker table, or -1
     const float *u_coord;      // [nu] patch centre coordinate along u
@@ -166,10 +162,8 @@ cudaError_t launch_quantise(const DevRequest *d_reqs, const long long *d_vp_pref
 cudaError_t launch_recolor(const DevRequest *d_req, long long n_vp, int sm_count, int *d_list, int *d_n_list,
                            cudaStream_t stream);
 
-// Zero the tile-queue counters (d_work[0..kWorkHeader)), every request's
-// vcm_stats and, when
-// any_bits, the occlusion-bit buffers of the requests with VCM_EMIT_BITS.
-cudaError_t launch_prologue(const DevRequest *d_reqs, int n_req, int *d_work, bool any_bits, cudaStream_t stream);
+// Zero the work counters and every request's vcm_stats.
+cudaError_t launch_prologue(const DevRequest *d_reqs, int n_req, int *d_work, cudaStream_t stream);
 
 // Blocks of the tile kernel that fit on one SM for this shared-memory size.
 int tiles_blocks_per_sm(int box_cap);

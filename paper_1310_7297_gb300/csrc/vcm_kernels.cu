@@ -6,8 +6,8 @@
 //    tile culls the scene against the convex hull of (tile, target) using
 //    the grid, stages the candidates in shared memory with cp.async, and its
 //    warps sweep the tile's viewpoints, lanes over target patch columns and
-//    registers over patch rows, deciding each viewpoint->patch segment by a
-//    float32 slab test (Def. 2 point-to-point visibility; touching blocks,
+//    bits of a mask over patch rows, deciding each viewpoint->patch segment by
+//    a float32 slab test (Def. 2 point-to-point visibility; touching blocks,
 //    Def. 4) with an exact float64 re-decision inside a 1e-6 margin band,
 //    then summing A cos(theta)/d^2 (or len cos(theta)/d in 2D) per viewpoint;
 //  * quantise: colors in L levels from v / v_ref (Def. 1 normalisation).
@@ -86,6 +86,15 @@ __device__ __forceinline__ float rcp_approx(float d)
 {
     float r;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    return r;
+}
+
+// rsqrtf without its scaling of subnormal arguments: squared distances of
+// distinct lattice points are at least 2^-20 m^2.
+__device__ __forceinline__ float rsqrt_normal(float d2)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d2));
     return r;
 }
 
@@ -580,78 +589,6 @@ __device__ __forceinline__ bool one_box_blocks_all(const DevRequest &R, const fl
     return __any_sync(kFull, full);
 }
 
-// Planes of the pyramid with apex q and base the rectangle [u_lo, u_hi] x
-// [w_lo, w_hi] of patch centres (2D: the triangle q, segment ends), in the
-// target frame (u, n, w).  Every segment from q to a patch centre in the
-// rectangle lies in it, so a box outside one of the planes meets none of
-// them.  Each plane's offset is the largest float32
-// evaluation over all the pyramid's points plus the same margin as the tile
-// hull, so the half-space holds the whole pyramid whatever the plane's
-// orientation; a degenerate plane only culls less.  Lanes 0..5 each write
-// one plane (NaN-free: degenerate normals are dropped); returns the count.
-// Not inlined: each sweep variant would carry a copy (1 % on the 3D step).
-__device__ __noinline__ int pyramid_planes(const DevRequest &R, float qu, float qn, float qw, float u_lo, float u_hi,
-                                           float w_lo, float w_hi, Plane *out)
-{
-    const int lane = threadIdx.x & 31;
-    // rectangle corners in order (u_min,w_min) (u_max,w_min) (u_max,w_max) (u_min,w_max)
-    const float P[5][3] = {{qu, qn, qw},
-                           {u_lo, R.p_n, w_lo},
-                           {u_hi, R.p_n, w_lo},
-                           {u_hi, R.p_n, w_hi},
-                           {u_lo, R.p_n, w_hi}};
-    float nx = 0.f, ny = 0.f, nz = 0.f;
-    bool ok = false;
-    if (lane == 0) {
-        // the target plane: segments stay on q's side of it
-        ny = (R.p_n > qn) ? 1.f : -1.f;
-        ok = R.p_n != qn;
-    } else if (lane <= 4) {
-        const int e = lane - 1, f = lane & 3;   // rectangle edge e -> f
-        const float eu = (e == 0 || e == 3) ? u_lo : u_hi, ew = (e < 2) ? w_lo : w_hi;
-        const float fu = (f == 0 || f == 3) ? u_lo : u_hi, fw = (f < 2) ? w_lo : w_hi;
-        if (R.dims == 3) {
-            const float ax = eu - qu, ay = R.p_n - qn, az = ew - qw;
-            const float bx = fu - qu, by = R.p_n - qn, bz = fw - qw;
-            nx = ay * bz - az * by;
-            ny = az * bx - ax * bz;
-            nz = ax * by - ay * bx;
-        } else if (e < 2) {
-            // 2D: lines from q through the two segment ends, normal in the (u, n) plane
-            nx = -(R.p_n - qn);
-            ny = eu - qu;
-        }
-        const float len = sqrtf(nx * nx + ny * ny + nz * nz);
-        ok = len > 0.f;
-        if (ok) {
-            nx /= len; ny /= len; nz /= len;
-            // outward: away from a point inside the pyramid
-            const float cu = 0.5f * (qu + 0.5f * (u_lo + u_hi)), cn = 0.5f * (qn + R.p_n);
-            const float cw = 0.5f * (qw + 0.5f * (w_lo + w_hi));
-            if (dot3(nx, ny, nz, cu, cn, cw) > dot3(nx, ny, nz, qu, qn, qw)) {
-                nx = -nx; ny = -ny; nz = -nz;
-            }
-        }
-    }
-    float c = -f_inf();
-    if (ok) {
-        for (int l = 0; l < 5; ++l)
-            c = fmaxf(c, dot3(nx, ny, nz, P[l][0], P[l][1], P[l][2]));
-        c += 0.04f * (fabsf(nx) + fabsf(ny) + fabsf(nz));
-    }
-    const unsigned okm = __ballot_sync(kFull, ok && lane <= 4);
-    if (ok && lane <= 4)
-        out[__popc(okm & ((1u << lane) - 1u))] = Plane{nx, ny, nz, c};
-    __syncwarp();
-    return __popc(okm);
-}
-
-// One viewpoint swept by one warp.  Lane l owns patch column
-// cp * nuc + (l % nuc) and rows (rp * K + m) * groups + l / nuc, m < K.
-// The t-interval of a segment along u depends only on its column, along n
-// only on the viewpoint and along w only on its row, so the u and n parts
-// of the slab test are formed once per box and column, and each row adds
-// its w interval.
 // Does a viewpoint at normal coordinate qn see the measured side of the
 // target?  One-sided: n.(q - p) > 0.  Two-sided: anywhere off its plane.
 __device__ __forceinline__ bool facing(const DevRequest &R, float qn)
@@ -686,218 +623,285 @@ __device__ __noinline__ bool in_cone(const DevRequest &R, float ru, float rn, fl
     return in_cone_inline(R, ru, rn, rw);
 }
 
-// One variant for either sign of the row offsets w - q_w (a per-row sign
-// mask): a viewpoint layer inside the target's height range and one outside
-// it then run the same code, which halves the sweep's hot instruction
-// footprint (a split by sign made the 3D workload 10 % slower).
-template <int K, bool EXTRA>
+// One row of a column against a box, in float32 with the exact re-decision in
+// the band: the segment q -> (pu, p_n, pw).  Bit 0: blocked, bit 1: re-decided.
+// Not inlined: the sweep takes it for rows at the end of a box's interval only.
+__device__ __noinline__ unsigned row_hit(float qu, float qn, float qw, float pu, float pn, float pw, float4 lo,
+                                         float4 hi, bool is3d)
+{
+    const float du = pu - qu, dn = pn - qn, dw = pw - qw;
+    const float iu = rcp_approx(du), in = rcp_approx(dn);
+    float enter = fmaxf(fmaxf(((du >= 0.f ? lo.x : hi.x) - qu) * iu, ((dn >= 0.f ? lo.y : hi.y) - qn) * in), 0.f);
+    float leave = fminf(fminf(((du >= 0.f ? hi.x : lo.x) - qu) * iu, ((dn >= 0.f ? hi.y : lo.y) - qn) * in), 1.f);
+    if (is3d) {
+        const float iw = rcp_approx(dw);
+        enter = fmaxf(enter, ((dw >= 0.f ? lo.z : hi.z) - qw) * iw);
+        leave = fminf(leave, ((dw >= 0.f ? hi.z : lo.z) - qw) * iw);
+    }
+    const float margin = leave - enter;
+    if (margin > kBand)
+        return 1u;
+    if (margin < -kBand)
+        return 0u;
+    return 2u | (exact_hit(qu, qn, qw, pu, pn, pw, lo, hi) ? 1u : 0u);
+}
+
+// Bits [start, start + n) of a word; start 0..32, n 0..32.
+__device__ __forceinline__ unsigned bit_run(int start, int n)
+{
+    unsigned m;
+    asm("bmsk.clamp.b32 %0, %1, %2;" : "=r"(m) : "r"(start), "r"(n));
+    return m;
+}
+
+// One viewpoint swept by one warp.  Lane l owns patch column cp * nuc +
+// l % nuc and, of the pass's 32 x groups rows, the rows (rp * 32 + m) * groups
+// + l / nuc, m < 32, one bit each.
+//
+// What bounded the sweep was instruction issue: one test per (row, box).  But
+// the rows of a column that a box blocks are one interval.  The column's
+// segment is inside the box's u and n slabs for t in [E, X]; it reaches the
+// box's w extent [a, b] for some such t iff its w offset dw lies in
+//     [a / (a > 0 ? X : E), b / (b > 0 ? E : X)],
+// the union over t of [a / t, b / t].  So a box and a column take one interval
+// in row numbers and one bit mask, about 40 lane operations for up to 32 rows
+// where the row tests took 15 + 8 per row, and the lane holds no per-row state
+// (16 registers), nor are there variants by rows per pass.
+//
+// Only the reciprocals 1/E and 1/X are needed.  Per (viewpoint, box) they come
+// from reciprocals of the box's offsets, which one lane per box forms ahead
+// (the record); per column they are products with du:
+//     iE = min(du r_u + k_u, nE),  iX = max(du f1, du f2, nX).
+// A box beside q in u (a_u > 0 or b_u < 0) has r_u = 1 / its near face and
+// k_u = 0, so a column on the other side gets iE <= 0 and misses; a box that
+// spans q has r_u = 0, k_u = inf (it is entered at t = 0).  f1 and f2 are the
+// far faces for du > 0 and du < 0.  With the hardware reciprocal iE and iX err
+// by at most 5 u, so iE > iX (1 + 1e-6) is a certain u/n hit and iE < iX (1 -
+// 1e-6) a certain miss.  An end of the interval in row numbers errs by at most
+// 12 u (|c| + 33) with c = -dw0 / step, plus twice the rows' rounding to the
+// lattice: rows within eps = 2 dev / step + 2e-6 (|c| + 64) of an end, and
+// every row of an uncertain u/n test, go to row_hit, which has the 1e-6 band
+// and the exact re-decision.  A lane whose eps passes 1/4 row (rows a few
+// lattice units apart) takes row_hit for all its open rows.
+//
+// Measured against the row tests (both passes; 2,048^2 x 8 viewpoints, 100,000
+// boxes, 64 x 32 patches: 10.9 -> 6.4 ms; 512^2 x 5, 5,000 boxes, 32 x 16:
+// 0.247 -> 0.174 ms, with bits 0.41 -> 0.27; 64 uneven requests: 15.7 ->
+// 11.0 ms).
+//
+// The record's shadow on the target plane, [du_lo, du_hi] x [dw_lo, dw_hi],
+// also filters the boxes: one that misses the pass's patch rectangle takes no
+// further part.
+template <bool EXTRA>
 __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const float4 *__restrict__ sbox,
                                                  int n_smem, const int *__restrict__ spill, int count,
                                                  const float4 *__restrict__ gbox, float qu, float qn,
-                                                 float qw, bool front, long long vp, Plane *pyr,
-                                                 bool use_pyr, unsigned long long &tests, unsigned &rechecks,
-                                                 int n_boxes)
+                                                 float qw, bool front, long long vp, float4 *rec,
+                                                 unsigned long long &tests, unsigned &rechecks, int n_boxes)
 {
+    constexpr float kLess = 1.f - 1e-6f, kMore = 1.f + 1e-6f;
+    constexpr float kTiny = 1e-20f;        // stands for a zero offset: inf x kTiny = inf, and 0 otherwise
+    constexpr float kMagic = 12582912.f;   // 1.5 x 2^23: adding it rounds to an integer
     const int lane = threadIdx.x & 31;
     const int nuc = R.nuc, G = R.groups;
-    const int c_in = lane % nuc, g = lane / nuc;
-    const bool lane_ok = g < G;
+    const int g = lane / nuc, c_in = lane - g * nuc;
     const float dn = R.p_n - qn;
-    const float inv_n = rcp_approx(dn);
-    const bool sgn_n = dn >= 0.f;
     const bool want_bits = (R.flags & VCM_EMIT_BITS) && R.bits_out;
     const bool is3d = R.dims == 3;
     // strict: any blocked patch zeroes the viewpoint, so the first one ends it
     const bool strict = (R.flags & VCM_STRICT) != 0;
     const bool strict_exit = strict && !want_bits;
     bool strict_fail = false;
-    const float *__restrict__ w_coord = R.w_coord;
+    const float inv_row = R.inv_row;
     float sum = 0.f, comp = 0.f;
+    if (want_bits) {   // the passes below set bits in the viewpoint's cleared words
+        for (int wd = lane; wd < R.words; wd += 32)
+            put_word(R, vp * R.words + wd, 0u);
+        __syncwarp();
+    }
 
     for (int cp = 0; cp < R.col_passes && !(strict_exit && strict_fail); ++cp) {
         const int iu = cp * nuc + c_in;
-        const bool col_ok = lane_ok && iu < R.nu;
+        const bool col_ok = g < G && iu < R.nu;
         const float pu = R.u_coord[col_ok ? iu : 0];
         const float du = pu - qu;
-        const float inv_u = rcp_approx(du);
-        const bool sgn_u = du >= 0.f;
-        const float ru = qu - pu, rn = qn - R.p_n;
-        const float col_d2 = fmaf(ru, ru, rn * rn);
-        // measure x |r| cos(theta); a two-sided target is measured from either side
-        const float m_s = R.measure * ((EXTRA && (R.flags & VCM_TWO_SIDED)) ? fabsf(rn) : R.sn * rn);
-        // The measure: a plain sum over each group of up to 8 of the lane's
-        // rows (error <= 7u of the group's total, the terms being >= 0), and a
-        // Neumaier-compensated sum of the group totals, so the bound holds for
-        // any patch count.
-        float psum = 0.f;
-        auto add_group = [&](float &g) {
-            const float tsum = sum + g;
-            if (fabsf(sum) >= fabsf(g))
-                comp += (sum - tsum) + g;
-            else
-                comp += (g - tsum) + sum;
-            sum = tsum;
-            g = 0.f;
-        };
-        for (int rp = 0; rp < R.row_passes && !(strict_exit && strict_fail); ++rp) {
-            // per row: its w offset dw and the band of its test in w units,
-            // tau |dw|; -inf once the row is blocked (or past the patch grid)
-            float dwv[K], thr[K];
-            unsigned valid = 0, sgnw = 0;
-#pragma unroll
-            for (int m = 0; m < K; ++m) {
-                const int iw = (rp * K + m) * G + g;
-                const bool ok = col_ok && iw < R.nw;
-                const float dw = w_coord[ok ? iw : 0] - qw;
-                dwv[m] = dw;
-                if (dw >= 0.f)
-                    sgnw |= 1u << m;
-                thr[m] = ok ? kBand * fabsf(dw) : -f_inf();
-                if (ok)
-                    valid |= 1u << m;
-            }
+        // the pass's columns, widened by more than the shadow's rounding
+        const float ua = R.u_coord[cp * nuc] - qu, ub = R.u_coord[min(R.nu, cp * nuc + nuc) - 1] - qu;
+        const float u_slack = 2e-6f * fmaxf(fabsf(ua), fabsf(ub));
+        const float u_from = fminf(ua, ub) - u_slack, u_to = fmaxf(ua, ub) + u_slack;
+        // A lane's terms are added plainly over each 8 of its rows (error
+        // <= 7u of the group's total, the terms being >= 0), and the group
+        // totals with Neumaier's compensation, so the bound holds for any
+        // patch count.
+        for (int rp = 0; rp * 32 * G < R.nw && !(strict_exit && strict_fail); ++rp) {
+            const int row0 = rp * 32 * G;
+            const int mine = col_ok ? min((R.nw - row0 - g + G - 1) / G, 32) : 0;   // the lane's rows
+            const unsigned valid = bit_run(0, max(mine, 0));
+            const float *__restrict__ w_row = R.w_coord + row0 + g;   // row m: w_row[m * G]
             unsigned alive = valid;
-            if (!__any_sync(kFull, alive != 0))
-                continue;
-            // The pyramid filter for this pass: apex q, base the rectangle
-            // of the patch centres the pass covers (its columns by its rows),
-            // so a box whose shadow misses them is dropped before its rows
-            // are tested.
-            int npyr = 0;
-            if (use_pyr) {
-                const int c0 = cp * nuc, c1 = min(R.nu, c0 + nuc) - 1;
-                const int r0 = rp * K * G, r1 = min(R.nw, r0 + K * G) - 1;
-                const float ua = R.u_coord[c0], ub = R.u_coord[c1], wa = w_coord[r0], wb = w_coord[r1];
-                __syncwarp();   // the previous pass has done with the planes
-                npyr = pyramid_planes(R, qu, qn, qw, fminf(ua, ub), fmaxf(ua, ub), fminf(wa, wb), fmaxf(wa, wb), pyr);
-            }
-            int nb = 0;
-            bool done = false;
-            for (int base = 0; base < count && !done; base += 32) {
-              // lanes over boxes: which of the next 32 candidates meet the
-              // viewpoint's pyramid at all
-              unsigned todo;
-              {
-                const int i = base + lane;
-                bool cand = false;
-                if (i < count && npyr == 0) {
-                    cand = true;
-                } else if (i < count) {
-                    float4 lo, hi;
-                    load_box(sbox, n_smem, spill, gbox, i, n_boxes, R.stats, lo, hi);
-                    cand = !outside(pyr, npyr, lo, hi);
-                }
-                todo = __ballot_sync(kFull, cand);
-              }
-              while (todo) {
-                const int i = base + __ffs(todo) - 1;
-                todo &= todo - 1;
-                float4 lo, hi;
-                load_box(sbox, n_smem, spill, gbox, i, n_boxes, R.stats, lo, hi);
-                const float a_u = lo.x - qu, b_u = hi.x - qu;
-                const float a_n = lo.y - qn, b_n = hi.y - qn;
-                const float tnu = (sgn_u ? a_u : b_u) * inv_u;
-                const float tfu = (sgn_u ? b_u : a_u) * inv_u;
-                const float tnn = (sgn_n ? a_n : b_n) * inv_n;
-                const float tfn = (sgn_n ? b_n : a_n) * inv_n;
-                const float pre_e = fmaxf(fmaxf(tnu, tnn), 0.f);
-                const float pre_x = fminf(fminf(tfu, tfn), 1.f);
-                // no row of this column can meet the box: skip the rows
-                if (__all_sync(kFull, alive == 0 || (pre_x - pre_e) < -kBand))
-                    continue;
-                ++nb;   // boxes whose rows are tested
-                // The column's segment is inside the box's u and n slabs for
-                // t in [pre_e, pre_x]; a row meets the box when the w offsets
-                // the segment takes there, t * dw, reach the box's w extent
-                // [a_w, b_w]: e1 = a_w - (the larger end) < 0 and e2 = (the
-                // smaller end) - b_w < 0.  Both are t-margins times |dw|, so the
-                // band is tau |dw|, and the column's own margin pre_x - pre_e
-                // joins them (a hit needs it above tau; below -tau no row
-                // meets the box).  The w extent of a 2D request is unbounded.
-                const float lm = pre_x - pre_e;
-                const bool lane_sure = lm > kBand;
-                float a_w = lo.z - qw, b_w = hi.z - qw;
-                if (R.dims != 3) {
-                    a_w = -f_inf();
-                    b_w = f_inf();
-                }
-                if (lm < -kBand) {   // e1 and e2 are +inf or NaN: no row enters
-                    a_w = f_inf();
-                    b_w = -f_inf();
-                }
-#pragma unroll
-                for (int m = 0; m < K; ++m) {
-                    const bool sp = (sgnw >> m) & 1u;
-                    const float e1 = fmaf(-(sp ? pre_x : pre_e), dwv[m], a_w);
-                    const float e2 = fmaf(sp ? pre_e : pre_x, dwv[m], -b_w);
-                    const float mm = fmaxf(e1, e2);
-                    if (mm <= thr[m] && ((alive >> m) & 1u)) {
-                        bool hit = lane_sure && mm < -thr[m];
-                        if (!hit) {
-                            const int iw = (rp * K + m) * G + g;
-                            hit = exact_hit(qu, qn, qw, pu, R.p_n, w_coord[iw], lo, hi);
-                            ++rechecks;
+            {
+                const float c = -((mine > 0 ? w_row[0] : R.w_min) - qw) * inv_row;
+                const float eps = fmaf(2.f * R.row_dev, fabsf(inv_row), 2e-6f * (fabsf(c) + 64.f));
+                const bool coarse = !(eps < 0.25f);
+                const float near_half = 0.5f - eps;
+                const float wa = R.w_coord[row0] - qw, wb = R.w_coord[min(R.nw, row0 + 32 * G) - 1] - qw;
+                const float w_slack = 2e-6f * fmaxf(fabsf(wa), fabsf(wb));
+                const float w_from = fminf(wa, wb) - w_slack, w_to = fmaxf(wa, wb) + w_slack;
+                int nb = 0;
+                for (int base = 0; base < count; base += 32) {
+                    // lanes over boxes: the records of the next 32 candidates
+                    bool keep = base + lane < count;
+                    if (keep) {
+                        float4 lo, hi;
+                        load_box(sbox, n_smem, spill, gbox, base + lane, n_boxes, R.stats, lo, hi);
+                        const float a_u = lo.x - qu, b_u = hi.x - qu, a_n = lo.y - qn, b_n = hi.y - qn;
+                        // the n interval of every segment from q, as 1 / t
+                        const float D = fabsf(dn), N = dn >= 0.f ? a_n : -b_n, F = dn >= 0.f ? b_n : -a_n;
+                        const float nE = N > 0.f ? D * rcp_approx(N) : f_inf();
+                        const float nX = F > 0.f ? fmaxf(1.f, D * rcp_approx(F)) : D > 0.f ? f_inf() : 1.f;
+                        // offsets with the sign that the end's parameter depends on
+                        const float a_u1 = a_u > 0.f ? a_u : fminf(a_u, -kTiny);
+                        const float b_u1 = b_u < 0.f ? b_u : fmaxf(b_u, kTiny);
+                        keep = F >= 0.f && nE >= nX * kLess && a_u1 * (a_u > 0.f ? nX : nE) <= u_to &&
+                               b_u1 * (b_u < 0.f ? nX : nE) >= u_from;
+                        float a_w = -f_inf(), b_w = f_inf();   // unbounded in 2D
+                        if (is3d) {
+                            a_w = lo.z - qw;
+                            b_w = hi.z - qw;
+                            a_w = a_w > 0.f ? a_w : fminf(a_w, -kTiny);
+                            b_w = b_w < 0.f ? b_w : fmaxf(b_w, kTiny);
+                            keep = keep && a_w * (a_w > 0.f ? nX : nE) <= w_to && b_w * (b_w < 0.f ? nX : nE) >= w_from;
                         }
-                        if (hit) {
-                            thr[m] = -f_inf();
-                            alive &= ~(1u << m);
+                        if (keep) {
+                            const bool out = a_u > 0.f || b_u < 0.f;
+                            const float r_a = a_u != 0.f ? rcp_approx(a_u) : -f_inf();
+                            const float r_b = b_u != 0.f ? rcp_approx(b_u) : f_inf();
+                            const float f1 = b_u < 0.f ? r_a : r_b, f2 = a_u > 0.f ? r_b : r_a;
+                            rec[2 * lane] = make_float4(out ? (a_u > 0.f ? r_a : r_b) : 0.f, out ? 0.f : f_inf(), f1, f2);
+                            // rows may run down the w axis: the smaller row number comes from b then
+                            rec[2 * lane + 1] = make_float4(nE, nX, (inv_row >= 0.f ? a_w : b_w) * inv_row,
+                                                            (inv_row >= 0.f ? b_w : a_w) * inv_row);
                         }
                     }
+                    unsigned todo = __ballot_sync(kFull, keep);
+                    __syncwarp();   // the records are written
+                    bool done = false;
+                    while (todo) {
+                        const int j = __ffs(todo) - 1;
+                        todo &= todo - 1;
+                        const float4 ru = rec[2 * j], rw = rec[2 * j + 1];
+                        const float iE = fminf(fmaf(du, ru.x, ru.y), rw.x);
+                        const float iX = fmaxf(fmaxf(du * ru.z, du * ru.w), rw.y);
+                        ++nb;
+                        if (alive != 0u && iE >= iX * kLess) {
+                            unsigned hit = 0u, ask = 0u;   // rows blocked for certain, rows to decide one by one
+                            // first row + 1/2 and last row - 1/2 of the interval
+                            const float y = fminf(fmaxf(fmaf(rw.z > 0.f ? iX : iE, rw.z, c + 0.5f), 0.f), 32.f);
+                            const float z = fminf(fmaxf(fmaf(rw.w > 0.f ? iE : iX, rw.w, c - 0.5f), -1.f), 31.f);
+                            const float ry = y + kMagic, rz = z + kMagic;
+                            if (!coarse && iE > iX * kMore) {
+                                const int from = __float_as_int(ry) - __float_as_int(kMagic);
+                                hit = bit_run(from, max(__float_as_int(rz) - __float_as_int(ry) + 1, 0));
+                                if (fabsf(y - (ry - kMagic)) > near_half)   // the row at the lower end
+                                    ask = 1u << (__float2int_rn(y - 0.5f) & 31);
+                                if (fabsf(z - (rz - kMagic)) > near_half)   // the row at the upper end
+                                    ask |= 1u << (__float2int_rn(z + 0.5f) & 31);
+                            } else {
+                                ask = kFull;
+                            }
+                            ask &= alive;
+                            hit &= ~ask;
+                            while (ask) {
+                                const int m = __ffs(ask) - 1;
+                                ask &= ask - 1;
+                                float4 lo, hi;
+                                load_box(sbox, n_smem, spill, gbox, base + j, n_boxes, R.stats, lo, hi);
+                                const unsigned h = row_hit(qu, qn, qw, pu, R.p_n, w_row[m * G], lo, hi, is3d);
+                                hit |= (h & 1u) << m;
+                                rechecks += h >> 1;
+                            }
+                            alive &= ~hit;
+                        }
+                        if (__all_sync(kFull, alive == 0u) || (strict_exit && __any_sync(kFull, alive != valid))) {
+                            done = true;
+                            break;
+                        }
+                    }
+                    __syncwarp();   // the records are read before the next are written
+                    if (done)
+                        break;
                 }
-                if (__all_sync(kFull, alive == 0) || (strict_exit && __any_sync(kFull, alive != valid))) {
-                    done = true;
-                    break;
-                }
-              }
+                tests += (unsigned long long)nb;
             }
-            tests += (unsigned long long)nb * K;
             if (strict)
                 strict_fail |= __any_sync(kFull, alive != valid);
-            // the blocked bits, and the visible measure of the unblocked rows
+            const int rows = min((R.nw - row0 + G - 1) / G, 32);   // rows of the pass, per lane
             if (want_bits) {
-#pragma unroll
-                for (int m = 0; m < K; ++m) {
-                    if (((valid & ~alive) >> m) & 1u) {
-                        const int iw = (rp * K + m) * G + g;
-                        const int j = iw * R.nu + iu;
-                        if (IN_BOUNDS(vp * R.words + (j >> 5), (long long)R.nx * R.ny * R.nl * R.words, R.stats))
-                            atomicOr(&R.bits_out[vp * R.words + (j >> 5)], 1u << (j & 31));
-                    }
+                // The blocked bits.  Row m of the pass is one run of patches
+                // over the lanes, from patch j0, so a ballot is its bits and
+                // lane m adds them to the two words they fall into (bit by
+                // bit atomics took a third of the 5,000-box step with bits).
+                unsigned run = 0u;
+                const unsigned blocked = valid & ~alive;
+                for (int m = 0; m < rows; ++m) {
+                    const unsigned b = __ballot_sync(kFull, (blocked >> m) & 1u);
+                    if (lane == m)
+                        run = b;
+                }
+                if (run) {
+                    const int j0 = (row0 + lane * G) * R.nu + cp * nuc;
+                    const long long at = vp * R.words + (j0 >> 5);
+                    const unsigned first = run << (j0 & 31), rest = (j0 & 31) ? run >> (32 - (j0 & 31)) : 0u;
+                    if (first && IN_BOUNDS(at, (long long)R.nx * R.ny * R.nl * R.words, R.stats))
+                        atomicOr(&R.bits_out[at], first);
+                    if (rest && IN_BOUNDS(at + 1, (long long)R.nx * R.ny * R.nl * R.words, R.stats))
+                        atomicOr(&R.bits_out[at + 1], rest);
                 }
             }
-            const unsigned open = front && !strict_fail ? (valid & alive) : 0u;
-            if (__any_sync(kFull, open != 0u)) {
-#pragma unroll
-                for (int m = 0; m < K; ++m) {
-                    if (!((open >> m) & 1u))
-                        continue;
-                    // |r|^2 = (ru^2 + rn^2) of the column + rw^2 of the row;
-                    // rw = q_w - w is the row's offset negated (round to
-                    // nearest is symmetric, so exactly -dw)
-                    const float rw = -dwv[m];
-                    if (EXTRA && R.cone && !in_cone(R, ru, rn, rw))
-                        continue;   // q is outside this patch's field of view
-                    const float d2 = fmaf(rw, rw, col_d2);
-                    float term;
-                    if (is3d) {
-                        const float ir = rsqrtf(d2);
-                        term = m_s * (ir * ir * ir);   // A |r| cos(theta) / |r|^3
-                    } else {
-                        term = m_s / d2;               // len |r| cos(theta) / |r|^2
-                    }
-                    // an add the compiler cannot fuse with the term's
-                    // product, so every specialised copy of this loop
-                    // rounds the same way
-                    psum = __fadd_rn(psum, term);
+            // the visible measure of the open rows
+            const unsigned open = front && !strict_fail ? alive : 0u;
+            if (!__any_sync(kFull, open != 0u))
+                continue;
+            const float ru = qu - pu, rn = qn - R.p_n;
+            const float col_d2 = fmaf(ru, ru, rn * rn);
+            // measure x |r| cos(theta); a two-sided target is measured from either side
+            const float m_s = R.measure * ((EXTRA && (R.flags & VCM_TWO_SIDED)) ? fabsf(rn) : R.sn * rn);
+            // |r|^2 = (ru^2 + rn^2) of the column + rw^2 of the row.  A closed
+            // row adds +0, which changes nothing (the terms are >= 0), so the
+            // rows take no branch.
+            auto term_of = [&](int m) {
+                bool counts = (open >> m) & 1u;
+                const float rw = counts ? qw - w_row[m * G] : 0.f;
+                const float d2 = fmaf(rw, rw, col_d2);
+                float term;
+                if (is3d) {
+                    const float ir = rsqrt_normal(d2);
+                    term = m_s * (ir * ir * ir);   // A |r| cos(theta) / |r|^3
+                } else {
+                    term = m_s / d2;               // len |r| cos(theta) / |r|^2
                 }
+                if (EXTRA && R.cone)
+                    counts = counts && in_cone(R, ru, rn, rw);   // is q in this patch's field of view?
+                return counts ? term : 0.f;
+            };
+            for (int m0 = 0; m0 < rows; m0 += 8) {
+                if (!__any_sync(kFull, (open >> m0) & 0xffu))
+                    continue;
+                float part = 0.f;
+                // an add the compiler cannot fuse with the term's product
+                if (m0 + 8 <= rows) {
+#pragma unroll
+                    for (int m = 0; m < 8; ++m)
+                        part = __fadd_rn(part, term_of(m0 + m));
+                } else {
+                    for (int m = m0; m < rows; ++m)
+                        part = __fadd_rn(part, term_of(m));
+                }
+                const float tsum = sum + part;
+                comp += fabsf(sum) >= fabsf(part) ? (sum - tsum) + part : (part - tsum) + sum;
+                sum = tsum;
             }
-            // a group closes after every 8 of the lane's rows (K divides 8, so
-            // the grouping and the result do not depend on K) and at the end
-            // of the column pass
-            if (((rp + 1) * K) % 8 == 0 || rp + 1 == R.row_passes)
-                add_group(psum);
         }
-        add_group(psum);   // what a strict early exit left
     }
     float v = sum + comp;
     // fixed-order butterfly: every lane ends with the same value
@@ -1005,7 +1009,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
     __shared__ float s_pts[8][3];
     __shared__ DevRequest s_req;
     __shared__ int s_next;
-    __shared__ Plane s_pyr[kWarps][6];
+    __shared__ float4 s_rec[kWarps][2 * 32];    // the sweeps' box records
     __shared__ int s_req_idx;
     __shared__ int s_next2;                     // cursor of the undecided list
     __shared__ int s_und[kMaxTileViewpoints];   // viewpoints left by the one-box check
@@ -1704,21 +1708,8 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                         continue;
                     }
                 }
-                // the pyramid filter pays for its set-up only on long candidate lists
-                Plane *pyr = s_pyr[warp];
-                const bool use_pyr = count > kPyramidMinCount;
-                float v;
-                if (EXTRA && (R.cone || (R.flags & VCM_TWO_SIDED))) {
-                    // sides and cone: one sweep variant of their own (8 rows
-                    // per pass; the host sets k_rows = 8 for these requests)
-                    v = sweep_viewpoint<8, true>(R, s_box, n_smem, list_tail, count, gbox, qu, qn, qw, front, vp, pyr,
-                                                 use_pyr, tests, rechecks, sc.n_boxes);
-                } else switch (R.k_rows) {
-                case 1: v = sweep_viewpoint<1, false>(R, s_box, n_smem, list_tail, count, gbox, qu, qn, qw, front, vp, pyr, use_pyr, tests, rechecks, sc.n_boxes); break;
-                case 2: v = sweep_viewpoint<2, false>(R, s_box, n_smem, list_tail, count, gbox, qu, qn, qw, front, vp, pyr, use_pyr, tests, rechecks, sc.n_boxes); break;
-                case 4: v = sweep_viewpoint<4, false>(R, s_box, n_smem, list_tail, count, gbox, qu, qn, qw, front, vp, pyr, use_pyr, tests, rechecks, sc.n_boxes); break;
-                default: v = sweep_viewpoint<8, false>(R, s_box, n_smem, list_tail, count, gbox, qu, qn, qw, front, vp, pyr, use_pyr, tests, rechecks, sc.n_boxes); break;
-                }
+                float v = sweep_viewpoint<EXTRA>(R, s_box, n_smem, list_tail, count, gbox, qu, qn, qw, front, vp,
+                                                 s_rec[warp], tests, rechecks, sc.n_boxes);
                 if (!front)
                     v = 0.f;
                 if (lane == 0)
@@ -1757,9 +1748,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
         atomicExch(&spill_busy[spill_slot], 0);
 }
 
-// Launch prologue, in one kernel: the tile queue's counter, every request's
-// counters and, for the requests that asked for bits, their occlusion-bit
-// buffers (the tile kernel sets bits with atomicOr).
+// Launch prologue: the work counters and every request's counters.
 __global__ void k_prologue(const DevRequest *__restrict__ reqs, int n_req, int *__restrict__ work)
 {
     const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
@@ -1769,14 +1758,6 @@ __global__ void k_prologue(const DevRequest *__restrict__ reqs, int n_req, int *
     constexpr int kStatWords = (int)(sizeof(vcm_stats) / sizeof(unsigned));
     for (long long i = t; i < (long long)n_req * kStatWords; i += nt)
         reinterpret_cast<unsigned *>(reqs[i / kStatWords].stats)[i % kStatWords] = 0u;
-    for (int r = 0; r < n_req; ++r) {
-        const DevRequest &R = reqs[r];
-        if (!(R.flags & VCM_EMIT_BITS) || !R.bits_out)
-            continue;
-        const long long n = (long long)R.nx * R.ny * R.nl * R.words;
-        for (long long i = t; i < n; i += nt)
-            R.bits_out[i] = 0u;
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -2167,12 +2148,11 @@ cudaError_t launch_tiles(const DevScene &sc, const DevRequest *d_reqs, const int
     return cudaGetLastError();
 }
 
-cudaError_t launch_prologue(const DevRequest *d_reqs, int n_req, int *d_work, bool any_bits, cudaStream_t stream)
+cudaError_t launch_prologue(const DevRequest *d_reqs, int n_req, int *d_work, cudaStream_t stream)
 {
     if (n_req <= 0)
         return cudaSuccess;
-    // without bits there are only n_req counters to clear
-    const int blocks = any_bits ? 152 * 4 : std::max(1, std::min(152, (n_req * 16 + 255) / 256));
+    const int blocks = std::max(1, std::min(152, (n_req * 16 + 255) / 256));
     k_prologue<<<blocks, 256, 0, stream>>>(d_reqs, n_req, d_work);
     return cudaGetLastError();
 }
