@@ -363,6 +363,7 @@ void fill_shape(const Canon &c, const vcm_tune &t, DevRequest &d)
     d.nuc = std::min(c.nu, 32);
     d.groups = 32 / d.nuc;
     d.col_passes = (c.nu + d.nuc - 1) / d.nuc;
+    d.rows = (c.nw + d.groups - 1) / d.groups;
     d.inv_row = 1.f / ((float)d.groups * c.row_step);
     d.row_dev = c.row_dev;
     // Work sharing: chunks of 32 open viewpoints, published from a tile

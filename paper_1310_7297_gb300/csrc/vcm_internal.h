@@ -21,6 +21,7 @@ constexpr int kTileCheckMinPatches = 512;
 constexpr int kMaxPlanes = 32;            // separating planes kept per tile hull
 constexpr float kBand = 1e-6f;            // FP32 slab margin re-decided in FP64
 constexpr int kMaxBoxCap = 5000;          // candidate boxes a tile stages in shared memory
+constexpr int kRowCap = 512;              // patch rows staged in shared memory for the measure
 constexpr int kMaxTileViewpoints = 1024;  // viewpoints in one tile (tile_x * tile_y)
 constexpr int kClaimRounds = 4096;        // bounded retries of a spill-region claim (2 us pauses)
 
@@ -96,7 +97,7 @@ struct DevRequest {
     float measure;             // patch area (3D) or length (2D), metres
     int nx, ny, nl;            // viewpoint grid
     int tile_x, tile_y, tiles_x, tiles_y, n_tiles;
-    int nuc, groups, col_passes;   // lane mapping
+    int nuc, groups, col_passes, rows;   // lane mapping: columns and row groups of a pass, column passes, rows per lane
     float inv_row, row_dev;    // 1 / w step between a lane's rows; how far a row is off an even step
     int chunk_vp, min_publish;   // work sharing: viewpoints per chunk, open viewpoints to publish
     int blk_base;                // offset of its tile positions in the blocker table, or -1

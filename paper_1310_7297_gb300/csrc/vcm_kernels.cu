@@ -553,41 +553,12 @@ __device__ __noinline__ bool box_blocks_tile(const DevRequest &R, float4 lo, flo
     return true;
 }
 
-// True if one of the first `nb` (<= 32) staged boxes certainly blocks the
-// segments from q to all four extreme patch centres.  On the target plane the
-// points whose segment to q meets a convex box form a convex set (a segment
-// from q to any point between two blocked ones crosses the box between their
-// two hit points), and every patch centre lies in the rectangle spanned by
-// the extreme ones, so such a box blocks every patch.  Lanes take one box
-// each; only float32 margins above the band count, so the answer is exact.
-__device__ __forceinline__ bool one_box_blocks_all(const DevRequest &R, const float4 *__restrict__ sbox, int nb,
-                                                   float qu, float qn, float qw)
-{
-    const int lane = threadIdx.x & 31;
-    const float du0 = R.u_min - qu, du1 = R.u_max - qu;
-    const float dn = R.p_n - qn;
-    const float dw0 = R.w_min - qw, dw1 = R.w_max - qw;
-    bool full = false;
-    if (lane < nb) {
-        const float iu0 = rcp_approx(du0), iu1 = rcp_approx(du1), inn = rcp_approx(dn);
-        const float iw0 = rcp_approx(dw0), iw1 = rcp_approx(dw1);
-        const float4 lo = sbox[2 * lane], hi = sbox[2 * lane + 1];
-        const float au = lo.x - qu, bu = hi.x - qu, an = lo.y - qn, bn = hi.y - qn;
-        const float aw = lo.z - qw, bw = hi.z - qw;
-        const float nu0 = (du0 >= 0.f ? au : bu) * iu0, fu0 = (du0 >= 0.f ? bu : au) * iu0;
-        const float nu1 = (du1 >= 0.f ? au : bu) * iu1, fu1 = (du1 >= 0.f ? bu : au) * iu1;
-        const float nw0 = (dw0 >= 0.f ? aw : bw) * iw0, fw0 = (dw0 >= 0.f ? bw : aw) * iw0;
-        const float nw1 = (dw1 >= 0.f ? aw : bw) * iw1, fw1 = (dw1 >= 0.f ? bw : aw) * iw1;
-        const float e0 = fmaxf((dn >= 0.f ? an : bn) * inn, 0.f);
-        const float x0 = fminf((dn >= 0.f ? bn : an) * inn, 1.f);
-        const bool c00 = fminf(fminf(fu0, fw0), x0) - fmaxf(fmaxf(nu0, nw0), e0) > kBand;
-        const bool c10 = fminf(fminf(fu1, fw0), x0) - fmaxf(fmaxf(nu1, nw0), e0) > kBand;
-        const bool c01 = fminf(fminf(fu0, fw1), x0) - fmaxf(fmaxf(nu0, nw1), e0) > kBand;
-        const bool c11 = fminf(fminf(fu1, fw1), x0) - fmaxf(fmaxf(nu1, nw1), e0) > kBand;
-        full = c00 && c10 && c01 && c11;
-    }
-    return __any_sync(kFull, full);
-}
+// One-box check.  On the target plane the points whose segment to q meets a
+// convex box form a convex set (a segment from q to any point between two
+// blocked ones crosses the box between their two hit points), and every patch
+// centre lies in the rectangle spanned by the extreme ones, so a box that
+// blocks the four extreme patches blocks every patch.  Only margins above the
+// band count, so the answer is exact.
 
 // Does a viewpoint at normal coordinate qn see the measured side of the
 // target?  One-sided: n.(q - p) > 0.  Two-sided: anywhere off its plane.
@@ -684,27 +655,144 @@ __device__ __forceinline__ unsigned bit_run(int start, int n)
 // and the exact re-decision.  A lane whose eps passes 1/4 row (rows a few
 // lattice units apart) takes row_hit for all its open rows.
 //
-// Measured against the row tests (both passes; 2,048^2 x 8 viewpoints, 100,000
-// boxes, 64 x 32 patches: 10.9 -> 6.4 ms; 512^2 x 5, 5,000 boxes, 32 x 16:
-// 0.247 -> 0.174 ms, with bits 0.41 -> 0.27; 64 uneven requests: 15.7 ->
-// 11.0 ms).
+// The boxes are filtered once per viewpoint, one per lane: a box whose shadow
+// on the target plane, [du_lo, du_hi] x [dw_lo, dw_hi], misses the patch
+// rectangle takes no further part.  The one-box test of the kept boxes comes
+// from the same record: a box that certainly blocks the four extreme patches
+// blocks them all (the one-box check), and the viewpoint is decided.  A
+// viewpoint keeps its records over its column passes when at most 32 boxes
+// are left (nearly always: 1 to 5); otherwise each pass filters the list again.
 //
-// The record's shadow on the target plane, [du_lo, du_hi] x [dw_lo, dw_hi],
-// also filters the boxes: one that misses the pass's patch rectangle takes no
-// further part.
-template <bool EXTRA>
-__device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const float4 *__restrict__ sbox,
-                                                 int n_smem, const int *__restrict__ spill, int count,
-                                                 const float4 *__restrict__ gbox, float qu, float qn,
-                                                 float qw, bool front, long long vp, float4 *rec,
-                                                 unsigned long long &tests, unsigned &rechecks, int n_boxes)
+// Measured against the row tests (both passes; 2,048^2 x 8 viewpoints, 100,000
+// boxes, 64 x 32 patches: 10.9 -> 5.4 ms; 512^2 x 5, 5,000 boxes, 32 x 16:
+// 0.247 -> 0.164 ms, with bits 0.41 -> 0.267; 64 uneven requests: 15.7 ->
+// 8.9 ms).
+
+constexpr float kLess = 1.f - 1e-6f, kMore = 1.f + 1e-6f;
+
+// A rectangle of patch centres relative to a viewpoint, and the same widened
+// by more than a shadow's rounding.
+struct PatchRect {
+    float u0, u1, w0, w1;          // smallest and largest offset along u and w
+    float u_from, u_to, w_from, w_to;
+};
+__device__ __forceinline__ PatchRect patch_rect(float u0, float u1, float w0, float w1)
 {
-    constexpr float kLess = 1.f - 1e-6f, kMore = 1.f + 1e-6f;
-    constexpr float kTiny = 1e-20f;        // stands for a zero offset: inf x kTiny = inf, and 0 otherwise
+    const float su = 2e-6f * fmaxf(fabsf(u0), fabsf(u1)), sw = 2e-6f * fmaxf(fabsf(w0), fabsf(w1));
+    return PatchRect{u0, u1, w0, w1, u0 - su, u1 + su, w0 - sw, w1 + sw};
+}
+
+// The record of one box for a viewpoint, if its shadow meets the rectangle:
+// returns whether it does.  r0 = (r_u, k_u, f1, f2); r1 = (nE, nX, a, b) with a
+// and b the w offsets whose quotients bound the rows from below and above (for
+// rows that run down the w axis they trade places), in rows.
+__device__ __forceinline__ bool make_record(float4 lo, float4 hi, float qu, float qn, float qw, float dn, bool is3d,
+                                            float inv_row, const PatchRect &P, float4 &r0, float4 &r1)
+{
+    constexpr float kTiny = 1e-20f;   // stands for a zero offset: inf x kTiny = inf, and 0 otherwise
+    const float a_u = lo.x - qu, b_u = hi.x - qu, a_n = lo.y - qn, b_n = hi.y - qn;
+    // the n interval of every segment from q, as 1 / t
+    const float D = fabsf(dn), N = dn >= 0.f ? a_n : -b_n, F = dn >= 0.f ? b_n : -a_n;
+    const float nE = N > 0.f ? D * rcp_approx(N) : f_inf();
+    const float nX = F > 0.f ? fmaxf(1.f, D * rcp_approx(F)) : D > 0.f ? f_inf() : 1.f;
+    // offsets with the sign that the end's parameter depends on
+    const float a_u1 = a_u > 0.f ? a_u : fminf(a_u, -kTiny), b_u1 = b_u < 0.f ? b_u : fmaxf(b_u, kTiny);
+    bool keep = F >= 0.f && nE >= nX * kLess && a_u1 * (a_u > 0.f ? nX : nE) <= P.u_to &&
+                b_u1 * (b_u < 0.f ? nX : nE) >= P.u_from;
+    float a_w = -f_inf(), b_w = f_inf();   // unbounded in 2D
+    if (is3d) {
+        a_w = lo.z - qw;
+        b_w = hi.z - qw;
+        a_w = a_w > 0.f ? a_w : fminf(a_w, -kTiny);
+        b_w = b_w < 0.f ? b_w : fmaxf(b_w, kTiny);
+        keep = keep && a_w * (a_w > 0.f ? nX : nE) <= P.w_to && b_w * (b_w < 0.f ? nX : nE) >= P.w_from;
+    }
+    if (!keep)
+        return false;
+    const bool out = a_u > 0.f || b_u < 0.f;
+    const float r_a = a_u != 0.f ? rcp_approx(a_u) : -f_inf(), r_b = b_u != 0.f ? rcp_approx(b_u) : f_inf();
+    r0 = make_float4(out ? (a_u > 0.f ? r_a : r_b) : 0.f, out ? 0.f : f_inf(), b_u < 0.f ? r_a : r_b,
+                     a_u > 0.f ? r_b : r_a);
+    r1 = make_float4(nE, nX, (inv_row >= 0.f ? a_w : b_w) * inv_row, (inv_row >= 0.f ? b_w : a_w) * inv_row);
+    return true;
+}
+
+// True if a recorded box certainly blocks all four corners of the rectangle.
+// Along w the bound of the smaller offset's side is a / dw > 0 only with a > 0.
+__device__ __forceinline__ bool record_blocks_rect(float4 r0, float4 r1, float inv_row, const PatchRect &P)
+{
+    const float e0 = fminf(fmaf(P.u0, r0.x, r0.y), r1.x), e1 = fminf(fmaf(P.u1, r0.x, r0.y), r1.x);
+    const float x0 = fmaxf(fmaxf(P.u0 * r0.z, P.u0 * r0.w), r1.y), x1 = fmaxf(fmaxf(P.u1 * r0.z, P.u1 * r0.w), r1.y);
+    // per column the w offsets it blocks for certain: (from, to), as in the sweep
+    const float row = fabsf(inv_row), a = inv_row >= 0.f ? r1.z : -r1.w, b = inv_row >= 0.f ? r1.w : -r1.z;
+    const float from = fmaxf(a * (a > 0.f ? x0 : e0), a * (a > 0.f ? x1 : e1));
+    const float to = fminf(b * (b > 0.f ? e0 : x0), b * (b > 0.f ? e1 : x1));
+    return e0 > x0 * kMore && e1 > x1 * kMore && from < P.w_from * row && to > P.w_to * row;
+}
+
+// The filter of one pass for a viewpoint with more than 32 kept boxes: lanes
+// over the boxes [base, base + 32); returns the kept ones, records written.
+__device__ __noinline__ unsigned pass_records(const DevRequest &R, const float4 *__restrict__ sbox, int n_smem,
+                                              const int *__restrict__ spill, int count,
+                                              const float4 *__restrict__ gbox, float qu, float qn, float qw, int cp,
+                                              int row0, float4 *rec, int n_boxes, int base)
+{
+    const int lane = threadIdx.x & 31;
+    const float ua = R.u_coord[cp * R.nuc] - qu, ub = R.u_coord[min(R.nu, cp * R.nuc + R.nuc) - 1] - qu;
+    const float wa = R.w_coord[row0] - qw, wb = R.w_coord[min(R.nw, row0 + 32 * R.groups) - 1] - qw;
+    bool keep = base + lane < count;
+    if (keep) {
+        float4 lo, hi, r0, r1;
+        load_box(sbox, n_smem, spill, gbox, base + lane, n_boxes, R.stats, lo, hi);
+        keep = make_record(lo, hi, qu, qn, qw, R.p_n - qn, R.dims == 3, R.inv_row,
+                           patch_rect(fminf(ua, ub), fmaxf(ua, ub), fminf(wa, wb), fmaxf(wa, wb)), r0, r1);
+        if (keep) {
+            rec[2 * lane] = r0;
+            rec[2 * lane + 1] = r1;
+        }
+    }
+    return __ballot_sync(kFull, keep);
+}
+
+// A warp's lane mapping and the staged rows of a tile's request.
+struct LaneMap {
+    int c_in, g;     // the lane's column of a pass, and its row group
+    int rows;        // rows of its group (0 for the lanes past the last group)
+    const float *s_row;   // its rows in shared memory, in order; null if they do not fit
+};
+
+// One open patch's term of the visible measure.  |r|^2 is (ru^2 + rn^2) of the
+// column + rw^2 of the row.
+template <bool EXTRA, bool IS3D>
+__device__ __forceinline__ float measure_term(const DevRequest &R, float col_d2, float m_s, float ru, float rn,
+                                              float rw)
+{
+    const float d2 = fmaf(rw, rw, col_d2);
+    float term;
+    if (IS3D) {
+        const float ir = rsqrt_normal(d2);
+        term = m_s * (ir * ir * ir);   // A |r| cos(theta) / |r|^3
+    } else {
+        term = m_s / d2;               // len |r| cos(theta) / |r|^2
+    }
+    if (EXTRA && R.cone && !in_cone(R, ru, rn, rw))
+        term = 0.f;   // q is outside this patch's field of view
+    return term;
+}
+
+// Returns the viewpoint's value, or -1 if one box blocks every patch.
+template <bool EXTRA>
+__device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const LaneMap &M,
+                                                 const float4 *__restrict__ sbox, int n_smem,
+                                                 const int *__restrict__ spill, int count,
+                                                 const float4 *__restrict__ gbox, float qu, float qn,
+                                                 float qw, bool front, long long vp, float4 *rec, int *rec_id,
+                                                 unsigned long long &tests, unsigned long long &corners,
+                                                 unsigned &rechecks, int n_boxes)
+{
     constexpr float kMagic = 12582912.f;   // 1.5 x 2^23: adding it rounds to an integer
     const int lane = threadIdx.x & 31;
     const int nuc = R.nuc, G = R.groups;
-    const int g = lane / nuc, c_in = lane - g * nuc;
     const float dn = R.p_n - qn;
     const bool want_bits = (R.flags & VCM_EMIT_BITS) && R.bits_out;
     const bool is3d = R.dims == 3;
@@ -714,6 +802,38 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const floa
     bool strict_fail = false;
     const float inv_row = R.inv_row;
     float sum = 0.f, comp = 0.f;
+
+    // the boxes that can block a patch at all, and the one-box test of each
+    // (lists of at most 8 boxes were tested whole in the tile pass)
+    int n_rec = 0;
+    {
+        const PatchRect P = patch_rect(R.u_min - qu, R.u_max - qu, R.w_min - qw, R.w_max - qw);
+        for (int base = 0; base < count; base += 32) {
+            bool keep = base + lane < count, full = false;
+            float4 r0, r1;
+            if (keep) {
+                float4 lo, hi;
+                load_box(sbox, n_smem, spill, gbox, base + lane, n_boxes, R.stats, lo, hi);
+                keep = make_record(lo, hi, qu, qn, qw, dn, is3d, inv_row, P, r0, r1);
+                if (keep && count > 8)
+                    full = record_blocks_rect(r0, r1, inv_row, P);
+            }
+            const unsigned kept = __ballot_sync(kFull, keep);
+            if (kept == 0u)
+                continue;
+            corners += count > 8 ? 4 * __popc(kept) : 0;
+            if (__any_sync(kFull, full))
+                return -1.f;
+            const int at = n_rec + __popc(kept & ((1u << lane) - 1u));
+            if (keep && at < 32) {
+                rec[2 * at] = r0;
+                rec[2 * at + 1] = r1;
+                rec_id[at] = base + lane;
+            }
+            n_rec += __popc(kept);
+        }
+        __syncwarp();   // the records are written
+    }
     if (want_bits) {   // the passes below set bits in the viewpoint's cleared words
         for (int wd = lane; wd < R.words; wd += 32)
             put_word(R, vp * R.words + wd, 0u);
@@ -721,70 +841,37 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const floa
     }
 
     for (int cp = 0; cp < R.col_passes && !(strict_exit && strict_fail); ++cp) {
-        const int iu = cp * nuc + c_in;
-        const bool col_ok = g < G && iu < R.nu;
+        const int iu = cp * nuc + M.c_in;
+        const bool col_ok = iu < R.nu;
         const float pu = R.u_coord[col_ok ? iu : 0];
         const float du = pu - qu;
-        // the pass's columns, widened by more than the shadow's rounding
-        const float ua = R.u_coord[cp * nuc] - qu, ub = R.u_coord[min(R.nu, cp * nuc + nuc) - 1] - qu;
-        const float u_slack = 2e-6f * fmaxf(fabsf(ua), fabsf(ub));
-        const float u_from = fminf(ua, ub) - u_slack, u_to = fmaxf(ua, ub) + u_slack;
         // A lane's terms are added plainly over each 8 of its rows (error
         // <= 7u of the group's total, the terms being >= 0), and the group
         // totals with Neumaier's compensation, so the bound holds for any
         // patch count.
-        for (int rp = 0; rp * 32 * G < R.nw && !(strict_exit && strict_fail); ++rp) {
-            const int row0 = rp * 32 * G;
-            const int mine = col_ok ? min((R.nw - row0 - g + G - 1) / G, 32) : 0;   // the lane's rows
+        for (int r_at = 0; r_at < R.rows && !(strict_exit && strict_fail); r_at += 32) {
+            const int row0 = r_at * G;                          // the pass's first row
+            const int rows = min(R.rows - r_at, 32);            // its rows per lane
+            const int mine = col_ok ? min(M.rows - r_at, 32) : 0;
             const unsigned valid = bit_run(0, max(mine, 0));
-            const float *__restrict__ w_row = R.w_coord + row0 + g;   // row m: w_row[m * G]
+            const float *__restrict__ w_row = R.w_coord + row0 + M.g;   // row m: w_row[m * G]
             unsigned alive = valid;
-            {
+            if (n_rec > 0) {
                 const float c = -((mine > 0 ? w_row[0] : R.w_min) - qw) * inv_row;
                 const float eps = fmaf(2.f * R.row_dev, fabsf(inv_row), 2e-6f * (fabsf(c) + 64.f));
                 const bool coarse = !(eps < 0.25f);
                 const float near_half = 0.5f - eps;
-                const float wa = R.w_coord[row0] - qw, wb = R.w_coord[min(R.nw, row0 + 32 * G) - 1] - qw;
-                const float w_slack = 2e-6f * fmaxf(fabsf(wa), fabsf(wb));
-                const float w_from = fminf(wa, wb) - w_slack, w_to = fmaxf(wa, wb) + w_slack;
+                const bool fits = n_rec <= 32;
                 int nb = 0;
-                for (int base = 0; base < count; base += 32) {
-                    // lanes over boxes: the records of the next 32 candidates
-                    bool keep = base + lane < count;
-                    if (keep) {
-                        float4 lo, hi;
-                        load_box(sbox, n_smem, spill, gbox, base + lane, n_boxes, R.stats, lo, hi);
-                        const float a_u = lo.x - qu, b_u = hi.x - qu, a_n = lo.y - qn, b_n = hi.y - qn;
-                        // the n interval of every segment from q, as 1 / t
-                        const float D = fabsf(dn), N = dn >= 0.f ? a_n : -b_n, F = dn >= 0.f ? b_n : -a_n;
-                        const float nE = N > 0.f ? D * rcp_approx(N) : f_inf();
-                        const float nX = F > 0.f ? fmaxf(1.f, D * rcp_approx(F)) : D > 0.f ? f_inf() : 1.f;
-                        // offsets with the sign that the end's parameter depends on
-                        const float a_u1 = a_u > 0.f ? a_u : fminf(a_u, -kTiny);
-                        const float b_u1 = b_u < 0.f ? b_u : fmaxf(b_u, kTiny);
-                        keep = F >= 0.f && nE >= nX * kLess && a_u1 * (a_u > 0.f ? nX : nE) <= u_to &&
-                               b_u1 * (b_u < 0.f ? nX : nE) >= u_from;
-                        float a_w = -f_inf(), b_w = f_inf();   // unbounded in 2D
-                        if (is3d) {
-                            a_w = lo.z - qw;
-                            b_w = hi.z - qw;
-                            a_w = a_w > 0.f ? a_w : fminf(a_w, -kTiny);
-                            b_w = b_w < 0.f ? b_w : fmaxf(b_w, kTiny);
-                            keep = keep && a_w * (a_w > 0.f ? nX : nE) <= w_to && b_w * (b_w < 0.f ? nX : nE) >= w_from;
-                        }
-                        if (keep) {
-                            const bool out = a_u > 0.f || b_u < 0.f;
-                            const float r_a = a_u != 0.f ? rcp_approx(a_u) : -f_inf();
-                            const float r_b = b_u != 0.f ? rcp_approx(b_u) : f_inf();
-                            const float f1 = b_u < 0.f ? r_a : r_b, f2 = a_u > 0.f ? r_b : r_a;
-                            rec[2 * lane] = make_float4(out ? (a_u > 0.f ? r_a : r_b) : 0.f, out ? 0.f : f_inf(), f1, f2);
-                            // rows may run down the w axis: the smaller row number comes from b then
-                            rec[2 * lane + 1] = make_float4(nE, nX, (inv_row >= 0.f ? a_w : b_w) * inv_row,
-                                                            (inv_row >= 0.f ? b_w : a_w) * inv_row);
-                        }
+                for (int base = 0; base < (fits ? 1 : count); base += 32) {
+                    unsigned todo;
+                    if (fits) {
+                        todo = bit_run(0, n_rec);
+                    } else {
+                        todo = pass_records(R, sbox, n_smem, spill, count, gbox, qu, qn, qw, cp, row0, rec, n_boxes,
+                                            base);
+                        __syncwarp();   // the records are written
                     }
-                    unsigned todo = __ballot_sync(kFull, keep);
-                    __syncwarp();   // the records are written
                     bool done = false;
                     while (todo) {
                         const int j = __ffs(todo) - 1;
@@ -815,7 +902,8 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const floa
                                 const int m = __ffs(ask) - 1;
                                 ask &= ask - 1;
                                 float4 lo, hi;
-                                load_box(sbox, n_smem, spill, gbox, base + j, n_boxes, R.stats, lo, hi);
+                                load_box(sbox, n_smem, spill, gbox, fits ? rec_id[j] : base + j, n_boxes, R.stats, lo,
+                                         hi);
                                 const unsigned h = row_hit(qu, qn, qw, pu, R.p_n, w_row[m * G], lo, hi, is3d);
                                 hit |= (h & 1u) << m;
                                 rechecks += h >> 1;
@@ -827,7 +915,7 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const floa
                             break;
                         }
                     }
-                    __syncwarp();   // the records are read before the next are written
+                    __syncwarp();   // the records are read before others are written
                     if (done)
                         break;
                 }
@@ -835,7 +923,6 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const floa
             }
             if (strict)
                 strict_fail |= __any_sync(kFull, alive != valid);
-            const int rows = min((R.nw - row0 + G - 1) / G, 32);   // rows of the pass, per lane
             if (want_bits) {
                 // The blocked bits.  Row m of the pass is one run of patches
                 // over the lanes, from patch j0, so a ballot is its bits and
@@ -866,40 +953,43 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const floa
             const float col_d2 = fmaf(ru, ru, rn * rn);
             // measure x |r| cos(theta); a two-sided target is measured from either side
             const float m_s = R.measure * ((EXTRA && (R.flags & VCM_TWO_SIDED)) ? fabsf(rn) : R.sn * rn);
-            // |r|^2 = (ru^2 + rn^2) of the column + rw^2 of the row.  A closed
-            // row adds +0, which changes nothing (the terms are >= 0), so the
-            // rows take no branch.
-            auto term_of = [&](int m) {
-                bool counts = (open >> m) & 1u;
-                const float rw = counts ? qw - w_row[m * G] : 0.f;
-                const float d2 = fmaf(rw, rw, col_d2);
-                float term;
-                if (is3d) {
-                    const float ir = rsqrt_normal(d2);
-                    term = m_s * (ir * ir * ir);   // A |r| cos(theta) / |r|^3
-                } else {
-                    term = m_s / d2;               // len |r| cos(theta) / |r|^2
-                }
-                if (EXTRA && R.cone)
-                    counts = counts && in_cone(R, ru, rn, rw);   // is q in this patch's field of view?
-                return counts ? term : 0.f;
-            };
-            for (int m0 = 0; m0 < rows; m0 += 8) {
-                if (!__any_sync(kFull, (open >> m0) & 0xffu))
-                    continue;
-                float part = 0.f;
-                // an add the compiler cannot fuse with the term's product
-                if (m0 + 8 <= rows) {
-#pragma unroll
-                    for (int m = 0; m < 8; ++m)
-                        part = __fadd_rn(part, term_of(m0 + m));
-                } else {
-                    for (int m = m0; m < rows; ++m)
-                        part = __fadd_rn(part, term_of(m));
-                }
+            // Eight rows' terms in row order.  A closed row adds +0, which
+            // changes nothing (the terms are >= 0), so the rows take no
+            // branch; the add must not fuse with the term's product.
+            auto close_group = [&](float part) {
                 const float tsum = sum + part;
                 comp += fabsf(sum) >= fabsf(part) ? (sum - tsum) + part : (part - tsum) + sum;
                 sum = tsum;
+            };
+            if (is3d) {
+                for (int m0 = 0; m0 < rows; m0 += 8) {
+                    const unsigned o8 = open >> m0;
+                    if (!__any_sync(kFull, o8 & 0xffu))
+                        continue;
+                    float part = 0.f;
+                    if (M.s_row && m0 + 8 <= rows) {
+                        const float4 *s4 = reinterpret_cast<const float4 *>(M.s_row + r_at + m0);
+                        const float4 wa = s4[0], wb = s4[1];
+                        const float w8[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+                        float t8[8];
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            t8[k] = measure_term<EXTRA, true>(R, col_d2, m_s, ru, rn, qw - w8[k]);
+#pragma unroll
+                        for (int k = 0; k < 8; ++k)
+                            part = __fadd_rn(part, (o8 & (1u << k)) ? t8[k] : 0.f);
+                    } else {
+                        for (int m = m0; m < min(m0 + 8, rows); ++m) {
+                            const bool counts = (open >> m) & 1u;
+                            const float w = M.s_row ? M.s_row[r_at + m] : counts ? w_row[m * G] : 0.f;
+                            const float t = measure_term<EXTRA, true>(R, col_d2, m_s, ru, rn, qw - w);
+                            part = __fadd_rn(part, counts ? t : 0.f);
+                        }
+                    }
+                    close_group(part);
+                }
+            } else {   // one row
+                close_group(open & 1u ? measure_term<EXTRA, false>(R, col_d2, m_s, ru, rn, 0.f) : 0.f);
             }
         }
     }
@@ -1010,6 +1100,8 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
     __shared__ DevRequest s_req;
     __shared__ int s_next;
     __shared__ float4 s_rec[kWarps][2 * 32];    // the sweeps' box records
+    __shared__ int s_rec_id[kWarps][32];
+    __shared__ __align__(16) float s_row[kRowCap];   // the request's rows, row groups apart
     __shared__ int s_req_idx;
     __shared__ int s_next2;                     // cursor of the undecided list
     __shared__ int s_und[kMaxTileViewpoints];   // viewpoints left by the one-box check
@@ -1504,12 +1596,19 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
             cp_async16(&s_box[2 * i], src);
             cp_async16(&s_box[2 * i + 1], src + 1);
         }
+        // the request's rows, for the measure: lane group g's rows side by side
+        const int row_stride = R.groups * ((R.rows + 3) / 4 * 4) <= kRowCap ? (R.rows + 3) / 4 * 4 : 0;
+        for (int i = tid; i < R.nw && row_stride > 0; i += kThreads) {
+            const int m = i / R.groups;
+            s_row[(i - m * R.groups) * row_stride + m] = R.w_coord[i];
+        }
         cp_async_wait_all();
         __syncthreads();
 
         // sweep: warps take the tile's viewpoints one at a time
-        unsigned long long tests = 0, corner_tests = 0;
-        unsigned rechecks = 0, shortcuts = 0;
+        unsigned long long tests = 0;     // of the warp's sweeps: a box and the 32 columns of its lanes
+        unsigned long long corners = 0;   // of the warp's sweeps
+        unsigned corner_tests = 0, rechecks = 0, shortcuts = 0;
         float vmax = 0.f;
 
         // Whole-tile check.  For a fixed patch, the viewpoints whose segment
@@ -1675,6 +1774,12 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
             }
         }
         // then the undecided viewpoints, one per warp at a time
+        LaneMap M;
+        M.g = lane / R.nuc;
+        M.c_in = M.g < R.groups ? lane - M.g * R.nuc : R.nu;   // lanes past the last group own no column
+        M.g = min(M.g, R.groups - 1);
+        M.rows = (R.nw - M.g + R.groups - 1) / R.groups;
+        M.s_row = row_stride > 0 ? s_row + M.g * row_stride : nullptr;
         for (;;) {
             int k = 0;
             if (lane == 0)
@@ -1691,25 +1796,21 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                 const float qn = R.an == 0 ? qx : (R.an == 1 ? qy : zq);
                 const float qw = R.dims == 3 ? (R.aw == 0 ? qx : (R.aw == 1 ? qy : zq)) : 0.f;
                 const bool front = facing(R, qn);
-                if (n_smem > 8) {
-                    const int nb_short = min(n_smem, 32);
-                    if (lane < nb_short)
-                        corner_tests += 4;
-                    if (one_box_blocks_all(R, s_box, nb_short, qu, qn, qw)) {
-                        if (lane == 0) {
-                            put_v(R, vp, 0.f);
-                            ++shortcuts;
-                        }
-                        if (want_bits)
-                            for (int wd = lane; wd < R.words; wd += 32) {
-                                const int rem = R.P - 32 * wd;
-                                put_word(R, vp * R.words + wd, rem >= 32 ? 0xffffffffu : ((1u << rem) - 1u));
-                            }
-                        continue;
+                float v = sweep_viewpoint<EXTRA>(R, M, s_box, n_smem, list_tail, count, gbox, qu, qn, qw, front, vp,
+                                                 s_rec[warp], s_rec_id[warp], tests, corners, rechecks,
+                                                 sc.n_boxes);
+                if (v < 0.f) {   // one box blocks every patch
+                    if (lane == 0) {
+                        put_v(R, vp, 0.f);
+                        ++shortcuts;
                     }
+                    if (want_bits)
+                        for (int wd = lane; wd < R.words; wd += 32) {
+                            const int rem = R.P - 32 * wd;
+                            put_word(R, vp * R.words + wd, rem >= 32 ? 0xffffffffu : ((1u << rem) - 1u));
+                        }
+                    continue;
                 }
-                float v = sweep_viewpoint<EXTRA>(R, s_box, n_smem, list_tail, count, gbox, qu, qn, qw, front, vp,
-                                                 s_rec[warp], tests, rechecks, sc.n_boxes);
                 if (!front)
                     v = 0.f;
                 if (lane == 0)
@@ -1718,25 +1819,29 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
             }
         }
         // per-tile counters
-        for (int off = 16; off > 0; off >>= 1) {
-            tests += __shfl_xor_sync(kFull, tests, off);
-            corner_tests += __shfl_xor_sync(kFull, corner_tests, off);
-            shortcuts += __shfl_xor_sync(kFull, shortcuts, off);
-            vmax = fmaxf(vmax, __shfl_xor_sync(kFull, vmax, off));
+        corner_tests = __reduce_add_sync(kFull, corner_tests);
+        shortcuts = __reduce_add_sync(kFull, shortcuts);
+        rechecks = __reduce_add_sync(kFull, rechecks);
+        if (viewer) {   // the lanes' own cells
+            for (int off = 16; off > 0; off >>= 1)
+                tests += __shfl_xor_sync(kFull, tests, off);
+        } else {
+            tests *= 32;
         }
+        corners += corner_tests;
+        const unsigned vmax_bits = __reduce_max_sync(kFull, __float_as_uint(vmax));   // v >= 0
         if (lane == 0) {
-            atomicMax(&R.stats->vmax_bits, __float_as_uint(vmax));
+            if (vmax_bits)
+                atomicMax(&R.stats->vmax_bits, vmax_bits);
             if (tests)
                 atomicAdd(&R.stats->slab_tests, tests);
-            if (corner_tests)
-                atomicAdd(&R.stats->corner_tests, corner_tests);
+            if (corners)
+                atomicAdd(&R.stats->corner_tests, corners);
             if (shortcuts)
                 atomicAdd(&R.stats->shortcut_viewpoints, (unsigned long long)shortcuts);
+            if (rechecks)
+                atomicAdd(&R.stats->rechecked, (unsigned long long)rechecks);
         }
-        for (int off = 16; off > 0; off >>= 1)
-            rechecks += __shfl_xor_sync(kFull, rechecks, off);
-        if (lane == 0 && rechecks)
-            atomicAdd(&R.stats->rechecked, (unsigned long long)rechecks);
         if (tid == 0) {
             if (!CHUNKS)
                 atomicAdd(&R.stats->boxes_listed, (unsigned long long)count);
