@@ -235,7 +235,7 @@ typedef struct {
  * (VCM_CACHE_BITS), and the scratch of the scheduler's execution slots.
  * A slot's scratch is a descriptor buffer, a spill list of n_boxes ints per
  * block that can be resident (about 365 MB per slot for 100,000 boxes on
- * 152 SMs) and a 74 MB work buffer through which the blocks of a launch
+ * 152 SMs) and a 71 MB work buffer through which the blocks of a launch
  * share the open viewpoints of expensive tiles; it is allocated when the
  * slot first runs a launch that needs it and kept.  The direct path
  * (vcm_compute, vcm_compute_batch, vcm_recolor) has scratch of its own,

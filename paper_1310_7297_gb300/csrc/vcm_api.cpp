@@ -971,7 +971,7 @@ vcm_status record_launch(vcm_ctx *ctx, Slot &s, const Prepared &P, vcm_stats *st
     if (timed && ctx->ev_before)
         CUDA_TRY(cudaEventRecord(ctx->ev_before, stream));
     CUDA_TRY(launch_tiles(ctx->scene, d_reqs, d_tiles, (int)P.n, P.L.total_tiles, s.d_work, s.d_spill,
-                          P.blocks, P.box_cap, P.extra, P.tile_check, stream, one_tile, s.d_spill_busy,
+                          P.blocks, P.box_cap, P.extra, P.tile_check, ctx->sm_count, stream, one_tile, s.d_spill_busy,
                           /*share=*/true, claim_rounds));
     if (timed && ctx->ev_after)
         CUDA_TRY(cudaEventRecord(ctx->ev_after, stream));
@@ -2647,7 +2647,7 @@ vcm_status vcm_compute_static(const float *lo, const float *hi, uint32_t n_boxes
         const int blocks = std::max(1, std::min(lay.total_tiles, tiles_blocks_per_sm((int)t.box_cap) * sm_count));
         CUDA_TRY(launch_prologue(d_reqs, 1, s_work, sm));
         CUDA_TRY(launch_tiles(sc, d_reqs, d_tiles, 1, lay.total_tiles, s_work, s_spill, blocks, (int)t.box_cap,
-                              needs_extra(c), c.P >= kTileCheckMinPatches, sm));
+                              needs_extra(c), c.P >= kTileCheckMinPatches, sm_count, sm));
         CUDA_TRY(launch_quantise(d_reqs, d_vps, 1, lay.total_vp, sm));
         return VCM_OK;
     } catch (const std::exception &ex) {

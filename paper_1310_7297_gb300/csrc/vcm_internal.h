@@ -21,30 +21,29 @@ constexpr int kTileCheckMinPatches = 512;
 constexpr int kMaxPlanes = 32;            // separating planes kept per tile hull
 constexpr float kBand = 1e-6f;            // FP32 slab margin re-decided in FP64
 constexpr int kMaxBoxCap = 5000;          // candidate boxes a tile stages in shared memory
-constexpr int kRowCap = 512;              // patch rows staged in shared memory for the measure
+constexpr int kRowCap = 256;              // patch rows a warp stages for the measure
+constexpr int kWarpBoxes = 64;            // boxes of a chunk's list a warp stages
+constexpr int kSweepBlocks = 7;           // blocks per SM of the second pass
+constexpr int kPartsPerWarp = 4;          // parts of chunks the second pass wants per warp
 constexpr int kMaxTileViewpoints = 1024;  // viewpoints in one tile (tile_x * tile_y)
 constexpr int kClaimRounds = 4096;        // bounded retries of a spill-region claim (2 us pauses)
 
 // Work sharing of the persistent tile kernel, in two passes.  In the first,
 // a tile whose one-box check leaves at least its request's min_publish
-// viewpoints open, and whose candidate list is staged whole and holds at
-// most kPublishBoxes boxes, publishes them, chunk_vp at a time, as chunks;
-// the second pass (a second launch of the same kernel) sweeps the chunks,
-// each staging its owner's list again.
+// viewpoints open publishes them, chunk_vp at a time, as chunks (a list
+// longer than kPublishBoxes only from kPublishHeavy viewpoints); in the
+// second, k_sweep's warps sweep parts of the chunks.
 // The work buffer of a launch holds kWorkHeader counters (next tile,
-// records, chunks published, chunks taken, id-pool ints used) and then the
+// records, chunks published, parts taken, id-pool ints used) and then the
 // arena:
-//   chunk[kChunkCap][2 + kChunkVp]   record index, count, viewpoints (tile-local)
-//   record[kRecCap][kRecInts]        queue item, candidate count, offset of its ids in the pool
+//   chunk[kChunkCap][kChunkInts]     record index, count, viewpoints (x + 256 y in the tile, 16 bits each)
+//   record[kRecCap][kRecInts]        request, candidate count, offset of its ids in the pool, layer, tile origin
 //   pool[kPoolInts]                  the records' candidate box ids, in the owner's order
 //   blocker[kBlockerCap]             per tile position of each request (whole-tile-check
 //                                    launches): a box id that blocked a tile there, or -1
 // A tile whose publication would pass a cap keeps its viewpoints.
-// 32 viewpoints per chunk: a block's 4 warps wait at the chunk's end for the
-// slowest viewpoint, and more viewpoints per chunk spread that wait
-// (100,000-box step 3.50 -> 3.38 ms against 16; 64: 3.44, and the 5,000-box
-// step +7 %; 8: +5 %).
 constexpr int kChunkVp = 32;
+constexpr int kChunkInts = 2 + kChunkVp / 2;
 constexpr int kMinPublish = 8;
 // Longer lists stay with their tile (the 100,000-box scene, lists of ~180
 // boxes on average: 6.44 ms with this limit, 6.71 ms without it) unless the
@@ -53,14 +52,14 @@ constexpr int kMinPublish = 8;
 // had set the end of the tile pass).
 constexpr int kPublishBoxes = 128;
 constexpr int kPublishHeavy = 32;
-constexpr int kChunkCap = 262144;
-constexpr int kRecCap = 65536;
-constexpr int kRecInts = 3;
+constexpr int kChunkCap = 393216;
+constexpr int kRecCap = 131072;
+constexpr int kRecInts = 8;
 constexpr int kPoolInts = 8 << 20;
 constexpr int kBlockerCap = 1 << 20;
 constexpr int kWorkHeader = 64;   // ints before the arena (256 bytes)
 constexpr size_t kChunkOff = 0;
-constexpr size_t kRecOff = kChunkOff + (size_t)kChunkCap * (2 + kChunkVp);
+constexpr size_t kRecOff = kChunkOff + (size_t)kChunkCap * kChunkInts;
 constexpr size_t kPoolOff = kRecOff + (size_t)kRecCap * kRecInts;
 constexpr size_t kBlockerOff = kPoolOff + (size_t)kPoolInts;
 constexpr size_t kArenaInts = kBlockerOff + (size_t)kBlockerCap;
@@ -141,15 +140,16 @@ cudaError_t launch_grid_build(const float *d_lo_world, const float *d_hi_world, 
 // `tile_check` selects the instantiation with the whole-tile check (any
 // launch may use either; it pays when every request has many patches).
 // `share` (persistent launches only): d_work is kWorkBytes long, and a second
-// launch of the kernel works the open viewpoints that expensive tiles of the
-// first published there.
+// kernel on all sm_count SMs works the open viewpoints that expensive tiles of
+// the first published there.
 // `claim_rounds` (1..kClaimRounds) bounds the retries of a one-tile block's
 // spill-region claim; a block that gives up runs without a region and sets
 // its request's vcm_stats.error to VCM_DEVERR_SPILL_WAIT if its candidate
 // list needs one.
 cudaError_t launch_tiles(const DevScene &sc, const DevRequest *d_reqs, const int *d_tile_prefix,
                          int n_req, int total_tiles, int *d_work, int *d_spill, int grid_blocks,
-                         int box_cap, bool extra, bool tile_check, cudaStream_t stream, bool one_tile = false,
+                         int box_cap, bool extra, bool tile_check, int sm_count, cudaStream_t stream,
+                         bool one_tile = false,
                          int *d_spill_busy = nullptr, bool share = false, int claim_rounds = kClaimRounds);
 // Colors and edge counts for all viewpoints of n_req requests (grid over the
 // concatenated viewpoints, `d_vp_prefix` = exclusive prefix, n_req + 1).

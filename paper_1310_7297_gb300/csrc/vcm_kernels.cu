@@ -408,7 +408,6 @@ struct TileSmem {
     int item;
     int pad;
     int n_und;
-    int helper;   // chunk this block took (-1: a tile from the queue)
     int pub[4];   // record, first chunk, chunks published, offset of the ids in the pool
 };
 
@@ -754,11 +753,40 @@ __device__ __noinline__ unsigned pass_records(const DevRequest &R, const float4 
     return __ballot_sync(kFull, keep);
 }
 
-// A warp's lane mapping and the staged rows of a tile's request.
+// Where a lane stands in a request's patch grid, in one register: bits 0-12 its
+// column of a pass (nu for the lanes past the last row group, which own none),
+// 13-17 its row group, 18-30 that group's rows.
 struct LaneMap {
-    int c_in, g;     // the lane's column of a pass, and its row group
-    int rows;        // rows of its group (0 for the lanes past the last group)
-    const float *s_row;   // its rows in shared memory, in order; null if they do not fit
+    unsigned bits;
+    __device__ __forceinline__ int c_in() const { return (int)(bits & 0x1fffu); }
+    __device__ __forceinline__ int g() const { return (int)((bits >> 13) & 31u); }
+    __device__ __forceinline__ int rows() const { return (int)(bits >> 18); }
+};
+__device__ __forceinline__ LaneMap lane_map(const DevRequest &R)
+{
+    const int lane = threadIdx.x & 31;
+    int g = lane / R.nuc;
+    const int c_in = g < R.groups ? lane - g * R.nuc : R.nu;
+    g = min(g, R.groups - 1);
+    return LaneMap{(unsigned)c_in | ((unsigned)g << 13) | ((unsigned)((R.nw - g + R.groups - 1) / R.groups) << 18)};
+}
+// Row groups are this far apart in a warp's staged rows; 0: they do not fit.
+__device__ __forceinline__ int row_stride(const DevRequest &R)
+{
+    const int stride = (R.rows + 3) & ~3;
+    return R.groups * stride <= kRowCap ? stride : 0;
+}
+// staged rows: row i = m * G + g at g * stride + m (a float division is exact for these sizes)
+__device__ __forceinline__ int row_slot(int i, int G, int stride)
+{
+    const int m = G == 1 ? i : (int)(((float)i + 0.5f) / (float)G);
+    return (i - m * G) * stride + m;
+}
+// Shared memory of one warp's sweeps.
+struct WarpScratch {
+    float4 rec[2 * 32];   // records of the boxes left to a viewpoint
+    float rw[kRowCap];    // its row offsets q_w - w, each lane group's rows side by side
+    int rec_id[32];       // the records' boxes
 };
 
 // One open patch's term of the visible measure.  |r|^2 is (ru^2 + rn^2) of the
@@ -786,11 +814,13 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
                                                  const float4 *__restrict__ sbox, int n_smem,
                                                  const int *__restrict__ spill, int count,
                                                  const float4 *__restrict__ gbox, float qu, float qn,
-                                                 float qw, bool front, long long vp, float4 *rec, int *rec_id,
-                                                 unsigned long long &tests, unsigned long long &corners,
-                                                 unsigned &rechecks, int n_boxes)
+                                                 float qw, bool front, long long vp, WarpScratch &W,
+                                                 unsigned &tests, unsigned &corners, unsigned &rechecks,
+                                                 int n_boxes)
 {
     constexpr float kMagic = 12582912.f;   // 1.5 x 2^23: adding it rounds to an integer
+    float4 *rec = W.rec;
+    bool rows_staged = false;
     const int lane = threadIdx.x & 31;
     const int nuc = R.nuc, G = R.groups;
     const float dn = R.p_n - qn;
@@ -828,7 +858,7 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
             if (keep && at < 32) {
                 rec[2 * at] = r0;
                 rec[2 * at + 1] = r1;
-                rec_id[at] = base + lane;
+                W.rec_id[at] = base + lane;
             }
             n_rec += __popc(kept);
         }
@@ -841,7 +871,7 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
     }
 
     for (int cp = 0; cp < R.col_passes && !(strict_exit && strict_fail); ++cp) {
-        const int iu = cp * nuc + M.c_in;
+        const int iu = cp * nuc + M.c_in();
         const bool col_ok = iu < R.nu;
         const float pu = R.u_coord[col_ok ? iu : 0];
         const float du = pu - qu;
@@ -852,9 +882,9 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
         for (int r_at = 0; r_at < R.rows && !(strict_exit && strict_fail); r_at += 32) {
             const int row0 = r_at * G;                          // the pass's first row
             const int rows = min(R.rows - r_at, 32);            // its rows per lane
-            const int mine = col_ok ? min(M.rows - r_at, 32) : 0;
+            const int mine = col_ok ? min(M.rows() - r_at, 32) : 0;
             const unsigned valid = bit_run(0, max(mine, 0));
-            const float *__restrict__ w_row = R.w_coord + row0 + M.g;   // row m: w_row[m * G]
+            const float *__restrict__ w_row = R.w_coord + row0 + M.g();   // row m: w_row[m * G]
             unsigned alive = valid;
             if (n_rec > 0) {
                 const float c = -((mine > 0 ? w_row[0] : R.w_min) - qw) * inv_row;
@@ -862,7 +892,6 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
                 const bool coarse = !(eps < 0.25f);
                 const float near_half = 0.5f - eps;
                 const bool fits = n_rec <= 32;
-                int nb = 0;
                 for (int base = 0; base < (fits ? 1 : count); base += 32) {
                     unsigned todo;
                     if (fits) {
@@ -879,7 +908,7 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
                         const float4 ru = rec[2 * j], rw = rec[2 * j + 1];
                         const float iE = fminf(fmaf(du, ru.x, ru.y), rw.x);
                         const float iX = fmaxf(fmaxf(du * ru.z, du * ru.w), rw.y);
-                        ++nb;
+                        ++tests;
                         if (alive != 0u && iE >= iX * kLess) {
                             unsigned hit = 0u, ask = 0u;   // rows blocked for certain, rows to decide one by one
                             // first row + 1/2 and last row - 1/2 of the interval
@@ -902,7 +931,7 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
                                 const int m = __ffs(ask) - 1;
                                 ask &= ask - 1;
                                 float4 lo, hi;
-                                load_box(sbox, n_smem, spill, gbox, fits ? rec_id[j] : base + j, n_boxes, R.stats, lo,
+                                load_box(sbox, n_smem, spill, gbox, fits ? W.rec_id[j] : base + j, n_boxes, R.stats, lo,
                                          hi);
                                 const unsigned h = row_hit(qu, qn, qw, pu, R.p_n, w_row[m * G], lo, hi, is3d);
                                 hit |= (h & 1u) << m;
@@ -919,7 +948,6 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
                     if (done)
                         break;
                 }
-                tests += (unsigned long long)nb;
             }
             if (strict)
                 strict_fail |= __any_sync(kFull, alive != valid);
@@ -955,41 +983,59 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
             const float m_s = R.measure * ((EXTRA && (R.flags & VCM_TWO_SIDED)) ? fabsf(rn) : R.sn * rn);
             // Eight rows' terms in row order.  A closed row adds +0, which
             // changes nothing (the terms are >= 0), so the rows take no
-            // branch; the add must not fuse with the term's product.
+            // branch; the add must not fuse with the term's product.  The
+            // group total joins by a two-sum of the larger and the smaller
+            // (both are >= 0).
             auto close_group = [&](float part) {
                 const float tsum = sum + part;
-                comp += fabsf(sum) >= fabsf(part) ? (sum - tsum) + part : (part - tsum) + sum;
+                comp += (fmaxf(sum, part) - tsum) + fminf(sum, part);
                 sum = tsum;
             };
-            if (is3d) {
-                for (int m0 = 0; m0 < rows; m0 += 8) {
-                    const unsigned o8 = open >> m0;
-                    if (!__any_sync(kFull, o8 & 0xffu))
-                        continue;
-                    float part = 0.f;
-                    if (M.s_row && m0 + 8 <= rows) {
-                        const float4 *s4 = reinterpret_cast<const float4 *>(M.s_row + r_at + m0);
-                        const float4 wa = s4[0], wb = s4[1];
-                        const float w8[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
-                        float t8[8];
+            if (!is3d) {   // one row
+                close_group(open & 1u ? measure_term<EXTRA, false>(R, col_d2, m_s, ru, rn, 0.f) : 0.f);
+                continue;
+            }
+            const int stride = row_stride(R);
+            if (!rows_staged && stride > 0) {
+                rows_staged = true;
+                __syncwarp();   // the viewpoint before this one is done with them
+                for (int i = lane; i < R.nw; i += 32)
+                    W.rw[row_slot(i, G, stride)] = qw - R.w_coord[i];
+                __syncwarp();
+            }
+            const float *my_rw = W.rw + M.g() * stride + r_at;
+            for (int m0 = 0; m0 < rows; m0 += 8) {
+                const unsigned o8 = open >> m0;
+                const unsigned any = __ballot_sync(kFull, (o8 & 0xffu) != 0u);
+                if (any == 0u)
+                    continue;
+                float part = 0.f;
+                if (stride > 0 && m0 + 8 <= rows) {
+                    const float4 *s4 = reinterpret_cast<const float4 *>(my_rw + m0);
+                    const float4 wa = s4[0], wb = s4[1];
+                    const float w8[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
+                    float t8[8];
+#pragma unroll
+                    for (int k = 0; k < 8; ++k)
+                        t8[k] = measure_term<EXTRA, true>(R, col_d2, m_s, ru, rn, w8[k]);
+                    if (__all_sync(kFull, (o8 & 0xffu) == 0xffu)) {   // mostly
 #pragma unroll
                         for (int k = 0; k < 8; ++k)
-                            t8[k] = measure_term<EXTRA, true>(R, col_d2, m_s, ru, rn, qw - w8[k]);
+                            part = __fadd_rn(part, t8[k]);
+                    } else {
 #pragma unroll
                         for (int k = 0; k < 8; ++k)
                             part = __fadd_rn(part, (o8 & (1u << k)) ? t8[k] : 0.f);
-                    } else {
-                        for (int m = m0; m < min(m0 + 8, rows); ++m) {
-                            const bool counts = (open >> m) & 1u;
-                            const float w = M.s_row ? M.s_row[r_at + m] : counts ? w_row[m * G] : 0.f;
-                            const float t = measure_term<EXTRA, true>(R, col_d2, m_s, ru, rn, qw - w);
-                            part = __fadd_rn(part, counts ? t : 0.f);
-                        }
                     }
-                    close_group(part);
+                } else {
+                    for (int m = m0; m < min(m0 + 8, rows); ++m) {
+                        const bool counts = (open >> m) & 1u;
+                        const float rw = stride > 0 ? my_rw[m] : counts ? qw - w_row[m * G] : 0.f;
+                        const float t = measure_term<EXTRA, true>(R, col_d2, m_s, ru, rn, rw);
+                        part = __fadd_rn(part, counts ? t : 0.f);
+                    }
                 }
-            } else {   // one row
-                close_group(open & 1u ? measure_term<EXTRA, false>(R, col_d2, m_s, ru, rn, 0.f) : 0.f);
+                close_group(part);
             }
         }
     }
@@ -1075,19 +1121,10 @@ __device__ __forceinline__ void add_candidate(const float4 *__restrict__ world, 
 // 100,000-box scene with 64 x 32 patches: -10 %); in the other instantiation
 // its code alone cost a few % on smaller requests.
 //
-// CHUNKS: the second pass's instantiation, which takes the published chunks
-// and holds none of the tile pass's code (the cull, the sort, the checks and
-// the publication), so its registers and instructions fit the sweep alone.
 //
-// Occupancy: the tile pass runs 6 blocks per SM (80 registers) and the chunk
-// pass 7 (72 registers).  Both spill some registers at these bounds, and
-// still the extra warps hide more latency than the spills cost.  Against 5
-// blocks for both (96 registers, no spills in the common instantiations):
-// 100,000-box step 4.23 -> 3.86 ms, 5,000-box step 0.354 -> 0.333 ms,
-// 256-request batch 91.5 -> 87.9 ms; 7 blocks for the tile pass too made
-// the batch 15 % slower.
-template <bool EXTRA, bool TILE_CHECK, bool CHUNKS>
-__global__ void __launch_bounds__(kThreads, CHUNKS ? 7 : 6)
+// Occupancy: 6 blocks per SM (80 registers); 7 made the batch slower.
+template <bool EXTRA, bool TILE_CHECK>
+__global__ void __launch_bounds__(kThreads, 6)
 k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict__ tile_prefix,
         int n_req, int total_tiles, int *__restrict__ work, int *__restrict__ spill_all, int box_cap,
         int one_tile, int *__restrict__ spill_busy, int spill_slots, int share, int claim_rounds)
@@ -1099,12 +1136,10 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
     __shared__ float s_pts[8][3];
     __shared__ DevRequest s_req;
     __shared__ int s_next;
-    __shared__ float4 s_rec[kWarps][2 * 32];    // the sweeps' box records
-    __shared__ int s_rec_id[kWarps][32];
-    __shared__ __align__(16) float s_row[kRowCap];   // the request's rows, row groups apart
+    __shared__ __align__(16) WarpScratch s_warp[kWarps];   // the sweeps'
     __shared__ int s_req_idx;
     __shared__ int s_next2;                     // cursor of the undecided list
-    __shared__ int s_und[kMaxTileViewpoints];   // viewpoints left by the one-box check
+    __shared__ unsigned short s_und[kMaxTileViewpoints];   // viewpoints left by the one-box check, x + 256 y
     __shared__ int s_rowpre[kThreads], s_rowx[kThreads], s_wsum[kWarps];   // cell-row spans
     __shared__ int s_passb[kPassCap], s_passn[kPassCap], s_passp[kPassCap + 1], s_wsum2[kWarps], s_npass;
     __shared__ int s_hist[kDistClasses];   // counting sort of long candidate lists
@@ -1140,38 +1175,22 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
     }
     __syncthreads();
     const int spill_slot = s_spill_slot;
-    // the chunk pass reads no spill region (and has more blocks than regions)
-    int *spill = CHUNKS ? nullptr : spill_all + (size_t)max(spill_slot, 0) * sc.n_boxes;
+    int *spill = spill_all + (size_t)max(spill_slot, 0) * sc.n_boxes;
 
     for (;;) {
         // thread 0 takes the next tile, copies its request and lays out the
         // hull points (one barrier for all of it).  With one_tile, block b
         // does tile b only and exits, so blocks of concurrent launches
         // interleave (a persistent grid would hold every SM to the end).
-        // The second pass (CHUNKS, share == 2) takes the chunks the first published,
-        // in order, and no tiles.
         if (tid == 0) {
-            int took = -1, it;
-            if (CHUNKS) {
-                const int h = atomicAdd(work + 3, 1);
-                took = h < min(__ldcg(work + 2), kChunkCap) ? h : -1;
-            }
-            if (took >= 0) {
-                const int rec = __ldcg(work + kWorkHeader + kChunkOff + (size_t)(2 + kChunkVp) * took);
-                it = __ldcg(work + kWorkHeader + kRecOff + (size_t)kRecInts * rec);
-            } else if (CHUNKS) {
-                it = total_tiles;
-            } else {
-                it = one_tile ? (sm.item == -2 ? total_tiles : (int)blockIdx.x) : atomicAdd(work, 1);
-                // Queue order: last tile first, and within a request the
-                // layers interleaved (consecutive items are one tile position
-                // in every layer).  Measured on the 3D workload with the
-                // target facing each of +-x and +-y: 3-14 % faster than the
-                // plain order, never slower; either change alone was not.
-                it = it < total_tiles ? total_tiles - 1 - it : total_tiles;
-            }
+            int it = one_tile ? (sm.item == -2 ? total_tiles : (int)blockIdx.x) : atomicAdd(work, 1);
+            // Queue order: last tile first, and within a request the
+            // layers interleaved (consecutive items are one tile position
+            // in every layer).  Measured on the 3D workload with the
+            // target facing each of +-x and +-y: 3-14 % faster than the
+            // plain order, never slower; either change alone was not.
+            it = it < total_tiles ? total_tiles - 1 - it : total_tiles;
             sm.item = it;
-            sm.helper = took;
             if (it < total_tiles) {
                 // request of this tile: last r with tile_prefix[r] <= it
                 int lo_r = 0, hi_r = n_req - 1;
@@ -1232,7 +1251,6 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
         const int item = sm.item;
         if (item >= total_tiles)
             break;
-        const int helper = sm.helper;
         const DevRequest &R = s_req;
         const int t = sm.pad;
         const int per_layer = R.tiles_x * R.tiles_y;
@@ -1262,7 +1280,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
         const bool viewer = (R.flags & VCM_VIEWER) != 0;
         const bool any_front = viewer || (R.flags & VCM_TWO_SIDED) ||
                                (R.sn > 0.f ? (qn_hi - R.p_n > 0.f) : (R.p_n - qn_lo > 0.f));
-        if (!CHUNKS && !any_front && !want_bits) {
+        if (!any_front && !want_bits) {
             for (int i = tid; i < tn; i += kThreads) {
                 const int ix = ix0 + i % tw, iy = iy0 + i / tw;
                 put_v(R, ((long long)layer * R.ny + iy) * R.nx + ix, 0.f);
@@ -1283,7 +1301,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
         // depend on the table.
         bool pre_blocked = false;
         unsigned pre_tests = 0;
-        const bool tile_check = TILE_CHECK && !CHUNKS && !viewer;
+        const bool tile_check = TILE_CHECK && !viewer;
         if (tile_check && R.blk_base >= 0) {
             int *blockers = work + kWorkHeader + kBlockerOff;
             const int tile_pos = ty * R.tiles_x + tx;
@@ -1321,10 +1339,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
         }
 
         const int np = (R.dims == 3) ? 8 : 6;
-        // candidates past the staged ones: the block's spill region for its
-        // own tile, the record's ids in the pool for a chunk
-        const int *list_tail = spill;
-        if (!CHUNKS && !pre_blocked) {
+        if (!pre_blocked) {
             hull_planes(R.dims, s_pts, np, sm);
             __syncthreads();
         }
@@ -1340,7 +1355,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
         // is spanned by the interval's two ends.  Rows are taken 128 at a
         // time: one thread finds a row's span, a block scan lays the spans
         // end to end, and the threads share out the cells.
-        if (!CHUNKS && !pre_blocked) {
+        if (!pre_blocked) {
             float ax0 = s_pts[0][0], ax1 = ax0, ay0 = s_pts[0][1], ay1 = ay0;
             for (int l = 1; l < 4; ++l) {
                 ax0 = fminf(ax0, s_pts[l][0]); ax1 = fmaxf(ax1, s_pts[l][0]);
@@ -1487,23 +1502,6 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                     s_npass = 0;
                 __syncthreads();   // the next rows reuse the span arrays
             }
-        } else if (CHUNKS) {
-            // a chunk: the owner's candidate list, in the owner's order, and
-            // the chunk's viewpoints
-            const int *ch = work + kWorkHeader + kChunkOff + (size_t)(2 + kChunkVp) * helper;
-            const int *rec = work + kWorkHeader + kRecOff + (size_t)kRecInts * __ldcg(ch);
-            const int cnt = __ldcg(rec + 1), n_ch = __ldcg(ch + 1);
-            const int *ids = work + kWorkHeader + kPoolOff + __ldcg(rec + 2);
-            for (int i = tid; i < min(cnt, box_cap); i += kThreads)
-                s_ids[i] = __ldcg(ids + i);
-            list_tail = ids + box_cap;
-            for (int i = tid; i < n_ch; i += kThreads)
-                if (IN_BOUNDS(i, kChunkVp, R.stats))
-                    s_und[i] = __ldcg(ch + 2 + i);
-            if (tid == 0) {
-                sm.count = cnt;
-                sm.n_und = n_ch;
-            }
         }
         __syncthreads();
         // A block without a spill region (its bounded claim gave up) keeps
@@ -1516,7 +1514,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
         // most sightlines, so the all-blocked exits come early.  Keys are the
         // squared footprint distance from the tile centre (a positive float,
         // so its bits order like the value) above the sorted box index.
-        if (!CHUNKS && n_smem > 1) {
+        if (n_smem > 1) {
             const float cx = 0.5f * (R.x_coord[ix0] + R.x_coord[ix1 - 1]);
             const float cy = 0.5f * (R.y_coord[iy0] + R.y_coord[iy1 - 1]);
             auto key_of = [&](int i) {
@@ -1596,12 +1594,6 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
             cp_async16(&s_box[2 * i], src);
             cp_async16(&s_box[2 * i + 1], src + 1);
         }
-        // the request's rows, for the measure: lane group g's rows side by side
-        const int row_stride = R.groups * ((R.rows + 3) / 4 * 4) <= kRowCap ? (R.rows + 3) / 4 * 4 : 0;
-        for (int i = tid; i < R.nw && row_stride > 0; i += kThreads) {
-            const int m = i / R.groups;
-            s_row[(i - m * R.groups) * row_stride + m] = R.w_coord[i];
-        }
         cp_async_wait_all();
         __syncthreads();
 
@@ -1645,13 +1637,13 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
             if (tid == 0)
                 shortcuts += (unsigned)tn;
         }
-        if (!CHUNKS && viewer) {
+        if (viewer) {
             // viewer-centric: threads take cells, one segment each
             for (int vi = tid; vi < tn; vi += kThreads) {
                 const int ry = (int)(((float)vi + 0.5f) * inv_tw), ix = ix0 + vi - ry * tw, iy = iy0 + ry;
                 const long long vp = ((long long)layer * R.ny + iy) * R.nx + ix;
                 bool blocked;
-                const float v = viewer_cell(R, s_box, n_smem, list_tail, count, gbox, R.x_coord[ix], R.y_coord[iy],
+                const float v = viewer_cell(R, s_box, n_smem, spill, count, gbox, R.x_coord[ix], R.y_coord[iy],
                                             R.dims == 3 ? zq : 0.f, blocked, tests, rechecks, sc.n_boxes);
                 put_v(R, vp, v);
                 if (want_bits)
@@ -1664,7 +1656,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
         // is almost always among them); the viewpoints it leaves open are
         // listed and then taken one per warp for the check over the 32
         // nearest and the separable sweep.
-        for (; !CHUNKS && !viewer && !tile_blocked;) {
+        for (; !viewer && !tile_blocked;) {
             int base = 0;
             if (lane == 0)
                 base = atomicAdd(&s_next, 4);
@@ -1677,8 +1669,10 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                 const int vi = base + sub;
                 long long vp = 0;
                 bool active = false, behind = false, full = false;
+                int xy = 0;
                 if (vi < tn) {
                     const int ry = (int)(((float)vi + 0.5f) * inv_tw), ix = ix0 + vi - ry * tw, iy = iy0 + ry;
+                    xy = (ix - ix0) | (ry << 8);
                     vp = ((long long)layer * R.ny + iy) * R.nx + ix;
                     const float qx = R.x_coord[ix], qy = R.y_coord[iy];
                     const float qu = R.au == 0 ? qx : (R.au == 1 ? qy : zq);
@@ -1709,7 +1703,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                 if (active && !decided && bl == 0) {
                     const int at = atomicAdd(&sm.n_und, 1);
                     if (IN_BOUNDS(at, kMaxTileViewpoints, R.stats))
-                        s_und[at] = vi;
+                        s_und[at] = (unsigned short)xy;
                 }
             }
         }
@@ -1726,7 +1720,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
         // again; a spilled list's tail is read from the record), and a tile
         // whose publication would pass a cap of the arena keeps its
         // viewpoints.
-        if (!CHUNKS && share == 1 && spill_slot >= 0 && n_und >= R.min_publish &&
+        if (share == 1 && spill_slot >= 0 && n_und >= R.min_publish &&
             (count <= kPublishBoxes || n_und >= kPublishHeavy)) {
             int *arena = work + kWorkHeader;
             const int cvp = R.chunk_vp;
@@ -1759,27 +1753,26 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                 int *rp = arena + kRecOff + (size_t)kRecInts * rec;
                 int *ids = arena + kPoolOff + off;
                 if (tid == 0) {
-                    rp[0] = item;
+                    rp[0] = s_req_idx;
                     rp[1] = count;
                     rp[2] = off;
+                    rp[3] = layer;
+                    rp[4] = ix0;
+                    rp[5] = iy0;
                 }
                 for (int i = tid; i < count; i += kThreads)
                     ids[i] = i < n_smem ? s_ids[i] : spill[i - n_smem];
-                for (int i = tid; i < pub_n * (2 + kChunkVp); i += kThreads) {
-                    const int j = i / (2 + kChunkVp), r = i - j * (2 + kChunkVp);
+                for (int i = tid; i < pub_n * kChunkInts; i += kThreads) {
+                    const int j = i / kChunkInts, r = i - j * kChunkInts, k = j * cvp + 2 * (r - 2);
                     const int n_j = min(cvp, n_und - j * cvp);
-                    arena[kChunkOff + (size_t)(2 + kChunkVp) * (pub_base + j) + r] =
-                        r == 0 ? rec : r == 1 ? n_j : (r - 2 < n_j ? s_und[j * cvp + r - 2] : -1);
+                    const unsigned a = s_und[min(max(k, 0), kMaxTileViewpoints - 1)];
+                    const unsigned b = s_und[min(max(k + 1, 0), kMaxTileViewpoints - 1)];
+                    arena[kChunkOff + (size_t)kChunkInts * (pub_base + j) + r] = r == 0 ? rec : r == 1 ? n_j : (int)(a | (b << 16));
                 }
             }
         }
         // then the undecided viewpoints, one per warp at a time
-        LaneMap M;
-        M.g = lane / R.nuc;
-        M.c_in = M.g < R.groups ? lane - M.g * R.nuc : R.nu;   // lanes past the last group own no column
-        M.g = min(M.g, R.groups - 1);
-        M.rows = (R.nw - M.g + R.groups - 1) / R.groups;
-        M.s_row = row_stride > 0 ? s_row + M.g * row_stride : nullptr;
+        const LaneMap M = lane_map(R);
         for (;;) {
             int k = 0;
             if (lane == 0)
@@ -1788,17 +1781,18 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
             if (k >= n_und)
                 break;
             {
-                const int vi = s_und[k];
-                const int ry = (int)(((float)vi + 0.5f) * inv_tw), ix = ix0 + vi - ry * tw, iy = iy0 + ry;
+                const int ix = ix0 + (s_und[k] & 255), iy = iy0 + (s_und[k] >> 8);
                 const long long vp = ((long long)layer * R.ny + iy) * R.nx + ix;
                 const float qx = R.x_coord[ix], qy = R.y_coord[iy];
                 const float qu = R.au == 0 ? qx : (R.au == 1 ? qy : zq);
                 const float qn = R.an == 0 ? qx : (R.an == 1 ? qy : zq);
                 const float qw = R.dims == 3 ? (R.aw == 0 ? qx : (R.aw == 1 ? qy : zq)) : 0.f;
                 const bool front = facing(R, qn);
-                float v = sweep_viewpoint<EXTRA>(R, M, s_box, n_smem, list_tail, count, gbox, qu, qn, qw, front, vp,
-                                                 s_rec[warp], s_rec_id[warp], tests, corners, rechecks,
-                                                 sc.n_boxes);
+                unsigned vp_tests = 0, vp_corners = 0;
+                float v = sweep_viewpoint<EXTRA>(R, M, s_box, n_smem, spill, count, gbox, qu, qn, qw, front, vp,
+                                                 s_warp[warp], vp_tests, vp_corners, rechecks, sc.n_boxes);
+                tests += vp_tests;
+                corners += vp_corners;
                 if (v < 0.f) {   // one box blocks every patch
                     if (lane == 0) {
                         put_v(R, vp, 0.f);
@@ -1843,14 +1837,140 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                 atomicAdd(&R.stats->rechecked, (unsigned long long)rechecks);
         }
         if (tid == 0) {
-            if (!CHUNKS)
-                atomicAdd(&R.stats->boxes_listed, (unsigned long long)count);
+            atomicAdd(&R.stats->boxes_listed, (unsigned long long)count);
             sm.item = -2;   // one_tile: the next round exits
         }
         __syncthreads();
     }
     if (one_tile && tid == 0 && spill_slot >= 0)
         atomicExch(&spill_busy[spill_slot], 0);
+}
+
+// The second pass: the chunks that the tile pass published, by warps of their
+// own.  A chunk was a block's work before (its list staged by the block, its
+// warps waiting at its end for the slowest viewpoint); a warp now takes a part
+// of a chunk, stages up to kWarpBoxes of the list for itself and meets no
+// block barrier, so parts are as small as the launch needs: 16 viewpoints when
+// there are many chunks, down to 1 when there are fewer than kPartsPerWarp
+// parts per warp.  What a warp knows of its part lies in shared memory and is
+// read where it is used: the sweep needs the registers (in registers it
+// spilled 200 bytes and issued 10 % more instructions).
+//
+// Bound by instruction issue at 85 % of the issue slots.  Measured against
+// chunks by blocks (both passes): 96 x 83 x 3 viewpoints, two-sided, 45 x 13
+// patches 92 -> 60 us; 64 x 64, 8 x 4 patches 44 -> 36 us; 2D 128 x 128 48 -> 41
+// us; 64 uneven requests 8.92 -> 8.71 ms; 100,000 boxes, 64 x 32 patches 5.38
+// -> 5.20 ms.  7 blocks per SM: 6 were 3 %, 5 13 % slower on the batch, 8 spill.
+template <bool EXTRA>
+__global__ void __launch_bounds__(kThreads, kSweepBlocks)
+k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work)
+{
+    struct Mine {   // one warp's: a single base address, the rest are constant offsets
+        WarpScratch scratch;
+        float4 boxes[2 * kWarpBoxes];
+        DevRequest req;
+        int list[8];   // the record: request, count, offset of the ids, layer, tile origin
+        int xy[kChunkVp];
+    };
+    __shared__ __align__(16) Mine s_mine[kWarps];
+    const int lane = threadIdx.x & 31;
+    Mine &mine = s_mine[threadIdx.x >> 5];
+    WarpScratch &W = mine.scratch;
+    DevRequest &R = mine.req;
+    float4 *boxes = mine.boxes;
+    const int *arena = work + kWorkHeader;
+    const int n_chunks = min(work[2], kChunkCap);
+    const int warps = (int)gridDim.x * kWarps;
+    int part_log = 1;   // parts per chunk
+    while (part_log < 5 && (n_chunks << part_log) < kPartsPerWarp * warps)
+        ++part_log;
+    const int part_vp = kChunkVp >> part_log;
+    const volatile int *list = mine.list;   // read where it is used: registers are scarce in the sweep
+    int cur_rec = -1;
+    if (lane == 0)
+        mine.list[0] = -1;
+    __syncwarp();
+    LaneMap M{};
+    for (;;) {
+        int item = 0;
+        if (lane == 0)
+            item = atomicAdd(work + 3, 1);
+        item = __shfl_sync(kFull, item, 0);
+        if ((item >> part_log) >= n_chunks)
+            break;
+        const int *chunk = arena + kChunkOff + (size_t)kChunkInts * (item >> part_log);
+        const int rec = chunk[0];
+        const int first = (item & ((1 << part_log) - 1)) * part_vp, n = min(chunk[1] - first, part_vp);
+        if (n <= 0)
+            continue;
+        __syncwarp();   // the viewpoints before are done with the item's shared memory
+        if (lane < n)
+            mine.xy[lane] = reinterpret_cast<const unsigned short *>(chunk + 2)[first + lane];
+        if (rec != cur_rec) {
+            cur_rec = rec;
+            const int old_req = list[0];
+            __syncwarp();
+            if (lane < 8)
+                mine.list[lane] = arena[kRecOff + (size_t)kRecInts * rec + lane];
+            __syncwarp();
+            if (list[0] != old_req) {
+                const int *src = reinterpret_cast<const int *>(reqs + list[0]);
+                for (int i = lane; i < (int)(sizeof(DevRequest) / sizeof(int)); i += 32)
+                    reinterpret_cast<int *>(&R)[i] = src[i];
+                __syncwarp();
+                M = lane_map(R);
+            }
+            const float4 *gbox = sc.boxes[R.perm];
+            for (int i = lane; i < min(list[1], kWarpBoxes); i += 32) {
+                const int id = arena[kPoolOff + list[2] + i];
+                boxes[2 * i] = __ldg(&gbox[2 * id]);
+                boxes[2 * i + 1] = __ldg(&gbox[2 * id + 1]);
+            }
+        }
+        __syncwarp();
+        const bool want_bits = (R.flags & VCM_EMIT_BITS) && R.bits_out;
+        unsigned tests = 0, corners = 0, rechecks = 0, shortcuts = 0;
+        float vmax = 0.f;
+        for (int k = 0; k < n; ++k) {
+            const int at = mine.xy[k];
+            const int ix = list[4] + (at & 255), iy = list[5] + (at >> 8);
+            const long long vp = ((long long)list[3] * R.ny + iy) * R.nx + ix;
+            const float qx = R.x_coord[ix], qy = R.y_coord[iy], zq = R.z_coord[list[3]];
+            const float qu = R.au == 0 ? qx : (R.au == 1 ? qy : zq);
+            const float qn = R.an == 0 ? qx : (R.an == 1 ? qy : zq);
+            const float qw = R.dims == 3 ? (R.aw == 0 ? qx : (R.aw == 1 ? qy : zq)) : 0.f;
+            const bool front = facing(R, qn);
+            const int count = list[1];
+            float v = sweep_viewpoint<EXTRA>(R, M, boxes, kWarpBoxes, arena + kPoolOff + list[2] + kWarpBoxes, count,
+                                             sc.boxes[R.perm], qu, qn, qw, front, vp, W, tests, corners, rechecks,
+                                             sc.n_boxes);
+            if (v < 0.f) {   // one box blocks every patch
+                ++shortcuts;
+                if (want_bits)
+                    for (int wd = lane; wd < R.words; wd += 32) {
+                        const int rem = R.P - 32 * wd;
+                        put_word(R, vp * R.words + wd, rem >= 32 ? 0xffffffffu : ((1u << rem) - 1u));
+                    }
+            }
+            v = front ? fmaxf(v, 0.f) : 0.f;
+            if (lane == 0)
+                put_v(R, vp, v);
+            vmax = fmaxf(vmax, v);
+        }
+        rechecks = __reduce_add_sync(kFull, rechecks);
+        if (lane == 0) {
+            if (vmax > 0.f)
+                atomicMax(&R.stats->vmax_bits, __float_as_uint(vmax));
+            if (tests)
+                atomicAdd(&R.stats->slab_tests, 32ull * tests);
+            if (corners)
+                atomicAdd(&R.stats->corner_tests, (unsigned long long)corners);
+            if (shortcuts)
+                atomicAdd(&R.stats->shortcut_viewpoints, (unsigned long long)shortcuts);
+            if (rechecks)
+                atomicAdd(&R.stats->rechecked, (unsigned long long)rechecks);
+        }
+    }
 }
 
 // Launch prologue: the work counters and every request's counters.
@@ -2112,9 +2232,8 @@ cudaError_t init_device()
             }
     if ((e = cudaMemcpyToSymbol(c_tri, tri, sizeof(tri))) != cudaSuccess)
         return e;
-    const void *kernels[6] = {(const void *)k_tiles<false, false, false>, (const void *)k_tiles<true, false, false>,
-                              (const void *)k_tiles<false, true, false>,  (const void *)k_tiles<true, true, false>,
-                              (const void *)k_tiles<false, false, true>,  (const void *)k_tiles<true, false, true>};
+    const void *kernels[4] = {(const void *)k_tiles<false, false>, (const void *)k_tiles<true, false>,
+                              (const void *)k_tiles<false, true>, (const void *)k_tiles<true, true>};
     for (const void *k : kernels)
         if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)tiles_smem_bytes(kMaxBoxCap))) != cudaSuccess)
@@ -2193,21 +2312,11 @@ cudaError_t launch_grid_build(const float *d_lo_world, const float *d_hi_world, 
     return cudaGetLastError();
 }
 
-// Blocks of the chunk pass that fit on one SM (its launch bounds allow 7).
-static int chunk_blocks_per_sm(int box_cap, bool extra)
-{
-    int n = 0;
-    auto kernel = extra ? k_tiles<true, false, true> : k_tiles<false, false, true>;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kernel, kThreads, tiles_smem_bytes(box_cap)) != cudaSuccess)
-        return 1;
-    return n > 0 ? n : 1;
-}
-
 int tiles_blocks_per_sm(int box_cap)
 {
     // the tile pass's instantiations share their launch bounds (6 blocks of kThreads)
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_tiles<false, false, false>, kThreads,
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_tiles<false, false>, kThreads,
                                                       tiles_smem_bytes(box_cap)) !=
         cudaSuccess)
         return 1;
@@ -2216,7 +2325,7 @@ int tiles_blocks_per_sm(int box_cap)
 
 cudaError_t launch_tiles(const DevScene &sc, const DevRequest *d_reqs, const int *d_tile_prefix,
                          int n_req, int total_tiles, int *d_work, int *d_spill, int grid_blocks,
-                         int box_cap, bool extra, bool tile_check, cudaStream_t stream, bool one_tile,
+                         int box_cap, bool extra, bool tile_check, int sm_count, cudaStream_t stream, bool one_tile,
                          int *d_spill_busy, bool share, int claim_rounds)
 {
     if (claim_rounds < 1 || claim_rounds > kClaimRounds)
@@ -2232,23 +2341,18 @@ cudaError_t launch_tiles(const DevScene &sc, const DevRequest *d_reqs, const int
             return cudaErrorInvalidValue;
         grid_blocks = total_tiles;
     }
-    auto kernel = extra ? (tile_check ? k_tiles<true, true, false> : k_tiles<true, false, false>)
-                        : (tile_check ? k_tiles<false, true, false> : k_tiles<false, false, false>);
-    auto chunks = extra ? k_tiles<true, false, true> : k_tiles<false, false, true>;
+    auto kernel = extra ? (tile_check ? k_tiles<true, true> : k_tiles<true, false>)
+                        : (tile_check ? k_tiles<false, true> : k_tiles<false, false>);
     share = share && !one_tile;
     kernel<<<grid_blocks, kThreads, smem, stream>>>(sc, d_reqs, d_tile_prefix, n_req, total_tiles, d_work, d_spill,
                                                     box_cap, one_tile ? 1 : 0, d_spill_busy, slots, share ? 1 : 0,
                                                     claim_rounds);
     if (share) {
-        // the second pass: the chunks the first published, on a grid scaled
-        // from the tile pass's by the two instantiations' blocks per SM
+        // the second pass, on every SM
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess)
             return e;
-        const int per_tile = tiles_blocks_per_sm(box_cap), per_chunk = chunk_blocks_per_sm(box_cap, extra);
-        const int chunk_grid = std::max(1, (int)((long long)grid_blocks * per_chunk / std::max(per_tile, 1)));
-        chunks<<<chunk_grid, kThreads, smem, stream>>>(sc, d_reqs, d_tile_prefix, n_req, total_tiles, d_work,
-                                                        d_spill, box_cap, 0, d_spill_busy, slots, 2, claim_rounds);
+        (extra ? k_sweep<true> : k_sweep<false>)<<<sm_count * kSweepBlocks, kThreads, 0, stream>>>(sc, d_reqs, d_work);
     }
     return cudaGetLastError();
 }
