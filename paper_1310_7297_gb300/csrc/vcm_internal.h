@@ -18,7 +18,6 @@ constexpr int kDistClasses = 128;            // distance classes of the candidat
 // check (and the recorded-blocker pre-check): from 512, the 5,000-box step
 // with 32 x 16 patches went 0.319 -> 0.305 ms (the bar was 1,024).
 constexpr int kTileCheckMinPatches = 512;
-constexpr int kMaxPlanes = 32;            // separating planes kept per tile hull
 constexpr float kBand = 1e-6f;            // FP32 slab margin re-decided in FP64
 constexpr int kMaxBoxCap = 5000;          // candidate boxes a tile stages in shared memory
 constexpr int kRowCap = 256;              // patch rows a warp stages for the measure

@@ -331,31 +331,59 @@ __global__ void k_cell_bounds(const float4 *__restrict__ boxes, const int *__res
 __device__ __forceinline__ float4 world_box_lo(const DevScene &sc, int s) { return __ldg(&sc.boxes[0][2 * s]); }
 __device__ __forceinline__ float4 world_box_hi(const DevScene &sc, int s) { return __ldg(&sc.boxes[0][2 * s + 1]); }
 
-struct __align__(16) Plane {
-    float x, y, z, c;
+// The union of every segment from a tile's viewpoints A to the target's patch
+// rectangle B, both axis-aligned boxes: conv(A, B), which is the union over t
+// in [0, 1] of the boxes (1 - t) A + t B.  An axis-aligned box [lo, hi] meets it
+// iff some t in [0, 1] satisfies, on each axis,
+//     t (B_hi - A_hi) >= lo - A_hi   and   t (B_lo - A_lo) <= hi - A_lo,
+// six linear bounds on t.  Each is an entry (t >= m e + o) or an exit (t <= m e
+// + o) of the box's edge e by the sign of its slope; the other one gets m = 0
+// and an infinite o, so a test is 12 fused multiply-adds and as many minima,
+// without a branch.  A and B are widened by 0.04 m, more than ten times the
+// rounding of an edge's bound in metres at 16,384 m (about 2^-24 x 16384 x 3),
+// so a box that meets the hull is never dropped.
+//
+// The separating planes of the hull that this replaces took 56 candidate normals
+// per tile and up to 20 plane tests per box, and dropped fewer boxes.  Tile
+// kernels before and after: 512^2 x 5 viewpoints, 5,000 boxes 0.164 -> 0.150 ms
+// (viewer-centric 0.107 -> 0.079 ms); 2,048^2 x 8, 100,000 boxes 5.20 -> 4.63 ms
+// (the tile pass 2.47 -> 1.91 ms); 64 uneven requests 8.72 -> 8.30 ms.
+struct Swept {
+    float m[6][2], o[6][2];   // bound (axis, lo or hi edge): entry, exit
 };
-
-// n . v, the single evaluation used for hull vertices and box corners alike.
-__device__ __forceinline__ float dot3(float nx, float ny, float nz, float x, float y, float z)
+// Slopes below this many metres count as 0: the bound then holds for every t
+// or for none.
+__device__ __forceinline__ void swept_bound(Swept &S, int k, float a, float b, bool upper_edge)
 {
-    return fmaf(nx, x, fmaf(ny, y, nz * z));
+    const float d = b - a;
+    const float inv = fabsf(d) < 1e-3f ? 1e30f : rcp_approx(d);
+    const bool entry = (fabsf(d) < 1e-3f || d > 0.f) != upper_edge;
+    S.m[k][0] = entry ? inv : 0.f;
+    S.o[k][0] = entry ? -a * inv : -f_inf();
+    S.m[k][1] = entry ? 0.f : inv;
+    S.o[k][1] = entry ? f_inf() : -a * inv;
 }
-
-// True if the box [lo, hi] lies strictly outside one of the hull's planes.
-// Each plane's offset was raised by more than twice the worst float32 error
-// of dot3 at these coordinate magnitudes, so a box that meets the hull is
-// never reported outside.
-__device__ __forceinline__ bool outside(const Plane *__restrict__ pl, int np, float4 lo, float4 hi)
+__device__ __forceinline__ Swept make_swept(const float (*A)[2], const float (*B)[2])
 {
-    for (int i = 0; i < np; ++i) {
-        Plane p = pl[i];
-        float x = p.x >= 0.f ? lo.x : hi.x;
-        float y = p.y >= 0.f ? lo.y : hi.y;
-        float z = p.z >= 0.f ? lo.z : hi.z;
-        if (dot3(p.x, p.y, p.z, x, y, z) > p.c)
-            return true;
+    constexpr float kPad = 0.04f;
+    Swept S;
+#pragma unroll
+    for (int ax = 0; ax < 3; ++ax) {
+        swept_bound(S, 2 * ax, A[ax][1] + kPad, B[ax][1] + kPad, false);   // lower edge against the upper sides
+        swept_bound(S, 2 * ax + 1, A[ax][0] - kPad, B[ax][0] - kPad, true);
     }
-    return false;
+    return S;
+}
+__device__ __forceinline__ bool swept_meets(const Swept &S, float4 lo, float4 hi)
+{
+    const float e[6] = {lo.x, hi.x, lo.y, hi.y, lo.z, hi.z};
+    float from = 0.f, to = 1.f;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+        from = fmaxf(from, fmaf(e[k], S.m[k][0], S.o[k][0]));
+        to = fminf(to, fmaf(e[k], S.m[k][1], S.o[k][1]));
+    }
+    return from <= to;
 }
 
 // Exact re-decision of one segment against one box, in float64.  Inputs are
@@ -399,11 +427,7 @@ __device__ __noinline__ bool exact_hit(float qu, float qn, float qw, float pu, f
     return en * xd <= xn * ed;
 }
 
-__constant__ unsigned char c_tri[56][3];
-
 struct TileSmem {
-    Plane planes[kMaxPlanes];
-    int n_planes;
     int count;
     int item;
     int pad;
@@ -419,95 +443,6 @@ __device__ __forceinline__ void cp_async16(void *smem_dst, const void *gmem_src)
 __device__ __forceinline__ void cp_async_wait_all()
 {
     asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;\n" ::: "memory");
-}
-
-// Candidate planes of the hull of points P[0..np): for every point triple
-// (3D) or pair (2D) whose plane leaves all points on one side, the outward
-// normal; of coplanar points only the first triple is kept.  Any normal gives
-// a valid half-space once its offset covers every point (below), so float32
-// is enough to find them.
-__device__ void hull_planes(int dims, const float (*P)[3], int np, TileSmem &sm)
-{
-    const int t = threadIdx.x;
-    float scale = 0.f;
-    for (int a = 1; a < np; ++a)
-        for (int k = 0; k < 3; ++k)
-            scale = fmaxf(scale, fabsf(P[a][k] - P[0][k]));
-    scale = fmaxf(scale, 1.f);
-    const int n_cand = (dims == 3) ? 56 : 15;
-    if (t < n_cand) {
-        int i, j, k = -1;
-        float n[3];
-        if (dims == 3) {
-            i = c_tri[t][0]; j = c_tri[t][1]; k = c_tri[t][2];
-            float e1[3], e2[3];
-            for (int c = 0; c < 3; ++c) {
-                e1[c] = P[j][c] - P[i][c];
-                e2[c] = P[k][c] - P[i][c];
-            }
-            n[0] = e1[1] * e2[2] - e1[2] * e2[1];
-            n[1] = e1[2] * e2[0] - e1[0] * e2[2];
-            n[2] = e1[0] * e2[1] - e1[1] * e2[0];
-        } else {
-            // pairs (i < j) of 6 points in a fixed order
-            int idx = t;
-            i = 0;
-            while (idx >= np - 1 - i) {
-                idx -= np - 1 - i;
-                ++i;
-            }
-            j = i + 1 + idx;
-            n[0] = -(P[j][1] - P[i][1]);
-            n[1] = P[j][0] - P[i][0];
-            n[2] = 0.f;
-        }
-        const float len = sqrtf(n[0] * n[0] + n[1] * n[1] + n[2] * n[2]);
-        const int last = (dims == 3) ? k : j;
-        if (len > 1e-6f * scale * scale) {
-            const float tol = 1e-5f * len * scale;
-            bool pos = false, neg = false, dup = false;
-            for (int l = 0; l < np; ++l) {
-                const float s = n[0] * (P[l][0] - P[i][0]) + n[1] * (P[l][1] - P[i][1]) +
-                                n[2] * (P[l][2] - P[i][2]);
-                if (s > tol)
-                    pos = true;
-                if (s < -tol)
-                    neg = true;
-                if (fabsf(s) <= tol && l < last && l != i && l != j && l != k)
-                    dup = true;
-            }
-            if (!(pos && neg) && !dup) {
-                for (int side = 0; side < 2; ++side) {
-                    // side 0: n outward (all points at s <= 0); side 1: -n outward
-                    if ((side == 0 && pos) || (side == 1 && neg))
-                        continue;
-                    const float sg = side ? -1.f : 1.f;
-                    const float nx = sg * n[0] / len, ny = sg * n[1] / len, nz = sg * n[2] / len;
-                    float c = -f_inf();
-                    for (int l = 0; l < np; ++l)
-                        c = fmaxf(c, dot3(nx, ny, nz, P[l][0], P[l][1], P[l][2]));
-                    c += 0.04f * (fabsf(nx) + fabsf(ny) + fabsf(nz));
-                    const int slot = atomicAdd(&sm.n_planes, 1);
-                    if (slot < kMaxPlanes)
-                        sm.planes[slot] = Plane{nx, ny, nz, c};
-                }
-            }
-        }
-    }
-    // the six (four in 2D) axis planes of the hull's bounding box
-    if (t >= 64 && t < 64 + 2 * dims) {
-        const int ax = (t - 64) >> 1;
-        const bool upper = ((t - 64) & 1) == 0;
-        float m = P[0][ax];
-        for (int l = 1; l < np; ++l)
-            m = upper ? fmaxf(m, P[l][ax]) : fminf(m, P[l][ax]);
-        float n3[3] = {0.f, 0.f, 0.f};
-        n3[ax] = upper ? 1.f : -1.f;
-        const float c = (upper ? m : -m) + 0.04f;
-        const int slot = atomicAdd(&sm.n_planes, 1);
-        if (slot < kMaxPlanes)
-            sm.planes[slot] = Plane{n3[0], n3[1], n3[2], c};
-    }
 }
 
 // True if the box [lo, hi] (target frame) certainly (margin > band) blocks
@@ -1089,13 +1024,13 @@ __device__ __forceinline__ float viewer_cell(const DevRequest &R, const float4 *
 }
 
 
-// Cull one box against the hull planes and, if it may matter, add it to the
-// tile's candidate list (shared memory, then the block's spill region).
-__device__ __forceinline__ void add_candidate(const float4 *__restrict__ world, const Plane *planes, int n_planes,
-                                              int s, TileSmem &sm, int *s_ids, int box_cap, int *spill,
+// If a box may matter to the tile, add it to the tile's candidate list (shared
+// memory, then the block's spill region).
+__device__ __forceinline__ void add_candidate(const float4 *__restrict__ world, const Swept &hull, int s,
+                                              TileSmem &sm, int *s_ids, int box_cap, int *spill,
                                               int spill_slot, const DevRequest &R, int n_boxes)
 {
-    if (outside(planes, n_planes, world[2 * s], world[2 * s + 1]))
+    if (!swept_meets(hull, world[2 * s], world[2 * s + 1]))
         return;
     const int pos = atomicAdd(&sm.count, 1);
     if (pos < box_cap)
@@ -1133,7 +1068,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
     float4 *s_box = reinterpret_cast<float4 *>(smem_raw);
     int *s_ids = reinterpret_cast<int *>(smem_raw + (size_t)box_cap * 32);
     __shared__ TileSmem sm;
-    __shared__ float s_pts[8][3];
+    __shared__ float s_A[3][2], s_B[3][2];   // the tile's viewpoints and the target's patch rectangle: world axis, low and high
     __shared__ DevRequest s_req;
     __shared__ int s_next;
     __shared__ __align__(16) WarpScratch s_warp[kWarps];   // the sweeps'
@@ -1218,33 +1153,20 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                 const int x0 = tx0 * Q.tile_x, x1 = min(Q.nx, x0 + Q.tile_x) - 1;
                 const int y0 = ty0 * Q.tile_y, y1 = min(Q.ny, y0 + Q.tile_y) - 1;
                 const float z = Q.z_coord[ly];
-                sm.n_planes = 0;
                 sm.count = 0;
                 sm.n_und = 0;
                 s_next = 0;
                 s_next2 = 0;
-                const float X[2] = {Q.x_coord[x0], Q.x_coord[x1]};
-                const float Y[2] = {Q.y_coord[y0], Q.y_coord[y1]};
-                for (int c = 0; c < 4; ++c) {
-                    s_pts[c][0] = X[c & 1];
-                    s_pts[c][1] = Y[c >> 1];
-                    s_pts[c][2] = (Q.dims == 3) ? z : 0.f;
-                }
-                if (Q.dims == 3) {
-                    const float U[2] = {Q.u_min, Q.u_max}, W[2] = {Q.w_min, Q.w_max};
-                    for (int c = 0; c < 4; ++c) {
-                        s_pts[4 + c][Q.au] = U[c & 1];
-                        s_pts[4 + c][Q.aw] = W[c >> 1];
-                        s_pts[4 + c][Q.an] = Q.p_n;
-                    }
-                } else {
-                    const float U[2] = {Q.u_min, Q.u_max};
-                    for (int c = 0; c < 2; ++c) {
-                        s_pts[4 + c][Q.au] = U[c];
-                        s_pts[4 + c][Q.an] = Q.p_n;
-                        s_pts[4 + c][2] = 0.f;
-                    }
-                }
+                s_A[0][0] = Q.x_coord[x0];
+                s_A[0][1] = Q.x_coord[x1];
+                s_A[1][0] = Q.y_coord[y0];
+                s_A[1][1] = Q.y_coord[y1];
+                s_A[2][0] = s_A[2][1] = Q.dims == 3 ? z : 0.f;
+                s_B[Q.au][0] = Q.u_min;
+                s_B[Q.au][1] = Q.u_max;
+                s_B[Q.an][0] = s_B[Q.an][1] = Q.p_n;
+                s_B[Q.aw][0] = Q.w_min;   // 0 in 2D
+                s_B[Q.aw][1] = Q.w_max;
             }
         }
         __syncthreads();
@@ -1321,8 +1243,8 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                         const float4 *gb = sc.boxes[R.perm];
                         // the tile's corners from shared memory at each use, so that
                         // they are not held in registers through the cull
-                        const float qx = (corner & 1) ? s_pts[1][0] : s_pts[0][0];
-                        const float qy = (corner & 2) ? s_pts[2][1] : s_pts[0][1];
+                        const float qx = s_A[0][corner & 1];
+                        const float qy = s_A[1][corner >> 1];
                         const float qu = R.au == 0 ? qx : (R.au == 1 ? qy : zq);
                         const float qn = R.an == 0 ? qx : (R.an == 1 ? qy : zq);
                         const float qw = R.dims == 3 ? (R.aw == 0 ? qx : (R.aw == 1 ? qy : zq)) : 0.f;
@@ -1338,13 +1260,6 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
             pre_blocked = __syncthreads_or(full) != 0;
         }
 
-        const int np = (R.dims == 3) ? 8 : 6;
-        if (!pre_blocked) {
-            hull_planes(R.dims, s_pts, np, sm);
-            __syncthreads();
-        }
-        const int n_planes = min(sm.n_planes, kMaxPlanes);
-
         // walk the grid cells under the hull's footprint.  In the xy plane
         // the footprint is the convex hull of two axis-aligned rectangles,
         // A (the tile's viewpoints) and B (the target's shadow on the
@@ -1356,16 +1271,9 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
         // time: one thread finds a row's span, a block scan lays the spans
         // end to end, and the threads share out the cells.
         if (!pre_blocked) {
-            float ax0 = s_pts[0][0], ax1 = ax0, ay0 = s_pts[0][1], ay1 = ay0;
-            for (int l = 1; l < 4; ++l) {
-                ax0 = fminf(ax0, s_pts[l][0]); ax1 = fmaxf(ax1, s_pts[l][0]);
-                ay0 = fminf(ay0, s_pts[l][1]); ay1 = fmaxf(ay1, s_pts[l][1]);
-            }
-            float bx0 = s_pts[4][0], bx1 = bx0, by0 = s_pts[4][1], by1 = by0;
-            for (int l = 5; l < np; ++l) {
-                bx0 = fminf(bx0, s_pts[l][0]); bx1 = fmaxf(bx1, s_pts[l][0]);
-                by0 = fminf(by0, s_pts[l][1]); by1 = fmaxf(by1, s_pts[l][1]);
-            }
+            const float ax0 = s_A[0][0], ax1 = s_A[0][1], ay0 = s_A[1][0], ay1 = s_A[1][1];
+            const float bx0 = s_B[0][0], bx1 = s_B[0][1], by0 = s_B[1][0], by1 = s_B[1][1];
+            const Swept hull = make_swept(s_A, s_B);
             // how far a cell's boxes reach past the cell, plus 1 m: far more
             // than the rounding of any quantity below (coordinates are
             // within 2^14 m), so no cell that can hold an occluder is missed
@@ -1436,7 +1344,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                             t += step;
                     const int cell = (r0 + t) * sc.gnx + s_rowx[t] + (c - s_rowpre[t]);
                     const int b = sc.cell_start[cell], e = sc.cell_start[cell + 1];
-                    if (b == e || outside(sm.planes, n_planes, sc.cell_lo[cell], sc.cell_hi[cell]))
+                    if (b == e || !swept_meets(hull, sc.cell_lo[cell], sc.cell_hi[cell]))
                         continue;
                     const int k = atomicAdd(&s_npass, 1);
                     if (k < kPassCap) {
@@ -1445,8 +1353,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                         continue;
                     }
                     for (int s = b; s < e; ++s)   // list full: this cell's boxes here
-                        add_candidate(world, sm.planes, n_planes, s, sm, s_ids, box_cap, spill, spill_slot, R,
-                                      sc.n_boxes);
+                        add_candidate(world, hull, s, sm, s_ids, box_cap, spill, spill_slot, R, sc.n_boxes);
                 }
                 __syncthreads();
                 // (b) exclusive scan of the listed cells' box counts
@@ -1495,8 +1402,8 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                     for (int step = kPassCap / 2; step > 0; step >>= 1)
                         if (s_passp[k + step] <= i)
                             k += step;
-                    add_candidate(world, sm.planes, n_planes, s_passb[k] + (i - s_passp[k]), sm, s_ids, box_cap,
-                                  spill, spill_slot, R, sc.n_boxes);
+                    add_candidate(world, hull, s_passb[k] + (i - s_passp[k]), sm, s_ids, box_cap, spill, spill_slot, R,
+                                  sc.n_boxes);
                 }
                 if (tid == 0)
                     s_npass = 0;
@@ -1615,8 +1522,8 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
         if (tile_check && !pre_blocked) {
             bool full = false;
             if (tid < min(n_smem, kThreads)) {
-                full = box_blocks_tile(R, s_box[2 * tid], s_box[2 * tid + 1], s_pts[0][0], s_pts[1][0], s_pts[0][1],
-                                       s_pts[2][1], zq);
+                full = box_blocks_tile(R, s_box[2 * tid], s_box[2 * tid + 1], s_A[0][0], s_A[0][1], s_A[1][0],
+                                       s_A[1][1], zq);
                 corner_tests += 16;
                 if (full && R.blk_base >= 0)   // for the tiles of this position and its neighbours
                     work[kWorkHeader + kBlockerOff + R.blk_base + ty * R.tiles_x + tx] = s_ids[tid];
@@ -2220,18 +2127,6 @@ cudaError_t init_device()
         return e;
     if (dev >= 0 && dev < 64 && done[dev])
         return cudaSuccess;
-    unsigned char tri[56][3];
-    int n = 0;
-    for (int i = 0; i < 8; ++i)
-        for (int j = i + 1; j < 8; ++j)
-            for (int k = j + 1; k < 8; ++k) {
-                tri[n][0] = (unsigned char)i;
-                tri[n][1] = (unsigned char)j;
-                tri[n][2] = (unsigned char)k;
-                ++n;
-            }
-    if ((e = cudaMemcpyToSymbol(c_tri, tri, sizeof(tri))) != cudaSuccess)
-        return e;
     const void *kernels[4] = {(const void *)k_tiles<false, false>, (const void *)k_tiles<true, false>,
                               (const void *)k_tiles<false, true>, (const void *)k_tiles<true, true>};
     for (const void *k : kernels)
