@@ -233,7 +233,7 @@ typedef struct {
  * device memory of the asynchronous path (0 = 64 GiB): the result buffers
  * of admitted requests, the occlusion bits kept for recolouring
  * (VCM_CACHE_BITS), and the scratch of the scheduler's execution slots.
- * A slot's scratch is a descriptor buffer, a spill list of n_boxes ints per
+ * A slot's scratch is a descriptor buffer, a spill list of n_boxes ids per
  * block that can be resident (about 365 MB per slot for 100,000 boxes on
  * 152 SMs) and a 71 MB work buffer through which the blocks of a launch
  * share the open viewpoints of expensive tiles; it is allocated when the
@@ -391,7 +391,7 @@ vcm_status vcm_autotune(vcm_ctx *ctx, const vcm_request *samples, uint32_t n, vc
 vcm_status vcm_set_tune(vcm_ctx *ctx, const vcm_tune *tune);
 
 /* Launch shape the context would use for this request launched alone
- * (a launch with fewer tiles than four waves of resident blocks has its
+ * (a launch with fewer tiles than three waves of resident blocks has its
  * tiles shrunk, 16 x 16 -> 16 x 8 -> 8 x 8 -> 8 x 4, unless a shape is
  * forced with vcm_set_tune). */
 vcm_status vcm_get_tune(vcm_ctx *ctx, const vcm_request *req, vcm_tune *out);

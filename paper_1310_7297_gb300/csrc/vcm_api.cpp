@@ -366,13 +366,6 @@ void fill_shape(const Canon &c, const vcm_tune &t, DevRequest &d)
     d.rows = (c.nw + d.groups - 1) / d.groups;
     d.inv_row = 1.f / ((float)d.groups * c.row_step);
     d.row_dev = c.row_dev;
-    // Work sharing: chunks of 32 open viewpoints, published from a tile
-    // with at least 8 open.  Smaller chunks for requests with many patches
-    // (about the same work per chunk) were slower: each chunk stages its
-    // owner's candidate list again (100,000-box scene, 64 x 32 patches:
-    // 8 viewpoints +7 %, 4 viewpoints +26 %; publishing from 4 open +0.5 %).
-    d.chunk_vp = kChunkVp;
-    d.min_publish = kMinPublish;
     d.tile_x = (int)std::max(1u, t.tile_x);
     d.tile_y = (int)std::max(1u, t.tile_y);
     d.tiles_x = (c.nx + d.tile_x - 1) / d.tile_x;
@@ -461,7 +454,7 @@ struct Slot {
     size_t desc_cap = 0;
     int *d_work = nullptr;
     int *d_spill = nullptr;
-    size_t spill_cap = 0;   // ints
+    size_t spill_cap = 0;   // bytes
     int *d_spill_busy = nullptr;   // spill-region claims of one-tile launches
     size_t spill_busy_cap = 0;
     bool high_priority = false;
@@ -742,19 +735,28 @@ void fill_desc(char *h, const char *d_base, const Layout &L, const std::vector<c
 // Device bytes of a slot's scratch.
 size_t slot_bytes(const Slot &s)
 {
-    return s.desc_cap + (s.d_work ? kWorkBytes : 0) + (s.spill_cap + s.spill_busy_cap) * sizeof(int) +
+    return s.desc_cap + (s.d_work ? kWorkBytes : 0) + s.spill_cap + s.spill_busy_cap * sizeof(int) +
            s.stats_cap * sizeof(vcm_stats);
 }
 
+// Resident blocks of the tile pass for a staged-box count.  Scenes whose box
+// ids take 4 bytes run at most 6 per SM, so that their spill lists take no
+// more memory than 8 per SM do with 3 bytes.
+int resident_blocks(const vcm_ctx *ctx, int box_cap)
+{
+    const int per_sm = tiles_blocks_per_sm(box_cap);
+    return (spill_id_bytes((int)ctx->n_boxes) == 4 ? std::min(per_sm, 6) : per_sm) * ctx->sm_count;
+}
+
 // Scratch one scheduler slot needs for the current scene: the work arena,
-// a spill list of n_boxes ints for every block that can be resident (at the
+// a spill list of n_boxes ids for every block that can be resident (at the
 // smallest shared-memory size, the most blocks), their claim words, 256
 // stats entries and 1 MB of descriptors.
 size_t slot_scratch_need(const vcm_ctx *ctx)
 {
-    const size_t blocks = (size_t)tiles_blocks_per_sm(32) * (size_t)ctx->sm_count;
-    return kWorkBytes + blocks * (std::max<uint32_t>(ctx->n_boxes, 1) + 1) * sizeof(int) + 256 * sizeof(vcm_stats) +
-           ((size_t)1 << 20);
+    const size_t blocks = (size_t)resident_blocks(ctx, 32);
+    const size_t region = spill_region_bytes((int)ctx->n_boxes, spill_id_bytes((int)ctx->n_boxes));
+    return kWorkBytes + blocks * (region + sizeof(int)) + 256 * sizeof(vcm_stats) + ((size_t)1 << 20);
 }
 
 vcm_status ensure_slot_impl(vcm_ctx *ctx, Slot &s, size_t desc_bytes, size_t n_stats, int grid_blocks,
@@ -765,11 +767,12 @@ vcm_status ensure_slot_impl(vcm_ctx *ctx, Slot &s, size_t desc_bytes, size_t n_s
         // first launch (what admission charged: slot_scratch_need), so a
         // later, larger launch does not regrow it: a cudaFree would wait
         // for the device while the context lock is held.
-        grid_blocks = std::max(grid_blocks, tiles_blocks_per_sm(32) * ctx->sm_count);
+        grid_blocks = std::max(grid_blocks, resident_blocks(ctx, 32));
         desc_bytes = std::max<size_t>(desc_bytes, (size_t)1 << 19);
         n_stats = std::max<size_t>(n_stats, 256);
     }
-    const size_t spill_need = (size_t)grid_blocks * std::max<uint32_t>(ctx->n_boxes, 1);
+    const size_t spill_need =
+        (size_t)grid_blocks * spill_region_bytes((int)ctx->n_boxes, spill_id_bytes((int)ctx->n_boxes));
     const bool grow = desc_bytes > s.desc_cap || spill_need > s.spill_cap || n_stats > s.stats_cap ||
                       !s.d_work || (size_t)grid_blocks > s.spill_busy_cap;
     if (!grow)
@@ -805,7 +808,7 @@ vcm_status ensure_slot_impl(vcm_ctx *ctx, Slot &s, size_t desc_bytes, size_t n_s
     if (spill_need > s.spill_cap) {
         if (s.d_spill) cudaFree(s.d_spill);
         s.d_spill = nullptr;
-        CUDA_TRY(cudaMalloc(&s.d_spill, spill_need * sizeof(int)));
+        CUDA_TRY(cudaMalloc(&s.d_spill, spill_need));
         s.spill_cap = spill_need;
     }
     if ((size_t)grid_blocks > s.spill_busy_cap) {
@@ -851,16 +854,18 @@ int launch_box_cap(const std::vector<vcm_tune> &shapes)
 
 // A launch with few tiles leaves SMs idle while its expensive tiles run
 // (a tile is one block's work item): shrink the tiles, 16 x 16 -> 16 x 8 ->
-// 8 x 8 -> 8 x 4, until the launch holds four waves of resident blocks.
+// 8 x 8 -> 8 x 4, until the launch holds kTileWaves waves of resident blocks.
 // Measured on the 64 requests of the serving pool, each launched alone: the
 // sum of their times 45.3 ms -> 26.1 ms (the best shape per request would
 // give 25.7 ms); a 124 x 124 x 5 grid with 64 x 32 patches 3.28 -> 0.30 ms.
 // Launches with many tiles (the 3D workloads, batches) keep their shapes.
-void shrink_small_launch(vcm_ctx *ctx, const std::vector<const Canon *> &cs, std::vector<vcm_tune> &shapes)
+// `list_cap`: as of launch_tiles.
+void shrink_small_launch(int sm_count, const std::vector<const Canon *> &cs, std::vector<vcm_tune> &shapes,
+                         int list_cap = 0)
 {
-    if (ctx->forced || cs.empty())
+    if (cs.empty())
         return;
-    const long long target = 4LL * tiles_blocks_per_sm(launch_box_cap(shapes)) * ctx->sm_count;
+    const long long target = kTileWaves * tiles_blocks_per_sm(launch_box_cap(shapes), list_cap) * sm_count;
     for (;;) {
         long long total = 0;
         for (size_t i = 0; i < cs.size(); ++i) {
@@ -887,8 +892,7 @@ void shrink_small_launch(vcm_ctx *ctx, const std::vector<const Canon *> &cs, std
 
 int grid_blocks_for(vcm_ctx *ctx, int box_cap, int total_tiles)
 {
-    const int per_sm = tiles_blocks_per_sm(box_cap);
-    return std::max(1, std::min(total_tiles, per_sm * ctx->sm_count));
+    return std::max(1, std::min(total_tiles, resident_blocks(ctx, box_cap)));
 }
 
 struct Prepared {
@@ -913,8 +917,8 @@ vcm_status prepare_launch(vcm_ctx *ctx, Slot &s, const std::vector<const Canon *
     if (!ctx->built)
         return fail(VCM_E_STATE, "vcm_build has not been called for the current scene");
     std::vector<vcm_tune> shapes = shapes_in;
-    if (adapt)
-        shrink_small_launch(ctx, cs, shapes);
+    if (adapt && !ctx->forced)
+        shrink_small_launch(ctx->sm_count, cs, shapes);
     P.L = layout_for(cs, shapes);
     P.box_cap = launch_box_cap(shapes);
     P.blocks = grid_blocks_for(ctx, P.box_cap, P.L.total_tiles);
@@ -955,7 +959,7 @@ vcm_status record_launch(vcm_ctx *ctx, Slot &s, const Prepared &P, vcm_stats *st
     (void)stats;   // the descriptors point into it; the prologue clears it
     CUDA_TRY(launch_prologue(d_reqs, (int)P.n, s.d_work, stream));
     if (P.tile_check && P.L.blocker_ints > 0)   // no blocker recorded yet (-1)
-        CUDA_TRY(cudaMemsetAsync(s.d_work + kWorkHeader + kBlockerOff, 0xFF, (size_t)P.L.blocker_ints * sizeof(int),
+        CUDA_TRY(cudaMemsetAsync(s.d_work + kWorkHeader + Arena().blocker_off(), 0xFF, (size_t)P.L.blocker_ints * sizeof(int),
                                  stream));
     // the tile kernel starts after another launch's kernels (see launch_group)
     if (after) {
@@ -2439,7 +2443,8 @@ vcm_status vcm_get_tune(vcm_ctx *ctx, const vcm_request *req, vcm_tune *out)
         return st;
     std::lock_guard<std::mutex> g(ctx->mu);
     std::vector<vcm_tune> shapes{shape_for(ctx, c)};
-    shrink_small_launch(ctx, {&c}, shapes);
+    if (!ctx->forced)
+        shrink_small_launch(ctx->sm_count, {&c}, shapes);
     *out = shapes[0];
     out->patch_k = (uint32_t)rows_per_pass(c, *out);
     return VCM_OK;
@@ -2578,10 +2583,18 @@ vcm_status vcm_compute_static(const float *lo, const float *hi, uint32_t n_boxes
         size_t cap = 0;
         CUDA_TRY(static_scratch(&base, &cap));
         const size_t nb = std::max<uint32_t>(n, 1);
+        int sm_count = 1, dev = 0;
+        CUDA_TRY(cudaGetDevice(&dev));
+        CUDA_TRY(cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev));
+        // Boxes past the staged ones are listed in shared memory, which holds
+        // the ids of all of them: no spill (staging every box took 54 KB per
+        // block for 1,500 boxes, so 3 blocks per SM).
         vcm_tune t = default_tune();
-        t.box_cap = (uint32_t)std::max<size_t>(32, nb);   // every candidate list fits: no spill
+        t.box_cap = (uint32_t)std::min<size_t>(std::max<size_t>(32, nb), t.box_cap);
+        const int list_cap = (int)std::max<size_t>(32, nb);
         std::vector<const Canon *> cs{&c};
         std::vector<vcm_tune> shapes{t};
+        shrink_small_launch(sm_count, cs, shapes, list_cap);
         const Layout lay = layout_for(cs, shapes);
         size_t off = 0;
         auto take = [&](size_t bytes) {
@@ -2602,11 +2615,20 @@ vcm_status vcm_compute_static(const float *lo, const float *hi, uint32_t n_boxes
         float4 *s_cell_lo = reinterpret_cast<float4 *>(take((size_t)n_cells * sizeof(float4)));
         float4 *s_cell_hi = reinterpret_cast<float4 *>(take((size_t)n_cells * sizeof(float4)));
         unsigned *s_overhang = reinterpret_cast<unsigned *>(take(sizeof(unsigned)));
-        int *s_work = reinterpret_cast<int *>(take(kWorkHeader * sizeof(int)));   // counters only: no sharing
-        int *s_spill = reinterpret_cast<int *>(take(256));   // never written: lists fit box_cap
+        int *s_spill = reinterpret_cast<int *>(take(256));   // never written: lists fit list_cap
         char *s_desc = take(lay.bytes);
+        int *s_work = reinterpret_cast<int *>(take(kWorkHeader * sizeof(int)));
         if (off > cap)
             return fail(VCM_E_ARG, "request needs %zu bytes of static scratch, the array has %zu", off, cap);
+        // what is left is the arena through which the second pass takes the
+        // open viewpoints (96 x 96 x 2 viewpoints, 1,500 boxes, 16 x 8 patches:
+        // the call's device work 165 -> 130 us, with the smaller tiles above)
+        Arena arena;
+        arena.rec_cap = std::min(lay.total_tiles, 8192);
+        arena.chunk_cap = (int)std::min<long long>(lay.total_vp / kChunkVp + lay.total_tiles, 32768);
+        const size_t left = (cap - off) / sizeof(int);
+        const bool share = arena.pool_off() < left;
+        arena.pool_ints = share ? (int)std::min<size_t>(left - arena.pool_off(), (size_t)kPoolInts) : 0;
 
         cudaStream_t sm = static_cast<cudaStream_t>(stream);
         // pageable host sources: each copy has consumed its source when it returns
@@ -2641,13 +2663,12 @@ vcm_status vcm_compute_static(const float *lo, const float *hi, uint32_t n_boxes
         const DevRequest *d_reqs = reinterpret_cast<const DevRequest *>(s_desc + lay.off_reqs);
         const int *d_tiles = reinterpret_cast<const int *>(s_desc + lay.off_tiles);
         const long long *d_vps = reinterpret_cast<const long long *>(s_desc + lay.off_vps);
-        int sm_count = 1, dev = 0;
-        CUDA_TRY(cudaGetDevice(&dev));
-        CUDA_TRY(cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev));
-        const int blocks = std::max(1, std::min(lay.total_tiles, tiles_blocks_per_sm((int)t.box_cap) * sm_count));
+        const int blocks =
+            std::max(1, std::min(lay.total_tiles, tiles_blocks_per_sm((int)t.box_cap, list_cap) * sm_count));
         CUDA_TRY(launch_prologue(d_reqs, 1, s_work, sm));
         CUDA_TRY(launch_tiles(sc, d_reqs, d_tiles, 1, lay.total_tiles, s_work, s_spill, blocks, (int)t.box_cap,
-                              needs_extra(c), c.P >= kTileCheckMinPatches, sm_count, sm));
+                              needs_extra(c), c.P >= kTileCheckMinPatches, sm_count, sm, false, nullptr, share, kClaimRounds,
+                              arena, list_cap));
         CUDA_TRY(launch_quantise(d_reqs, d_vps, 1, lay.total_vp, sm));
         return VCM_OK;
     } catch (const std::exception &ex) {

@@ -22,49 +22,69 @@ constexpr float kBand = 1e-6f;            // FP32 slab margin re-decided in FP64
 constexpr int kMaxBoxCap = 5000;          // candidate boxes a tile stages in shared memory
 constexpr int kRowCap = 256;              // patch rows a warp stages for the measure
 constexpr int kWarpBoxes = 64;            // boxes of a chunk's list a warp stages
+constexpr int kTileBlocks = 8;            // blocks per SM of the tile pass
+constexpr long long kTileWaves = 3;         // waves of resident blocks below which a launch's tiles shrink
+constexpr int kKeptWarps = 2;             // warps that sweep the viewpoints a tile keeps
 constexpr int kSweepBlocks = 7;           // blocks per SM of the second pass
 constexpr int kPartsPerWarp = 4;          // parts of chunks the second pass wants per warp
 constexpr int kMaxTileViewpoints = 1024;  // viewpoints in one tile (tile_x * tile_y)
 constexpr int kClaimRounds = 4096;        // bounded retries of a spill-region claim (2 us pauses)
 
 // Work sharing of the persistent tile kernel, in two passes.  In the first,
-// a tile whose one-box check leaves at least its request's min_publish
-// viewpoints open publishes them, chunk_vp at a time, as chunks (a list
-// longer than kPublishBoxes only from kPublishHeavy viewpoints); in the
-// second, k_sweep's warps sweep parts of the chunks.
+// the tiles publish the viewpoints their checks leave open, kChunkVp at a time,
+// as chunks; in the second, k_sweep's warps sweep parts of the chunks.
 // The work buffer of a launch holds kWorkHeader counters (next tile,
 // records, chunks published, parts taken, id-pool ints used) and then the
 // arena:
-//   chunk[kChunkCap][kChunkInts]     record index, count, viewpoints (x + 256 y in the tile, 16 bits each)
+//   chunk[kChunkCap][kChunkInts]     32 x record index + count, viewpoints (x + 256 y in the tile, 16 bits each)
 //   record[kRecCap][kRecInts]        request, candidate count, offset of its ids in the pool, layer, tile origin
 //   pool[kPoolInts]                  the records' candidate box ids, in the owner's order
 //   blocker[kBlockerCap]             per tile position of each request (whole-tile-check
 //                                    launches): a box id that blocked a tile there, or -1
 // A tile whose publication would pass a cap keeps its viewpoints.
-constexpr int kChunkVp = 32;
-constexpr int kChunkInts = 2 + kChunkVp / 2;
-constexpr int kMinPublish = 8;
-// Longer lists stay with their tile (the 100,000-box scene, lists of ~180
-// boxes on average: 6.44 ms with this limit, 6.71 ms without it) unless the
-// tile has at least kPublishHeavy open viewpoints (32: 3.84 -> 3.82 ms
-// against 64; the tiles with 39-63 open viewpoints and lists just over 128
-// had set the end of the tile pass).
-constexpr int kPublishBoxes = 128;
-constexpr int kPublishHeavy = 32;
-constexpr int kChunkCap = 393216;
+constexpr int kChunkVp = 16;
+constexpr int kChunkInts = 1 + kChunkVp / 2;
+constexpr int kChunkCap = 800000;
 constexpr int kRecCap = 131072;
 constexpr int kRecInts = 8;
 constexpr int kPoolInts = 8 << 20;
 constexpr int kBlockerCap = 1 << 20;
 constexpr int kWorkHeader = 64;   // ints before the arena (256 bytes)
-constexpr size_t kChunkOff = 0;
-constexpr size_t kRecOff = kChunkOff + (size_t)kChunkCap * kChunkInts;
-constexpr size_t kPoolOff = kRecOff + (size_t)kRecCap * kRecInts;
-constexpr size_t kBlockerOff = kPoolOff + (size_t)kPoolInts;
-constexpr size_t kArenaInts = kBlockerOff + (size_t)kBlockerCap;
+// Where the parts of an arena lie (in ints, after the header).  The defaults are
+// those of a work buffer of kWorkBytes; vcm_compute_static lays out a smaller
+// one.
+struct Arena {
+    int chunk_cap = kChunkCap, rec_cap = kRecCap, pool_ints = kPoolInts;
+#ifdef __CUDACC__
+    __host__ __device__
+#endif
+    size_t rec_off() const { return (size_t)chunk_cap * kChunkInts; }
+#ifdef __CUDACC__
+    __host__ __device__
+#endif
+    size_t pool_off() const { return rec_off() + (size_t)rec_cap * kRecInts; }
+#ifdef __CUDACC__
+    __host__ __device__
+#endif
+    size_t blocker_off() const { return pool_off() + (size_t)pool_ints; }
+};
+constexpr size_t kArenaInts = (size_t)kChunkCap * kChunkInts + (size_t)kRecCap * kRecInts + (size_t)kPoolInts +
+                              (size_t)kBlockerCap;
 constexpr size_t kWorkBytes = (kWorkHeader + kArenaInts) * sizeof(int);
 
-inline size_t tiles_smem_bytes(int box_cap) { return (size_t)box_cap * (32 + 4); }
+// Bytes per id of a spill region, and of a block's region (a multiple of 4).
+int spill_id_bytes(int n_boxes);
+#ifdef __CUDACC__
+__host__ __device__
+#endif
+inline size_t spill_region_bytes(int n_boxes, int id_bytes)
+{
+    return ((size_t)(n_boxes > 0 ? n_boxes : 1) * id_bytes + 3) & ~(size_t)3;
+}
+
+// Dynamic shared memory of the tile kernel: box_cap staged boxes, and the ids
+// of list_cap candidates.
+inline size_t tiles_smem_bytes(int box_cap, int list_cap) { return (size_t)box_cap * 32 + (size_t)list_cap * 4; }
 
 // Device view of the scene and its uniform-grid index.  Boxes are sorted by
 // grid cell; `boxes[perm]` holds the same boxes with their coordinates
@@ -97,7 +117,6 @@ struct DevRequest {
     int tile_x, tile_y, tiles_x, tiles_y, n_tiles;
     int nuc, groups, col_passes, rows;   // lane mapping: columns and row groups of a pass, column passes, rows per lane
     float inv_row, row_dev;    // 1 / w step between a lane's rows; how far a row is off an even step
-    int chunk_vp, min_publish;   // work sharing: viewpoints per chunk, open viewpoints to publish
     int blk_base;                // offset of its tile positions in the blocker table, or -1
     const float *u_coord;      // [nu] patch centre coordinate along u
     const float *w_coord;      // [nw] along w (one 0 in 2D)
@@ -133,14 +152,18 @@ cudaError_t launch_grid_build(const float *d_lo_world, const float *d_hi_world, 
 // interleave block by block; grid_blocks must then be at least the number of
 // blocks that can be resident at once, and `d_spill_busy` (grid_blocks ints,
 // all zero between launches) hands out the spill regions.  `d_spill` holds
-// grid_blocks * n_boxes ints for candidate lists longer than box_cap.
+// grid_blocks regions of spill_region_bytes for candidate lists longer than box_cap.
 // `extra` must be set when any request is two-sided or has a field-of-view
 // cone: it selects the tile kernel's instantiation that handles them.
 // `tile_check` selects the instantiation with the whole-tile check (any
 // launch may use either; it pays when every request has many patches).
-// `share` (persistent launches only): d_work is kWorkBytes long, and a second
+// `share` (persistent launches only): d_work holds `arena` behind its header
+// (kWorkBytes for the default one), and a second
 // kernel on all sm_count SMs works the open viewpoints that expensive tiles of
 // the first published there.
+// `list_cap` > box_cap: the ids of candidates past the staged boxes are kept in
+// shared memory, which must then hold every box of the scene (d_spill is not
+// used); otherwise they spill.
 // `claim_rounds` (1..kClaimRounds) bounds the retries of a one-tile block's
 // spill-region claim; a block that gives up runs without a region and sets
 // its request's vcm_stats.error to VCM_DEVERR_SPILL_WAIT if its candidate
@@ -149,7 +172,8 @@ cudaError_t launch_tiles(const DevScene &sc, const DevRequest *d_reqs, const int
                          int n_req, int total_tiles, int *d_work, int *d_spill, int grid_blocks,
                          int box_cap, bool extra, bool tile_check, int sm_count, cudaStream_t stream,
                          bool one_tile = false,
-                         int *d_spill_busy = nullptr, bool share = false, int claim_rounds = kClaimRounds);
+                         int *d_spill_busy = nullptr, bool share = false, int claim_rounds = kClaimRounds,
+                         const Arena &arena = Arena(), int list_cap = 0);
 // Colors and edge counts for all viewpoints of n_req requests (grid over the
 // concatenated viewpoints, `d_vp_prefix` = exclusive prefix, n_req + 1).
 cudaError_t launch_quantise(const DevRequest *d_reqs, const long long *d_vp_prefix, int n_req,
@@ -166,7 +190,7 @@ cudaError_t launch_recolor(const DevRequest *d_req, long long n_vp, int sm_count
 cudaError_t launch_prologue(const DevRequest *d_reqs, int n_req, int *d_work, cudaStream_t stream);
 
 // Blocks of the tile kernel that fit on one SM for this shared-memory size.
-int tiles_blocks_per_sm(int box_cap);
+int tiles_blocks_per_sm(int box_cap, int list_cap = 0);
 
 // One-time per-device setup (constant tables, kernel attributes); must run
 // before any launch is captured into a graph.

@@ -44,10 +44,36 @@ __device__ __noinline__ bool in_bounds_slow(long long i, long long n, vcm_stats 
 #define IN_BOUNDS(i, n, st) true
 #endif
 
+// The ids of a candidate list past its staged boxes: ints, or 3 bytes each in a
+// spill region (scenes of less than 2^24 boxes: 8 blocks per SM then spill
+// into what 6 blocks needed with ints).
+struct Tail {
+    const void *p;
+    int bytes;
+    __device__ __forceinline__ int operator[](int i) const
+    {
+        if (bytes == 4)
+            return static_cast<const int *>(p)[i];
+        const unsigned char *b = static_cast<const unsigned char *>(p) + 3 * (size_t)i;
+        return (int)(b[0] | (b[1] << 8) | (b[2] << 16));
+    }
+    __device__ __forceinline__ void put(int i, int id) const
+    {
+        if (bytes == 4) {
+            static_cast<int *>(const_cast<void *>(p))[i] = id;
+            return;
+        }
+        unsigned char *b = static_cast<unsigned char *>(const_cast<void *>(p)) + 3 * (size_t)i;
+        b[0] = (unsigned char)id;
+        b[1] = (unsigned char)(id >> 8);
+        b[2] = (unsigned char)(id >> 16);
+    }
+};
+
 // Box i of a tile's candidate list: staged in shared memory, or (past
-// n_smem) through its id in the block's spill region.  The checked build
+// n_smem) through its id in the list's tail.  The checked build
 // replaces an out-of-range id by an empty box, which blocks nothing.
-__device__ __forceinline__ void load_box(const float4 *__restrict__ sbox, int n_smem, const int *__restrict__ spill,
+__device__ __forceinline__ void load_box(const float4 *__restrict__ sbox, int n_smem, Tail spill,
                                          const float4 *__restrict__ gbox, int i, int n_boxes, vcm_stats *st,
                                          float4 &lo, float4 &hi)
 {
@@ -667,7 +693,7 @@ __device__ __forceinline__ bool record_blocks_rect(float4 r0, float4 r1, float i
 // The filter of one pass for a viewpoint with more than 32 kept boxes: lanes
 // over the boxes [base, base + 32); returns the kept ones, records written.
 __device__ __noinline__ unsigned pass_records(const DevRequest &R, const float4 *__restrict__ sbox, int n_smem,
-                                              const int *__restrict__ spill, int count,
+                                              Tail spill, int count,
                                               const float4 *__restrict__ gbox, float qu, float qn, float qw, int cp,
                                               int row0, float4 *rec, int n_boxes, int base)
 {
@@ -747,7 +773,7 @@ __device__ __forceinline__ float measure_term(const DevRequest &R, float col_d2,
 template <bool EXTRA>
 __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const LaneMap &M,
                                                  const float4 *__restrict__ sbox, int n_smem,
-                                                 const int *__restrict__ spill, int count,
+                                                 Tail spill, int count,
                                                  const float4 *__restrict__ gbox, float qu, float qn,
                                                  float qw, bool front, long long vp, WarpScratch &W,
                                                  unsigned &tests, unsigned &corners, unsigned &rechecks,
@@ -982,12 +1008,44 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
     return strict_fail ? 0.f : v;
 }
 
+// One open viewpoint, at (ix, iy) of a layer: swept, and its outputs written.
+// Returns its value.
+template <bool EXTRA>
+__device__ __forceinline__ float sweep_one(const DevRequest &R, const LaneMap &M, int ix, int iy, int layer, float zq,
+                                           bool want_bits, const float4 *__restrict__ sbox, int n_smem,
+                                           Tail spill, int count, const float4 *__restrict__ gbox,
+                                           WarpScratch &W, unsigned &tests, unsigned &corners, unsigned &rechecks,
+                                           unsigned &shortcuts, int n_boxes)
+{
+    const int lane = threadIdx.x & 31;
+    const long long vp = ((long long)layer * R.ny + iy) * R.nx + ix;
+    const float qx = R.x_coord[ix], qy = R.y_coord[iy];
+    const float qu = R.au == 0 ? qx : (R.au == 1 ? qy : zq);
+    const float qn = R.an == 0 ? qx : (R.an == 1 ? qy : zq);
+    const float qw = R.dims == 3 ? (R.aw == 0 ? qx : (R.aw == 1 ? qy : zq)) : 0.f;
+    const bool front = facing(R, qn);
+    float v = sweep_viewpoint<EXTRA>(R, M, sbox, n_smem, spill, count, gbox, qu, qn, qw, front, vp, W, tests, corners,
+                                     rechecks, n_boxes);
+    if (v < 0.f) {   // one box blocks every patch
+        ++shortcuts;
+        if (want_bits)
+            for (int wd = lane; wd < R.words; wd += 32) {
+                const int rem = R.P - 32 * wd;
+                put_word(R, vp * R.words + wd, rem >= 32 ? 0xffffffffu : ((1u << rem) - 1u));
+            }
+    }
+    v = front ? fmaxf(v, 0.f) : 0.f;
+    if (lane == 0)
+        put_v(R, vp, v);
+    return v;
+}
+
 // Viewer-centric cell (VCM_VIEWER): one segment from the cell q to the
 // viewer p (world frame) against the candidate boxes, nearest first; the
 // cell's value is the visual angle (2D, Eq. 1) or solid angle (3D) of an
 // object of size S at distance D facing the viewer, 0 when blocked or D = 0.
 __device__ __forceinline__ float viewer_cell(const DevRequest &R, const float4 *__restrict__ sbox, int n_smem,
-                                             const int *__restrict__ spill, int count,
+                                             Tail spill, int count,
                                              const float4 *__restrict__ gbox, float qx, float qy, float qz,
                                              bool &blocked, unsigned long long &tests, unsigned &rechecks,
                                              int n_boxes)
@@ -1027,42 +1085,94 @@ __device__ __forceinline__ float viewer_cell(const DevRequest &R, const float4 *
 // If a box may matter to the tile, add it to the tile's candidate list (shared
 // memory, then the block's spill region).
 __device__ __forceinline__ void add_candidate(const float4 *__restrict__ world, const Swept &hull, int s,
-                                              TileSmem &sm, int *s_ids, int box_cap, int *spill,
+                                              TileSmem &sm, int *s_ids, int list_cap, Tail spill,
                                               int spill_slot, const DevRequest &R, int n_boxes)
 {
     if (!swept_meets(hull, world[2 * s], world[2 * s + 1]))
         return;
     const int pos = atomicAdd(&sm.count, 1);
-    if (pos < box_cap)
+    if (pos < list_cap)
         s_ids[pos] = s;
     else if (spill_slot >= 0) {
-        if (IN_BOUNDS(pos - box_cap, n_boxes, R.stats))
-            spill[pos - box_cap] = s;
+        if (IN_BOUNDS(pos - list_cap, n_boxes, R.stats))
+            spill.put(pos - list_cap, s);
     } else {
         R.stats->error = VCM_DEVERR_SPILL_WAIT;   // no spill region: the result is flagged
     }
 }
 
-// EXTRA: the instantiation for launches that hold a two-sided or cone
-// request; the common one carries none of that code (the tile kernel is
-// sensitive to its instruction footprint).
-// Five blocks per SM: the compiler then fits the kernel in 94 registers
-// without spilling, and the fifth block hides more of the dependency and
-// barrier latency that bound it (4 -> 5 blocks: 3D step -5 %, a 256-request
-// batch -11 %; 6 blocks spill and lose on large scenes).
+// Shared memory of the tile pass that its phases use in turn: the walk over the
+// grid cells and the sort, then (rarely) the sweeps of sweep_kept.
+union TileScratch {
+    struct {
+        int rowpre[kThreads], rowx[kThreads], wsum[kWarps];   // cell-row spans
+        int passb[kPassCap], passn[kPassCap], passp[kPassCap + 1], wsum2[kWarps];   // listed cells
+        int hist[kDistClasses];   // counting sort of long candidate lists
+    } walk;
+    WarpScratch sweep[kKeptWarps];
+};
+
+// The open viewpoints that a tile does not publish (launches without a second
+// pass, or an arena that is full), swept by the tile's first warps.  Not
+// inlined: the tile pass then holds none of the sweep's registers.
+__device__ __noinline__ void sweep_kept(const DevRequest &R, TileScratch &T, const float4 *__restrict__ sbox,
+                                        int n_smem, Tail spill, int count,
+                                        const float4 *__restrict__ gbox, const unsigned short *und, int *next,
+                                        int n_und, int ix0, int iy0, int layer, int n_boxes)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp >= kKeptWarps)
+        return;
+    const LaneMap M = lane_map(R);
+    const bool want_bits = (R.flags & VCM_EMIT_BITS) && R.bits_out;
+    const float zq = R.z_coord[layer];
+    unsigned long long tests = 0, corners = 0;
+    unsigned rechecks = 0, shortcuts = 0;
+    float vmax = 0.f;
+    for (;;) {
+        int k = 0;
+        if (lane == 0)
+            k = atomicAdd(next, 1);
+        k = __shfl_sync(kFull, k, 0);
+        if (k >= n_und)
+            break;
+        unsigned vp_tests = 0, vp_corners = 0;
+        const float v = sweep_one<true>(R, M, ix0 + (und[k] & 255), iy0 + (und[k] >> 8), layer, zq, want_bits, sbox,
+                                        n_smem, spill, count, gbox, T.sweep[warp], vp_tests, vp_corners, rechecks,
+                                        shortcuts, n_boxes);
+        vmax = fmaxf(vmax, v);
+        tests += vp_tests;
+        corners += vp_corners;
+    }
+    rechecks = __reduce_add_sync(kFull, rechecks);
+    if (lane == 0) {
+        atomicMax(&R.stats->vmax_bits, __float_as_uint(vmax));
+        atomicAdd(&R.stats->slab_tests, 32 * tests);
+        atomicAdd(&R.stats->corner_tests, corners);
+        if (shortcuts)
+            atomicAdd(&R.stats->shortcut_viewpoints, (unsigned long long)shortcuts);
+        if (rechecks)
+            atomicAdd(&R.stats->rechecked, (unsigned long long)rechecks);
+    }
+}
+
 // TILE_CHECK: the instantiation with the whole-tile check below, for
 // launches whose requests all have many patches (the host picks it).  It
 // decides whole tiles, which pays when a viewpoint's own work is large (the
 // 100,000-box scene with 64 x 32 patches: -10 %); in the other instantiation
 // its code alone cost a few % on smaller requests.
 //
-//
-// Occupancy: 6 blocks per SM (80 registers); 7 made the batch slower.
-template <bool EXTRA, bool TILE_CHECK>
-__global__ void __launch_bounds__(kThreads, 6)
+// The pass holds no sweep: every viewpoint its checks leave open goes to the
+// second pass (sweep_kept takes what does not fit).  It waits on latency (queue
+// and cell loads, block barriers), so blocks per SM decide: 8 at 64 registers,
+// where the sweep's registers allowed 6.  2,048^2 x 8 viewpoints, 100,000 boxes:
+// 1.91 -> 1.47 ms for this pass; 512^2 x 5, 5,000 boxes 72 -> 61 us.  With 7 and 6
+// blocks 1.57 and 1.72 ms; 9 blocks (56 registers) spill, 2 % slower.
+template <bool TILE_CHECK>
+__global__ void __launch_bounds__(kThreads, kTileBlocks)
 k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict__ tile_prefix,
-        int n_req, int total_tiles, int *__restrict__ work, int *__restrict__ spill_all, int box_cap,
-        int one_tile, int *__restrict__ spill_busy, int spill_slots, int share, int claim_rounds)
+        int n_req, int total_tiles, int *__restrict__ work, Arena ar, unsigned char *__restrict__ spill_all, int id_bytes, int box_cap,
+        int list_cap, int one_tile, int *__restrict__ spill_busy, int spill_slots, int share, int claim_rounds)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4 *s_box = reinterpret_cast<float4 *>(smem_raw);
@@ -1071,14 +1181,11 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
     __shared__ float s_A[3][2], s_B[3][2];   // the tile's viewpoints and the target's patch rectangle: world axis, low and high
     __shared__ DevRequest s_req;
     __shared__ int s_next;
-    __shared__ __align__(16) WarpScratch s_warp[kWarps];   // the sweeps'
-    __shared__ int s_req_idx;
+    __shared__ __align__(16) TileScratch s_scratch;
+    __shared__ int s_req_idx, s_npass;
     __shared__ int s_next2;                     // cursor of the undecided list
     __shared__ unsigned short s_und[kMaxTileViewpoints];   // viewpoints left by the one-box check, x + 256 y
-    __shared__ int s_rowpre[kThreads], s_rowx[kThreads], s_wsum[kWarps];   // cell-row spans
-    __shared__ int s_passb[kPassCap], s_passn[kPassCap], s_passp[kPassCap + 1], s_wsum2[kWarps], s_npass;
-    __shared__ int s_hist[kDistClasses];   // counting sort of long candidate lists
-
+    auto &walk = s_scratch.walk;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     __shared__ int s_spill_slot;
     if (tid == 0) {
@@ -1110,7 +1217,28 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
     }
     __syncthreads();
     const int spill_slot = s_spill_slot;
-    int *spill = spill_all + (size_t)max(spill_slot, 0) * sc.n_boxes;
+    const Tail spill{spill_all + (size_t)max(spill_slot, 0) * spill_region_bytes(sc.n_boxes, id_bytes), id_bytes};
+    // candidates past the staged boxes: ids in shared memory where these hold
+    // every box of the scene (list_cap > box_cap), else the spill region
+    const Tail tail = list_cap > box_cap ? Tail{s_ids + box_cap, 4} : spill;
+    // counters, added to a request's when its last tile in a row is done
+    vcm_stats *acc = nullptr;
+    unsigned corner_tests = 0, shortcuts = 0;
+    unsigned long long listed = 0;   // thread 0's
+    auto flush = [&] {
+        corner_tests = __reduce_add_sync(kFull, corner_tests);
+        shortcuts = __reduce_add_sync(kFull, shortcuts);
+        if (acc && lane == 0) {
+            if (corner_tests)
+                atomicAdd(&acc->corner_tests, (unsigned long long)corner_tests);
+            if (shortcuts)
+                atomicAdd(&acc->shortcut_viewpoints, (unsigned long long)shortcuts);
+        }
+        if (acc && tid == 0)
+            atomicAdd(&acc->boxes_listed, listed);
+        corner_tests = shortcuts = 0;
+        listed = 0;
+    };
 
     for (;;) {
         // thread 0 takes the next tile, copies its request and lays out the
@@ -1173,6 +1301,10 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
         const int item = sm.item;
         if (item >= total_tiles)
             break;
+        if (s_req.stats != acc) {
+            flush();
+            acc = s_req.stats;
+        }
         const DevRequest &R = s_req;
         const int t = sm.pad;
         const int per_layer = R.tiles_x * R.tiles_y;
@@ -1225,7 +1357,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
         unsigned pre_tests = 0;
         const bool tile_check = TILE_CHECK && !viewer;
         if (tile_check && R.blk_base >= 0) {
-            int *blockers = work + kWorkHeader + kBlockerOff;
+            int *blockers = work + kWorkHeader + ar.blocker_off();
             const int tile_pos = ty * R.tiles_x + tx;
             bool full = false;
             if (warp == 0) {
@@ -1322,38 +1454,38 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                         incl += t;
                 }
                 if (lane == 31)
-                    s_wsum[warp] = incl;
+                    walk.wsum[warp] = incl;
                 __syncthreads();
                 int before = 0, total = 0;
 #pragma unroll
                 for (int w2 = 0; w2 < kWarps; ++w2) {
-                    before += w2 < warp ? s_wsum[w2] : 0;
-                    total += s_wsum[w2];
+                    before += w2 < warp ? walk.wsum[w2] : 0;
+                    total += walk.wsum[w2];
                 }
-                s_rowpre[tid] = before + incl - width;
-                s_rowx[tid] = xa;
+                walk.rowpre[tid] = before + incl - width;
+                walk.rowx[tid] = xa;
                 __syncthreads();
                 // (a) threads over cells: the cells whose bounds meet the
                 // hull are listed (box range start and length)
                 for (int c = tid; c < total; c += kThreads) {
-                    // the row of cell c: the last t with s_rowpre[t] <= c
+                    // the row of cell c: the last t with walk.rowpre[t] <= c
                     int t = 0;
 #pragma unroll
                     for (int step = kThreads / 2; step > 0; step >>= 1)
-                        if (s_rowpre[t + step] <= c)
+                        if (walk.rowpre[t + step] <= c)
                             t += step;
-                    const int cell = (r0 + t) * sc.gnx + s_rowx[t] + (c - s_rowpre[t]);
+                    const int cell = (r0 + t) * sc.gnx + walk.rowx[t] + (c - walk.rowpre[t]);
                     const int b = sc.cell_start[cell], e = sc.cell_start[cell + 1];
                     if (b == e || !swept_meets(hull, sc.cell_lo[cell], sc.cell_hi[cell]))
                         continue;
                     const int k = atomicAdd(&s_npass, 1);
                     if (k < kPassCap) {
-                        s_passb[k] = b;
-                        s_passn[k] = e - b;
+                        walk.passb[k] = b;
+                        walk.passn[k] = e - b;
                         continue;
                     }
                     for (int s = b; s < e; ++s)   // list full: this cell's boxes here
-                        add_candidate(world, hull, s, sm, s_ids, box_cap, spill, spill_slot, R, sc.n_boxes);
+                        add_candidate(world, hull, s, sm, s_ids, list_cap, spill, spill_slot, R, sc.n_boxes);
                 }
                 __syncthreads();
                 // (b) exclusive scan of the listed cells' box counts
@@ -1363,7 +1495,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
 #pragma unroll
                     for (int q = 0; q < kPassCap / kThreads; ++q) {
                         const int k = tid * (kPassCap / kThreads) + q;
-                        cnt[q] = k < n_pass ? s_passn[k] : 0;
+                        cnt[q] = k < n_pass ? walk.passn[k] : 0;
                         local += cnt[q];
                     }
                     int incl = local;
@@ -1374,35 +1506,35 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                             incl += t;
                     }
                     if (lane == 31)
-                        s_wsum2[warp] = incl;
+                        walk.wsum2[warp] = incl;
                     __syncthreads();
                     int run = 0, all = 0;
 #pragma unroll
                     for (int w2 = 0; w2 < kWarps; ++w2) {
-                        run += w2 < warp ? s_wsum2[w2] : 0;
-                        all += s_wsum2[w2];
+                        run += w2 < warp ? walk.wsum2[w2] : 0;
+                        all += walk.wsum2[w2];
                     }
                     run += incl - local;
 #pragma unroll
                     for (int q = 0; q < kPassCap / kThreads; ++q) {
                         const int k = tid * (kPassCap / kThreads) + q;
-                        s_passp[k] = k < n_pass ? run : INT_MAX;
+                        walk.passp[k] = k < n_pass ? run : INT_MAX;
                         run += cnt[q];
                     }
                     if (tid == 0)
-                        s_passp[kPassCap] = all;
+                        walk.passp[kPassCap] = all;
                 }
                 __syncthreads();
                 // (c) threads over the listed cells' boxes
-                const int n_boxes_listed = s_passp[kPassCap];
+                const int n_boxes_listed = walk.passp[kPassCap];
                 for (int i = tid; i < n_boxes_listed; i += kThreads) {
-                    // the cell of box i: the last k with s_passp[k] <= i
+                    // the cell of box i: the last k with walk.passp[k] <= i
                     int k = 0;
 #pragma unroll
                     for (int step = kPassCap / 2; step > 0; step >>= 1)
-                        if (s_passp[k + step] <= i)
+                        if (walk.passp[k + step] <= i)
                             k += step;
-                    add_candidate(world, hull, s_passb[k] + (i - s_passp[k]), sm, s_ids, box_cap, spill, spill_slot, R,
+                    add_candidate(world, hull, walk.passb[k] + (i - walk.passp[k]), sm, s_ids, list_cap, spill, spill_slot, R,
                                   sc.n_boxes);
                 }
                 if (tid == 0)
@@ -1414,7 +1546,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
         // A block without a spill region (its bounded claim gave up) keeps
         // only the candidates it staged: its request is already flagged
         // (vcm_stats.error), and it reads no region it does not own.
-        const int count = spill_slot >= 0 ? sm.count : min(sm.count, box_cap);
+        const int count = spill_slot >= 0 ? sm.count : min(sm.count, list_cap);
         const int n_smem = min(count, box_cap);
         const float4 *gbox = sc.boxes[R.perm];
         // near-first order of the staged candidates: nearby boxes block the
@@ -1455,12 +1587,12 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                 int *cls_rank = reinterpret_cast<int *>(s_box);   // s_box is free until staging
                 int *placed = cls_rank + n_smem;
                 for (int i = tid; i < kDistClasses; i += kThreads)
-                    s_hist[i] = 0;
+                    walk.hist[i] = 0;
                 __syncthreads();
                 for (int i = tid; i < n_smem; i += kThreads) {
                     const unsigned bits = (unsigned)(key_of(i) >> 32);   // float bits of d^2 >= 0
                     const int c = (int)min((unsigned)(kDistClasses - 1), bits > 0x3f800000u ? (bits - 0x3f800000u) >> 21 : 0u);
-                    cls_rank[i] = (c << 24) | atomicAdd(&s_hist[c], 1);
+                    cls_rank[i] = (c << 24) | atomicAdd(&walk.hist[c], 1);
                 }
                 __syncthreads();
                 if (warp == 0) {
@@ -1468,7 +1600,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                     int cnt[kDistClasses / 32], sum = 0;
 #pragma unroll
                     for (int q = 0; q < kDistClasses / 32; ++q) {
-                        cnt[q] = s_hist[lane * (kDistClasses / 32) + q];
+                        cnt[q] = walk.hist[lane * (kDistClasses / 32) + q];
                         sum += cnt[q];
                     }
                     int incl = sum;
@@ -1481,14 +1613,14 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                     int run = incl - sum;
 #pragma unroll
                     for (int q = 0; q < kDistClasses / 32; ++q) {
-                        s_hist[lane * (kDistClasses / 32) + q] = run;
+                        walk.hist[lane * (kDistClasses / 32) + q] = run;
                         run += cnt[q];
                     }
                 }
                 __syncthreads();
                 for (int i = tid; i < n_smem; i += kThreads) {
                     const int cr = cls_rank[i];
-                    placed[s_hist[cr >> 24] + (cr & 0xffffff)] = s_ids[i];
+                    placed[walk.hist[cr >> 24] + (cr & 0xffffff)] = s_ids[i];
                 }
                 __syncthreads();
                 for (int i = tid; i < n_smem; i += kThreads)
@@ -1503,12 +1635,6 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
         }
         cp_async_wait_all();
         __syncthreads();
-
-        // sweep: warps take the tile's viewpoints one at a time
-        unsigned long long tests = 0;     // of the warp's sweeps: a box and the 32 columns of its lanes
-        unsigned long long corners = 0;   // of the warp's sweeps
-        unsigned corner_tests = 0, rechecks = 0, shortcuts = 0;
-        float vmax = 0.f;
 
         // Whole-tile check.  For a fixed patch, the viewpoints whose segment
         // to it meets a convex box form a convex set (the box's shadow seen
@@ -1526,36 +1652,56 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                                        s_A[1][1], zq);
                 corner_tests += 16;
                 if (full && R.blk_base >= 0)   // for the tiles of this position and its neighbours
-                    work[kWorkHeader + kBlockerOff + R.blk_base + ty * R.tiles_x + tx] = s_ids[tid];
+                    work[kWorkHeader + ar.blocker_off() + R.blk_base + ty * R.tiles_x + tx] = s_ids[tid];
             }
             tile_blocked = __syncthreads_or(full) != 0;
         }
         if (tile_blocked) {
             for (int i = tid; i < tn; i += kThreads) {
-                const int ix = ix0 + i % tw, iy = iy0 + i / tw;
-                const long long vp = ((long long)layer * R.ny + iy) * R.nx + ix;
-                put_v(R, vp, 0.f);
-                if (want_bits)
-                    for (int wd = 0; wd < R.words; ++wd) {
-                        const int rem = R.P - 32 * wd;
-                        put_word(R, vp * R.words + wd, rem >= 32 ? 0xffffffffu : ((1u << rem) - 1u));
+                const int ry = (int)(((float)i + 0.5f) * inv_tw);
+                put_v(R, ((long long)layer * R.ny + iy0 + ry) * R.nx + ix0 + i - ry * tw, 0.f);
+            }
+            if (want_bits) {   // a row of the tile is one run of words
+                const int row_words = tw * R.words, rem = R.P & 31;
+                const float inv_words = 1.0f / (float)R.words;   // (exact as above: row_words < 2^20)
+                const unsigned last = rem ? (1u << rem) - 1u : 0xffffffffu;
+                for (int y = iy0; y < iy1; ++y) {
+                    const long long at = (((long long)layer * R.ny + y) * R.nx + ix0) * R.words;
+                    for (int i = tid; i < row_words; i += kThreads) {
+                        const int k = (int)(((float)i + 0.5f) * inv_words);   // viewpoint of word i
+                        put_word(R, at + i, i - k * R.words == R.words - 1 ? last : 0xffffffffu);
                     }
+                }
             }
             if (tid == 0)
                 shortcuts += (unsigned)tn;
         }
         if (viewer) {
             // viewer-centric: threads take cells, one segment each
+            unsigned long long tests = 0;
+            unsigned rechecks = 0;
+            float vmax = 0.f;
             for (int vi = tid; vi < tn; vi += kThreads) {
                 const int ry = (int)(((float)vi + 0.5f) * inv_tw), ix = ix0 + vi - ry * tw, iy = iy0 + ry;
                 const long long vp = ((long long)layer * R.ny + iy) * R.nx + ix;
                 bool blocked;
-                const float v = viewer_cell(R, s_box, n_smem, spill, count, gbox, R.x_coord[ix], R.y_coord[iy],
+                const float v = viewer_cell(R, s_box, n_smem, tail, count, gbox, R.x_coord[ix], R.y_coord[iy],
                                             R.dims == 3 ? zq : 0.f, blocked, tests, rechecks, sc.n_boxes);
                 put_v(R, vp, v);
                 if (want_bits)
                     put_word(R, vp, blocked ? 1u : 0u);
                 vmax = fmaxf(vmax, v);
+            }
+            for (int off = 16; off > 0; off >>= 1)
+                tests += __shfl_xor_sync(kFull, tests, off);
+            rechecks = __reduce_add_sync(kFull, rechecks);
+            const unsigned vmax_bits = __reduce_max_sync(kFull, __float_as_uint(vmax));   // v >= 0
+            if (lane == 0) {
+                atomicMax(&R.stats->vmax_bits, vmax_bits);
+                if (tests)
+                    atomicAdd(&R.stats->slab_tests, tests);
+                if (rechecks)
+                    atomicAdd(&R.stats->rechecked, (unsigned long long)rechecks);
             }
         }
         // First every viewpoint gets the one-box check, four per warp with
@@ -1616,32 +1762,25 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
         }
         __syncthreads();
         int n_und = (viewer || tile_blocked) ? 0 : sm.n_und;
-        // Work sharing, first pass (share == 1): a tile with at least
-        // R.min_publish open viewpoints publishes them, in chunks of up to
-        // R.chunk_vp, with its candidate list (when the list is staged
-        // whole), and the second pass sweeps them.  Without it a few hundred
-        // tiles of mostly visible viewpoints set the end of the launch (3D
-        // workload: 100-290 us each against 17 us for the median tile).  A
-        // tile with a list longer than kPublishBoxes publishes only with at
-        // least kPublishHeavy open viewpoints (each chunk stages the list
-        // again; a spilled list's tail is read from the record), and a tile
-        // whose publication would pass a cap of the arena keeps its
-        // viewpoints.
-        if (share == 1 && spill_slot >= 0 && n_und >= R.min_publish &&
-            (count <= kPublishBoxes || n_und >= kPublishHeavy)) {
+        // Work sharing (share == 1): the tile's open viewpoints go to the
+        // second pass in chunks, with the tile's candidate list: swept here,
+        // a few hundred tiles of mostly visible viewpoints set the end of the
+        // launch (100-290 us each against 17 us for the median tile).  What
+        // would pass a cap of the arena stays.
+        if (share == 1 && spill_slot >= 0 && n_und > 0) {
             int *arena = work + kWorkHeader;
-            const int cvp = R.chunk_vp;
             if (tid == 0) {
-                const int want = (n_und + cvp - 1) / cvp;
-                int rec = kRecCap, base = 0, got = 0, off = 0;
+                const int want = (n_und + kChunkVp - 1) / kChunkVp;
+                int rec = ar.rec_cap, base = 0, got = 0, off = 0;
                 // counters move only while their caps are not reached
-                if (__ldcg(work + 1) < kRecCap && __ldcg(work + 4) < kPoolInts && __ldcg(work + 2) < kChunkCap) {
+                if (__ldcg(work + 1) < ar.rec_cap && __ldcg(work + 4) < ar.pool_ints &&
+                    __ldcg(work + 2) < ar.chunk_cap) {
                     rec = atomicAdd(work + 1, 1);
-                    if (rec < kRecCap) {
+                    if (rec < ar.rec_cap) {
                         off = atomicAdd(work + 4, count);
-                        if (off <= kPoolInts - count) {
+                        if (off <= ar.pool_ints - count) {
                             base = atomicAdd(work + 2, want);
-                            got = max(0, min(want, kChunkCap - base));
+                            got = max(0, min(want, ar.chunk_cap - base));
                         }
                     }
                 }
@@ -1649,7 +1788,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                 sm.pub[1] = base;
                 sm.pub[2] = got;
                 sm.pub[3] = off;
-                s_next2 = min(n_und, got * cvp);   // the tile keeps the rest
+                s_next2 = min(n_und, got * kChunkVp);   // the tile keeps the rest
                 if (got > 0)
                     atomicAdd(&R.stats->shared_viewpoints, (unsigned long long)s_next2);
             }
@@ -1657,8 +1796,8 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
             const int pub_n = sm.pub[2];
             if (pub_n > 0) {
                 const int rec = sm.pub[0], pub_base = sm.pub[1], off = sm.pub[3];
-                int *rp = arena + kRecOff + (size_t)kRecInts * rec;
-                int *ids = arena + kPoolOff + off;
+                int *rp = arena + ar.rec_off() + (size_t)kRecInts * rec;
+                int *ids = arena + ar.pool_off() + off;
                 if (tid == 0) {
                     rp[0] = s_req_idx;
                     rp[1] = count;
@@ -1668,87 +1807,27 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                     rp[5] = iy0;
                 }
                 for (int i = tid; i < count; i += kThreads)
-                    ids[i] = i < n_smem ? s_ids[i] : spill[i - n_smem];
+                    ids[i] = i < n_smem ? s_ids[i] : tail[i - n_smem];
                 for (int i = tid; i < pub_n * kChunkInts; i += kThreads) {
-                    const int j = i / kChunkInts, r = i - j * kChunkInts, k = j * cvp + 2 * (r - 2);
-                    const int n_j = min(cvp, n_und - j * cvp);
+                    const int j = i / kChunkInts, r = i - j * kChunkInts, k = j * kChunkVp + 2 * (r - 1);
+                    const int n_j = min(kChunkVp, n_und - j * kChunkVp);
                     const unsigned a = s_und[min(max(k, 0), kMaxTileViewpoints - 1)];
                     const unsigned b = s_und[min(max(k + 1, 0), kMaxTileViewpoints - 1)];
-                    arena[kChunkOff + (size_t)kChunkInts * (pub_base + j) + r] = r == 0 ? rec : r == 1 ? n_j : (int)(a | (b << 16));
+                    arena[(size_t)kChunkInts * (pub_base + j) + r] =
+                        r == 0 ? rec * 32 + n_j : (int)(a | (b << 16));
                 }
             }
         }
-        // then the undecided viewpoints, one per warp at a time
-        const LaneMap M = lane_map(R);
-        for (;;) {
-            int k = 0;
-            if (lane == 0)
-                k = atomicAdd(&s_next2, 1);
-            k = __shfl_sync(kFull, k, 0);
-            if (k >= n_und)
-                break;
-            {
-                const int ix = ix0 + (s_und[k] & 255), iy = iy0 + (s_und[k] >> 8);
-                const long long vp = ((long long)layer * R.ny + iy) * R.nx + ix;
-                const float qx = R.x_coord[ix], qy = R.y_coord[iy];
-                const float qu = R.au == 0 ? qx : (R.au == 1 ? qy : zq);
-                const float qn = R.an == 0 ? qx : (R.an == 1 ? qy : zq);
-                const float qw = R.dims == 3 ? (R.aw == 0 ? qx : (R.aw == 1 ? qy : zq)) : 0.f;
-                const bool front = facing(R, qn);
-                unsigned vp_tests = 0, vp_corners = 0;
-                float v = sweep_viewpoint<EXTRA>(R, M, s_box, n_smem, spill, count, gbox, qu, qn, qw, front, vp,
-                                                 s_warp[warp], vp_tests, vp_corners, rechecks, sc.n_boxes);
-                tests += vp_tests;
-                corners += vp_corners;
-                if (v < 0.f) {   // one box blocks every patch
-                    if (lane == 0) {
-                        put_v(R, vp, 0.f);
-                        ++shortcuts;
-                    }
-                    if (want_bits)
-                        for (int wd = lane; wd < R.words; wd += 32) {
-                            const int rem = R.P - 32 * wd;
-                            put_word(R, vp * R.words + wd, rem >= 32 ? 0xffffffffu : ((1u << rem) - 1u));
-                        }
-                    continue;
-                }
-                if (!front)
-                    v = 0.f;
-                if (lane == 0)
-                    put_v(R, vp, v);
-                vmax = fmaxf(vmax, v);
-            }
-        }
-        // per-tile counters
-        corner_tests = __reduce_add_sync(kFull, corner_tests);
-        shortcuts = __reduce_add_sync(kFull, shortcuts);
-        rechecks = __reduce_add_sync(kFull, rechecks);
-        if (viewer) {   // the lanes' own cells
-            for (int off = 16; off > 0; off >>= 1)
-                tests += __shfl_xor_sync(kFull, tests, off);
-        } else {
-            tests *= 32;
-        }
-        corners += corner_tests;
-        const unsigned vmax_bits = __reduce_max_sync(kFull, __float_as_uint(vmax));   // v >= 0
-        if (lane == 0) {
-            if (vmax_bits)
-                atomicMax(&R.stats->vmax_bits, vmax_bits);
-            if (tests)
-                atomicAdd(&R.stats->slab_tests, tests);
-            if (corners)
-                atomicAdd(&R.stats->corner_tests, corners);
-            if (shortcuts)
-                atomicAdd(&R.stats->shortcut_viewpoints, (unsigned long long)shortcuts);
-            if (rechecks)
-                atomicAdd(&R.stats->rechecked, (unsigned long long)rechecks);
-        }
+        if (s_next2 < n_und)
+            sweep_kept(R, s_scratch, s_box, n_smem, tail, count, gbox, s_und, &s_next2, n_und, ix0, iy0, layer,
+                       sc.n_boxes);
         if (tid == 0) {
-            atomicAdd(&R.stats->boxes_listed, (unsigned long long)count);
+            listed += (unsigned)count;
             sm.item = -2;   // one_tile: the next round exits
         }
         __syncthreads();
     }
+    flush();
     if (one_tile && tid == 0 && spill_slot >= 0)
         atomicExch(&spill_busy[spill_slot], 0);
 }
@@ -1770,7 +1849,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
 // -> 5.20 ms.  7 blocks per SM: 6 were 3 %, 5 13 % slower on the batch, 8 spill.
 template <bool EXTRA>
 __global__ void __launch_bounds__(kThreads, kSweepBlocks)
-k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work)
+k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work, Arena ar)
 {
     struct Mine {   // one warp's: a single base address, the rest are constant offsets
         WarpScratch scratch;
@@ -1786,10 +1865,10 @@ k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work
     DevRequest &R = mine.req;
     float4 *boxes = mine.boxes;
     const int *arena = work + kWorkHeader;
-    const int n_chunks = min(work[2], kChunkCap);
+    const int n_chunks = min(work[2], ar.chunk_cap);
     const int warps = (int)gridDim.x * kWarps;
-    int part_log = 1;   // parts per chunk
-    while (part_log < 5 && (n_chunks << part_log) < kPartsPerWarp * warps)
+    int part_log = 0;   // parts per chunk
+    while (part_log < 4 && (n_chunks << part_log) < kPartsPerWarp * warps)
         ++part_log;
     const int part_vp = kChunkVp >> part_log;
     const volatile int *list = mine.list;   // read where it is used: registers are scarce in the sweep
@@ -1805,20 +1884,20 @@ k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work
         item = __shfl_sync(kFull, item, 0);
         if ((item >> part_log) >= n_chunks)
             break;
-        const int *chunk = arena + kChunkOff + (size_t)kChunkInts * (item >> part_log);
-        const int rec = chunk[0];
-        const int first = (item & ((1 << part_log) - 1)) * part_vp, n = min(chunk[1] - first, part_vp);
+        const int *chunk = arena + (size_t)kChunkInts * (item >> part_log);
+        const int rec = chunk[0] >> 5;
+        const int first = (item & ((1 << part_log) - 1)) * part_vp, n = min((chunk[0] & 31) - first, part_vp);
         if (n <= 0)
             continue;
         __syncwarp();   // the viewpoints before are done with the item's shared memory
         if (lane < n)
-            mine.xy[lane] = reinterpret_cast<const unsigned short *>(chunk + 2)[first + lane];
+            mine.xy[lane] = reinterpret_cast<const unsigned short *>(chunk + 1)[first + lane];
         if (rec != cur_rec) {
             cur_rec = rec;
             const int old_req = list[0];
             __syncwarp();
             if (lane < 8)
-                mine.list[lane] = arena[kRecOff + (size_t)kRecInts * rec + lane];
+                mine.list[lane] = arena[ar.rec_off() + (size_t)kRecInts * rec + lane];
             __syncwarp();
             if (list[0] != old_req) {
                 const int *src = reinterpret_cast<const int *>(reqs + list[0]);
@@ -1829,7 +1908,7 @@ k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work
             }
             const float4 *gbox = sc.boxes[R.perm];
             for (int i = lane; i < min(list[1], kWarpBoxes); i += 32) {
-                const int id = arena[kPoolOff + list[2] + i];
+                const int id = arena[ar.pool_off() + list[2] + i];
                 boxes[2 * i] = __ldg(&gbox[2 * id]);
                 boxes[2 * i + 1] = __ldg(&gbox[2 * id + 1]);
             }
@@ -1839,29 +1918,11 @@ k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work
         unsigned tests = 0, corners = 0, rechecks = 0, shortcuts = 0;
         float vmax = 0.f;
         for (int k = 0; k < n; ++k) {
-            const int at = mine.xy[k];
-            const int ix = list[4] + (at & 255), iy = list[5] + (at >> 8);
-            const long long vp = ((long long)list[3] * R.ny + iy) * R.nx + ix;
-            const float qx = R.x_coord[ix], qy = R.y_coord[iy], zq = R.z_coord[list[3]];
-            const float qu = R.au == 0 ? qx : (R.au == 1 ? qy : zq);
-            const float qn = R.an == 0 ? qx : (R.an == 1 ? qy : zq);
-            const float qw = R.dims == 3 ? (R.aw == 0 ? qx : (R.aw == 1 ? qy : zq)) : 0.f;
-            const bool front = facing(R, qn);
-            const int count = list[1];
-            float v = sweep_viewpoint<EXTRA>(R, M, boxes, kWarpBoxes, arena + kPoolOff + list[2] + kWarpBoxes, count,
-                                             sc.boxes[R.perm], qu, qn, qw, front, vp, W, tests, corners, rechecks,
+            const int at = mine.xy[k], layer = list[3];
+            const float v = sweep_one<EXTRA>(R, M, list[4] + (at & 255), list[5] + (at >> 8), layer, R.z_coord[layer],
+                                             want_bits, boxes, kWarpBoxes,
+                                             Tail{arena + ar.pool_off() + list[2] + kWarpBoxes, 4}, list[1], sc.boxes[R.perm], W, tests, corners, rechecks, shortcuts,
                                              sc.n_boxes);
-            if (v < 0.f) {   // one box blocks every patch
-                ++shortcuts;
-                if (want_bits)
-                    for (int wd = lane; wd < R.words; wd += 32) {
-                        const int rem = R.P - 32 * wd;
-                        put_word(R, vp * R.words + wd, rem >= 32 ? 0xffffffffu : ((1u << rem) - 1u));
-                    }
-            }
-            v = front ? fmaxf(v, 0.f) : 0.f;
-            if (lane == 0)
-                put_v(R, vp, v);
             vmax = fmaxf(vmax, v);
         }
         rechecks = __reduce_add_sync(kFull, rechecks);
@@ -2127,11 +2188,10 @@ cudaError_t init_device()
         return e;
     if (dev >= 0 && dev < 64 && done[dev])
         return cudaSuccess;
-    const void *kernels[4] = {(const void *)k_tiles<false, false>, (const void *)k_tiles<true, false>,
-                              (const void *)k_tiles<false, true>, (const void *)k_tiles<true, true>};
+    const void *kernels[2] = {(const void *)k_tiles<false>, (const void *)k_tiles<true>};
     for (const void *k : kernels)
         if ((e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)tiles_smem_bytes(kMaxBoxCap))) != cudaSuccess)
+                                      (int)tiles_smem_bytes(kMaxBoxCap, kMaxBoxCap))) != cudaSuccess)
             return e;
     if (dev >= 0 && dev < 64)
         done[dev] = true;
@@ -2207,21 +2267,23 @@ cudaError_t launch_grid_build(const float *d_lo_world, const float *d_hi_world, 
     return cudaGetLastError();
 }
 
-int tiles_blocks_per_sm(int box_cap)
+int tiles_blocks_per_sm(int box_cap, int list_cap)
 {
-    // the tile pass's instantiations share their launch bounds (6 blocks of kThreads)
+    // the tile pass's instantiations share their launch bounds
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_tiles<false, false>, kThreads,
-                                                      tiles_smem_bytes(box_cap)) !=
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_tiles<false>, kThreads,
+                                                      tiles_smem_bytes(box_cap, std::max(list_cap, box_cap))) !=
         cudaSuccess)
         return 1;
     return n > 0 ? n : 1;
 }
 
+int spill_id_bytes(int n_boxes) { return n_boxes < (1 << 24) ? 3 : 4; }
+
 cudaError_t launch_tiles(const DevScene &sc, const DevRequest *d_reqs, const int *d_tile_prefix,
                          int n_req, int total_tiles, int *d_work, int *d_spill, int grid_blocks,
                          int box_cap, bool extra, bool tile_check, int sm_count, cudaStream_t stream, bool one_tile,
-                         int *d_spill_busy, bool share, int claim_rounds)
+                         int *d_spill_busy, bool share, int claim_rounds, const Arena &arena, int list_cap)
 {
     if (claim_rounds < 1 || claim_rounds > kClaimRounds)
         return cudaErrorInvalidValue;
@@ -2229,25 +2291,26 @@ cudaError_t launch_tiles(const DevScene &sc, const DevRequest *d_reqs, const int
         return cudaSuccess;
     if (box_cap < 1 || box_cap > kMaxBoxCap)
         return cudaErrorInvalidValue;
-    const size_t smem = tiles_smem_bytes(box_cap);
+    list_cap = std::max(list_cap, box_cap);
+    const size_t smem = tiles_smem_bytes(box_cap, list_cap);
     const int slots = grid_blocks;   // spill regions: the resident-block bound
     if (one_tile) {
         if (!d_spill_busy)
             return cudaErrorInvalidValue;
         grid_blocks = total_tiles;
     }
-    auto kernel = extra ? (tile_check ? k_tiles<true, true> : k_tiles<true, false>)
-                        : (tile_check ? k_tiles<false, true> : k_tiles<false, false>);
+    auto kernel = tile_check ? k_tiles<true> : k_tiles<false>;
     share = share && !one_tile;
-    kernel<<<grid_blocks, kThreads, smem, stream>>>(sc, d_reqs, d_tile_prefix, n_req, total_tiles, d_work, d_spill,
-                                                    box_cap, one_tile ? 1 : 0, d_spill_busy, slots, share ? 1 : 0,
+    kernel<<<grid_blocks, kThreads, smem, stream>>>(sc, d_reqs, d_tile_prefix, n_req, total_tiles, d_work, arena,
+                                                    reinterpret_cast<unsigned char *>(d_spill),
+                                                    spill_id_bytes(sc.n_boxes), box_cap, list_cap, one_tile ? 1 : 0, d_spill_busy, slots, share ? 1 : 0,
                                                     claim_rounds);
     if (share) {
         // the second pass, on every SM
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess)
             return e;
-        (extra ? k_sweep<true> : k_sweep<false>)<<<sm_count * kSweepBlocks, kThreads, 0, stream>>>(sc, d_reqs, d_work);
+        (extra ? k_sweep<true> : k_sweep<false>)<<<sm_count * kSweepBlocks, kThreads, 0, stream>>>(sc, d_reqs, d_work, arena);
     }
     return cudaGetLastError();
 }
