@@ -901,7 +901,7 @@ struct Prepared {
     int blocks = 0;
     size_t n = 0;
     bool extra = false;   // a request is two-sided or has a field-of-view cone
-    bool tile_check = false;   // every request has many patches: whole-tile check
+    bool tile_check = false;   // every request has many patches: recorded blockers
 };
 
 bool needs_extra(const Canon &c) { return c.cone || (c.flags & VCM_TWO_SIDED); }

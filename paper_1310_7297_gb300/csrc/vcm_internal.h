@@ -14,16 +14,19 @@ constexpr int kWarps = 4;                 // warps per block of the tile kernel
 constexpr int kThreads = kWarps * 32;
 constexpr int kPassCap = 2 * kThreads;       // cells listed per round of the grid walk
 constexpr int kDistClasses = 128;            // distance classes of the candidate counting sort
-// Launches whose requests all have this many patches use the whole-tile
-// check (and the recorded-blocker pre-check): from 512, the 5,000-box step
-// with 32 x 16 patches went 0.319 -> 0.305 ms (the bar was 1,024).
-constexpr int kTileCheckMinPatches = 512;
+// Launches whose requests all have this many patches look at recorded blockers
+// before a tile's cull.  With the node checks it pays where lists are long and
+// walks deep (100,000 boxes, 64 x 32 patches: 1.51 -> 1.42 ms on a mostly
+// hidden target, 3.40 -> 3.46 ms on a mostly visible one); at 512 patches it
+// cost 4 % (5,000 boxes: 0.189 -> 0.197 ms).
+constexpr int kTileCheckMinPatches = 1024;
 constexpr float kBand = 1e-6f;            // FP32 slab margin re-decided in FP64
 constexpr int kMaxBoxCap = 5000;          // candidate boxes a tile stages in shared memory
 constexpr int kRowCap = 256;              // patch rows a warp stages for the measure
 constexpr int kWarpBoxes = 64;            // boxes of a chunk's list a warp stages
 constexpr int kTileBlocks = 8;            // blocks per SM of the tile pass
 constexpr long long kTileWaves = 3;         // waves of resident blocks below which a launch's tiles shrink
+constexpr int kNodeBoxes = 64;             // nearest candidates that the tile's nodes test
 constexpr int kKeptWarps = 2;             // warps that sweep the viewpoints a tile keeps
 constexpr int kSweepBlocks = 7;           // blocks per SM of the second pass
 constexpr int kPartsPerWarp = 4;          // parts of chunks the second pass wants per warp
@@ -39,7 +42,7 @@ constexpr int kClaimRounds = 4096;        // bounded retries of a spill-region c
 //   chunk[kChunkCap][kChunkInts]     32 x record index + count, viewpoints (x + 256 y in the tile, 16 bits each)
 //   record[kRecCap][kRecInts]        request, candidate count, offset of its ids in the pool, layer, tile origin
 //   pool[kPoolInts]                  the records' candidate box ids, in the owner's order
-//   blocker[kBlockerCap]             per tile position of each request (whole-tile-check
+//   blocker[kBlockerCap]             per tile position of each request (many-patch
 //                                    launches): a box id that blocked a tile there, or -1
 // A tile whose publication would pass a cap keeps its viewpoints.
 constexpr int kChunkVp = 16;
@@ -155,7 +158,7 @@ cudaError_t launch_grid_build(const float *d_lo_world, const float *d_hi_world, 
 // grid_blocks regions of spill_region_bytes for candidate lists longer than box_cap.
 // `extra` must be set when any request is two-sided or has a field-of-view
 // cone: it selects the tile kernel's instantiation that handles them.
-// `tile_check` selects the instantiation with the whole-tile check (any
+// `tile_check` selects the instantiation that looks at recorded blockers (any
 // launch may use either; it pays when every request has many patches).
 // `share` (persistent launches only): d_work holds `arena` behind its header
 // (kWorkBytes for the default one), and a second
