@@ -528,7 +528,7 @@ struct vcm_ctx {
     bool built = false;
     unsigned long long scene_gen = 0;   // bumped by every vcm_build
     float4 *d_perm[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
-    int *d_cell_start = nullptr, *d_cell_of = nullptr, *d_count = nullptr, *d_cursor = nullptr, *d_order = nullptr;
+    int *d_cell_start = nullptr, *d_cell_of = nullptr, *d_count = nullptr, *d_order = nullptr;
     float4 *d_cell_lo = nullptr, *d_cell_hi = nullptr;
     unsigned *d_overhang = nullptr;
     DevScene scene{};
@@ -1090,14 +1090,13 @@ void free_scene(vcm_ctx *ctx)
     cudaFree(ctx->d_cell_start);
     cudaFree(ctx->d_cell_of);
     cudaFree(ctx->d_count);
-    cudaFree(ctx->d_cursor);
     cudaFree(ctx->d_order);
     cudaFree(ctx->d_cell_lo);
     cudaFree(ctx->d_cell_hi);
     cudaFree(ctx->d_overhang);
     cudaFree(ctx->d_recolor_list);
     cudaFree(ctx->d_recolor_n);
-    ctx->d_cell_start = ctx->d_cell_of = ctx->d_count = ctx->d_cursor = ctx->d_order = nullptr;
+    ctx->d_cell_start = ctx->d_cell_of = ctx->d_count = ctx->d_order = nullptr;
     ctx->d_cell_lo = ctx->d_cell_hi = nullptr;
     ctx->d_overhang = nullptr;
     ctx->lo_cap = ctx->idx_box_cap = ctx->idx_cell_cap = 0;
@@ -2059,15 +2058,13 @@ vcm_status vcm_build(vcm_ctx *ctx, float grid_cell_m)
         if ((size_t)n_cells + 1 > ctx->idx_cell_cap) {
             cudaFree(ctx->d_cell_start);
             cudaFree(ctx->d_count);
-            cudaFree(ctx->d_cursor);
             cudaFree(ctx->d_cell_lo);
             cudaFree(ctx->d_cell_hi);
-            ctx->d_cell_start = ctx->d_count = ctx->d_cursor = nullptr;
+            ctx->d_cell_start = ctx->d_count = nullptr;
             ctx->d_cell_lo = ctx->d_cell_hi = nullptr;
             ctx->idx_cell_cap = 0;
             CUDA_TRY(cudaMalloc(&ctx->d_cell_start, sizeof(int) * (n_cells + 1)));
             CUDA_TRY(cudaMalloc(&ctx->d_count, sizeof(int) * n_cells));
-            CUDA_TRY(cudaMalloc(&ctx->d_cursor, sizeof(int) * n_cells));
             CUDA_TRY(cudaMalloc(&ctx->d_cell_lo, sizeof(float4) * n_cells));
             CUDA_TRY(cudaMalloc(&ctx->d_cell_hi, sizeof(float4) * n_cells));
             ctx->idx_cell_cap = (size_t)n_cells + 1;
@@ -2075,7 +2072,7 @@ vcm_status vcm_build(vcm_ctx *ctx, float grid_cell_m)
         if (!ctx->d_overhang)
             CUDA_TRY(cudaMalloc(&ctx->d_overhang, sizeof(unsigned)));
         CUDA_TRY(launch_grid_build(ctx->d_lo, ctx->d_hi, (int)n, ctx->dims, (float)x0, (float)y0, (float)cell, gnx,
-                                   gny, ctx->d_cell_of, ctx->d_count, ctx->d_cursor, ctx->d_order,
+                                   gny, ctx->d_cell_of, ctx->d_count, ctx->d_order,
                                    ctx->d_cell_start, ctx->d_perm, ctx->d_cell_lo, ctx->d_cell_hi,
                                    ctx->d_overhang, ctx->aux));
         CUDA_TRY(cudaStreamSynchronize(ctx->aux));
@@ -2610,7 +2607,6 @@ vcm_status vcm_compute_static(const float *lo, const float *hi, uint32_t n_boxes
         int *s_cell_of = reinterpret_cast<int *>(take(nb * sizeof(int)));
         int *s_order = reinterpret_cast<int *>(take(nb * sizeof(int)));
         int *s_count = reinterpret_cast<int *>(take((size_t)n_cells * sizeof(int)));
-        int *s_cursor = reinterpret_cast<int *>(take((size_t)n_cells * sizeof(int)));
         int *s_start = reinterpret_cast<int *>(take((size_t)(n_cells + 1) * sizeof(int)));
         float4 *s_cell_lo = reinterpret_cast<float4 *>(take((size_t)n_cells * sizeof(float4)));
         float4 *s_cell_hi = reinterpret_cast<float4 *>(take((size_t)n_cells * sizeof(float4)));
@@ -2635,7 +2631,7 @@ vcm_status vcm_compute_static(const float *lo, const float *hi, uint32_t n_boxes
         CUDA_TRY(cudaMemcpyAsync(s_lo, L.data(), nb * 3 * sizeof(float), cudaMemcpyHostToDevice, sm));
         CUDA_TRY(cudaMemcpyAsync(s_hi, H.data(), nb * 3 * sizeof(float), cudaMemcpyHostToDevice, sm));
         CUDA_TRY(launch_grid_build(s_lo, s_hi, (int)n, dims, (float)x0, (float)y0, (float)cell, gnx, gny, s_cell_of,
-                                   s_count, s_cursor, s_order, s_start, s_perm, s_cell_lo, s_cell_hi, s_overhang, sm));
+                                   s_count, s_order, s_start, s_perm, s_cell_lo, s_cell_hi, s_overhang, sm));
         DevScene sc{};
         for (int p = 0; p < 6; ++p)
             sc.boxes[p] = s_perm[p];

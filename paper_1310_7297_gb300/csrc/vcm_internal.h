@@ -144,7 +144,7 @@ struct DevRequest {
 // `stream` and return the launch status.
 cudaError_t launch_grid_build(const float *d_lo_world, const float *d_hi_world, int n, int dims,
                               float gx0, float gy0, float cell, int gnx, int gny,
-                              int *d_cell_of, int *d_count, int *d_cursor, int *d_order,
+                              int *d_cell_of, int *d_count, int *d_order,
                               int *d_cell_start, float4 *const *d_perm_boxes, float4 *d_cell_lo,
                               float4 *d_cell_hi, unsigned *d_overhang_bits, cudaStream_t stream);
 

@@ -1,7 +1,7 @@
 // vcm_kernels.cu -- sm_103a kernels of the visibility color map engine.
 //
 //  * grid build: boxes bucketed by footprint centre into a uniform 2D grid
-//    (count -> scan -> scatter -> per-cell sort -> permuted copies -> bounds);
+//    (count -> scan -> scatter -> permuted copies in box order -> bounds);
 //  * tile kernel: persistent blocks draw viewpoint tiles from a queue; each
 //    tile culls the scene against the convex hull of (tile, target) using
 //    the grid, stages the candidates in shared memory with cp.async, and its
@@ -146,6 +146,57 @@ __global__ void k_box_cell(const float *__restrict__ lo, const float *__restrict
     atomicAdd(&count[c], 1);
 }
 
+// Exclusive scan of count[0..n) into start[0..n] by one block, for at most
+// kScanOneMax cells: 4,096 a round, 4 per thread.  At these sizes the three
+// kernels below are three launch latencies (15 us against 5).
+constexpr int kScanOneThreads = 1024;
+constexpr int kScanOneMax = 65536;
+__global__ void __launch_bounds__(kScanOneThreads) k_scan_one(const int *__restrict__ count, int n,
+                                                              int *__restrict__ start)
+{
+    __shared__ int s_warp[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int carry = 0;
+    for (int base = 0; base < n; base += 4 * kScanOneThreads) {
+        const int i = base + 4 * threadIdx.x;
+        int v[4], local = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            v[k] = i + k < n ? count[i + k] : 0;
+            local += v[k];
+        }
+        int incl = local;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int t = __shfl_up_sync(kFull, incl, off);
+            if (lane >= off)
+                incl += t;
+        }
+        if (lane == 31)
+            s_warp[warp] = incl;
+        __syncthreads();
+        const int w = s_warp[lane];
+        int wincl = w;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const int t = __shfl_up_sync(kFull, wincl, off);
+            if (lane >= off)
+                wincl += t;
+        }
+        int run = carry + incl - local + __shfl_sync(kFull, wincl - w, warp);
+        carry += __shfl_sync(kFull, wincl, 31);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (i + k < n)
+                start[i + k] = run;
+            run += v[k];
+        }
+        __syncthreads();   // s_warp is reused
+    }
+    if (threadIdx.x == 0)
+        start[n] = carry;
+}
+
 // Exclusive scan of count[0..n) into start[0..n] in three kernels: block
 // sums of kScanChunk elements, a one-block scan of the block sums (at most
 // 1024 of them: n <= 4M cells), then each block's scan with its offset.
@@ -236,90 +287,45 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_down(const int *__restric
     }
 }
 
+// Each box takes a place in its cell, in any order (the counts run down to 0).
 __global__ void k_scatter(const int *__restrict__ cell_of, int n, const int *__restrict__ start,
-                          int *__restrict__ cursor, int *__restrict__ order)
+                          int *__restrict__ count, int *__restrict__ order)
 {
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n)
         return;
     int c = cell_of[i];
-    int pos = start[c] + atomicAdd(&cursor[c], 1);
-    order[pos] = i;
+    order[start[c] + atomicSub(&count[c], 1) - 1] = i;
 }
-
-// Deterministic order inside each cell: ascending box index (the scatter's
-// atomics leave it arbitrary).  Blocks take contiguous ranges of cells, a
-// thread each: a cell of at most kSmallCell boxes is sorted in place by its
-// thread; larger cells are listed, and the whole block sorts each of them by
-// rank (the rank of an id is the number of smaller ids in its cell; ids are
-// unique), writing to `tmp` (free after the scatter) and copying back.
-constexpr int kSmallCell = 32;
-
-__global__ void __launch_bounds__(kScanThreads) k_sort_cells(const int *__restrict__ start, int n_cells,
-                                                             int *__restrict__ order, int *__restrict__ tmp)
-{
-    __shared__ int s_big[kScanThreads];
-    __shared__ int s_n_big;
-    for (int c0 = blockIdx.x * kScanThreads; c0 < n_cells; c0 += gridDim.x * kScanThreads) {
-        if (threadIdx.x == 0)
-            s_n_big = 0;
-        __syncthreads();
-        const int c = c0 + threadIdx.x;
-        if (c < n_cells) {
-            const int b = start[c], e = start[c + 1];
-            if (e - b > kSmallCell) {
-                s_big[atomicAdd(&s_n_big, 1)] = c;
-            } else {
-                for (int i = b + 1; i < e; ++i) {
-                    const int v = order[i];
-                    int j = i - 1;
-                    while (j >= b && order[j] > v) {
-                        order[j + 1] = order[j];
-                        --j;
-                    }
-                    order[j + 1] = v;
-                }
-            }
-        }
-        __syncthreads();
-        const int n_big = s_n_big;
-        for (int k = 0; k < n_big; ++k) {
-            const int cb = s_big[k];
-            const int b = start[cb], e = start[cb + 1];
-            for (int i = b + threadIdx.x; i < e; i += kScanThreads) {
-                const int v = order[i];
-                int rank = 0;
-                for (int j = b; j < e; ++j)
-                    rank += order[j] < v;
-                tmp[b + rank] = v;
-            }
-            __syncthreads();
-            for (int i = b + threadIdx.x; i < e; i += kScanThreads)
-                order[i] = tmp[i];
-            __syncthreads();
-        }
-    }
-}
-
-__constant__ int c_perm[6][3] = {{0, 1, 2}, {0, 2, 1}, {1, 0, 2}, {1, 2, 0}, {2, 0, 1}, {2, 1, 0}};
 
 struct PermPtrs {
     float4 *p[6];
 };
 
+// The permuted copies, in ascending box index inside each cell (the scatter's
+// atomics leave the order arbitrary): a box's place is the number of smaller
+// indices in its cell, counted by its thread.  Cells hold a few boxes, and in a
+// crowded one the threads of a warp read the same list.  (Sorting the cells in
+// place first, a thread each, was a kernel of 18 us of dependent loads.)
 __global__ void k_write_boxes(const float *__restrict__ lo, const float *__restrict__ hi, int n,
+                              const int *__restrict__ cell_of, const int *__restrict__ start,
                               const int *__restrict__ order, PermPtrs out)
 {
-    int s = blockIdx.x * blockDim.x + threadIdx.x;
-    if (s >= n)
+    int at = blockIdx.x * blockDim.x + threadIdx.x;
+    if (at >= n)
         return;
-    int id = order[s];
-    float L[3] = {lo[3 * id], lo[3 * id + 1], lo[3 * id + 2]};
-    float H[3] = {hi[3 * id], hi[3 * id + 1], hi[3 * id + 2]};
+    const int id = order[at], c = cell_of[id];
+    const int b = start[c], e = start[c + 1];
+    const float L[3] = {lo[3 * id], lo[3 * id + 1], lo[3 * id + 2]};
+    const float H[3] = {hi[3 * id], hi[3 * id + 1], hi[3 * id + 2]};
+    int s = b;
+    for (int j = b; j < e; ++j)
+        s += order[j] < id;
+#pragma unroll
     for (int p = 0; p < 6; ++p) {
-        const int *a = c_perm[p];
-        out.p[p][2 * s] = make_float4(L[a[0]], L[a[1]], L[a[2]], __int_as_float(id));
-        out.p[p][2 * s + 1] = make_float4(H[a[0]], H[a[1]], H[a[2]], 0.f);
+        const int a0 = p >> 1, a1 = (p & 1) ? (a0 == 2 ? 1 : 2) : (a0 == 0 ? 1 : 0), a2 = 3 - a0 - a1;
+        out.p[p][2 * s] = make_float4(L[a0], L[a1], L[a2], __int_as_float(id));
+        out.p[p][2 * s + 1] = make_float4(H[a0], H[a1], H[a2], 0.f);
     }
 }
 
@@ -328,26 +334,30 @@ __global__ void k_cell_bounds(const float4 *__restrict__ boxes, const int *__res
                               float4 *__restrict__ cell_lo, float4 *__restrict__ cell_hi,
                               unsigned *__restrict__ overhang_bits)
 {
-    int c = blockIdx.x * blockDim.x + threadIdx.x;
-    if (c >= gnx * gny)
-        return;
+    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    const bool in = c < gnx * gny;
     float4 lo = make_float4(f_inf(), f_inf(), f_inf(), 0.f);
     float4 hi = make_float4(-f_inf(), -f_inf(), -f_inf(), 0.f);
-    int b = start[c], e = start[c + 1];
+    const int b = in ? start[c] : 0, e = in ? start[c + 1] : 0;
     for (int s = b; s < e; ++s) {
         float4 l = boxes[2 * s], h = boxes[2 * s + 1];
         lo.x = fminf(lo.x, l.x); lo.y = fminf(lo.y, l.y); lo.z = fminf(lo.z, l.z);
         hi.x = fmaxf(hi.x, h.x); hi.y = fmaxf(hi.y, h.y); hi.z = fmaxf(hi.z, h.z);
     }
-    cell_lo[c] = lo;
-    cell_hi[c] = hi;
-    if (e > b) {
-        int ix = c % gnx, iy = c / gnx;
-        float x0 = gx0 + ix * cell, y0 = gy0 + iy * cell;
-        float oh = fmaxf(fmaxf(x0 - lo.x, hi.x - (x0 + cell)), fmaxf(y0 - lo.y, hi.y - (y0 + cell)));
-        oh = fmaxf(oh, 0.f);
-        atomicMax(overhang_bits, __float_as_uint(oh));
+    if (in) {
+        cell_lo[c] = lo;
+        cell_hi[c] = hi;
     }
+    float oh = 0.f;
+    if (e > b) {
+        const int ix = c % gnx, iy = c / gnx;
+        const float x0 = gx0 + ix * cell, y0 = gy0 + iy * cell;
+        oh = fmaxf(fmaxf(x0 - lo.x, hi.x - (x0 + cell)), fmaxf(y0 - lo.y, hi.y - (y0 + cell)));
+        oh = fmaxf(oh, 0.f);
+    }
+    const unsigned most = __reduce_max_sync(kFull, __float_as_uint(oh));
+    if ((threadIdx.x & 31) == 0 && most)
+        atomicMax(overhang_bits, most);
 }
 
 // ---------------------------------------------------------------------------
@@ -2382,7 +2392,7 @@ cudaError_t static_scratch(void **ptr, size_t *bytes)
 
 cudaError_t launch_grid_build(const float *d_lo_world, const float *d_hi_world, int n, int dims,
                               float gx0, float gy0, float cell, int gnx, int gny,
-                              int *d_cell_of, int *d_count, int *d_cursor, int *d_order,
+                              int *d_cell_of, int *d_count, int *d_order,
                               int *d_cell_start, float4 *const *d_perm_boxes, float4 *d_cell_lo,
                               float4 *d_cell_hi, unsigned *d_overhang_bits, cudaStream_t stream)
 {
@@ -2391,29 +2401,30 @@ cudaError_t launch_grid_build(const float *d_lo_world, const float *d_hi_world, 
     const int tb = 256;
     cudaError_t e;
     if ((e = cudaMemsetAsync(d_count, 0, sizeof(int) * n_cells, stream)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(d_cursor, 0, sizeof(int) * n_cells, stream)) != cudaSuccess) return e;
     if ((e = cudaMemsetAsync(d_overhang_bits, 0, sizeof(unsigned), stream)) != cudaSuccess) return e;
     if (n > 0)
         k_box_cell<<<(n + tb - 1) / tb, tb, 0, stream>>>(d_lo_world, d_hi_world, n, gx0, gy0, 1.0f / cell,
                                                           gnx, gny, d_cell_of, d_count);
-    // exclusive scan of the counts; its block sums live in d_cell_lo, which
-    // k_cell_bounds writes only at the end (16 bytes per cell, 4 per block sum)
-    const int n_scan_blocks = (n_cells + kScanChunk - 1) / kScanChunk;
-    if (n_scan_blocks > 1024)
-        return cudaErrorInvalidValue;
-    int *block_sum = reinterpret_cast<int *>(d_cell_lo);
-    k_scan_reduce<<<n_scan_blocks, kScanThreads, 0, stream>>>(d_count, n_cells, block_sum);
-    k_scan_top<<<1, 1024, 0, stream>>>(block_sum, n_scan_blocks, n_cells, d_cell_start);
-    k_scan_down<<<n_scan_blocks, kScanThreads, 0, stream>>>(d_count, n_cells, block_sum, d_cell_start);
+    if (n_cells <= kScanOneMax) {
+        k_scan_one<<<1, kScanOneThreads, 0, stream>>>(d_count, n_cells, d_cell_start);
+    } else {
+        // its block sums live in d_cell_lo, which k_cell_bounds writes only at
+        // the end (16 bytes per cell, 4 per block sum)
+        const int n_scan_blocks = (n_cells + kScanChunk - 1) / kScanChunk;
+        if (n_scan_blocks > 1024)
+            return cudaErrorInvalidValue;
+        int *block_sum = reinterpret_cast<int *>(d_cell_lo);
+        k_scan_reduce<<<n_scan_blocks, kScanThreads, 0, stream>>>(d_count, n_cells, block_sum);
+        k_scan_top<<<1, 1024, 0, stream>>>(block_sum, n_scan_blocks, n_cells, d_cell_start);
+        k_scan_down<<<n_scan_blocks, kScanThreads, 0, stream>>>(d_count, n_cells, block_sum, d_cell_start);
+    }
     if (n > 0) {
-        k_scatter<<<(n + tb - 1) / tb, tb, 0, stream>>>(d_cell_of, n, d_cell_start, d_cursor, d_order);
-        // d_cell_of is free after the scatter: the sort's scratch for large cells
-        const int sort_blocks = std::min((n_cells + kScanThreads - 1) / kScanThreads, 152 * 8);
-        k_sort_cells<<<sort_blocks, kScanThreads, 0, stream>>>(d_cell_start, n_cells, d_order, d_cell_of);
+        k_scatter<<<(n + tb - 1) / tb, tb, 0, stream>>>(d_cell_of, n, d_cell_start, d_count, d_order);
         PermPtrs pp;
         for (int p = 0; p < 6; ++p)
             pp.p[p] = d_perm_boxes[p];
-        k_write_boxes<<<(n + tb - 1) / tb, tb, 0, stream>>>(d_lo_world, d_hi_world, n, d_order, pp);
+        k_write_boxes<<<(n + 127) / 128, 128, 0, stream>>>(d_lo_world, d_hi_world, n, d_cell_of, d_cell_start, d_order,
+                                                           pp);
     }
     k_cell_bounds<<<(n_cells + tb - 1) / tb, tb, 0, stream>>>(d_perm_boxes[0], d_cell_start, gnx, gny,
                                                                gx0, gy0, cell, d_cell_lo, d_cell_hi,
