@@ -450,6 +450,7 @@ class PinnedPool {
 struct Slot {
     cudaStream_t stream = nullptr;
     cudaEvent_t desc_copied = nullptr;
+    bool desc_pending = false;   // an upload from h_desc has been enqueued, desc_copied marks its end
     char *d_desc = nullptr, *h_desc = nullptr;
     size_t desc_cap = 0;
     int *d_work = nullptr;
@@ -541,8 +542,7 @@ struct vcm_ctx {
     std::vector<std::unique_ptr<Slot>> slots;   // scheduler
     uint32_t max_batch = 64;
     cudaEvent_t ev_before = nullptr, ev_after = nullptr;   // optional timing of the tile kernel
-    int *d_recolor_list = nullptr;   // vcm_recolor: viewpoints that need a measure, and their count
-    int *d_recolor_n = nullptr;
+    int *d_recolor_list = nullptr;   // vcm_recolor: viewpoints that need a measure
     size_t recolor_cap = 0;
     PinnedPool pinned;
     cudaStream_t aux = nullptr;
@@ -895,6 +895,37 @@ int grid_blocks_for(vcm_ctx *ctx, int box_cap, int total_tiles)
     return std::max(1, std::min(total_tiles, resident_blocks(ctx, box_cap)));
 }
 
+// Wait until the pinned descriptors may be rewritten.
+vcm_status desc_free(Slot &s)
+{
+    if (s.desc_pending)
+        CUDA_TRY(cudaEventSynchronize(s.desc_copied));
+    s.desc_pending = false;
+    return VCM_OK;
+}
+
+// Bring the descriptors in h_desc to the device and clear the launch's
+// counters: as the prologue's parameters where they fit, else by a copy.  A
+// captured launch always copies (a graph replays it with the arena's contents
+// then); its caller records desc_copied after the graph launch.
+vcm_status upload_desc(Slot &s, const Layout &L, size_t n, long long n_blockers, cudaStream_t stream,
+                       bool capturing = false)
+{
+    int *blockers = s.d_work + kWorkHeader + Arena().blocker_off();
+    if (!capturing && L.bytes <= (size_t)kDescParamBytes) {
+        CUDA_TRY(launch_prologue_desc(s.h_desc, L.bytes, s.d_desc, (int)n, s.d_work, blockers, n_blockers, stream));
+        return VCM_OK;
+    }
+    CUDA_TRY(cudaMemcpyAsync(s.d_desc, s.h_desc, L.bytes, cudaMemcpyHostToDevice, stream));
+    // An event recorded inside a stream capture cannot be waited on later.
+    if (!capturing)
+        CUDA_TRY(cudaEventRecord(s.desc_copied, stream));
+    s.desc_pending = true;
+    CUDA_TRY(launch_prologue(reinterpret_cast<const DevRequest *>(s.d_desc + L.off_reqs), (int)n, s.d_work, blockers,
+                             n_blockers, stream));
+    return VCM_OK;
+}
+
 struct Prepared {
     Layout L;
     int box_cap = 0;
@@ -932,8 +963,8 @@ vcm_status prepare_launch(vcm_ctx *ctx, Slot &s, const std::vector<const Canon *
     vcm_status st = ensure_slot(ctx, s, P.L.bytes, cs.size(), P.blocks, sync_stream);
     if (st != VCM_OK)
         return st;
-    // the previous upload from h_desc must have completed before rewriting it
-    CUDA_TRY(cudaEventSynchronize(s.desc_copied));
+    if ((st = desc_free(s)) != VCM_OK)
+        return st;
     fill_desc(s.h_desc, s.d_desc, P.L, cs, shapes, v, color, bits, stats, P.box_cap);
     return VCM_OK;
 }
@@ -947,20 +978,13 @@ vcm_status record_launch(vcm_ctx *ctx, Slot &s, const Prepared &P, vcm_stats *st
                          cudaEvent_t after = nullptr)
 {
     Range range("vcm record launch");
-    CUDA_TRY(cudaMemcpyAsync(s.d_desc, s.h_desc, P.L.bytes, cudaMemcpyHostToDevice, stream));
-    // An event recorded inside a stream capture cannot be waited on later;
-    // a captured launch records it after the graph launch instead.
-    if (!capturing)
-        CUDA_TRY(cudaEventRecord(s.desc_copied, stream));
-
+    (void)stats;   // the descriptors point into it; the prologue clears it
+    const vcm_status up = upload_desc(s, P.L, P.n, P.tile_check ? P.L.blocker_ints : 0, stream, capturing);
+    if (up != VCM_OK)
+        return up;
     const DevRequest *d_reqs = reinterpret_cast<const DevRequest *>(s.d_desc + P.L.off_reqs);
     const int *d_tiles = reinterpret_cast<const int *>(s.d_desc + P.L.off_tiles);
     const long long *d_vps = reinterpret_cast<const long long *>(s.d_desc + P.L.off_vps);
-    (void)stats;   // the descriptors point into it; the prologue clears it
-    CUDA_TRY(launch_prologue(d_reqs, (int)P.n, s.d_work, stream));
-    if (P.tile_check && P.L.blocker_ints > 0)   // no blocker recorded yet (-1)
-        CUDA_TRY(cudaMemsetAsync(s.d_work + kWorkHeader + Arena().blocker_off(), 0xFF, (size_t)P.L.blocker_ints * sizeof(int),
-                                 stream));
     // the tile kernel starts after another launch's kernels (see launch_group)
     if (after) {
         CUDA_TRY(cudaStreamWaitEvent(stream, after, 0));
@@ -976,7 +1000,7 @@ vcm_status record_launch(vcm_ctx *ctx, Slot &s, const Prepared &P, vcm_stats *st
         CUDA_TRY(cudaEventRecord(ctx->ev_before, stream));
     CUDA_TRY(launch_tiles(ctx->scene, d_reqs, d_tiles, (int)P.n, P.L.total_tiles, s.d_work, s.d_spill,
                           P.blocks, P.box_cap, P.extra, P.tile_check, ctx->sm_count, stream, one_tile, s.d_spill_busy,
-                          /*share=*/true, claim_rounds));
+                          /*share=*/true, claim_rounds, Arena(), 0, /*overlap=*/after == nullptr));
     if (timed && ctx->ev_after)
         CUDA_TRY(cudaEventRecord(ctx->ev_after, stream));
     if (hold_spill)
@@ -1029,6 +1053,7 @@ vcm_status enqueue_graph(vcm_ctx *ctx, Slot &s, const std::vector<const Canon *>
     if (!direct_only && s.exec[f] && s.key[f] == key) {
         CUDA_TRY(cudaGraphLaunch(s.exec[f], s.stream));
         CUDA_TRY(cudaEventRecord(s.desc_copied, s.stream));
+        s.desc_pending = true;
         return VCM_OK;
     }
     if (direct_only || s.last_key[f] != key) {
@@ -1095,7 +1120,6 @@ void free_scene(vcm_ctx *ctx)
     cudaFree(ctx->d_cell_hi);
     cudaFree(ctx->d_overhang);
     cudaFree(ctx->d_recolor_list);
-    cudaFree(ctx->d_recolor_n);
     ctx->d_cell_start = ctx->d_cell_of = ctx->d_count = ctx->d_order = nullptr;
     ctx->d_cell_lo = ctx->d_cell_hi = nullptr;
     ctx->d_overhang = nullptr;
@@ -1469,15 +1493,16 @@ void launch_recolor_group(vcm_ctx *ctx, Slot &s, std::vector<std::shared_ptr<Tic
     t.form = VCM_FORM_RECOLOR;
     vcm_status st = ensure_slot(ctx, s, L.bytes, 1, 1, s.stream);
     auto body = [&]() -> vcm_status {
-        CUDA_TRY(cudaEventSynchronize(s.desc_copied));
+        vcm_status ready = desc_free(s);
+        if (ready != VCM_OK)
+            return ready;
         float *vv[1] = {t.d_v};
         uint8_t *cc[1] = {t.d_color};
         uint32_t *bb[1] = {e->d_bits};   // read only in k_recolor
         fill_desc(s.h_desc, s.d_desc, L, cs, shapes, vv, cc, bb, s.d_stats, 256, /*blockers=*/false);
         CUDA_TRY(cudaEventRecord(s.t0, s.stream));
-        CUDA_TRY(cudaMemcpyAsync(s.d_desc, s.h_desc, L.bytes, cudaMemcpyHostToDevice, s.stream));
-        CUDA_TRY(cudaEventRecord(s.desc_copied, s.stream));
-        CUDA_TRY(cudaMemsetAsync(s.d_stats, 0, sizeof(vcm_stats), s.stream));
+        if ((ready = upload_desc(s, L, 1, 0, s.stream)) != VCM_OK)
+            return ready;
         s.chained = false;
         if (after) {
             CUDA_TRY(cudaStreamWaitEvent(s.stream, after, 0));
@@ -1486,9 +1511,9 @@ void launch_recolor_group(vcm_ctx *ctx, Slot &s, std::vector<std::shared_ptr<Tic
         }
         const DevRequest *d_reqs = reinterpret_cast<const DevRequest *>(s.d_desc + L.off_reqs);
         const long long *d_vps = reinterpret_cast<const long long *>(s.d_desc + L.off_vps);
-        int *list = nullptr;   // the viewpoints that need a measure, and their count
-        CUDA_TRY(cudaMallocAsync((void **)&list, sizeof(int) * ((size_t)c.n_vp + 1), s.stream));
-        const cudaError_t le = launch_recolor(d_reqs, c.n_vp, ctx->sm_count, list, list + c.n_vp, s.stream);
+        int *list = nullptr;   // the viewpoints that need a measure; their count is the first work counter
+        CUDA_TRY(cudaMallocAsync((void **)&list, sizeof(int) * (size_t)c.n_vp, s.stream));
+        const cudaError_t le = launch_recolor(d_reqs, c.n_vp, ctx->sm_count, list, s.d_work, s.stream);
         cudaFreeAsync(list, s.stream);
         CUDA_TRY(le);
         CUDA_TRY(launch_quantise(d_reqs, d_vps, 1, c.n_vp, s.stream));
@@ -2473,8 +2498,8 @@ vcm_status vcm_recolor(vcm_ctx *ctx, const vcm_request *req, const uint32_t *d_b
         const Layout L = layout_for(cs, shapes);
         if ((st = ensure_slot(ctx, s, L.bytes, 1, 1, strm)) != VCM_OK)
             return st;
-        // the previous upload from the pinned descriptors must have completed
-        CUDA_TRY(cudaEventSynchronize(s.desc_copied));
+        if ((st = desc_free(s)) != VCM_OK)
+            return st;
         if ((size_t)c.n_vp > ctx->recolor_cap) {
             // earlier work may still read the old list
             CUDA_TRY(cudaDeviceSynchronize());
@@ -2484,20 +2509,17 @@ vcm_status vcm_recolor(vcm_ctx *ctx, const vcm_request *req, const uint32_t *d_b
             CUDA_TRY(cudaMalloc(&ctx->d_recolor_list, sizeof(int) * (size_t)c.n_vp));
             ctx->recolor_cap = (size_t)c.n_vp;
         }
-        if (!ctx->d_recolor_n)
-            CUDA_TRY(cudaMalloc(&ctx->d_recolor_n, sizeof(int)));
         float *vv[1] = {d_v};
         uint8_t *cc[1] = {d_color};
         uint32_t *bb[1] = {const_cast<uint32_t *>(d_bits)};   // read only in k_recolor
         fill_desc(s.h_desc, s.d_desc, L, cs, shapes, vv, cc, bb, d_stats, 256, /*blockers=*/false);
-        CUDA_TRY(cudaMemcpyAsync(s.d_desc, s.h_desc, L.bytes, cudaMemcpyHostToDevice, strm));
-        CUDA_TRY(cudaEventRecord(s.desc_copied, strm));
-        CUDA_TRY(cudaMemsetAsync(d_stats, 0, sizeof(vcm_stats), strm));
+        if ((st = upload_desc(s, L, 1, 0, strm)) != VCM_OK)
+            return st;
         const DevRequest *d_reqs = reinterpret_cast<const DevRequest *>(s.d_desc + L.off_reqs);
         const long long *d_vps = reinterpret_cast<const long long *>(s.d_desc + L.off_vps);
         if (ctx->ev_before)
             CUDA_TRY(cudaEventRecord(ctx->ev_before, strm));
-        CUDA_TRY(launch_recolor(d_reqs, c.n_vp, ctx->sm_count, ctx->d_recolor_list, ctx->d_recolor_n, strm));
+        CUDA_TRY(launch_recolor(d_reqs, c.n_vp, ctx->sm_count, ctx->d_recolor_list, s.d_work, strm));
         if (ctx->ev_after)
             CUDA_TRY(cudaEventRecord(ctx->ev_after, strm));
         CUDA_TRY(launch_quantise(d_reqs, d_vps, 1, c.n_vp, strm));
@@ -2543,7 +2565,9 @@ vcm_status vcm_compute_static(const float *lo, const float *hi, uint32_t n_boxes
                         "grid_nx + grid_ny + n_layers = %d)", VCM_STATIC_MAX_COORDS, c.coord_count());
         // boxes: lattice checks, world copy n x 3, bounds and largest extent
         const uint32_t n = n_boxes;
-        std::vector<float> L((size_t)std::max<uint32_t>(n, 1) * 3, 0.f), H(L.size(), 0.f);
+        const size_t n3 = (size_t)std::max<uint32_t>(n, 1) * 3;
+        std::vector<float> corners(2 * n3, 0.f);   // low ones, then high ones
+        float *const L = corners.data(), *const H = L + n3;
         double x0 = 0, x1 = 1, y0 = 0, y1 = 1, ext = 0;
         if (n) {
             x0 = y0 = 1e30;
@@ -2599,8 +2623,8 @@ vcm_status vcm_compute_static(const float *lo, const float *hi, uint32_t n_boxes
             off = align_up(off + bytes, 256);
             return static_cast<char *>(base) + at;
         };
-        float *s_lo = reinterpret_cast<float *>(take(nb * 3 * sizeof(float)));
-        float *s_hi = reinterpret_cast<float *>(take(nb * 3 * sizeof(float)));
+        float *s_lo = reinterpret_cast<float *>(take(corners.size() * sizeof(float)));
+        float *s_hi = s_lo + n3;
         float4 *s_perm[6];
         for (auto &p : s_perm)
             p = reinterpret_cast<float4 *>(take(nb * 2 * sizeof(float4)));
@@ -2627,9 +2651,8 @@ vcm_status vcm_compute_static(const float *lo, const float *hi, uint32_t n_boxes
         arena.pool_ints = share ? (int)std::min<size_t>(left - arena.pool_off(), (size_t)kPoolInts) : 0;
 
         cudaStream_t sm = static_cast<cudaStream_t>(stream);
-        // pageable host sources: each copy has consumed its source when it returns
-        CUDA_TRY(cudaMemcpyAsync(s_lo, L.data(), nb * 3 * sizeof(float), cudaMemcpyHostToDevice, sm));
-        CUDA_TRY(cudaMemcpyAsync(s_hi, H.data(), nb * 3 * sizeof(float), cudaMemcpyHostToDevice, sm));
+        // a pageable host source: the copy has consumed it when it returns
+        CUDA_TRY(cudaMemcpyAsync(s_lo, L, corners.size() * sizeof(float), cudaMemcpyHostToDevice, sm));
         CUDA_TRY(launch_grid_build(s_lo, s_hi, (int)n, dims, (float)x0, (float)y0, (float)cell, gnx, gny, s_cell_of,
                                    s_count, s_order, s_start, s_perm, s_cell_lo, s_cell_hi, s_overhang, sm));
         DevScene sc{};
@@ -2655,13 +2678,17 @@ vcm_status vcm_compute_static(const float *lo, const float *hi, uint32_t n_boxes
         uint8_t *cc[1] = {d_color};
         uint32_t *bb[1] = {d_bits};
         fill_desc(hdesc.data(), s_desc, lay, cs, shapes, vv, cc, bb, d_stats, (int)t.box_cap, /*blockers=*/false);
-        CUDA_TRY(cudaMemcpyAsync(s_desc, hdesc.data(), lay.bytes, cudaMemcpyHostToDevice, sm));
         const DevRequest *d_reqs = reinterpret_cast<const DevRequest *>(s_desc + lay.off_reqs);
         const int *d_tiles = reinterpret_cast<const int *>(s_desc + lay.off_tiles);
         const long long *d_vps = reinterpret_cast<const long long *>(s_desc + lay.off_vps);
         const int blocks =
             std::max(1, std::min(lay.total_tiles, tiles_blocks_per_sm((int)t.box_cap, list_cap) * sm_count));
-        CUDA_TRY(launch_prologue(d_reqs, 1, s_work, sm));
+        if (lay.bytes <= (size_t)kDescParamBytes) {
+            CUDA_TRY(launch_prologue_desc(hdesc.data(), lay.bytes, s_desc, 1, s_work, nullptr, 0, sm));
+        } else {
+            CUDA_TRY(cudaMemcpyAsync(s_desc, hdesc.data(), lay.bytes, cudaMemcpyHostToDevice, sm));
+            CUDA_TRY(launch_prologue(d_reqs, 1, s_work, nullptr, 0, sm));
+        }
         CUDA_TRY(launch_tiles(sc, d_reqs, d_tiles, 1, lay.total_tiles, s_work, s_spill, blocks, (int)t.box_cap,
                               needs_extra(c), c.P >= kTileCheckMinPatches, sm_count, sm, false, nullptr, share, kClaimRounds,
                               arena, list_cap));

@@ -167,6 +167,8 @@ cudaError_t launch_grid_build(const float *d_lo_world, const float *d_hi_world, 
 // `list_cap` > box_cap: the ids of candidates past the staged boxes are kept in
 // shared memory, which must then hold every box of the scene (d_spill is not
 // used); otherwise they spill.
+// `overlap` false: the tile kernel is not launched ahead of the end of what is
+// before it on the stream (k_sweep and the other kernels of a call are).
 // `claim_rounds` (1..kClaimRounds) bounds the retries of a one-tile block's
 // spill-region claim; a block that gives up runs without a region and sets
 // its request's vcm_stats.error to VCM_DEVERR_SPILL_WAIT if its candidate
@@ -176,7 +178,7 @@ cudaError_t launch_tiles(const DevScene &sc, const DevRequest *d_reqs, const int
                          int box_cap, bool extra, bool tile_check, int sm_count, cudaStream_t stream,
                          bool one_tile = false,
                          int *d_spill_busy = nullptr, bool share = false, int claim_rounds = kClaimRounds,
-                         const Arena &arena = Arena(), int list_cap = 0);
+                         const Arena &arena = Arena(), int list_cap = 0, bool overlap = true);
 // Colors and edge counts for all viewpoints of n_req requests (grid over the
 // concatenated viewpoints, `d_vp_prefix` = exclusive prefix, n_req + 1).
 cudaError_t launch_quantise(const DevRequest *d_reqs, const long long *d_vp_prefix, int n_req,
@@ -185,12 +187,19 @@ cudaError_t launch_quantise(const DevRequest *d_reqs, const long long *d_vp_pref
 // Values of one request (d_req[0]) recomputed from the occlusion bits its
 // bits_out points at (read only); colors then come from launch_quantise.
 // d_list: n_vp ints of scratch for the viewpoints that need a measure, and
-// d_n_list their count (n_vp <= INT_MAX).
+// d_n_list their count, 0 before (n_vp <= INT_MAX).
 cudaError_t launch_recolor(const DevRequest *d_req, long long n_vp, int sm_count, int *d_list, int *d_n_list,
                            cudaStream_t stream);
 
-// Zero the work counters and every request's vcm_stats.
-cudaError_t launch_prologue(const DevRequest *d_reqs, int n_req, int *d_work, cudaStream_t stream);
+// Zero the work counters (d_work[0..5)) and every request's vcm_stats, and set
+// n_blockers entries of the blocker table to -1.
+cudaError_t launch_prologue(const DevRequest *d_reqs, int n_req, int *d_work, int *d_blockers, long long n_blockers,
+                            cudaStream_t stream);
+// The same, and write the descriptors (host memory, consumed before the call
+// returns; `bytes` at most kDescParamBytes) to d_desc, 16-byte aligned.
+constexpr int kDescParamBytes = 32512;   // a kernel's parameters hold 32,764 bytes
+cudaError_t launch_prologue_desc(const void *h_desc, size_t bytes, void *d_desc, int n_req, int *d_work, int *d_blockers,
+                                 long long n_blockers, cudaStream_t stream);
 
 // Blocks of the tile kernel that fit on one SM for this shared-memory size.
 int tiles_blocks_per_sm(int box_cap, int list_cap = 0);

@@ -16,13 +16,29 @@
 #include <cfloat>
 #include <climits>
 #include <cstdio>
+#include <cstring>
+#include <map>
 #include <mutex>
+#include <utility>
 
 namespace vcm {
 
 namespace {
 
 constexpr unsigned kFull = 0xFFFFFFFFu;
+
+// The kernels of a call follow one another closely, so each is launched ahead of
+// the end of the one before it (programmatic stream serialization) and waits
+// here until that one has completed with its writes visible.  Every thread of
+// every kernel waits, so a kernel's end implies those before it.  The kernel
+// before lets go when its blocks exit: letting go at its start put waiting
+// blocks beside the persistent passes (64 uneven requests +1 %).  Without the
+// launch attribute this does nothing.  512^2 x 5 viewpoints, 5,000 boxes: 126 ->
+// 117 us per call; a 2D map of 128 x 128 36 -> 28 us.
+__device__ __forceinline__ void after_previous_kernel()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
 
 __device__ __forceinline__ float f_inf() { return __int_as_float(0x7f800000); }
 
@@ -132,6 +148,7 @@ __global__ void k_box_cell(const float *__restrict__ lo, const float *__restrict
                            float gx0, float gy0, float inv_cell, int gnx, int gny,
                            int *__restrict__ cell_of, int *__restrict__ count)
 {
+    after_previous_kernel();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n)
         return;
@@ -152,8 +169,10 @@ __global__ void k_box_cell(const float *__restrict__ lo, const float *__restrict
 constexpr int kScanOneThreads = 1024;
 constexpr int kScanOneMax = 65536;
 __global__ void __launch_bounds__(kScanOneThreads) k_scan_one(const int *__restrict__ count, int n,
-                                                              int *__restrict__ start)
+                                                              int *__restrict__ start,
+                                                              unsigned *__restrict__ overhang_bits)
 {
+    after_previous_kernel();
     __shared__ int s_warp[32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int carry = 0;
@@ -193,8 +212,10 @@ __global__ void __launch_bounds__(kScanOneThreads) k_scan_one(const int *__restr
         }
         __syncthreads();   // s_warp is reused
     }
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0) {
         start[n] = carry;
+        *overhang_bits = 0u;   // k_cell_bounds accumulates it
+    }
 }
 
 // Exclusive scan of count[0..n) into start[0..n] in three kernels: block
@@ -234,6 +255,7 @@ __device__ __forceinline__ int block_exclusive_scan(int x, int &total)
 __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const int *__restrict__ count, int n,
                                                               int *__restrict__ block_sum)
 {
+    after_previous_kernel();
     const int base = blockIdx.x * kScanChunk;
     int local = 0;
     for (int i = threadIdx.x; i < kScanChunk && base + i < n; i += kScanThreads)
@@ -247,8 +269,9 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_reduce(const int *__restr
 // One block: exclusive scan of the n_blocks (<= 1024) block sums in place;
 // start[n] gets the grand total.
 __global__ void __launch_bounds__(1024) k_scan_top(int *__restrict__ block_sum, int n_blocks, int n,
-                                                   int *__restrict__ start)
+                                                   int *__restrict__ start, unsigned *__restrict__ overhang_bits)
 {
+    after_previous_kernel();
     __shared__ int s_part[1024];
     const int t = threadIdx.x;
     const int x = t < n_blocks ? block_sum[t] : 0;
@@ -262,13 +285,16 @@ __global__ void __launch_bounds__(1024) k_scan_top(int *__restrict__ block_sum, 
     }
     if (t < n_blocks)
         block_sum[t] = s_part[t] - x;
-    if (t == 1023)
+    if (t == 1023) {
         start[n] = s_part[t];
+        *overhang_bits = 0u;   // k_cell_bounds accumulates it
+    }
 }
 
 __global__ void __launch_bounds__(kScanThreads) k_scan_down(const int *__restrict__ count, int n,
                                                             const int *__restrict__ block_off, int *__restrict__ start)
 {
+    after_previous_kernel();
     // each thread owns kScanItems consecutive elements of the block's chunk
     const int base = blockIdx.x * kScanChunk + threadIdx.x * kScanItems;
     int v[kScanItems], local = 0;
@@ -291,6 +317,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan_down(const int *__restric
 __global__ void k_scatter(const int *__restrict__ cell_of, int n, const int *__restrict__ start,
                           int *__restrict__ count, int *__restrict__ order)
 {
+    after_previous_kernel();
     int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n)
         return;
@@ -311,6 +338,7 @@ __global__ void k_write_boxes(const float *__restrict__ lo, const float *__restr
                               const int *__restrict__ cell_of, const int *__restrict__ start,
                               const int *__restrict__ order, PermPtrs out)
 {
+    after_previous_kernel();
     int at = blockIdx.x * blockDim.x + threadIdx.x;
     if (at >= n)
         return;
@@ -334,6 +362,7 @@ __global__ void k_cell_bounds(const float4 *__restrict__ boxes, const int *__res
                               float4 *__restrict__ cell_lo, float4 *__restrict__ cell_hi,
                               unsigned *__restrict__ overhang_bits)
 {
+    after_previous_kernel();
     const int c = blockIdx.x * blockDim.x + threadIdx.x;
     const bool in = c < gnx * gny;
     float4 lo = make_float4(f_inf(), f_inf(), f_inf(), 0.f);
@@ -1203,6 +1232,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
         int n_req, int total_tiles, int *__restrict__ work, Arena ar, unsigned char *__restrict__ spill_all, int id_bytes, int box_cap,
         int list_cap, int one_tile, int *__restrict__ spill_busy, int spill_slots, int share, int claim_rounds)
 {
+    after_previous_kernel();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4 *s_box = reinterpret_cast<float4 *>(smem_raw);
     int *s_ids = reinterpret_cast<int *>(smem_raw + (size_t)box_cap * 32);
@@ -1964,6 +1994,7 @@ template <bool EXTRA>
 __global__ void __launch_bounds__(kThreads, kSweepBlocks)
 k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work, Arena ar)
 {
+    after_previous_kernel();
     struct Mine {   // one warp's: a single base address, the rest are constant offsets
         WarpScratch scratch;
         float4 boxes[2 * kWarpBoxes];
@@ -2054,16 +2085,43 @@ k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work
     }
 }
 
-// Launch prologue: the work counters and every request's counters.
-__global__ void k_prologue(const DevRequest *__restrict__ reqs, int n_req, int *__restrict__ work)
+// Launch prologue: the work counters, every request's counters, and -1 in the
+// launch's part of the blocker table.
+__device__ __forceinline__ void prologue(const DevRequest *reqs, int n_req, int *__restrict__ work,
+                                         int *__restrict__ blockers, int n_blockers)
 {
-    const long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-    const long long nt = (long long)gridDim.x * blockDim.x;
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
     if (t < 5)
-        work[t] = 0;   // next tile, records, chunks published, chunks taken, id-pool ints used
+        work[t] = 0;   // next tile, records, chunks published, parts taken, id-pool ints used
     constexpr int kStatWords = (int)(sizeof(vcm_stats) / sizeof(unsigned));
-    for (long long i = t; i < (long long)n_req * kStatWords; i += nt)
+    for (int i = t; i < n_req * kStatWords; i += nt)
         reinterpret_cast<unsigned *>(reqs[i / kStatWords].stats)[i % kStatWords] = 0u;
+    for (int i = t; i < n_blockers; i += nt)
+        blockers[i] = -1;
+}
+__global__ void k_prologue(const DevRequest *__restrict__ reqs, int n_req, int *__restrict__ work,
+                           int *__restrict__ blockers, int n_blockers)
+{
+    after_previous_kernel();
+    prologue(reqs, n_req, work, blockers, n_blockers);
+}
+
+// The same for descriptors that fit a kernel's parameters: it also writes them
+// to device memory.  An upload from pinned memory is a copy-engine operation
+// that the first kernel waits for, and its buffer has to be waited for before
+// the next call: 49 -> 36 us per 2D map of 128 x 128.
+template <int BYTES>
+struct DescBlob {
+    uint4 v[BYTES / 16];
+};
+template <int BYTES>
+__global__ void k_prologue_desc(const __grid_constant__ DescBlob<BYTES> blob, int n16, uint4 *__restrict__ dst, int n_req,
+                                int *__restrict__ work, int *__restrict__ blockers, int n_blockers)
+{
+    after_previous_kernel();
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n16; i += gridDim.x * blockDim.x)
+        dst[i] = blob.v[i];
+    prologue(reinterpret_cast<const DevRequest *>(blob.v), n_req, work, blockers, n_blockers);
 }
 
 // ---------------------------------------------------------------------------
@@ -2100,6 +2158,7 @@ __device__ __forceinline__ void recolor_point(const DevRequest &R, unsigned vp, 
 __global__ void __launch_bounds__(256) k_recolor_scan(const DevRequest *__restrict__ reqs, int *__restrict__ list,
                                                       int *__restrict__ n_list)
 {
+    after_previous_kernel();
     __shared__ DevRequest s_r;
     if (threadIdx.x == 0)
         s_r = reqs[0];
@@ -2174,6 +2233,7 @@ __global__ void __launch_bounds__(256) k_recolor_scan(const DevRequest *__restri
 __global__ void __launch_bounds__(256) k_recolor_measure(const DevRequest *__restrict__ reqs,
                                                          const int *__restrict__ list, const int *__restrict__ n_list)
 {
+    after_previous_kernel();
     __shared__ DevRequest s_r;
     __shared__ float s_w[kRowCap];
     if (threadIdx.x == 0)
@@ -2279,30 +2339,50 @@ __device__ __forceinline__ unsigned char quantise_one(float v, float vref, int L
 
 // Four consecutive viewpoints per thread: one 16-byte load of values and one
 // 4-byte store of colors when the four belong to one request and both
-// addresses are aligned, else one at a time.
+// addresses are aligned, else one at a time.  A block takes a run of
+// viewpoints and looks its request up once; for each group of four on its own
+// the search took more than the colors (64 requests, 46 M viewpoints: 124 -> @
+// us).
 __global__ void k_quantise(const DevRequest *__restrict__ reqs, const long long *__restrict__ vp_prefix,
                            int n_req, long long total)
 {
-    for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; 4 * g < total;
-         g += (long long)gridDim.x * blockDim.x) {
+    after_previous_kernel();
+    const long long groups = (total + 3) / 4;
+    const long long from = groups * blockIdx.x / gridDim.x, to = groups * (blockIdx.x + 1) / gridDim.x;
+    int lo_r = 0, hi_r = n_req - 1;
+    while (lo_r < hi_r) {
+        const int mid = (lo_r + hi_r + 1) >> 1;
+        if (vp_prefix[mid] <= 4 * from)
+            lo_r = mid;
+        else
+            hi_r = mid - 1;
+    }
+    int held = -1, L = 2;
+    long long first = 0, n_vp = 0;
+    float vref = 0.f;
+    const float *v_out = nullptr;
+    unsigned char *color_out = nullptr;
+    vcm_stats *stats = nullptr;
+    for (long long g = from + threadIdx.x; g < to; g += blockDim.x) {
         const long long i0 = 4 * g;
-        int lo_r = 0, hi_r = n_req - 1;
-        while (lo_r < hi_r) {
-            int mid = (lo_r + hi_r + 1) >> 1;
-            if (vp_prefix[mid] <= i0)
-                lo_r = mid;
-            else
-                hi_r = mid - 1;
+        while (lo_r + 1 < n_req && vp_prefix[lo_r + 1] <= i0)
+            ++lo_r;
+        if (lo_r != held) {
+            held = lo_r;
+            const DevRequest &R = reqs[lo_r];
+            first = vp_prefix[lo_r];
+            n_vp = vp_prefix[lo_r + 1] - first;
+            stats = R.stats;
+            vref = R.v_ref_given > 0.f ? R.v_ref_given : __uint_as_float(stats->vmax_bits);
+            L = R.levels;
+            v_out = R.v_out;
+            color_out = R.color_out;
         }
-        const DevRequest &R = reqs[lo_r];
-        const long long local0 = i0 - vp_prefix[lo_r];
-        const long long n_vp = vp_prefix[lo_r + 1] - vp_prefix[lo_r];
-        const float vref = R.v_ref_given > 0.f ? R.v_ref_given : __uint_as_float(R.stats->vmax_bits);
-        const int L = R.levels;
+        const long long local0 = i0 - first;
         if (local0 == 0)
-            R.stats->v_ref = vref;
-        const float *vsrc = R.v_out + local0;
-        unsigned char *cdst = R.color_out ? R.color_out + local0 : nullptr;
+            stats->v_ref = vref;
+        const float *vsrc = v_out + local0;
+        unsigned char *cdst = color_out ? color_out + local0 : nullptr;
         if (local0 + 4 <= n_vp && (reinterpret_cast<uintptr_t>(vsrc) & 15u) == 0 &&
             (reinterpret_cast<uintptr_t>(cdst) & 3u) == 0) {
             const float4 v4 = *reinterpret_cast<const float4 *>(vsrc);
@@ -2311,17 +2391,17 @@ __global__ void k_quantise(const DevRequest *__restrict__ reqs, const long long 
                                ((unsigned)quantise_one(v4.y, vref, L, e1) << 8) |
                                ((unsigned)quantise_one(v4.z, vref, L, e2) << 16) |
                                ((unsigned)quantise_one(v4.w, vref, L, e3) << 24);
-            if (cdst && IN_BOUNDS(local0 + 3, (long long)R.nx * R.ny * R.nl, R.stats))
+            if (cdst && IN_BOUNDS(local0 + 3, n_vp, stats))
                 *reinterpret_cast<unsigned *>(cdst) = c;
             const unsigned n_edge = (unsigned)e0 + (unsigned)e1 + (unsigned)e2 + (unsigned)e3;
             if (n_edge)   // rare; lanes of one warp may belong to different requests
-                atomicAdd(&R.stats->edge_cells, n_edge);
+                atomicAdd(&stats->edge_cells, n_edge);
             continue;
         }
         // one at a time: the group's last viewpoints may start the next requests
         for (long long i = i0; i < i0 + 4 && i < total; ++i) {
             while (lo_r + 1 < n_req && vp_prefix[lo_r + 1] <= i)
-                ++lo_r;
+                ++lo_r;   // (the next group looks its request up again)
             const DevRequest &Q = reqs[lo_r];
             const long long local = i - vp_prefix[lo_r];
             const float qref = Q.v_ref_given > 0.f ? Q.v_ref_given : __uint_as_float(Q.stats->vmax_bits);
@@ -2390,6 +2470,25 @@ cudaError_t static_scratch(void **ptr, size_t *bytes)
     return cudaSuccess;
 }
 
+// Launch with programmatic stream serialization (see after_previous_kernel).
+// `overlap` false: an ordinary launch.
+template <typename... KArgs, typename... Args>
+static cudaError_t launch(void (*kernel)(KArgs...), int grid, int block, size_t smem, cudaStream_t stream, bool overlap,
+                          Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
+}
+
 cudaError_t launch_grid_build(const float *d_lo_world, const float *d_hi_world, int n, int dims,
                               float gx0, float gy0, float cell, int gnx, int gny,
                               int *d_cell_of, int *d_count, int *d_order,
@@ -2401,12 +2500,13 @@ cudaError_t launch_grid_build(const float *d_lo_world, const float *d_hi_world, 
     const int tb = 256;
     cudaError_t e;
     if ((e = cudaMemsetAsync(d_count, 0, sizeof(int) * n_cells, stream)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(d_overhang_bits, 0, sizeof(unsigned), stream)) != cudaSuccess) return e;
-    if (n > 0)
-        k_box_cell<<<(n + tb - 1) / tb, tb, 0, stream>>>(d_lo_world, d_hi_world, n, gx0, gy0, 1.0f / cell,
-                                                          gnx, gny, d_cell_of, d_count);
+    if (n > 0 && (e = launch(k_box_cell, (n + tb - 1) / tb, tb, 0, stream, true, d_lo_world, d_hi_world, n, gx0, gy0,
+                             1.0f / cell, gnx, gny, d_cell_of, d_count)) != cudaSuccess)
+        return e;
     if (n_cells <= kScanOneMax) {
-        k_scan_one<<<1, kScanOneThreads, 0, stream>>>(d_count, n_cells, d_cell_start);
+        if ((e = launch(k_scan_one, 1, kScanOneThreads, 0, stream, true, d_count, n_cells, d_cell_start,
+                        d_overhang_bits)) != cudaSuccess)
+            return e;
     } else {
         // its block sums live in d_cell_lo, which k_cell_bounds writes only at
         // the end (16 bytes per cell, 4 per block sum)
@@ -2414,33 +2514,48 @@ cudaError_t launch_grid_build(const float *d_lo_world, const float *d_hi_world, 
         if (n_scan_blocks > 1024)
             return cudaErrorInvalidValue;
         int *block_sum = reinterpret_cast<int *>(d_cell_lo);
-        k_scan_reduce<<<n_scan_blocks, kScanThreads, 0, stream>>>(d_count, n_cells, block_sum);
-        k_scan_top<<<1, 1024, 0, stream>>>(block_sum, n_scan_blocks, n_cells, d_cell_start);
-        k_scan_down<<<n_scan_blocks, kScanThreads, 0, stream>>>(d_count, n_cells, block_sum, d_cell_start);
+        if ((e = launch(k_scan_reduce, n_scan_blocks, kScanThreads, 0, stream, true, d_count, n_cells, block_sum)) !=
+                cudaSuccess ||
+            (e = launch(k_scan_top, 1, 1024, 0, stream, true, block_sum, n_scan_blocks, n_cells, d_cell_start,
+                        d_overhang_bits)) != cudaSuccess ||
+            (e = launch(k_scan_down, n_scan_blocks, kScanThreads, 0, stream, true, d_count, n_cells, block_sum,
+                        d_cell_start)) != cudaSuccess)
+            return e;
     }
     if (n > 0) {
-        k_scatter<<<(n + tb - 1) / tb, tb, 0, stream>>>(d_cell_of, n, d_cell_start, d_count, d_order);
         PermPtrs pp;
         for (int p = 0; p < 6; ++p)
             pp.p[p] = d_perm_boxes[p];
-        k_write_boxes<<<(n + 127) / 128, 128, 0, stream>>>(d_lo_world, d_hi_world, n, d_cell_of, d_cell_start, d_order,
-                                                           pp);
+        if ((e = launch(k_scatter, (n + tb - 1) / tb, tb, 0, stream, true, d_cell_of, n, d_cell_start, d_count,
+                        d_order)) != cudaSuccess ||
+            (e = launch(k_write_boxes, (n + 127) / 128, 128, 0, stream, true, d_lo_world, d_hi_world, n, d_cell_of,
+                        d_cell_start, d_order, pp)) != cudaSuccess)
+            return e;
     }
-    k_cell_bounds<<<(n_cells + tb - 1) / tb, tb, 0, stream>>>(d_perm_boxes[0], d_cell_start, gnx, gny,
-                                                               gx0, gy0, cell, d_cell_lo, d_cell_hi,
-                                                               d_overhang_bits);
-    return cudaGetLastError();
+    return launch(k_cell_bounds, (n_cells + tb - 1) / tb, tb, 0, stream, true, d_perm_boxes[0], d_cell_start, gnx, gny,
+                  gx0, gy0, cell, d_cell_lo, d_cell_hi, d_overhang_bits);
 }
 
+// Blocks of the tile pass per SM by shared memory (the instantiations share
+// their launch bounds).  The runtime's answer is kept: it is a property of the
+// device and the kernel, and asking took 2 us, four times per call.
 int tiles_blocks_per_sm(int box_cap, int list_cap)
 {
-    // the tile pass's instantiations share their launch bounds
-    int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_tiles<false>, kThreads,
-                                                      tiles_smem_bytes(box_cap, std::max(list_cap, box_cap))) !=
-        cudaSuccess)
+    static std::mutex mu;
+    static std::map<std::pair<int, size_t>, int> known;
+    const size_t smem = tiles_smem_bytes(box_cap, std::max(list_cap, box_cap));
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess)
         return 1;
-    return n > 0 ? n : 1;
+    std::lock_guard<std::mutex> g(mu);
+    const auto it = known.find({dev, smem});
+    if (it != known.end())
+        return it->second;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_tiles<false>, kThreads, smem) != cudaSuccess)
+        return 1;
+    n = n > 0 ? n : 1;
+    known[{dev, smem}] = n;   // (box_cap takes at most kMaxBoxCap values)
+    return n;
 }
 
 int spill_id_bytes(int n_boxes) { return n_boxes < (1 << 24) ? 3 : 4; }
@@ -2448,7 +2563,8 @@ int spill_id_bytes(int n_boxes) { return n_boxes < (1 << 24) ? 3 : 4; }
 cudaError_t launch_tiles(const DevScene &sc, const DevRequest *d_reqs, const int *d_tile_prefix,
                          int n_req, int total_tiles, int *d_work, int *d_spill, int grid_blocks,
                          int box_cap, bool extra, bool tile_check, int sm_count, cudaStream_t stream, bool one_tile,
-                         int *d_spill_busy, bool share, int claim_rounds, const Arena &arena, int list_cap)
+                         int *d_spill_busy, bool share, int claim_rounds, const Arena &arena, int list_cap,
+                         bool overlap)
 {
     if (claim_rounds < 1 || claim_rounds > kClaimRounds)
         return cudaErrorInvalidValue;
@@ -2466,27 +2582,53 @@ cudaError_t launch_tiles(const DevScene &sc, const DevRequest *d_reqs, const int
     }
     auto kernel = tile_check ? k_tiles<true> : k_tiles<false>;
     share = share && !one_tile;
-    kernel<<<grid_blocks, kThreads, smem, stream>>>(sc, d_reqs, d_tile_prefix, n_req, total_tiles, d_work, arena,
-                                                    reinterpret_cast<unsigned char *>(d_spill),
-                                                    spill_id_bytes(sc.n_boxes), box_cap, list_cap, one_tile ? 1 : 0, d_spill_busy, slots, share ? 1 : 0,
-                                                    claim_rounds);
-    if (share) {
-        // the second pass, on every SM
-        const cudaError_t e = cudaGetLastError();
-        if (e != cudaSuccess)
-            return e;
-        (extra ? k_sweep<true> : k_sweep<false>)<<<sm_count * kSweepBlocks, kThreads, 0, stream>>>(sc, d_reqs, d_work, arena);
-    }
-    return cudaGetLastError();
+    cudaError_t e = launch(kernel, grid_blocks, kThreads, smem, stream, overlap, sc, d_reqs, d_tile_prefix, n_req,
+                           total_tiles, d_work, arena, reinterpret_cast<unsigned char *>(d_spill),
+                           spill_id_bytes(sc.n_boxes), box_cap, list_cap, one_tile ? 1 : 0, d_spill_busy, slots,
+                           share ? 1 : 0, claim_rounds);
+    if (e == cudaSuccess && share)   // the second pass, on every SM
+        e = launch(extra ? k_sweep<true> : k_sweep<false>, sm_count * kSweepBlocks, kThreads, 0, stream, true, sc,
+                   d_reqs, d_work, arena);
+    return e;
 }
 
-cudaError_t launch_prologue(const DevRequest *d_reqs, int n_req, int *d_work, cudaStream_t stream)
+static int prologue_blocks(size_t desc_bytes, int n_req, long long n_blockers)
+{
+    const long long items = std::max(std::max((long long)desc_bytes / 16, 18LL * n_req), n_blockers / 8);
+    return (int)std::max<long long>(1, std::min<long long>(152, (items + 255) / 256));
+}
+
+cudaError_t launch_prologue(const DevRequest *d_reqs, int n_req, int *d_work, int *d_blockers, long long n_blockers,
+                            cudaStream_t stream)
 {
     if (n_req <= 0)
         return cudaSuccess;
-    const int blocks = std::max(1, std::min(152, (n_req * 16 + 255) / 256));
-    k_prologue<<<blocks, 256, 0, stream>>>(d_reqs, n_req, d_work);
-    return cudaGetLastError();
+    return launch(k_prologue, prologue_blocks(0, n_req, n_blockers), 256, 0, stream, false, d_reqs, n_req, d_work,
+                  d_blockers, (int)n_blockers);
+}
+
+template <int BYTES>
+static cudaError_t prologue_desc(const void *h_desc, size_t bytes, void *d_desc, int n_req, int *d_work, int *d_blockers,
+                                 long long n_blockers, cudaStream_t stream)
+{
+    DescBlob<BYTES> blob;
+    std::memcpy(&blob, h_desc, bytes);
+    return launch(k_prologue_desc<BYTES>, prologue_blocks(bytes, n_req, n_blockers), 256, 0, stream, true, blob,
+                  (int)((bytes + 15) / 16), static_cast<uint4 *>(d_desc), n_req, d_work, d_blockers, (int)n_blockers);
+}
+
+cudaError_t launch_prologue_desc(const void *h_desc, size_t bytes, void *d_desc, int n_req, int *d_work, int *d_blockers,
+                                 long long n_blockers, cudaStream_t stream)
+{
+    if (n_req <= 0)
+        return cudaSuccess;
+    if (bytes <= 4096)
+        return prologue_desc<4096>(h_desc, bytes, d_desc, n_req, d_work, d_blockers, n_blockers, stream);
+    if (bytes <= 16384)
+        return prologue_desc<16384>(h_desc, bytes, d_desc, n_req, d_work, d_blockers, n_blockers, stream);
+    if (bytes <= kDescParamBytes)
+        return prologue_desc<kDescParamBytes>(h_desc, bytes, d_desc, n_req, d_work, d_blockers, n_blockers, stream);
+    return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_quantise(const DevRequest *d_reqs, const long long *d_vp_prefix, int n_req,
@@ -2497,8 +2639,7 @@ cudaError_t launch_quantise(const DevRequest *d_reqs, const long long *d_vp_pref
     long long blocks = ((total_vp + 3) / 4 + 255) / 256;   // four viewpoints per thread
     if (blocks > 152 * 16)
         blocks = 152 * 16;
-    k_quantise<<<(int)blocks, 256, 0, stream>>>(d_reqs, d_vp_prefix, n_req, total_vp);
-    return cudaGetLastError();
+    return launch(k_quantise, (int)blocks, 256, 0, stream, true, d_reqs, d_vp_prefix, n_req, total_vp);
 }
 
 cudaError_t launch_recolor(const DevRequest *d_req, long long n_vp, int sm_count, int *d_list, int *d_n_list,
@@ -2506,18 +2647,14 @@ cudaError_t launch_recolor(const DevRequest *d_req, long long n_vp, int sm_count
 {
     if (n_vp <= 0)
         return cudaSuccess;
-    cudaError_t e = cudaMemsetAsync(d_n_list, 0, sizeof(int), stream);
-    if (e != cudaSuccess)
-        return e;
     long long blocks = (n_vp + 255) / 256;
     const long long cap = (long long)std::max(sm_count, 1) * 8;
     if (blocks > cap)
         blocks = cap;
-    k_recolor_scan<<<(int)blocks, 256, 0, stream>>>(d_req, d_list, d_n_list);
-    if ((e = cudaGetLastError()) != cudaSuccess)
+    const cudaError_t e = launch(k_recolor_scan, (int)blocks, 256, 0, stream, true, d_req, d_list, d_n_list);
+    if (e != cudaSuccess)
         return e;
-    k_recolor_measure<<<(int)cap, 256, 0, stream>>>(d_req, d_list, d_n_list);
-    return cudaGetLastError();
+    return launch(k_recolor_measure, (int)cap, 256, 0, stream, true, d_req, d_list, d_n_list);
 }
 
 }  // namespace vcm
