@@ -179,7 +179,7 @@ typedef struct {
     uint32_t error;                    /* VCM_DEVERR_*: nonzero if a device-side check failed */
     unsigned long long slab_tests;     /* slab tests executed in the sweep: a patch column against a box
                                           (VCM_VIEWER: a segment against a box) */
-    unsigned long long rechecked;      /* segment-box pairs re-decided by the exact float64 predicate */
+    unsigned long long rechecked;      /* segment-box pairs re-decided by the exact predicate */
     unsigned long long segments;       /* viewpoint-patch pairs decided (= viewpoints x patches) */
     unsigned long long boxes_listed;   /* sum over tiles of culled candidate-list lengths */
     unsigned long long corner_tests;   /* segment-box tests of the one-box-blocks-all check */

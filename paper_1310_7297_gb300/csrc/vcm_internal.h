@@ -20,7 +20,7 @@ constexpr int kDistClasses = 128;            // distance classes of the candidat
 // hidden target, 3.40 -> 3.46 ms on a mostly visible one); at 512 patches it
 // cost 4 % (5,000 boxes: 0.189 -> 0.197 ms).
 constexpr int kTileCheckMinPatches = 1024;
-constexpr float kBand = 1e-6f;            // FP32 slab margin re-decided in FP64
+constexpr float kBand = 1e-6f;            // FP32 slab margin that is re-decided exactly
 constexpr int kMaxBoxCap = 5000;          // candidate boxes a tile stages in shared memory
 constexpr int kRowCap = 256;              // patch rows a warp stages for the measure
 constexpr int kWarpBoxes = 64;            // boxes of a chunk's list a warp stages

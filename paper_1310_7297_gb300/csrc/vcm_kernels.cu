@@ -8,7 +8,7 @@
 //    warps sweep the tile's viewpoints, lanes over target patch columns and
 //    bits of a mask over patch rows, deciding each viewpoint->patch segment by
 //    a float32 slab test (Def. 2 point-to-point visibility; touching blocks,
-//    Def. 4) with an exact float64 re-decision inside a 1e-6 margin band,
+//    Def. 4) with an exact integer re-decision inside a 1e-6 margin band,
 //    then summing A cos(theta)/d^2 (or len cos(theta)/d in 2D) per viewpoint;
 //  * quantise: colors in L levels from v / v_ref (Def. 1 normalisation).
 #include "vcm_internal.h"
@@ -123,7 +123,7 @@ __device__ __forceinline__ void put_word(const DevRequest &R, long long at, uint
 
 // Hardware reciprocal, at most 1 ulp from 1/d (2^-23 relative); 1/(+0) = +inf.
 // The slab-test error bound with it is about 5 u per t value, 10 u per
-// margin, still inside the 1e-6 band that is re-decided in float64.
+// margin, still inside the 1e-6 band that is re-decided exactly.
 __device__ __forceinline__ float rcp_approx(float d)
 {
     float r;
@@ -451,45 +451,46 @@ __device__ __forceinline__ bool swept_meets(const Swept &S, float4 lo, float4 hi
     return from <= to;
 }
 
-// Exact re-decision of one segment against one box, in float64.  Inputs are
-// lattice values (multiples of 2^-10 m, |x| <= 2^14 m): differences are
-// exact and every product of two of them needs at most 52 significant bits,
-// so the comparisons below are exact.  The running lower bound en/ed and
-// upper bound xn/xd of the segment parameter t are kept as fractions with
-// positive denominators.
+// Exact re-decision of one segment against one box, in integers.  Inputs are
+// lattice values (multiples of 2^-10 m, |x| <= 2^14 m): in lattice units their
+// differences take 26 bits and a product of two of them 52, so the comparisons
+// below are exact.  The running lower bound en/ed and upper bound xn/xd of the
+// segment parameter t are kept as fractions with positive denominators.  (The
+// same in float64 is exact too, but took 2.8 us per call on the narrow FP64
+// pipe, and a column that grazes a box asked for 16 to 32 of them in a row:
+// 1 % of the sweep's warps set its end.  512^2 x 5 viewpoints, 5,000 boxes: both
+// passes 128 -> 105 us, strict 101 -> 68 us.)
 __device__ __noinline__ bool exact_hit(float qu, float qn, float qw, float pu, float pn, float pw,
                                        float4 lo, float4 hi)
 {
-    const double q[3] = {qu, qn, qw};
-    const double p[3] = {pu, pn, pw};
-    const double L[3] = {lo.x, lo.y, lo.z};
-    const double H[3] = {hi.x, hi.y, hi.z};
-    double en = 0.0, ed = 1.0, xn = 1.0, xd = 1.0;
+    constexpr float kUnits = (float)VCM_UNITS_PER_M;
+    const float q[3] = {qu, qn, qw};
+    const float p[3] = {pu, pn, pw};
+    const float L[3] = {lo.x, lo.y, lo.z};
+    const float H[3] = {hi.x, hi.y, hi.z};
+    int en = 0, ed = 1, xn = 1, xd = 1;
+#pragma unroll
     for (int k = 0; k < 3; ++k) {
-        const double d = p[k] - q[k];
-        const double a = L[k] - q[k];
-        const double b = H[k] - q[k];
-        if (d == 0.0) {
-            if (a > 0.0 || b < 0.0)
+        const int at = __float2int_rn(q[k] * kUnits);
+        const int d = __float2int_rn(p[k] * kUnits) - at;
+        const int a = __float2int_rn(L[k] * kUnits) - at;
+        const int b = __float2int_rn(H[k] * kUnits) - at;
+        if (d == 0) {
+            if (a > 0 || b < 0)
                 return false;
             continue;
         }
-        double ln, un, den;
-        if (d > 0.0) {
-            ln = a; un = b; den = d;
-        } else {
-            ln = -b; un = -a; den = -d;
-        }
-        if (ln * ed > en * den) {
+        const int ln = d > 0 ? a : -b, un = d > 0 ? b : -a, den = abs(d);
+        if ((long long)ln * ed > (long long)en * den) {
             en = ln;
             ed = den;
         }
-        if (un * xd < xn * den) {
+        if ((long long)un * xd < (long long)xn * den) {
             xn = un;
             xd = den;
         }
     }
-    return en * xd <= xn * ed;
+    return (long long)en * xd <= (long long)xn * ed;
 }
 
 struct TileSmem {
@@ -929,8 +930,8 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
                         const float iE = fminf(fmaf(du, ru.x, ru.y), rw.x);
                         const float iX = fmaxf(fmaxf(du * ru.z, du * ru.w), rw.y);
                         ++tests;
+                        unsigned hit = 0u, ask = 0u;   // rows blocked for certain, rows to decide one by one
                         if (alive != 0u && iE >= iX * kLess) {
-                            unsigned hit = 0u, ask = 0u;   // rows blocked for certain, rows to decide one by one
                             // first row + 1/2 and last row - 1/2 of the interval
                             const float y = fminf(fmaxf(fmaf(rw.z > 0.f ? iX : iE, rw.z, c + 0.5f), 0.f), 32.f);
                             const float z = fminf(fmaxf(fmaf(rw.w > 0.f ? iE : iX, rw.w, c - 0.5f), -1.f), 31.f);
@@ -947,18 +948,38 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
                             }
                             ask &= alive;
                             hit &= ~ask;
+                        }
+                        if (__any_sync(kFull, ask != 0u)) {   // rare
+                            float4 lo, hi;
+                            load_box(sbox, n_smem, spill, gbox, fits ? W.rec_id[j] : base + j, n_boxes, R.stats, lo,
+                                     hi);
+                            // a column with many such rows (it grazes the box): its rows over the lanes
+                            unsigned columns = __ballot_sync(kFull, __popc(ask) > 2);
+                            while (columns) {
+                                const int from = __ffs(columns) - 1;
+                                columns &= columns - 1;
+                                const float p_col = __shfl_sync(kFull, pu, from);
+                                const unsigned rows_of = __shfl_sync(kFull, ask, from);
+                                const int g_of = __shfl_sync(kFull, M.g(), from);
+                                unsigned h = 0u;
+                                if ((rows_of >> lane) & 1u)
+                                    h = row_hit(qu, qn, qw, p_col, R.p_n, R.w_coord[row0 + lane * G + g_of], lo, hi, is3d);
+                                rechecks += h >> 1;
+                                const unsigned blocked_rows = __ballot_sync(kFull, h & 1u);
+                                if (lane == from) {
+                                    hit |= blocked_rows;
+                                    ask = 0u;
+                                }
+                            }
                             while (ask) {
                                 const int m = __ffs(ask) - 1;
                                 ask &= ask - 1;
-                                float4 lo, hi;
-                                load_box(sbox, n_smem, spill, gbox, fits ? W.rec_id[j] : base + j, n_boxes, R.stats, lo,
-                                         hi);
                                 const unsigned h = row_hit(qu, qn, qw, pu, R.p_n, w_row[m * G], lo, hi, is3d);
                                 hit |= (h & 1u) << m;
                                 rechecks += h >> 1;
                             }
-                            alive &= ~hit;
                         }
+                        alive &= ~hit;
                         if (__all_sync(kFull, alive == 0u) || (strict_exit && __any_sync(kFull, alive != valid))) {
                             done = true;
                             break;
