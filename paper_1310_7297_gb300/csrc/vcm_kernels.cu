@@ -140,6 +140,31 @@ __device__ __forceinline__ float rsqrt_normal(float d2)
     return r;
 }
 
+// Two floats per operation (each rounded as the scalar one).
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float a, float b)
+{
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 x, float &a, float &b)
+{
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(x));
+}
+__device__ __forceinline__ f32x2 mul2(f32x2 a, f32x2 b)
+{
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c)
+{
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
 // ---------------------------------------------------------------------------
 // grid build
 // ---------------------------------------------------------------------------
@@ -805,7 +830,8 @@ __device__ __forceinline__ int row_slot(int i, int G, int stride)
 // Shared memory of one warp's sweeps.
 struct WarpScratch {
     float4 rec[2 * 32];   // records of the boxes left to a viewpoint
-    float rw[kRowCap];    // its row offsets q_w - w, each lane group's rows side by side
+    float rw[kRowCap];    // row offsets q_w - w, each lane group's rows side by side
+    float rw_of;          // the q_w they are for (NaN: none); viewpoints of a layer share them
     int rec_id[32];       // the records' boxes
 };
 
@@ -840,7 +866,6 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
 {
     constexpr float kMagic = 12582912.f;   // 1.5 x 2^23: adding it rounds to an integer
     float4 *rec = W.rec;
-    bool rows_staged = false;
     const int lane = threadIdx.x & 31;
     const int nuc = R.nuc, G = R.groups;
     const float dn = R.p_n - qn;
@@ -1037,11 +1062,12 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
                 continue;
             }
             const int stride = row_stride(R);
-            if (!rows_staged && stride > 0) {
-                rows_staged = true;
+            if (stride > 0 && !(W.rw_of == qw)) {
                 __syncwarp();   // the viewpoint before this one is done with them
                 for (int i = lane; i < R.nw; i += 32)
                     W.rw[row_slot(i, G, stride)] = qw - R.w_coord[i];
+                if (lane == 0)
+                    W.rw_of = qw;
                 __syncwarp();
             }
             const float *my_rw = W.rw + M.g() * stride + r_at;
@@ -1052,13 +1078,24 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
                     continue;
                 float part = 0.f;
                 if (stride > 0 && m0 + 8 <= rows) {
-                    const float4 *s4 = reinterpret_cast<const float4 *>(my_rw + m0);
-                    const float4 wa = s4[0], wb = s4[1];
-                    const float w8[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
                     float t8[8];
+                    if (EXTRA && cone == kConeMixed) {
 #pragma unroll
-                    for (int k = 0; k < 8; ++k)
-                        t8[k] = measure_term<EXTRA, true>(R, cone == kConeMixed, col_d2, m_s, ru, rn, w8[k]);
+                        for (int k = 0; k < 8; ++k)
+                            t8[k] = measure_term<EXTRA, true>(R, true, col_d2, m_s, ru, rn, my_rw[m0 + k]);
+                    } else {
+                        // measure_term two rows at a time: the sweep is bound by issue
+                        const ulonglong2 *s2 = reinterpret_cast<const ulonglong2 *>(my_rw + m0);
+                        const ulonglong2 wa = s2[0], wb = s2[1];
+                        const f32x2 w2[4] = {wa.x, wa.y, wb.x, wb.y}, c2 = pack2(col_d2, col_d2), m2 = pack2(m_s, m_s);
+#pragma unroll
+                        for (int k = 0; k < 4; ++k) {
+                            float d0, d1;
+                            unpack2(fma2(w2[k], w2[k], c2), d0, d1);
+                            const f32x2 ir = pack2(rsqrt_normal(d0), rsqrt_normal(d1));
+                            unpack2(mul2(m2, mul2(mul2(ir, ir), ir)), t8[2 * k], t8[2 * k + 1]);
+                        }
+                    }
                     if (__all_sync(kFull, (o8 & 0xffu) == 0xffu)) {   // mostly
 #pragma unroll
                         for (int k = 0; k < 8; ++k)
@@ -1088,27 +1125,26 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
     return strict_fail ? 0.f : v;
 }
 
-// One open viewpoint, at (ix, iy) of a layer: swept, and its outputs written.
-// Returns its value.
+// A viewpoint in the target frame.
+__device__ __forceinline__ float3 in_target_frame(const DevRequest &R, float qx, float qy, float zq)
+{
+    return make_float3(R.au == 0 ? qx : (R.au == 1 ? qy : zq), R.an == 0 ? qx : (R.an == 1 ? qy : zq),
+                       R.dims == 3 ? (R.aw == 0 ? qx : (R.aw == 1 ? qy : zq)) : 0.f);
+}
+
+// One open viewpoint q: swept, and its outputs written.  Returns its value.
 template <bool EXTRA>
-__device__ __forceinline__ float sweep_one(const DevRequest &R, const LaneMap &M, int ix, int iy, int layer, float zq,
-                                           bool want_bits, const float4 *__restrict__ sbox, int n_smem,
-                                           Tail spill, int count, const float4 *__restrict__ gbox,
-                                           WarpScratch &W, unsigned &tests, unsigned &corners, unsigned &rechecks,
-                                           unsigned &shortcuts, int n_boxes)
+__device__ __forceinline__ float sweep_one(const DevRequest &R, const LaneMap &M, float3 q, bool front, long long vp,
+                                           const float4 *__restrict__ sbox, int n_smem, Tail tail, int count,
+                                           const float4 *__restrict__ gbox, WarpScratch &W, unsigned &tests,
+                                           unsigned &corners, unsigned &rechecks, unsigned &shortcuts, int n_boxes)
 {
     const int lane = threadIdx.x & 31;
-    const long long vp = ((long long)layer * R.ny + iy) * R.nx + ix;
-    const float qx = R.x_coord[ix], qy = R.y_coord[iy];
-    const float qu = R.au == 0 ? qx : (R.au == 1 ? qy : zq);
-    const float qn = R.an == 0 ? qx : (R.an == 1 ? qy : zq);
-    const float qw = R.dims == 3 ? (R.aw == 0 ? qx : (R.aw == 1 ? qy : zq)) : 0.f;
-    const bool front = facing(R, qn);
-    float v = sweep_viewpoint<EXTRA>(R, M, sbox, n_smem, spill, count, gbox, qu, qn, qw, front, vp, W, tests, corners,
-                                     rechecks, n_boxes);
+    float v = sweep_viewpoint<EXTRA>(R, M, sbox, n_smem, tail, count, gbox, q.x, q.y, q.z, front, vp, W, tests,
+                                     corners, rechecks, n_boxes);
     if (v < 0.f) {   // one box blocks every patch
         ++shortcuts;
-        if (want_bits)
+        if ((R.flags & VCM_EMIT_BITS) && R.bits_out)
             for (int wd = lane; wd < R.words; wd += 32) {
                 const int rem = R.P - 32 * wd;
                 put_word(R, vp * R.words + wd, rem >= 32 ? 0xffffffffu : ((1u << rem) - 1u));
@@ -1206,8 +1242,10 @@ __device__ __noinline__ void sweep_kept(const DevRequest &R, TileScratch &T, con
     if (warp >= kKeptWarps)
         return;
     const LaneMap M = lane_map(R);
-    const bool want_bits = (R.flags & VCM_EMIT_BITS) && R.bits_out;
     const float zq = R.z_coord[layer];
+    if (lane == 0)
+        T.sweep[warp].rw_of = __int_as_float(0x7fffffff);
+    __syncwarp();
     unsigned long long tests = 0, corners = 0;
     unsigned rechecks = 0, shortcuts = 0;
     float vmax = 0.f;
@@ -1219,9 +1257,11 @@ __device__ __noinline__ void sweep_kept(const DevRequest &R, TileScratch &T, con
         if (k >= n_und)
             break;
         unsigned vp_tests = 0, vp_corners = 0;
-        const float v = sweep_one<true>(R, M, ix0 + (und[k] & 255), iy0 + (und[k] >> 8), layer, zq, want_bits, sbox,
-                                        n_smem, spill, count, gbox, T.sweep[warp], vp_tests, vp_corners, rechecks,
-                                        shortcuts, n_boxes);
+        const int ix = ix0 + (und[k] & 255), iy = iy0 + (und[k] >> 8);
+        const float3 q = in_target_frame(R, R.x_coord[ix], R.y_coord[iy], zq);
+        const float v = sweep_one<true>(R, M, q, facing(R, q.y), ((long long)layer * R.ny + iy) * R.nx + ix, sbox, n_smem,
+                                        spill, count, gbox, T.sweep[warp], vp_tests, vp_corners, rechecks, shortcuts,
+                                        n_boxes);
         vmax = fmaxf(vmax, v);
         tests += vp_tests;
         corners += vp_corners;
@@ -2006,11 +2046,14 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
 // read where it is used: the sweep needs the registers (in registers it
 // spilled 200 bytes and issued 10 % more instructions).
 //
-// Bound by instruction issue at 85 % of the issue slots.  Measured against
-// chunks by blocks (both passes): 96 x 83 x 3 viewpoints, two-sided, 45 x 13
-// patches 92 -> 60 us; 64 x 64, 8 x 4 patches 44 -> 36 us; 2D 128 x 128 48 -> 41
-// us; 64 uneven requests 8.92 -> 8.71 ms; 100,000 boxes, 64 x 32 patches 5.38
-// -> 5.20 ms.  7 blocks per SM: 6 were 3 %, 5 13 % slower on the batch, 8 spill.
+// Bound by instruction issue (79 % of the slots; 60 % with 5,000 boxes, where
+// the loads that begin a part show).  Against chunks by blocks (both passes): 96
+// x 83 x 3 viewpoints, two-sided, 45 x 13 patches 92 -> 60 us; 64 x 64, 8 x 4
+// patches 44 -> 36 us; 2D 128 x 128 48 -> 41 us; 64 uneven requests 8.92 -> 8.71
+// ms.  Since then the part's viewpoints are set up one per lane, rows are staged
+// once per layer and the measure takes two rows per operation: 64 requests 7.19
+// -> 6.16 ms, 100,000 boxes, 64 x 32 patches 3.44 -> 3.14 ms.  6 blocks per SM (80
+// registers): 7 spill (+6 %), 5 leave latency open (+8 %).
 template <bool EXTRA>
 __global__ void __launch_bounds__(kThreads, kSweepBlocks)
 k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work, Arena ar)
@@ -2020,8 +2063,9 @@ k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work
         WarpScratch scratch;
         float4 boxes[2 * kWarpBoxes];
         DevRequest req;
+        float4 q[kChunkVp];   // the part's viewpoints in the target frame; w: 1 in front of the target
+        long long vp[kChunkVp];
         int list[8];   // the record: request, count, offset of the ids, layer, tile origin
-        int xy[kChunkVp];
     };
     __shared__ __align__(16) Mine s_mine[kWarps];
     const int lane = threadIdx.x & 31;
@@ -2055,8 +2099,7 @@ k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work
         if (n <= 0)
             continue;
         __syncwarp();   // the viewpoints before are done with the item's shared memory
-        if (lane < n)
-            mine.xy[lane] = reinterpret_cast<const unsigned short *>(chunk + 1)[first + lane];
+        const int at = lane < n ? reinterpret_cast<const unsigned short *>(chunk + 1)[first + lane] : 0;
         if (rec != cur_rec) {
             cur_rec = rec;
             const int old_req = list[0];
@@ -2068,6 +2111,8 @@ k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work
                 const int *src = reinterpret_cast<const int *>(reqs + list[0]);
                 for (int i = lane; i < (int)(sizeof(DevRequest) / sizeof(int)); i += 32)
                     reinterpret_cast<int *>(&R)[i] = src[i];
+                if (lane == 0)
+                    W.rw_of = __int_as_float(0x7fffffff);
                 __syncwarp();
                 M = lane_map(R);
             }
@@ -2078,16 +2123,20 @@ k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work
                 boxes[2 * i + 1] = __ldg(&gbox[2 * id + 1]);
             }
         }
+        if (lane < n) {   // one per lane: 45 instructions for all of them
+            const int ix = list[4] + (at & 255), iy = list[5] + (at >> 8);
+            const float3 q = in_target_frame(R, R.x_coord[ix], R.y_coord[iy], R.z_coord[list[3]]);
+            mine.q[lane] = make_float4(q.x, q.y, q.z, facing(R, q.y) ? 1.f : 0.f);
+            mine.vp[lane] = ((long long)list[3] * R.ny + iy) * R.nx + ix;
+        }
         __syncwarp();
-        const bool want_bits = (R.flags & VCM_EMIT_BITS) && R.bits_out;
         unsigned tests = 0, corners = 0, rechecks = 0, shortcuts = 0;
         float vmax = 0.f;
         for (int k = 0; k < n; ++k) {
-            const int at = mine.xy[k], layer = list[3];
-            const float v = sweep_one<EXTRA>(R, M, list[4] + (at & 255), list[5] + (at >> 8), layer, R.z_coord[layer],
-                                             want_bits, boxes, kWarpBoxes,
-                                             Tail{arena + ar.pool_off() + list[2] + kWarpBoxes, 4}, list[1], sc.boxes[R.perm], W, tests, corners, rechecks, shortcuts,
-                                             sc.n_boxes);
+            const float4 q = mine.q[k];
+            const float v = sweep_one<EXTRA>(R, M, make_float3(q.x, q.y, q.z), q.w != 0.f, mine.vp[k], boxes, kWarpBoxes,
+                                             Tail{arena + ar.pool_off() + list[2] + kWarpBoxes, 4}, list[1],
+                                             sc.boxes[R.perm], W, tests, corners, rechecks, shortcuts, sc.n_boxes);
             vmax = fmaxf(vmax, v);
         }
         rechecks = __reduce_add_sync(kFull, rechecks);
