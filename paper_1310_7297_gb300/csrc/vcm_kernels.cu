@@ -521,7 +521,7 @@ __device__ __noinline__ bool exact_hit(float qu, float qn, float qw, float pu, f
 struct TileSmem {
     int count;
     int item;
-    int pad;
+    int layer, tx, ty;
     int n_und;
     int pub[4];   // record, first chunk, chunks published, offset of the ids in the pool
 };
@@ -1304,6 +1304,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
     __shared__ unsigned s_node[2][16];   // nodes' boxes, of this batch and the last
     __shared__ __align__(16) TileScratch s_scratch;
     __shared__ int s_req_idx, s_npass;
+    __shared__ unsigned long long s_listed, s_shared;   // counters of thread 0
     __shared__ int s_next2;                     // cursor of the undecided list
     __shared__ unsigned short s_und[kMaxTileViewpoints];   // viewpoints left by the one-box check, x + 256 y
     auto &walk = s_scratch.walk;
@@ -1312,6 +1313,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
     if (tid == 0) {
         s_req_idx = -1;
         s_npass = 0;
+        s_listed = s_shared = 0;
         sm.item = -1;
         // A persistent block owns spill region blockIdx.x.  A one-tile block
         // claims a free region for the length of its tile.  There are as
@@ -1345,7 +1347,6 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
     // counters, added to a request's when its last tile in a row is done
     vcm_stats *acc = nullptr;
     unsigned corner_tests = 0, shortcuts = 0;
-    unsigned long long listed = 0;   // thread 0's
     auto flush = [&] {
         corner_tests = __reduce_add_sync(kFull, corner_tests);
         shortcuts = __reduce_add_sync(kFull, shortcuts);
@@ -1355,10 +1356,13 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
             if (shortcuts)
                 atomicAdd(&acc->shortcut_viewpoints, (unsigned long long)shortcuts);
         }
-        if (acc && tid == 0)
-            atomicAdd(&acc->boxes_listed, listed);
+        if (acc && tid == 0) {
+            atomicAdd(&acc->boxes_listed, s_listed);
+            if (s_shared)
+                atomicAdd(&acc->shared_viewpoints, s_shared);
+            s_listed = s_shared = 0;
+        }
         corner_tests = shortcuts = 0;
-        listed = 0;
     };
 
     for (;;) {
@@ -1389,16 +1393,13 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                     s_req = reqs[lo_r];
                     s_req_idx = lo_r;
                 }
-                {
-                    // tile index within its request, layers interleaved
-                    const int t0 = it - tile_prefix[lo_r];
-                    const int nl = s_req.nl, pl = s_req.tiles_x * s_req.tiles_y;
-                    sm.pad = (t0 % nl) * pl + t0 / nl;
-                }
                 const DevRequest &Q = s_req;
-                const int t0 = sm.pad, pl = Q.tiles_x * Q.tiles_y;
-                const int ly = t0 / pl, t1 = t0 - ly * pl;
-                const int ty0 = t1 / Q.tiles_x, tx0 = t1 - ty0 * Q.tiles_x;
+                // tile index within its request, layers interleaved
+                const int t0 = it - tile_prefix[lo_r], pos = t0 / Q.nl, ly = t0 - pos * Q.nl;
+                const int ty0 = pos / Q.tiles_x, tx0 = pos - ty0 * Q.tiles_x;
+                sm.layer = ly;
+                sm.tx = tx0;
+                sm.ty = ty0;
                 const int x0 = tx0 * Q.tile_x, x1 = min(Q.nx, x0 + Q.tile_x) - 1;
                 const int y0 = ty0 * Q.tile_y, y1 = min(Q.ny, y0 + Q.tile_y) - 1;
                 const float z = Q.z_coord[ly];
@@ -1427,11 +1428,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
             acc = s_req.stats;
         }
         const DevRequest &R = s_req;
-        const int t = sm.pad;
-        const int per_layer = R.tiles_x * R.tiles_y;
-        const int layer = t / per_layer;
-        const int tt = t - layer * per_layer;
-        const int ty = tt / R.tiles_x, tx = tt - ty * R.tiles_x;
+        const int layer = sm.layer, tx = sm.tx, ty = sm.ty;
         const int ix0 = tx * R.tile_x, ix1 = min(R.nx, ix0 + R.tile_x);
         const int iy0 = ty * R.tile_y, iy1 = min(R.ny, iy0 + R.tile_y);
         const int tw = ix1 - ix0, tn = tw * (iy1 - iy0);
@@ -1976,16 +1973,19 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
             if (tid == 0) {
                 const int want = (n_und + kChunkVp - 1) / kChunkVp;
                 int rec = ar.rec_cap, base = 0, got = 0, off = 0;
-                // counters move only while their caps are not reached
+                // counters move only while their caps are not reached, and all at
+                // once (one round trip, not three): a tile whose record or ids did
+                // not fit leaves its chunks empty
                 if (__ldcg(work + 1) < ar.rec_cap && __ldcg(work + 4) < ar.pool_ints &&
                     __ldcg(work + 2) < ar.chunk_cap) {
                     rec = atomicAdd(work + 1, 1);
-                    if (rec < ar.rec_cap) {
-                        off = atomicAdd(work + 4, count);
-                        if (off <= ar.pool_ints - count) {
-                            base = atomicAdd(work + 2, want);
-                            got = max(0, min(want, ar.chunk_cap - base));
-                        }
+                    off = atomicAdd(work + 4, count);
+                    base = atomicAdd(work + 2, want);
+                    got = max(0, min(want, ar.chunk_cap - base));
+                    if (rec >= ar.rec_cap || off > ar.pool_ints - count) {
+                        for (int i = 0; i < got; ++i)
+                            arena[(size_t)kChunkInts * (base + i)] = 0;
+                        got = 0;
                     }
                 }
                 sm.pub[0] = rec;
@@ -1993,8 +1993,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                 sm.pub[2] = got;
                 sm.pub[3] = off;
                 s_next2 = min(n_und, got * kChunkVp);   // the tile keeps the rest
-                if (got > 0)
-                    atomicAdd(&R.stats->shared_viewpoints, (unsigned long long)s_next2);
+                s_shared += (unsigned)s_next2;
             }
             __syncthreads();
             const int pub_n = sm.pub[2];
@@ -2026,7 +2025,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
             sweep_kept(R, s_scratch, s_box, n_smem, tail, count, gbox, s_und, &s_next2, n_und, ix0, iy0, layer,
                        sc.n_boxes);
         if (tid == 0) {
-            listed += (unsigned)count;
+            s_listed += (unsigned)count;
             sm.item = -2;   // one_tile: the next round exits
         }
         __syncthreads();
