@@ -29,7 +29,7 @@ constexpr long long kTileWaves = 3;         // waves of resident blocks below wh
 constexpr int kNodeBoxes = 64;             // nearest candidates that the tile's nodes test
 constexpr int kKeptWarps = 2;             // warps that sweep the viewpoints a tile keeps
 constexpr int kSweepBlocks = 6;           // blocks per SM of the second pass
-constexpr int kPartsPerWarp = 4;          // parts of chunks the second pass wants per warp
+constexpr int kPartsPerWarp = 2;          // parts of chunks the second pass wants per warp
 constexpr int kMaxTileViewpoints = 1024;  // viewpoints in one tile (tile_x * tile_y)
 constexpr int kClaimRounds = 4096;        // bounded retries of a spill-region claim (2 us pauses)
 

@@ -2041,7 +2041,8 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
 // of a chunk, stages up to kWarpBoxes of the list for itself and meets no
 // block barrier, so parts are as small as the launch needs: 16 viewpoints when
 // there are many chunks, down to 1 when there are fewer than kPartsPerWarp
-// parts per warp.  What a warp knows of its part lies in shared memory and is
+// parts per warp (2: 4 or 6 parts were 8 % slower on a strict map, 1 was 4 to 8 %
+// slower on maps with bits).  What a warp knows of its part lies in shared memory and is
 // read where it is used: the sweep needs the registers (in registers it
 // spilled 200 bytes and issued 10 % more instructions).
 //
@@ -2208,15 +2209,18 @@ __global__ void k_prologue_desc(const __grid_constant__ DescBlob<BYTES> blob, in
 //     the bit words in registers.  The summation follows the tile kernel's:
 //     a compensated sum per lane, then a fixed-order butterfly.
 
-__device__ __forceinline__ void recolor_point(const DevRequest &R, unsigned vp, float &qu, float &qn, float &qw)
+struct GridPoint {
+    int ix, iy, layer;
+};
+__device__ __forceinline__ GridPoint grid_point(const DevRequest &R, unsigned vp)
 {
     const unsigned nxy = (unsigned)R.nx * (unsigned)R.ny;   // the request has less than 2^31 viewpoints
-    const unsigned layer = vp / nxy, rem = vp - layer * nxy;
-    const unsigned iy = rem / (unsigned)R.nx, ix = rem - iy * (unsigned)R.nx;
-    const float qx = R.x_coord[ix], qy = R.y_coord[iy], qz = R.dims == 3 ? R.z_coord[layer] : 0.f;
-    qu = R.au == 0 ? qx : (R.au == 1 ? qy : qz);
-    qn = R.an == 0 ? qx : (R.an == 1 ? qy : qz);
-    qw = R.dims == 3 ? (R.aw == 0 ? qx : (R.aw == 1 ? qy : qz)) : 0.f;
+    const unsigned layer = vp / nxy, rem = vp - layer * nxy, iy = rem / (unsigned)R.nx;
+    return GridPoint{(int)(rem - iy * (unsigned)R.nx), (int)iy, (int)layer};
+}
+__device__ __forceinline__ float3 recolor_point(const DevRequest &R, const GridPoint &g)
+{
+    return in_target_frame(R, R.x_coord[g.ix], R.y_coord[g.iy], R.dims == 3 ? R.z_coord[g.layer] : 0.f);
 }
 
 // Pass 1 is bound by reading the bits.  A warp takes 32 viewpoints, whose words
@@ -2235,40 +2239,58 @@ __global__ void __launch_bounds__(256) k_recolor_scan(const DevRequest *__restri
     const DevRequest &R = s_r;
     const int lane = threadIdx.x & 31;
     const long long n = (long long)R.nx * R.ny * R.nl;
-    const long long step = (long long)gridDim.x * blockDim.x;
     const bool strict = (R.flags & VCM_STRICT) != 0;
     const unsigned last_mask = (R.P & 31) ? ((1u << (R.P & 31)) - 1u) : 0xffffffffu;
     const int per = R.words >> 2;   // lanes per viewpoint
     const bool wide = (R.words & 3) == 0 && per <= 32 && (per & (per - 1)) == 0 &&
                       (reinterpret_cast<uintptr_t>(R.bits_out) & 15u) == 0;
     const int per_log = wide ? __ffs(per) - 1 : 0;
-    for (long long base = (long long)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += step) {
+    // a run of 32s of viewpoints per warp, walked along the grid's rows: the
+    // divisions are for the first
+    const int warps = gridDim.x * (blockDim.x >> 5), warp = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    const long long groups = (n + 31) >> 5, from = groups * warp / warps, to = groups * (warp + 1) / warps;
+    GridPoint g = grid_point(R, (unsigned)min(32 * from + lane, n - 1));
+    for (long long base = 32 * from; base < 32 * to; base += 32) {
         const long long vp = base + lane;
         bool front = false;
         if (vp < n) {
-            float qu, qn, qw;
-            recolor_point(R, (unsigned)vp, qu, qn, qw);
-            front = facing(R, qn);
+            front = facing(R, recolor_point(R, g).y);
+            g.ix += 32;
+            while (g.ix >= R.nx) {
+                g.ix -= R.nx;
+                if (++g.iy == R.ny) {
+                    g.iy = 0;
+                    if (++g.layer == R.nl)   // past the last viewpoint
+                        g.layer = 0;
+                }
+            }
         }
         const unsigned in_front = __ballot_sync(kFull, front);
         bool all_blocked = true, any_blocked = false;
         if (wide) {
             const int at_once = 32 >> per_log;   // viewpoints per load
-            const unsigned run = per == 32 ? kFull : (1u << per) - 1u;
-            for (int t = 0; t < per; ++t) {
-                if (((in_front >> (t * at_once)) & (at_once == 32 ? kFull : (1u << at_once) - 1u)) == 0u)
-                    continue;
-                const int mine = t * at_once + (lane >> per_log);   // the viewpoint whose words this lane reads
-                uint4 w = make_uint4(0u, 0u, 0u, 0u);
-                if (base + mine < n)
-                    w = __ldg(reinterpret_cast<const uint4 *>(R.bits_out + base * R.words) + t * 32 + lane);
+            const unsigned run = per == 32 ? kFull : (1u << per) - 1u, some = at_once == 32 ? kFull : (1u << at_once) - 1u;
+            for (int t0 = 0; t0 < per; t0 += 4) {
+                // up to four loads in flight
+                uint4 w[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const int t = t0 + q;
+                    w[q] = make_uint4(0u, 0u, 0u, 0u);
+                    if (t < per && ((in_front >> (t * at_once)) & some) != 0u && base + t * at_once + (lane >> per_log) < n)
+                        w[q] = __ldg(reinterpret_cast<const uint4 *>(R.bits_out + base * R.words) + t * 32 + lane);
+                }
                 const unsigned end = (lane & (per - 1)) == per - 1 ? last_mask : 0xffffffffu;
-                const unsigned full = __ballot_sync(kFull, (w.x & w.y & w.z) == 0xffffffffu && (w.w & end) == end);
-                const unsigned any = __ballot_sync(kFull, (w.x | w.y | w.z | (w.w & end)) != 0u);
-                if (lane / at_once == t) {   // this lane's viewpoint was among them
-                    const int sh = (lane & (at_once - 1)) << per_log;
-                    all_blocked = ((full >> sh) & run) == run;
-                    any_blocked = ((any >> sh) & run) != 0u;
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const unsigned full =
+                        __ballot_sync(kFull, (w[q].x & w[q].y & w[q].z) == 0xffffffffu && (w[q].w & end) == end);
+                    const unsigned any = __ballot_sync(kFull, (w[q].x | w[q].y | w[q].z | (w[q].w & end)) != 0u);
+                    if (lane / at_once == t0 + q) {   // this lane's viewpoint was among them
+                        const int sh = (lane & (at_once - 1)) << per_log;
+                        all_blocked = ((full >> sh) & run) == run;
+                        any_blocked = ((any >> sh) & run) != 0u;
+                    }
                 }
             }
         } else if (front) {
@@ -2297,8 +2319,8 @@ __global__ void __launch_bounds__(256) k_recolor_scan(const DevRequest *__restri
 // compensated sum.  Words without an open patch are skipped, the cone is
 // decided for the whole target where it can be (cone_class), rows come from
 // shared memory and a lane's column stays put where 32 is a multiple of the
-// columns.  512^2 x 5 viewpoints, 32 x 16 patches, 120 degree cone:
-// 107 -> 62 us.
+// columns; then a word takes 20 operations without a branch.  512^2 x 5
+// viewpoints, 32 x 16 patches, 120 degree cone: 107 -> 54 us.
 __global__ void __launch_bounds__(256) k_recolor_measure(const DevRequest *__restrict__ reqs,
                                                          const int *__restrict__ list, const int *__restrict__ n_list)
 {
@@ -2324,23 +2346,43 @@ __global__ void __launch_bounds__(256) k_recolor_measure(const DevRequest *__res
     float vmax = 0.f;
     for (int i = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < n; i += warps) {
         const int vq = list[i];
-        float qu, qn, qw;
-        recolor_point(R, (unsigned)vq, qu, qn, qw);
+        const float3 p = recolor_point(R, grid_point(R, (unsigned)vq));
+        const float qu = p.x, qn = p.y, qw = p.z;
         const uint32_t *words = R.bits_out + (long long)vq * n_words;
         const float rn = qn - R.p_n;
         const float m_s = R.measure * ((R.flags & VCM_TWO_SIDED) ? fabsf(rn) : R.sn * rn);
         const int cone = R.cone ? cone_class(R, qu, qn, qw) : kConeIn;
         float sum = 0.f, comp = 0.f;
-        if (cone != kConeOut) {
-            int iu = iu0, iw = iw0;
-            float ru = qu - __ldg(&R.u_coord[iu]), col_d2 = fmaf(ru, ru, rn * rn);
-            unsigned held = 0u;   // words k..k + 31 of this viewpoint, one per lane, open patches set
+        // a term joins by a two-sum of the larger and the smaller (both are >= 0)
+        auto add = [&](float term) {
+            const float tsum = __fadd_rn(sum, term);
+            comp += (fmaxf(sum, term) - tsum) + fminf(sum, term);
+            sum = tsum;
+        };
+        auto word = [&](int k, unsigned &held) {   // word k's open patches; words 32 at a time, one per lane
+            if ((k & 31) == 0) {
+                const int wd = k + lane;
+                held = wd < n_words ? ~__ldg(&words[wd]) & (wd == n_words - 1 ? last_mask : 0xffffffffu) : 0u;
+            }
+            return __shfl_sync(kFull, held, k & 31);
+        };
+        unsigned held = 0u;
+        float ru = qu - __ldg(&R.u_coord[iu0]), col_d2 = fmaf(ru, ru, rn * rn);
+        if (cone == kConeIn && is3d && du == 0 && rows_fit) {
+            // the lane's column stays; a closed patch adds +0, which changes nothing
             for (int k = 0; k < n_words; ++k) {
-                if ((k & 31) == 0) {
-                    const int wd = k + lane;
-                    held = wd < n_words ? ~__ldg(&words[wd]) & (wd == n_words - 1 ? last_mask : 0xffffffffu) : 0u;
+                const unsigned open = word(k, held);
+                if (open) {
+                    const float rw = qw - s_w[min(iw0 + k * dw, R.nw - 1)];
+                    const float ir = rsqrt_normal(fmaf(rw, rw, col_d2));
+                    const float term = m_s * (ir * ir * ir);
+                    add((open >> lane) & 1u ? term : 0.f);
                 }
-                const unsigned open = __shfl_sync(kFull, held, k & 31);
+            }
+        } else if (cone != kConeOut) {
+            int iu = iu0, iw = iw0;
+            for (int k = 0; k < n_words; ++k) {
+                const unsigned open = word(k, held);
                 if (open) {
                     if (du) {   // (otherwise the lane's column stays)
                         ru = qu - __ldg(&R.u_coord[iu]);
@@ -2350,17 +2392,8 @@ __global__ void __launch_bounds__(256) k_recolor_measure(const DevRequest *__res
                         const float rw = qw - (rows_fit ? s_w[iw] : __ldg(&R.w_coord[iw]));
                         if (cone == kConeIn || in_cone_inline(R, ru, rn, rw)) {
                             const float d2 = fmaf(rw, rw, col_d2);
-                            float term;
-                            if (is3d) {
-                                const float ir = rsqrt_normal(d2);
-                                term = m_s * (ir * ir * ir);
-                            } else {
-                                term = m_s / d2;
-                            }
-                            // (both are >= 0: the larger and the smaller give the rounding error)
-                            const float tsum = __fadd_rn(sum, term);
-                            comp += (fmaxf(sum, term) - tsum) + fminf(sum, term);
-                            sum = tsum;
+                            const float ir = rsqrt_normal(d2);
+                            add(is3d ? m_s * (ir * ir * ir) : m_s / d2);
                         }
                     }
                 }
