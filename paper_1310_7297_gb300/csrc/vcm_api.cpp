@@ -1046,7 +1046,7 @@ vcm_status enqueue_graph(vcm_ctx *ctx, Slot &s, const std::vector<const Canon *>
         ctx->scene_gen, P.L.off_reqs, P.L.off_tiles, P.L.off_vps, P.L.off_coords, P.L.bytes,
         (unsigned long long)P.L.total_tiles, (unsigned long long)P.L.total_vp, (unsigned long long)P.box_cap,
         (unsigned long long)P.blocks, P.n, (unsigned long long)P.extra, (unsigned long long)P.tile_check,
-        ptr(s.d_desc), ptr(s.h_desc), ptr(s.d_work), ptr(s.d_spill),
+        (unsigned long long)P.L.blocker_ints, ptr(s.d_desc), ptr(s.h_desc), ptr(s.d_work), ptr(s.d_spill),
         ptr(s.d_spill_busy), ptr(stats)};
     direct_only = direct_only || after != nullptr;   // a graph holds no wait on another stream's event
     s.chained = false;

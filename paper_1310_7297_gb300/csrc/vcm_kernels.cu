@@ -1967,8 +1967,9 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
         // second pass in chunks, with the tile's candidate list: swept here,
         // a few hundred tiles of mostly visible viewpoints set the end of the
         // launch (100-290 us each against 17 us for the median tile).  What
-        // would pass a cap of the arena stays.
-        if (share == 1 && spill_slot >= 0 && n_und > 0) {
+        // would pass a cap of the arena stays, as do lists so long that the pool's
+        // counter could pass 2^31 with one from every resident block.
+        if (share == 1 && spill_slot >= 0 && n_und > 0 && count <= kPublishMax) {
             int *arena = work + kWorkHeader;
             if (tid == 0) {
                 const int want = (n_und + kChunkVp - 1) / kChunkVp;
@@ -2227,7 +2228,7 @@ __device__ __forceinline__ float3 recolor_point(const DevRequest &R, const GridP
 // are one run: where a viewpoint's words are 4, 8, ... 128 and aligned, lanes read
 // 16 bytes each in order and ballots say which viewpoints are all or partly
 // blocked; runs of viewpoints behind the target are not read.  512^2 x 5
-// viewpoints of 16 words: 27 -> 24 us with one viewpoint per thread, 4 bytes a time, before.
+// viewpoints of 16 words: 24 us (27 with one viewpoint per thread, 4 bytes a time).
 __global__ void __launch_bounds__(256) k_recolor_scan(const DevRequest *__restrict__ reqs, int *__restrict__ list,
                                                       int *__restrict__ n_list)
 {

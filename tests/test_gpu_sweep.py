@@ -100,3 +100,40 @@ def test_2d_columns(ctx, pu):
     ctx.load_scene(sc)
     ctx.vcm_build(8.0)
     full_parity(ctx, sc, req2((0, 0), width=16 * U, pu=pu, origin=(-40 * U, -40 * U), step=(2 * U, 2 * U), n=(40, 40)))
+
+
+def test_more_boxes_per_viewpoint_than_records(ctx):
+    """300 posts between the viewpoints and the target: more boxes left to a
+    viewpoint than it keeps records for (32), and longer lists than a warp
+    stages (64)."""
+    posts = []
+    for i in range(60):
+        for j in range(5):
+            x, y = (i - 30) * U // 2 + 100 * j, (4 + 2 * j) * U
+            posts.append(((x, y, 0), (x + 77, y + 90, (6 + (i * 7 + j * 3) % 9) * U)))
+    sc = scene(3, posts)
+    ctx.load_scene(sc)
+    ctx.vcm_build(4.0)
+    r = req3((0, 0, 8 * U), width=20 * U, height=10 * U, pu=64, pw=40, origin=(-12 * U, 14 * U), step=(U, 2 * U),
+             n=(24, 12), layers=(2 * U, 9 * U))
+    _, gb, _, _, _ = full_parity(ctx, sc, r)
+    assert gb.any()
+
+
+def test_more_open_viewpoints_than_the_arena_holds(ctx):
+    """16.8 M viewpoints, nearly all open: the tiles sweep what the second
+    pass's arena (12.8 M) cannot take."""
+    from gpu_util import compare_bits, compare_v, gpu_run
+    from oracle import oracle as O
+
+    sc = field(77, (0, 0, 8 * U))
+    ctx.load_scene(sc)
+    ctx.vcm_build(10.0)
+    r = req3((0, 0, 8 * U), width=6 * U, height=4 * U, pu=4, pw=2, origin=(-2048 * U, -2048 * U), step=(U, U),
+             n=(4096, 4096), layers=(300 * U,), flags=8)   # two-sided: the whole grid faces the target
+    gv, _, gb, st = gpu_run(ctx, r, bits=True)
+    assert np.isfinite(gv).all() and 0 < st["shared_viewpoints"] < gv.size
+    idx = np.unique(np.concatenate([np.random.default_rng(1).choice(gv.size, 600), np.arange(0, gv.size, 65521)]))
+    ov, ob = O.run(sc, r, indices=idx, bits=True)
+    compare_bits(ob, gb[idx])
+    compare_v(ov, gv[idx])
