@@ -998,7 +998,7 @@ vcm_status record_launch(vcm_ctx *ctx, Slot &s, const Prepared &P, vcm_stats *st
         CUDA_TRY(cudaMemsetAsync(s.d_spill_busy, 1, s.spill_busy_cap * sizeof(int), stream));
     if (timed && ctx->ev_before)
         CUDA_TRY(cudaEventRecord(ctx->ev_before, stream));
-    CUDA_TRY(launch_tiles(ctx->scene, d_reqs, d_tiles, (int)P.n, P.L.total_tiles, s.d_work, s.d_spill,
+    CUDA_TRY(launch_tiles(ctx->scene, d_reqs, d_tiles, (int)P.n, P.L.total_tiles, P.L.total_vp, s.d_work, s.d_spill,
                           P.blocks, P.box_cap, P.extra, P.tile_check, ctx->sm_count, stream, one_tile, s.d_spill_busy,
                           /*share=*/true, claim_rounds, Arena(), 0, /*overlap=*/after == nullptr));
     if (timed && ctx->ev_after)
@@ -2689,7 +2689,7 @@ vcm_status vcm_compute_static(const float *lo, const float *hi, uint32_t n_boxes
             CUDA_TRY(cudaMemcpyAsync(s_desc, hdesc.data(), lay.bytes, cudaMemcpyHostToDevice, sm));
             CUDA_TRY(launch_prologue(d_reqs, 1, s_work, nullptr, 0, sm));
         }
-        CUDA_TRY(launch_tiles(sc, d_reqs, d_tiles, 1, lay.total_tiles, s_work, s_spill, blocks, (int)t.box_cap,
+        CUDA_TRY(launch_tiles(sc, d_reqs, d_tiles, 1, lay.total_tiles, lay.total_vp, s_work, s_spill, blocks, (int)t.box_cap,
                               needs_extra(c), c.P >= kTileCheckMinPatches, sm_count, sm, false, nullptr, share, kClaimRounds,
                               arena, list_cap));
         CUDA_TRY(launch_quantise(d_reqs, d_vps, 1, lay.total_vp, sm));

@@ -37,15 +37,16 @@ constexpr int kClaimRounds = 4096;        // bounded retries of a spill-region c
 // Work sharing of the persistent tile kernel, in two passes.  In the first,
 // the tiles publish the viewpoints their checks leave open, kChunkVp at a time,
 // as chunks; in the second, k_sweep's warps sweep parts of the chunks.
-// The work buffer of a launch holds kWorkHeader counters (next tile,
-// records, chunks published, parts taken, id-pool ints used) and then the
-// arena:
+// The work buffer of a launch holds kWorkHeader counters (next tile, and for
+// each round records, chunks published, parts taken, id-pool ints used) and
+// then the arena:
 //   chunk[kChunkCap][kChunkInts]     32 x record index + count, viewpoints (x + 256 y in the tile, 16 bits each)
 //   record[kRecCap][kRecInts]        request, candidate count, offset of its ids in the pool, layer, tile origin
 //   pool[kPoolInts]                  the records' candidate box ids, in the owner's order
 //   blocker[kBlockerCap]             per tile position of each request (many-patch
 //                                    launches): a box id that blocked a tile there, or -1
-// A tile whose publication would pass a cap keeps its viewpoints.
+// A launch with many more viewpoints than the arena holds runs in rounds of
+// both passes.  A tile whose publication would pass a cap keeps its viewpoints.
 constexpr int kChunkVp = 16;
 constexpr int kChunkInts = 1 + kChunkVp / 2;
 constexpr int kChunkCap = 800000;
@@ -54,6 +55,7 @@ constexpr int kRecInts = 8;
 constexpr int kPoolInts = 8 << 20;
 constexpr int kBlockerCap = 1 << 20;
 constexpr int kWorkHeader = 64;   // ints before the arena (256 bytes)
+constexpr int kMaxRounds = 15;    // rounds of a launch: 1 + 4 x 15 counters fit the header
 // Where the parts of an arena lie (in ints, after the header).  The defaults are
 // those of a work buffer of kWorkBytes; vcm_compute_static lays out a smaller
 // one.
@@ -175,7 +177,7 @@ cudaError_t launch_grid_build(const float *d_lo_world, const float *d_hi_world, 
 // its request's vcm_stats.error to VCM_DEVERR_SPILL_WAIT if its candidate
 // list needs one.
 cudaError_t launch_tiles(const DevScene &sc, const DevRequest *d_reqs, const int *d_tile_prefix,
-                         int n_req, int total_tiles, int *d_work, int *d_spill, int grid_blocks,
+                         int n_req, int total_tiles, long long total_vp, int *d_work, int *d_spill, int grid_blocks,
                          int box_cap, bool extra, bool tile_check, int sm_count, cudaStream_t stream,
                          bool one_tile = false,
                          int *d_spill_busy = nullptr, bool share = false, int claim_rounds = kClaimRounds,
@@ -192,7 +194,7 @@ cudaError_t launch_quantise(const DevRequest *d_reqs, const long long *d_vp_pref
 cudaError_t launch_recolor(const DevRequest *d_req, long long n_vp, int sm_count, int *d_list, int *d_n_list,
                            cudaStream_t stream);
 
-// Zero the work counters (d_work[0..5)) and every request's vcm_stats, and set
+// Zero the work counters (d_work[0..kWorkHeader)) and every request's vcm_stats, and set
 // n_blockers entries of the blocker table to -1.
 cudaError_t launch_prologue(const DevRequest *d_reqs, int n_req, int *d_work, int *d_blockers, long long n_blockers,
                             cudaStream_t stream);

@@ -1291,9 +1291,12 @@ template <bool TILE_CHECK>
 __global__ void __launch_bounds__(kThreads, kTileBlocks)
 k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict__ tile_prefix,
         int n_req, int total_tiles, int *__restrict__ work, Arena ar, unsigned char *__restrict__ spill_all, int id_bytes, int box_cap,
-        int list_cap, int one_tile, int *__restrict__ spill_busy, int spill_slots, int share, int claim_rounds)
+        int list_cap, int one_tile, int *__restrict__ spill_busy, int spill_slots, int share, int claim_rounds, int stop_at,
+        int round)
 {
     after_previous_kernel();
+    if (round > 0 && __syncthreads_or(__ldcg(work) >= total_tiles))
+        return;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     float4 *s_box = reinterpret_cast<float4 *>(smem_raw);
     int *s_ids = reinterpret_cast<int *>(smem_raw + (size_t)box_cap * 32);
@@ -1310,7 +1313,9 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
     auto &walk = s_scratch.walk;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     __shared__ int s_spill_slot;
+    __shared__ bool s_full;   // the arena is nearly full: the block leaves its other tiles to the next round
     if (tid == 0) {
+        s_full = false;
         s_req_idx = -1;
         s_npass = 0;
         s_listed = s_shared = 0;
@@ -1371,7 +1376,8 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
         // does tile b only and exits, so blocks of concurrent launches
         // interleave (a persistent grid would hold every SM to the end).
         if (tid == 0) {
-            int it = one_tile ? (sm.item == -2 ? total_tiles : (int)blockIdx.x) : atomicAdd(work, 1);
+            int it = s_full || (one_tile && sm.item == -2) ? total_tiles
+                     : one_tile ? (int)blockIdx.x : atomicAdd(work, 1);
             // Queue order: last tile first, and within a request the
             // layers interleaved (consecutive items are one tile position
             // in every layer).  Measured on the 3D workload with the
@@ -1977,11 +1983,12 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                 // counters move only while their caps are not reached, and all at
                 // once (one round trip, not three): a tile whose record or ids did
                 // not fit leaves its chunks empty
-                if (__ldcg(work + 1) < ar.rec_cap && __ldcg(work + 4) < ar.pool_ints &&
-                    __ldcg(work + 2) < ar.chunk_cap) {
-                    rec = atomicAdd(work + 1, 1);
-                    off = atomicAdd(work + 4, count);
-                    base = atomicAdd(work + 2, want);
+                int *ctr = work + 4 * round;
+                if (__ldcg(ctr + 1) < ar.rec_cap && __ldcg(ctr + 4) < ar.pool_ints &&
+                    __ldcg(ctr + 2) < ar.chunk_cap) {
+                    rec = atomicAdd(ctr + 1, 1);
+                    off = atomicAdd(ctr + 4, count);
+                    base = atomicAdd(ctr + 2, want);
                     got = max(0, min(want, ar.chunk_cap - base));
                     if (rec >= ar.rec_cap || off > ar.pool_ints - count) {
                         for (int i = 0; i < got; ++i)
@@ -1994,6 +2001,8 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                 sm.pub[2] = got;
                 sm.pub[3] = off;
                 s_next2 = min(n_und, got * kChunkVp);   // the tile keeps the rest
+                s_full = stop_at < INT_MAX &&
+                         (got < want || base + want > stop_at || off > ar.pool_ints - (ar.pool_ints >> 3));
                 s_shared += (unsigned)s_next2;
             }
             __syncthreads();
@@ -2057,7 +2066,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
 // registers): 7 spill (+6 %), 5 leave latency open (+8 %).
 template <bool EXTRA>
 __global__ void __launch_bounds__(kThreads, kSweepBlocks)
-k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work, Arena ar)
+k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work, Arena ar, int round)
 {
     after_previous_kernel();
     struct Mine {   // one warp's: a single base address, the rest are constant offsets
@@ -2075,7 +2084,10 @@ k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work
     DevRequest &R = mine.req;
     float4 *boxes = mine.boxes;
     const int *arena = work + kWorkHeader;
-    const int n_chunks = min(work[2], ar.chunk_cap);
+    int *ctr = work + 4 * round;
+    const int n_chunks = min(ctr[2], ar.chunk_cap);
+    if (n_chunks == 0)
+        return;
     const int warps = (int)gridDim.x * kWarps;
     int part_log = 0;   // parts per chunk
     while (part_log < 4 && (n_chunks << part_log) < kPartsPerWarp * warps)
@@ -2090,7 +2102,7 @@ k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work
     for (;;) {
         int item = 0;
         if (lane == 0)
-            item = atomicAdd(work + 3, 1);
+            item = atomicAdd(ctr + 3, 1);
         item = __shfl_sync(kFull, item, 0);
         if ((item >> part_log) >= n_chunks)
             break;
@@ -2162,8 +2174,8 @@ __device__ __forceinline__ void prologue(const DevRequest *reqs, int n_req, int 
                                          int *__restrict__ blockers, int n_blockers)
 {
     const int t = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
-    if (t < 5)
-        work[t] = 0;   // next tile, records, chunks published, parts taken, id-pool ints used
+    if (t < kWorkHeader)
+        work[t] = 0;
     constexpr int kStatWords = (int)(sizeof(vcm_stats) / sizeof(unsigned));
     for (int i = t; i < n_req * kStatWords; i += nt)
         reinterpret_cast<unsigned *>(reqs[i / kStatWords].stats)[i % kStatWords] = 0u;
@@ -2664,7 +2676,7 @@ int tiles_blocks_per_sm(int box_cap, int list_cap)
 int spill_id_bytes(int n_boxes) { return n_boxes < (1 << 24) ? 3 : 4; }
 
 cudaError_t launch_tiles(const DevScene &sc, const DevRequest *d_reqs, const int *d_tile_prefix,
-                         int n_req, int total_tiles, int *d_work, int *d_spill, int grid_blocks,
+                         int n_req, int total_tiles, long long total_vp, int *d_work, int *d_spill, int grid_blocks,
                          int box_cap, bool extra, bool tile_check, int sm_count, cudaStream_t stream, bool one_tile,
                          int *d_spill_busy, bool share, int claim_rounds, const Arena &arena, int list_cap,
                          bool overlap)
@@ -2685,13 +2697,30 @@ cudaError_t launch_tiles(const DevScene &sc, const DevRequest *d_reqs, const int
     }
     auto kernel = tile_check ? k_tiles<true> : k_tiles<false>;
     share = share && !one_tile;
-    cudaError_t e = launch(kernel, grid_blocks, kThreads, smem, stream, overlap, sc, d_reqs, d_tile_prefix, n_req,
-                           total_tiles, d_work, arena, reinterpret_cast<unsigned char *>(d_spill),
-                           spill_id_bytes(sc.n_boxes), box_cap, list_cap, one_tile ? 1 : 0, d_spill_busy, slots,
-                           share ? 1 : 0, claim_rounds);
-    if (e == cudaSuccess && share)   // the second pass, on every SM
-        e = launch(extra ? k_sweep<true> : k_sweep<false>, sm_count * kSweepBlocks, kThreads, 0, stream, true, sc,
-                   d_reqs, d_work, arena);
+    // A launch with many more viewpoints than the arena holds runs in rounds:
+    // when the arena is nearly full, each block stops after the tile it is at, the
+    // second pass empties it, and the tile pass takes the queue up again.  The
+    // last round runs to the queue's end whatever the arena holds; what does
+    // not fit there the tiles sweep themselves, with kKeptWarps warps per block.
+    // 256 requests, 49.3 M open viewpoints: 50.1 -> 35.0 ms.  A round that finds
+    // nothing left costs 8 us (33.5 M viewpoints with 0.3 M open: 1.282 ms in one
+    // round, 1.291 in two, 1.298 in three), so launches of up to four arenas'
+    // viewpoints (51 M), which seldom fill one, run in one, and longer ones
+    // have a round per two.
+    const int usable = std::max(arena.chunk_cap / 2, arena.chunk_cap - grid_blocks * (kMaxTileViewpoints / kChunkVp));
+    const long long rounds =
+        share && total_vp > 4LL * kChunkVp * arena.chunk_cap
+            ? std::min<long long>(kMaxRounds, 1 + total_vp / (2LL * kChunkVp * std::max(1, usable))) : 1;
+    cudaError_t e = cudaSuccess;
+    for (int r = 0; r < rounds && e == cudaSuccess; ++r) {
+        e = launch(kernel, grid_blocks, kThreads, smem, stream, overlap || r > 0, sc, d_reqs, d_tile_prefix, n_req,
+                   total_tiles, d_work, arena, reinterpret_cast<unsigned char *>(d_spill),
+                   spill_id_bytes(sc.n_boxes), box_cap, list_cap, one_tile ? 1 : 0, d_spill_busy, slots,
+                   share ? 1 : 0, claim_rounds, r + 1 < rounds ? usable : INT_MAX, r);
+        if (e == cudaSuccess && share)   // the second pass, on every SM
+            e = launch(extra ? k_sweep<true> : k_sweep<false>, sm_count * kSweepBlocks, kThreads, 0, stream, true,
+                       sc, d_reqs, d_work, arena, r);
+    }
     return e;
 }
 

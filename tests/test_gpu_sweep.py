@@ -120,19 +120,21 @@ def test_more_boxes_per_viewpoint_than_records(ctx):
     assert gb.any()
 
 
-def test_more_open_viewpoints_than_the_arena_holds(ctx):
-    """16.8 M viewpoints, nearly all open: the tiles sweep what the second
-    pass's arena (12.8 M) cannot take."""
+@pytest.mark.parametrize("n", (4096, 7232), ids=("one-round", "rounds"))
+def test_more_open_viewpoints_than_the_arena_holds(ctx, n):
+    """Nearly all viewpoints open, and more of them than the second pass's arena
+    (12.8 M) takes: the tiles sweep the rest of 16.8 M, 52.3 M run in rounds."""
     from gpu_util import compare_bits, compare_v, gpu_run
     from oracle import oracle as O
 
     sc = field(77, (0, 0, 8 * U))
     ctx.load_scene(sc)
     ctx.vcm_build(10.0)
-    r = req3((0, 0, 8 * U), width=6 * U, height=4 * U, pu=4, pw=2, origin=(-2048 * U, -2048 * U), step=(U, U),
-             n=(4096, 4096), layers=(300 * U,), flags=8)   # two-sided: the whole grid faces the target
+    r = req3((0, 0, 8 * U), width=6 * U, height=4 * U, pu=4, pw=2, origin=(-n // 2 * U, -n // 2 * U), step=(U, U),
+             n=(n, n), layers=(300 * U,), flags=8)   # two-sided: the whole grid faces the target
     gv, _, gb, st = gpu_run(ctx, r, bits=True)
     assert np.isfinite(gv).all() and 0 < st["shared_viewpoints"] < gv.size
+    assert n == 4096 or st["shared_viewpoints"] > 13000000
     idx = np.unique(np.concatenate([np.random.default_rng(1).choice(gv.size, 600), np.arange(0, gv.size, 65521)]))
     ov, ob = O.run(sc, r, indices=idx, bits=True)
     compare_bits(ob, gb[idx])
