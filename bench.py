@@ -57,8 +57,8 @@ OPS_PER_SLAB_TEST = {3: 19, 2: 13}
 ISSUED_OPS_PER_INTERVAL_TEST = 36
 ISSUED_OPS_PER_CORNER_TEST = 15
 L2_FLUSH_BYTES = 512 << 20
-# kernels of ours that one step launches: k_prologue, k_tiles (two passes:
-# the tiles, then the open viewpoints they published), k_quantise
+# kernels of ours that one step launches: k_prologue_desc, k_tiles (the tiles),
+# k_sweep (the open viewpoints they published), k_quantise
 LAUNCHES_PER_STEP = 4
 
 
@@ -86,7 +86,7 @@ PROFILE_3D = os.path.join(ROOT, "profiles", "k_tiles_3d_512x512x5_5000boxes.md")
 
 
 def profiled_traffic(profile):
-    """DRAM bytes per k_tiles launch (both passes) of the workload a
+    """DRAM bytes per launch of k_tiles and k_sweep, together, of the workload a
     committed ncu summary covers, or None if the kernel source has changed
     since that capture."""
     import hashlib
@@ -365,7 +365,7 @@ def time_direct(ctx, req, steps, warmup, stream, flush, sampler, what, preload_s
 
 
 def alu_roofline(stats, dims, kern_ms, sm_count, profile=None):
-    """ALU roofline of k_tiles (both passes): the device-counted slab tests
+    """ALU roofline of k_tiles and k_sweep: the device-counted slab tests
     x their algorithmic operations over the passes' CUDA-event time."""
     max_mhz = float(peaks().get("sm_max_mhz", 2070.0))
     peak = alu_peak_ops(sm_count, max_mhz)
@@ -376,7 +376,7 @@ def alu_roofline(stats, dims, kern_ms, sm_count, profile=None):
               stats["corner_tests"] * ISSUED_OPS_PER_CORNER_TEST) / kern_s
     return {"bound": "alu", "achieved": achieved / 1e12, "peak": peak / 1e12, "unit": "Tops/s",
             "frac": achieved / peak, "traffic": profiled_traffic(profile) if profile else None,
-            "kernel": "k_tiles (both passes)", "work_unit": "segment/box or column/box slab test",
+            "kernel": "k_tiles and k_sweep", "work_unit": "segment/box or column/box slab test",
             "ops_per_unit": OPS_PER_SLAB_TEST[dims],
             "issued_slab_ops": {"value": issued / 1e12, "frac": issued / peak,
                                 "ops_per_interval_test": ISSUED_OPS_PER_INTERVAL_TEST,

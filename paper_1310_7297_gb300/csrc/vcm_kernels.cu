@@ -2,14 +2,15 @@
 //
 //  * grid build: boxes bucketed by footprint centre into a uniform 2D grid
 //    (count -> scan -> scatter -> permuted copies in box order -> bounds);
-//  * tile kernel: persistent blocks draw viewpoint tiles from a queue; each
-//    tile culls the scene against the convex hull of (tile, target) using
-//    the grid, stages the candidates in shared memory with cp.async, and its
-//    warps sweep the tile's viewpoints, lanes over target patch columns and
-//    bits of a mask over patch rows, deciding each viewpoint->patch segment by
-//    a float32 slab test (Def. 2 point-to-point visibility; touching blocks,
-//    Def. 4) with an exact integer re-decision inside a 1e-6 margin band,
-//    then summing A cos(theta)/d^2 (or len cos(theta)/d in 2D) per viewpoint;
+//  * tile pass: persistent blocks draw viewpoint tiles from a queue; each tile
+//    culls the scene against the convex hull of (tile, target) using the
+//    grid, stages the candidates in shared memory with cp.async, decides the
+//    viewpoints that one box hides, and publishes the others;
+//  * sweep: warps take the published viewpoints, lanes over target patch columns
+//    and bits of a mask over patch rows, deciding each viewpoint->patch segment
+//    by float32 slab intervals (Def. 2 point-to-point visibility; touching
+//    blocks, Def. 4) with an exact integer re-decision inside a 1e-6 margin
+//    band, then summing A cos(theta)/d^2 (or len cos(theta)/d in 2D);
 //  * quantise: colors in L levels from v / v_ref (Def. 1 normalisation).
 #include "vcm_internal.h"
 
@@ -1230,8 +1231,8 @@ union TileScratch {
     WarpScratch sweep[kKeptWarps];
 };
 
-// The open viewpoints that a tile does not publish (launches without a second
-// pass, or an arena that is full), swept by the tile's first warps.  Not
+// The open viewpoints that a tile does not publish (no second pass, a full arena in
+// the last round, a list past the arena), swept by the tile's first warps.  Not
 // inlined: the tile pass then holds none of the sweep's registers.
 __device__ __noinline__ void sweep_kept(const DevRequest &R, TileScratch &T, const float4 *__restrict__ sbox,
                                         int n_smem, Tail spill, int count,
@@ -1372,7 +1373,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
 
     for (;;) {
         // thread 0 takes the next tile, copies its request and lays out the
-        // hull points (one barrier for all of it).  With one_tile, block b
+        // two rectangles of the cull (one barrier for all of it).  With one_tile, block b
         // does tile b only and exits, so blocks of concurrent launches
         // interleave (a persistent grid would hold every SM to the end).
         if (tid == 0) {
