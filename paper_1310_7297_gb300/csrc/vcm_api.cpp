@@ -2689,7 +2689,7 @@ vcm_status vcm_compute_static(const float *lo, const float *hi, uint32_t n_boxes
             CUDA_TRY(cudaMemcpyAsync(s_desc, hdesc.data(), lay.bytes, cudaMemcpyHostToDevice, sm));
             CUDA_TRY(launch_prologue(d_reqs, 1, s_work, nullptr, 0, sm));
         }
-        CUDA_TRY(launch_tiles(sc, d_reqs, d_tiles, 1, lay.total_tiles, lay.total_vp, s_work, s_spill, blocks, (int)t.box_cap,
+        CUDA_TRY(launch_tiles(sc, d_reqs, d_tiles, 1, lay.total_tiles, /*total_vp=*/0, s_work, s_spill, blocks, (int)t.box_cap,
                               needs_extra(c), c.P >= kTileCheckMinPatches, sm_count, sm, false, nullptr, share, kClaimRounds,
                               arena, list_cap));
         CUDA_TRY(launch_quantise(d_reqs, d_vps, 1, lay.total_vp, sm));

@@ -167,6 +167,9 @@ cudaError_t launch_grid_build(const float *d_lo_world, const float *d_hi_world, 
 // (kWorkBytes for the default one), and a second
 // kernel on all sm_count SMs works the open viewpoints that expensive tiles of
 // the first published there.
+// `total_vp`: the requests' viewpoints, from which the number of rounds follows;
+// 0: one round (vcm_compute_static: its arena is small, and rounds that find
+// nothing left would cost 8 us each).
 // `list_cap` > box_cap: the ids of candidates past the staged boxes are kept in
 // shared memory, which must then hold every box of the scene (d_spill is not
 // used); otherwise they spill.
