@@ -8,6 +8,12 @@
 
 #include "../../include/vcm.h"
 
+#ifdef __CUDACC__
+#define VCM_HD __host__ __device__
+#else
+#define VCM_HD
+#endif
+
 namespace vcm {
 
 constexpr int kWarps = 4;                 // warps per block of the tile kernel
@@ -62,18 +68,9 @@ constexpr int kMaxRounds = 15;    // rounds of a launch: 1 + 4 x 15 counters fit
 // one.
 struct Arena {
     int chunk_cap = kChunkCap, rec_cap = kRecCap, pool_ints = kPoolInts;
-#ifdef __CUDACC__
-    __host__ __device__
-#endif
-    size_t rec_off() const { return (size_t)chunk_cap * kChunkInts; }
-#ifdef __CUDACC__
-    __host__ __device__
-#endif
-    size_t pool_off() const { return rec_off() + (size_t)rec_cap * kRecInts; }
-#ifdef __CUDACC__
-    __host__ __device__
-#endif
-    size_t blocker_off() const { return pool_off() + (size_t)pool_ints; }
+    VCM_HD size_t rec_off() const { return (size_t)chunk_cap * kChunkInts; }
+    VCM_HD size_t pool_off() const { return rec_off() + (size_t)rec_cap * kRecInts; }
+    VCM_HD size_t blocker_off() const { return pool_off() + (size_t)pool_ints; }
 };
 constexpr size_t kArenaInts = (size_t)kChunkCap * kChunkInts + (size_t)kRecCap * kRecInts + (size_t)kPoolInts +
                               (size_t)kBlockerCap;
@@ -81,10 +78,7 @@ constexpr size_t kWorkBytes = (kWorkHeader + kArenaInts) * sizeof(int);
 
 // Bytes per id of a spill region, and of a block's region (a multiple of 4).
 int spill_id_bytes(int n_boxes);
-#ifdef __CUDACC__
-__host__ __device__
-#endif
-inline size_t spill_region_bytes(int n_boxes, int id_bytes)
+VCM_HD inline size_t spill_region_bytes(int n_boxes, int id_bytes)
 {
     return ((size_t)(n_boxes > 0 ? n_boxes : 1) * id_bytes + 3) & ~(size_t)3;
 }
@@ -143,6 +137,28 @@ struct DevRequest {
     float cone_c;              // cosine of its half-angle
     float cone_a[3];           // its unit axis, world x, y, z
 };
+
+// The rules that the checked build applies to what goes through the arena: the
+// places a tile publishes at, and what a chunk's first word, a record (its list's
+// ids and its layer among them) and a viewpoint of the chunk name.
+VCM_HD inline bool publication_in_bounds(const Arena &a, int rec, int chunk, int chunks, int ids, int n_ids)
+{
+    return rec >= 0 && rec < a.rec_cap && chunk >= 0 && chunks >= 0 && chunk <= a.chunk_cap - chunks && ids >= 0 &&
+           n_ids >= 0 && ids <= a.pool_ints - n_ids;
+}
+VCM_HD inline bool chunk_in_bounds(const Arena &a, int word)
+{
+    return word >= 0 && (word >> 5) < a.rec_cap && (word & 31) <= kChunkVp;
+}
+VCM_HD inline bool record_in_bounds(const Arena &a, const int *rec, const DevRequest *reqs, int n_req, int n_boxes)
+{
+    return rec[0] >= 0 && rec[0] < n_req && rec[1] >= 0 && rec[1] <= n_boxes && rec[2] >= 0 &&
+           rec[2] <= a.pool_ints - rec[1] && rec[3] >= 0 && rec[3] < reqs[rec[0]].nl;
+}
+VCM_HD inline bool viewpoint_in_bounds(const DevRequest &R, int ix, int iy)
+{
+    return ix >= 0 && ix < R.nx && iy >= 0 && iy < R.ny;
+}
 
 // Launch helpers implemented in vcm_kernels.cu.  All are asynchronous on
 // `stream` and return the launch status.

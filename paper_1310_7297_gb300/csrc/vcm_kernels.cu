@@ -57,8 +57,10 @@ __device__ __noinline__ bool in_bounds_slow(long long i, long long n, vcm_stats 
     return false;
 }
 #define IN_BOUNDS(i, n, st) in_bounds_slow((long long)(i), (long long)(n), (st))
+#define CHECKED(ok, st) in_bounds_slow((ok) ? 0 : 1, 1, (st))   // the same for a rule of vcm_internal.h
 #else
 #define IN_BOUNDS(i, n, st) true
+#define CHECKED(ok, st) true
 #endif
 
 // The ids of a candidate list past its staged boxes: ints, or 3 bytes each in a
@@ -2007,9 +2009,12 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                     got = max(0, min(want, ar.chunk_cap - base));
                     if (rec >= ar.rec_cap || off > ar.pool_ints - count) {
                         for (int i = 0; i < got; ++i)
-                            arena[(size_t)kChunkInts * (base + i)] = 0;
+                            if (IN_BOUNDS(base + i, ar.chunk_cap, R.stats))
+                                arena[(size_t)kChunkInts * (base + i)] = 0;
                         got = 0;
                     }
+                    if (got > 0 && !CHECKED(publication_in_bounds(ar, rec, base, got, off, count), R.stats))
+                        got = 0;
                 }
                 sm.pub[0] = rec;
                 sm.pub[1] = base;
@@ -2034,8 +2039,10 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
                     rp[4] = ix0;
                     rp[5] = iy0;
                 }
-                for (int i = tid; i < count; i += kThreads)
-                    ids[i] = i < n_smem ? s_ids[i] : tail[i - n_smem];
+                for (int i = tid; i < count; i += kThreads) {
+                    const int id = i < n_smem ? s_ids[i] : tail[i - n_smem];
+                    ids[i] = IN_BOUNDS(id, sc.n_boxes, R.stats) ? id : 0;
+                }
                 for (int i = tid; i < pub_n * kChunkInts; i += kThreads) {
                     const int j = i / kChunkInts, r = i - j * kChunkInts, k = j * kChunkVp + 2 * (r - 1);
                     const int n_j = min(kChunkVp, n_und - j * kChunkVp);
@@ -2081,7 +2088,7 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
 // registers): 7 spill (+6 %), 5 leave latency open (+8 %).
 template <bool EXTRA>
 __global__ void __launch_bounds__(kThreads, kSweepBlocks)
-k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work, Arena ar, int round)
+k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int n_req, int *__restrict__ work, Arena ar, int round)
 {
     after_previous_kernel();
     struct Mine {   // one warp's: a single base address, the rest are constant offsets
@@ -2122,6 +2129,9 @@ k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work
         if ((item >> part_log) >= n_chunks)
             break;
         const int *chunk = arena + (size_t)kChunkInts * (item >> part_log);
+        if (!IN_BOUNDS(item >> part_log, ar.chunk_cap, reqs[0].stats) ||
+            !CHECKED(chunk_in_bounds(ar, chunk[0]), reqs[0].stats))
+            continue;
         const int rec = chunk[0] >> 5;
         const int first = (item & ((1 << part_log) - 1)) * part_vp, n = min((chunk[0] & 31) - first, part_vp);
         if (n <= 0)
@@ -2129,6 +2139,9 @@ k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work
         __syncwarp();   // the viewpoints before are done with the item's shared memory
         const int at = lane < n ? reinterpret_cast<const unsigned short *>(chunk + 1)[first + lane] : 0;
         if (rec != cur_rec) {
+            if (!CHECKED(record_in_bounds(ar, arena + ar.rec_off() + (size_t)kRecInts * rec, reqs, n_req, sc.n_boxes),
+                         reqs[0].stats))
+                continue;
             cur_rec = rec;
             const int old_req = list[0];
             __syncwarp();
@@ -2147,12 +2160,19 @@ k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int *__restrict__ work
             const float4 *gbox = sc.boxes[R.perm];
             for (int i = lane; i < min(list[1], kWarpBoxes); i += 32) {
                 const int id = arena[ar.pool_off() + list[2] + i];
+                if (!IN_BOUNDS(id, sc.n_boxes, R.stats)) {   // an empty box
+                    boxes[2 * i] = make_float4(f_inf(), f_inf(), f_inf(), 0.f);
+                    boxes[2 * i + 1] = make_float4(-f_inf(), -f_inf(), -f_inf(), 0.f);
+                    continue;
+                }
                 boxes[2 * i] = __ldg(&gbox[2 * id]);
                 boxes[2 * i + 1] = __ldg(&gbox[2 * id + 1]);
             }
         }
         if (lane < n) {   // one per lane: 45 instructions for all of them
-            const int ix = list[4] + (at & 255), iy = list[5] + (at >> 8);
+            int ix = list[4] + (at & 255), iy = list[5] + (at >> 8);
+            if (!CHECKED(viewpoint_in_bounds(R, ix, iy), R.stats))
+                ix = iy = 0;
             const float3 q = in_target_frame(R, R.x_coord[ix], R.y_coord[iy], R.z_coord[list[3]]);
             mine.q[lane] = make_float4(q.x, q.y, q.z, facing(R, q.y) ? 1.f : 0.f);
             mine.vp[lane] = ((long long)list[3] * R.ny + iy) * R.nx + ix;
@@ -2734,7 +2754,7 @@ cudaError_t launch_tiles(const DevScene &sc, const DevRequest *d_reqs, const int
                    share ? 1 : 0, claim_rounds, r + 1 < rounds ? usable : INT_MAX, r);
         if (e == cudaSuccess && share)   // the second pass, on every SM
             e = launch(extra ? k_sweep<true> : k_sweep<false>, sm_count * kSweepBlocks, kThreads, 0, stream, true,
-                       sc, d_reqs, d_work, arena, r);
+                       sc, d_reqs, n_req, d_work, arena, r);
     }
     return e;
 }
