@@ -177,8 +177,9 @@ typedef struct {
     uint32_t vmax_bits;                /* largest v (float bits), accumulated on device */
     uint32_t edge_cells;               /* viewpoints within 1e-5 (relative) of a color bin edge */
     uint32_t error;                    /* VCM_DEVERR_*: nonzero if a device-side check failed */
-    unsigned long long slab_tests;     /* slab tests executed in the sweep: a patch column against a box
-                                          (VCM_VIEWER: a segment against a box) */
+    unsigned long long slab_tests;     /* slab tests executed in the sweep: a box against a patch column, or a
+                                          row group of it, with rows still open (rows decided one by one are
+                                          not counted again); VCM_VIEWER: a box against a segment */
     unsigned long long rechecked;      /* segment-box pairs re-decided by the exact predicate */
     unsigned long long segments;       /* viewpoint-patch pairs decided (= viewpoints x patches) */
     unsigned long long boxes_listed;   /* sum over tiles of culled candidate-list lengths */

@@ -971,7 +971,7 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
                         const float4 ru = rec[2 * j], rw = rec[2 * j + 1];
                         const float iE = fminf(fmaf(du, ru.x, ru.y), rw.x);
                         const float iX = fmaxf(fmaxf(du * ru.z, du * ru.w), rw.y);
-                        ++tests;
+                        tests += alive != 0u;
                         unsigned hit = 0u, ask = 0u;   // rows blocked for certain, rows to decide one by one
                         if (alive != 0u && iE >= iX * kLess) {
                             // first row + 1/2 and last row - 1/2 of the interval
@@ -1284,9 +1284,11 @@ __device__ __noinline__ void sweep_kept(const DevRequest &R, TileScratch &T, con
         corners += vp_corners;
     }
     rechecks = __reduce_add_sync(kFull, rechecks);
+    for (int off = 16; off > 0; off >>= 1)
+        tests += __shfl_xor_sync(kFull, tests, off);
     if (lane == 0) {
         atomicMax(&R.stats->vmax_bits, __float_as_uint(vmax));
-        atomicAdd(&R.stats->slab_tests, 32 * tests);
+        atomicAdd(&R.stats->slab_tests, tests);
         atomicAdd(&R.stats->corner_tests, corners);
         if (shortcuts)
             atomicAdd(&R.stats->shortcut_viewpoints, (unsigned long long)shortcuts);
@@ -2188,11 +2190,13 @@ k_sweep(DevScene sc, const DevRequest *__restrict__ reqs, int n_req, int *__rest
             vmax = fmaxf(vmax, v);
         }
         rechecks = __reduce_add_sync(kFull, rechecks);
+        // the lanes' tests, in two halves that cannot overflow
+        const unsigned low = __reduce_add_sync(kFull, tests & 0xffffu), high = __reduce_add_sync(kFull, tests >> 16);
         if (lane == 0) {
             if (vmax > 0.f)
                 atomicMax(&R.stats->vmax_bits, __float_as_uint(vmax));
-            if (tests)
-                atomicAdd(&R.stats->slab_tests, 32ull * tests);
+            if (low | high)
+                atomicAdd(&R.stats->slab_tests, ((unsigned long long)high << 16) + low);
             if (corners)
                 atomicAdd(&R.stats->corner_tests, (unsigned long long)corners);
             if (shortcuts)
