@@ -1513,7 +1513,7 @@ void launch_recolor_group(vcm_ctx *ctx, Slot &s, std::vector<std::shared_ptr<Tic
         const long long *d_vps = reinterpret_cast<const long long *>(s.d_desc + L.off_vps);
         int *list = nullptr;   // the viewpoints that need a measure; their count is the first work counter
         CUDA_TRY(cudaMallocAsync((void **)&list, sizeof(int) * (size_t)c.n_vp, s.stream));
-        const cudaError_t le = launch_recolor(d_reqs, c.n_vp, ctx->sm_count, list, s.d_work, s.stream);
+        const cudaError_t le = launch_recolor(d_reqs, c.n_vp, c.nw, ctx->sm_count, list, s.d_work, s.stream);
         cudaFreeAsync(list, s.stream);
         CUDA_TRY(le);
         CUDA_TRY(launch_quantise(d_reqs, d_vps, 1, c.n_vp, s.stream));
@@ -2519,7 +2519,7 @@ vcm_status vcm_recolor(vcm_ctx *ctx, const vcm_request *req, const uint32_t *d_b
         const long long *d_vps = reinterpret_cast<const long long *>(s.d_desc + L.off_vps);
         if (ctx->ev_before)
             CUDA_TRY(cudaEventRecord(ctx->ev_before, strm));
-        CUDA_TRY(launch_recolor(d_reqs, c.n_vp, ctx->sm_count, ctx->d_recolor_list, s.d_work, strm));
+        CUDA_TRY(launch_recolor(d_reqs, c.n_vp, c.nw, ctx->sm_count, ctx->d_recolor_list, s.d_work, strm));
         if (ctx->ev_after)
             CUDA_TRY(cudaEventRecord(ctx->ev_after, strm));
         CUDA_TRY(launch_quantise(d_reqs, d_vps, 1, c.n_vp, strm));

@@ -209,9 +209,9 @@ cudaError_t launch_quantise(const DevRequest *d_reqs, const long long *d_vp_pref
 
 // Values of one request (d_req[0]) recomputed from the occlusion bits its
 // bits_out points at (read only); colors then come from launch_quantise.
-// d_list: n_vp ints of scratch for the viewpoints that need a measure, and
-// d_n_list their count, 0 before (n_vp <= INT_MAX).
-cudaError_t launch_recolor(const DevRequest *d_req, long long n_vp, int sm_count, int *d_list, int *d_n_list,
+// n_rows: its patch rows.  d_list: n_vp ints of scratch for the viewpoints that
+// need a measure, and d_n_list their count, 0 before (n_vp <= INT_MAX).
+cudaError_t launch_recolor(const DevRequest *d_req, long long n_vp, int n_rows, int sm_count, int *d_list, int *d_n_list,
                            cudaStream_t stream);
 
 // Zero the work counters (d_work[0..kWorkHeader)) and every request's vcm_stats, and set
