@@ -995,8 +995,13 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
                             float4 lo, hi;
                             load_box(sbox, n_smem, spill, gbox, fits ? W.rec_id[j] : base + j, n_boxes, R.stats, lo,
                                      hi);
-                            // a column with many such rows (it grazes the box): its rows over the lanes
+                            // a column with many such rows (it grazes the box): its rows over the
+                            // lanes, where that takes fewer steps than every lane doing its own
+                            // (28 x 8 patches, 73,000 viewpoints that many boxes graze in all
+                            // columns: 257 us without the comparison, 111 with it)
                             unsigned columns = __ballot_sync(kFull, __popc(ask) > 2);
+                            if (__popc(columns) >= (int)__reduce_max_sync(kFull, (unsigned)__popc(ask)))
+                                columns = 0u;
                             while (columns) {
                                 const int from = __ffs(columns) - 1;
                                 columns &= columns - 1;
