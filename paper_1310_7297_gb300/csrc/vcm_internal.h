@@ -34,7 +34,13 @@ constexpr int kLongList = 256;            // longer lists are filtered as a view
 constexpr int kTileBlocks = 8;            // blocks per SM of the tile pass
 constexpr long long kTileWaves = 3;         // waves of resident blocks below which a launch's tiles shrink
 constexpr int kNodeBoxes = 64;             // nearest candidates that the tile's nodes test
-constexpr int kPublishMax = 1 << 20;        // longest list a tile publishes (x 8 blocks x 152 SMs < 2^31)
+#ifndef VCM_CHECKED
+constexpr int kPublishMax = 1 << 20;      // longest list a tile publishes (x 8 blocks x 152 SMs < 2^31)
+constexpr int kWideIds = 1 << 24;         // boxes from which a spill region's ids take 4 bytes, not 3
+#else   // the checked build's small scenes reach both sides of either limit
+constexpr int kPublishMax = 300;
+constexpr int kWideIds = 600;
+#endif
 constexpr int kKeptWarps = 2;             // warps that sweep the viewpoints a tile keeps
 constexpr int kSweepBlocks = 6;           // blocks per SM of the second pass
 constexpr int kPartsPerWarp = 2;          // parts of chunks the second pass wants per warp

@@ -2719,7 +2719,7 @@ int tiles_blocks_per_sm(int box_cap, int list_cap)
     return n;
 }
 
-int spill_id_bytes(int n_boxes) { return n_boxes < (1 << 24) ? 3 : 4; }
+int spill_id_bytes(int n_boxes) { return n_boxes < kWideIds ? 3 : 4; }
 
 cudaError_t launch_tiles(const DevScene &sc, const DevRequest *d_reqs, const int *d_tile_prefix,
                          int n_req, int total_tiles, long long total_vp, int *d_work, int *d_spill, int grid_blocks,
