@@ -223,7 +223,8 @@ def _raw_stream(stream, dev):
 
     if stream is not None:
         return stream.cuda_stream
-    return torch._C._cuda_getCurrentRawStream(dev.index)
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)   # private to torch
+    return raw(dev.index) if raw else torch.cuda.current_stream(dev).cuda_stream
 
 
 class Context:
