@@ -669,7 +669,7 @@ Layout layout_for(const std::vector<const Canon *> &cs, const std::vector<vcm_tu
 // Fill the pinned descriptor arena (host side) for a launch.
 void fill_desc(char *h, const char *d_base, const Layout &L, const std::vector<const Canon *> &cs,
                const std::vector<vcm_tune> &shapes, float *const *v, uint8_t *const *color,
-               uint32_t *const *bits, vcm_stats *stats, int box_cap, bool blockers = true)
+               uint32_t *const *bits, vcm_stats *stats, bool blockers = true)
 {
     const size_t n = cs.size();
     DevRequest *reqs = reinterpret_cast<DevRequest *>(h + L.off_reqs);
@@ -709,7 +709,6 @@ void fill_desc(char *h, const char *d_base, const Layout &L, const std::vector<c
         d.v_ref_given = c.v_ref;
         d.levels = c.levels;
         d.flags = c.flags;
-        d.box_cap = box_cap;
         d.cone = c.cone;
         d.cone_c = c.cone_c;
         for (int k = 0; k < 3; ++k)
@@ -965,20 +964,18 @@ vcm_status prepare_launch(vcm_ctx *ctx, Slot &s, const std::vector<const Canon *
         return st;
     if ((st = desc_free(s)) != VCM_OK)
         return st;
-    fill_desc(s.h_desc, s.d_desc, P.L, cs, shapes, v, color, bits, stats, P.box_cap);
+    fill_desc(s.h_desc, s.d_desc, P.L, cs, shapes, v, color, bits, stats);
     return VCM_OK;
 }
 
 // Device half: descriptor upload, counters, bit buffers, the persistent tile
 // kernel and the quantiser, in stream order.  The node sequence is the same
 // for every launch, so a captured graph can be updated in place.
-vcm_status record_launch(vcm_ctx *ctx, Slot &s, const Prepared &P, vcm_stats *stats, cudaStream_t stream,
-                         bool timed = false, bool capturing = false, bool one_tile = false,
-                         int claim_rounds = kClaimRounds, bool hold_spill = false,
-                         cudaEvent_t after = nullptr)
+vcm_status record_launch(vcm_ctx *ctx, Slot &s, const Prepared &P, cudaStream_t stream, bool timed = false,
+                         bool capturing = false, bool one_tile = false, int claim_rounds = kClaimRounds,
+                         bool hold_spill = false, cudaEvent_t after = nullptr)
 {
     Range range("vcm record launch");
-    (void)stats;   // the descriptors point into it; the prologue clears it
     const vcm_status up = upload_desc(s, P.L, P.n, P.tile_check ? P.L.blocker_ints : 0, stream, capturing);
     if (up != VCM_OK)
         return up;
@@ -1018,7 +1015,7 @@ vcm_status enqueue_launch(vcm_ctx *ctx, Slot &s, const std::vector<const Canon *
     vcm_status st = prepare_launch(ctx, s, cs, shapes, v, color, bits, stats, stream, P, adapt);
     if (st != VCM_OK)
         return st;
-    return record_launch(ctx, s, P, stats, stream, timed);
+    return record_launch(ctx, s, P, stream, timed);
 }
 
 // Same device work on the slot's stream.  A launch whose parameters equal
@@ -1059,12 +1056,12 @@ vcm_status enqueue_graph(vcm_ctx *ctx, Slot &s, const std::vector<const Canon *>
     if (direct_only || s.last_key[f] != key) {
         if (!direct_only)
             s.last_key[f] = key;
-        return record_launch(ctx, s, P, stats, s.stream, false, false, one_tile, claim_rounds, hold_spill, after);
+        return record_launch(ctx, s, P, s.stream, false, false, one_tile, claim_rounds, hold_spill, after);
     }
     s.key[f].clear();
     CUDA_TRY(cudaStreamBeginCapture(s.stream, cudaStreamCaptureModeRelaxed));
     // one_tile: one block per tile, so launches of other slots interleave
-    st = record_launch(ctx, s, P, stats, s.stream, false, true, one_tile);
+    st = record_launch(ctx, s, P, s.stream, false, true, one_tile);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(s.stream, &g);
     if (st != VCM_OK) {
@@ -1499,7 +1496,7 @@ void launch_recolor_group(vcm_ctx *ctx, Slot &s, std::vector<std::shared_ptr<Tic
         float *vv[1] = {t.d_v};
         uint8_t *cc[1] = {t.d_color};
         uint32_t *bb[1] = {e->d_bits};   // read only in k_recolor
-        fill_desc(s.h_desc, s.d_desc, L, cs, shapes, vv, cc, bb, s.d_stats, 256, /*blockers=*/false);
+        fill_desc(s.h_desc, s.d_desc, L, cs, shapes, vv, cc, bb, s.d_stats, /*blockers=*/false);
         CUDA_TRY(cudaEventRecord(s.t0, s.stream));
         if ((ready = upload_desc(s, L, 1, 0, s.stream)) != VCM_OK)
             return ready;
@@ -2512,7 +2509,7 @@ vcm_status vcm_recolor(vcm_ctx *ctx, const vcm_request *req, const uint32_t *d_b
         float *vv[1] = {d_v};
         uint8_t *cc[1] = {d_color};
         uint32_t *bb[1] = {const_cast<uint32_t *>(d_bits)};   // read only in k_recolor
-        fill_desc(s.h_desc, s.d_desc, L, cs, shapes, vv, cc, bb, d_stats, 256, /*blockers=*/false);
+        fill_desc(s.h_desc, s.d_desc, L, cs, shapes, vv, cc, bb, d_stats, /*blockers=*/false);
         if ((st = upload_desc(s, L, 1, 0, strm)) != VCM_OK)
             return st;
         const DevRequest *d_reqs = reinterpret_cast<const DevRequest *>(s.d_desc + L.off_reqs);
@@ -2677,7 +2674,7 @@ vcm_status vcm_compute_static(const float *lo, const float *hi, uint32_t n_boxes
         float *vv[1] = {d_v};
         uint8_t *cc[1] = {d_color};
         uint32_t *bb[1] = {d_bits};
-        fill_desc(hdesc.data(), s_desc, lay, cs, shapes, vv, cc, bb, d_stats, (int)t.box_cap, /*blockers=*/false);
+        fill_desc(hdesc.data(), s_desc, lay, cs, shapes, vv, cc, bb, d_stats, /*blockers=*/false);
         const DevRequest *d_reqs = reinterpret_cast<const DevRequest *>(s_desc + lay.off_reqs);
         const int *d_tiles = reinterpret_cast<const int *>(s_desc + lay.off_tiles);
         const long long *d_vps = reinterpret_cast<const long long *>(s_desc + lay.off_vps);

@@ -138,7 +138,6 @@ struct DevRequest {
     float v_ref_given;
     int levels;
     unsigned flags;
-    int box_cap;               // candidate boxes staged in shared memory
     int cone;                  // 1: a field-of-view cone masks the patches
     float cone_c;              // cosine of its half-angle
     float cone_a[3];           // its unit axis, world x, y, z
