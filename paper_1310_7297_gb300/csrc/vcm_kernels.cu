@@ -896,12 +896,11 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
     // the boxes that can block a patch at all, and the one-box test of each
     // (lists of at most 8 boxes were tested whole in the tile pass); long lists
     // are left to the passes
-    int n_rec = 0;
+    int n_rec = count > kLongList ? 33 : 0;
     {
-        const int head = count > kLongList ? 0 : count;
         const PatchRect P = patch_rect(R.u_min - qu, R.u_max - qu, R.w_min - qw, R.w_max - qw);
-        for (int base = 0; base < head; base += 32) {
-            bool keep = base + lane < head, full = false;
+        for (int base = n_rec ? count : 0; base < count; base += 32) {
+            bool keep = base + lane < count, full = false;
             float4 r0, r1;
             if (keep) {
                 float4 lo, hi;
@@ -924,7 +923,6 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
             }
             n_rec += __popc(kept);
         }
-        n_rec = head < count ? 33 : n_rec;
         __syncwarp();   // the records are written
     }
     if (want_bits) {   // the passes below set bits in the viewpoint's cleared words
@@ -1000,7 +998,7 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
                             // (28 x 8 patches, 73,000 viewpoints that many boxes graze in all
                             // columns: 257 us without the comparison, 111 with it)
                             unsigned columns = __ballot_sync(kFull, __popc(ask) > 2);
-                            if (__popc(columns) >= (int)__reduce_max_sync(kFull, (unsigned)__popc(ask)))
+                            if (columns && __popc(columns) >= (int)__reduce_max_sync(kFull, (unsigned)__popc(ask)))
                                 columns = 0u;
                             while (columns) {
                                 const int from = __ffs(columns) - 1;
