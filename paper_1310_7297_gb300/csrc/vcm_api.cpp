@@ -604,14 +604,16 @@ struct Ticket {
 
 namespace {
 
-// 16 x 16 viewpoints per tile: with the chunk phase taking the open
-// viewpoints of expensive tiles, larger tiles spread the cull (16 x 8 was
-// 2 % slower on the 3D workload and the 100,000-box scene, 4 % on the
-// 256-request mix; 32 x 8 and 32 x 16 were 40-90 % slower, 8 x 8 18 %).
-// 448 staged boxes: at 6 and 7 blocks per SM, less shared memory leaves more
-// L1 for the tile kernel's spilled registers (against 512: 100,000-box
-// step -0.5 %, 5,000-box step -2.1 %, 256-request batch -0.4 %; 1,024 was
-// 28 % slower on the 100,000-box scene).
+// 16 x 16 viewpoints per tile: the open ones go to the second pass, so a tile is
+// as large as its cull and node checks like.  512^2 x 5 viewpoints, 5,000 boxes
+// (two scenes) 102 / 75 us; 16 x 8 119 / 90, 8 x 8 158 / 127, 32 x 8 108 / 74,
+// 32 x 16 107 / 76, 32 x 32 141 / 111.  2,048^2 x 8, 100,000 boxes 3.18 / 1.81 ms;
+// 16 x 8 3.80 / 2.44, 32 x 16 3.47 / 2.28.  64 uneven requests 6.35 ms; 16 x 8
+// 7.02, 32 x 16 6.22.
+// 448 staged boxes (14 KB, and 2 KB of ids, per block at 8 blocks per SM): more
+// take L1 from the index and the box copies (1,024: 111 us, 3.58 ms and 6.85 ms
+// on the first of each of these), fewer leave more boxes behind ids (256: 101 us,
+// 3.17 / 1.82 ms, 6.33 ms).
 vcm_tune default_tune()
 {
     vcm_tune t;
@@ -627,9 +629,10 @@ vcm_tune shape_for(vcm_ctx *ctx, const Canon &c)
     if (ctx->forced)
         return ctx->forced_tune;
     if (c.flags & VCM_VIEWER) {
-        // one segment per cell: larger tiles spread the per-tile cull over
-        // more cells (3D workload, 512 x 512 x 5 cells: 16 x 8 0.20 ms,
-        // 32 x 8 0.14, 32 x 16 0.13, 32 x 32 0.16; 2,048 staged boxes slower)
+        // one segment per cell: larger tiles spread the cull over more cells.
+        // Maps of less than 1.9 M cells shrink them (shrink_small_launch), so
+        // that 512 x 512 x 5 cells run as 16 x 16: 65 us, 16 x 8 87, 32 x 8 73,
+        // 32 x 16 83; 1,024 staged boxes 79
         vcm_tune t{};
         t.tile_x = 32;
         t.tile_y = 16;
@@ -854,10 +857,9 @@ int launch_box_cap(const std::vector<vcm_tune> &shapes)
 // A launch with few tiles leaves SMs idle while its expensive tiles run
 // (a tile is one block's work item): shrink the tiles, 16 x 16 -> 16 x 8 ->
 // 8 x 8 -> 8 x 4, until the launch holds kTileWaves waves of resident blocks.
-// Measured on the 64 requests of the serving pool, each launched alone: the
-// sum of their times 45.3 ms -> 26.1 ms (the best shape per request would
-// give 25.7 ms); a 124 x 124 x 5 grid with 64 x 32 patches 3.28 -> 0.30 ms.
-// Launches with many tiles (the 3D workloads, batches) keep their shapes.
+// 64 x 64 viewpoints of 8 x 4 patches 42 -> 35 us, 97 x 83 x 3 of 45 x 13
+// two-sided 51 -> 40 us; launches with many tiles (512^2 x 5 viewpoints, batches)
+// keep their shapes: 102 us, and 119 with tiles of 16 x 8.
 // `list_cap`: as of launch_tiles.
 void shrink_small_launch(int sm_count, const std::vector<const Canon *> &cs, std::vector<vcm_tune> &shapes,
                          int list_cap = 0)

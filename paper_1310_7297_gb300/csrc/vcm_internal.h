@@ -21,10 +21,12 @@ constexpr int kThreads = kWarps * 32;
 constexpr int kPassCap = 2 * kThreads;       // cells listed per round of the grid walk
 constexpr int kDistClasses = 128;            // distance classes of the candidate counting sort
 // Launches whose requests all have this many patches look at recorded blockers
-// before a tile's cull.  With the node checks it pays where lists are long and
-// walks deep (100,000 boxes, 64 x 32 patches: 1.51 -> 1.42 ms on a mostly
-// hidden target, 3.40 -> 3.46 ms on a mostly visible one); at 512 patches it
-// cost 4 % (5,000 boxes: 0.189 -> 0.197 ms).
+// before a tile's cull.  What decides is how much of the map one box hides, which
+// the host does not know: 33.5 M viewpoints, 100,000 boxes and 64 x 32 patches
+// took 1.47 ms without and 1.28 with them where nearly all is hidden, 2.05 and
+// 2.04 where more is seen.  The line keeps them from the maps they were slower
+// for: 512^2 x 5 viewpoints, 5,000 boxes, 32 x 16 patches 80.0 -> 81.6 us, with
+// bits 146.5 -> 149.5.
 constexpr int kTileCheckMinPatches = 1024;
 constexpr float kBand = 1e-6f;            // FP32 slab margin that is re-decided exactly
 constexpr int kMaxBoxCap = 5000;          // candidate boxes a tile stages in shared memory

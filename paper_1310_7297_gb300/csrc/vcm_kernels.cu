@@ -715,8 +715,9 @@ __device__ __forceinline__ unsigned bit_run(int start, int n)
 // (512^2 viewpoints in 2D, 100,000 rectangles, lists of 1,900: 0.69 -> 0.31 ms,
 // strict 0.67 -> 0.17; 256^2 x 2, 100,000 posts, strict 0.26 -> 0.13).  The whole
 // list first is better for shorter ones: lists of 240 took 5 % longer with the
-// line at 128 boxes; so are wide targets that one box behind many others hides
-// (4.5 M viewpoints, lists of 440, a target of 100 m: 10.0 -> 13.1 ms).
+// line at 128 boxes.  It is better too where one box far down the list hides a
+// viewpoint (4.5 M viewpoints, lists of 440, a target of 100 m: 10.0 -> 13.1 ms;
+// 15 viewpoints, lists of 3,000: 0.17 -> 0.29 ms), which a sweep cannot know.
 //
 // Measured against the row tests (both passes; 2,048^2 x 8 viewpoints, 100,000
 // boxes, 64 x 32 patches: 10.9 -> 5.4 ms; 512^2 x 5, 5,000 boxes, 32 x 16:
@@ -893,9 +894,11 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
     float sum = 0.f, comp = 0.f;
     const int cone = EXTRA && R.cone ? cone_class(R, qu, qn, qw) : kConeIn;
 
-    // the boxes that can block a patch at all, and the one-box test of each
-    // (lists of at most 8 boxes were tested whole in the tile pass); long lists
-    // are left to the passes
+    // the boxes that can block a patch at all, and the one-box test of each; long
+    // lists are left to the passes.  Lists of at most 8 boxes go without the test:
+    // the tile's checks mostly had these boxes, and a box that blocks every patch
+    // closes the rows at its first interval anyway (with the test 73.1 us on
+    // 512^2 x 5 viewpoints and 5,000 boxes, 71.9 without)
     int n_rec = count > kLongList ? 33 : 0;
     {
         const PatchRect P = patch_rect(R.u_min - qu, R.u_max - qu, R.w_min - qw, R.w_max - qw);
@@ -1493,9 +1496,9 @@ k_tiles(DevScene sc, const DevRequest *__restrict__ reqs, const int *__restrict_
 
         // Shortcut from recorded blockers: a box that blocked this tile position on
         // another layer, or a neighbouring position, often blocks this tile
-        // too, so threads 0-4 test those first, against the same 16
-        // segments as the check below; a tile one of them blocks skips its
-        // cull.  Any tile writes the table, so which blocker it keeps is a
+        // too, so 20 lanes test five of those first, each against the four extreme
+        // patches from one of the tile's four corners; a tile one of them blocks
+        // skips its cull.  Any tile writes the table, so which blocker it keeps is a
         // race; a box counts only if it certainly blocks, so results do not
         // depend on the table.
         bool pre_blocked = false;
@@ -2257,9 +2260,9 @@ __global__ void k_prologue_desc(const __grid_constant__ DescBlob<BYTES> blob, in
 // (R.bits_out is read, not written): no occlusion test, only the sides, the
 // field-of-view cone, strictness and the measure.  Two passes, because the
 // viewpoints that need a measure cluster in the grid:
-//  1. one viewpoint per thread: the side test and the viewpoint's bit words
-//     (fully blocked, or in strict mode any patch blocked, gives v = 0);
-//     the others are appended to a list;
+//  1. a warp per 32 viewpoints: the side test of each and their bit words (fully
+//     blocked, or in strict mode any patch blocked, gives v = 0); the others are
+//     appended to a list;
 //  2. one warp per listed viewpoint, lanes over patches, the warp holding
 //     the bit words in registers.  The summation follows the tile kernel's:
 //     a compensated sum per lane, then a fixed-order butterfly.
@@ -2500,7 +2503,7 @@ __device__ __forceinline__ unsigned char quantise_one(float v, float vref, int L
 // 4-byte store of colors when the four belong to one request and both
 // addresses are aligned, else one at a time.  A block takes a run of
 // viewpoints and looks its request up once; for each group of four on its own
-// the search took more than the colors (64 requests, 46 M viewpoints: 124 -> @
+// the search took more than the colors (64 requests, 46 M viewpoints: 124 -> 121
 // us).
 __global__ void k_quantise(const DevRequest *__restrict__ reqs, const long long *__restrict__ vp_prefix,
                            int n_req, long long total)
@@ -2748,9 +2751,16 @@ cudaError_t launch_tiles(const DevScene &sc, const DevRequest *d_reqs, const int
     // not fit there the tiles sweep themselves, with kKeptWarps warps per block.
     // 256 requests, 49.3 M open viewpoints: 50.1 -> 35.0 ms.  A round that finds
     // nothing left costs 8 us (33.5 M viewpoints with 0.3 M open: 1.282 ms in one
-    // round, 1.291 in two, 1.298 in three), so launches of up to four arenas'
-    // viewpoints (51 M), which seldom fill one, run in one, and longer ones
-    // have a round per two.
+    // round, 1.291 in two, 1.298 in three).  What fills an arena (12.8 M) is open
+    // viewpoints, which the host does not know; launches of up to four arenas'
+    // viewpoints (51 M) run in one round, for maps of cities leave 1 to 9 % open,
+    // and longer ones have a round per two.  Open maps below the line pay for it,
+    // though less than when the tiles kept all they could not publish and swept it
+    // with every warp: 33.5 M viewpoints of 512 patches, 30 M open, 29.1 ms then,
+    // 17.4 now, 13.6 in three rounds; of 2,048 patches 88.9, 48.2 and 31.4; 16.8 M
+    // of 8 patches, 13.2 M open, 10.6, 7.4 and 7.1.  Static maps (an arena of
+    // 0.5 M, always one round): 8.4 M viewpoints of 512 patches, all open, 12.1 ms
+    // then, 7.6 now.
     const int usable = std::max(arena.chunk_cap / 2, arena.chunk_cap - grid_blocks * (kMaxTileViewpoints / kChunkVp));
     const long long rounds =
         share && total_vp > 4LL * kChunkVp * arena.chunk_cap
