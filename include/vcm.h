@@ -281,7 +281,10 @@ vcm_status vcm_build(vcm_ctx *ctx, float grid_cell_m);
  * (one vcm_stats).  Returns once the work is enqueued.  Calls on one
  * context share its scratch and must not overlap on the device; issue them
  * on one stream.  The first call for a larger shape may allocate scratch
- * (and synchronises the device once). */
+ * (and synchronises the device once).  On a stream that is being captured
+ * into a CUDA graph in global or thread-local mode this call, like
+ * vcm_compute_batch and vcm_recolor, returns VCM_E_CUDA (and the capture is
+ * invalid): a graph would keep using scratch that later calls replace. */
 vcm_status vcm_compute(vcm_ctx *ctx, const vcm_request *req, float *d_v, uint8_t *d_color,
                        uint32_t *d_bits, vcm_stats *d_stats, void *stream);
 

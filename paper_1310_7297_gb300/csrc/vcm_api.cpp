@@ -896,11 +896,24 @@ int grid_blocks_for(vcm_ctx *ctx, int box_cap, int total_tiles)
     return std::max(1, std::min(total_tiles, resident_blocks(ctx, box_cap)));
 }
 
-// Wait until the pinned descriptors may be rewritten.
-vcm_status desc_free(Slot &s)
+// Wait until the pinned descriptors may be rewritten.  A caller's stream that is
+// being captured takes the wait whether or not an upload is pending: only a
+// capture in relaxed mode permits it.  The others end here, before anything of the
+// call is captured; their graph would hold addresses of scratch that the context
+// frees when a later call needs more.
+vcm_status desc_free(Slot &s, cudaStream_t stream)
 {
-    if (s.desc_pending)
-        CUDA_TRY(cudaEventSynchronize(s.desc_copied));
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    CUDA_TRY(cudaStreamIsCapturing(stream, &cap));
+    if (s.desc_pending || cap != cudaStreamCaptureStatusNone) {
+        const cudaError_t e = cudaEventSynchronize(s.desc_copied);
+        if (e != cudaSuccess) {
+            (void)cudaGetLastError();   // returned here, and not to be met by a later call
+            return fail(VCM_E_CUDA, cap != cudaStreamCaptureStatusNone ? "stream is being captured: %s"
+                                                                       : "waiting for the last upload: %s",
+                        cudaGetErrorString(e));
+        }
+    }
     s.desc_pending = false;
     return VCM_OK;
 }
@@ -964,7 +977,7 @@ vcm_status prepare_launch(vcm_ctx *ctx, Slot &s, const std::vector<const Canon *
     vcm_status st = ensure_slot(ctx, s, P.L.bytes, cs.size(), P.blocks, sync_stream);
     if (st != VCM_OK)
         return st;
-    if ((st = desc_free(s)) != VCM_OK)
+    if ((st = desc_free(s, sync_stream)) != VCM_OK)
         return st;
     fill_desc(s.h_desc, s.d_desc, P.L, cs, shapes, v, color, bits, stats);
     return VCM_OK;
@@ -1492,7 +1505,7 @@ void launch_recolor_group(vcm_ctx *ctx, Slot &s, std::vector<std::shared_ptr<Tic
     t.form = VCM_FORM_RECOLOR;
     vcm_status st = ensure_slot(ctx, s, L.bytes, 1, 1, s.stream);
     auto body = [&]() -> vcm_status {
-        vcm_status ready = desc_free(s);
+        vcm_status ready = desc_free(s, s.stream);
         if (ready != VCM_OK)
             return ready;
         float *vv[1] = {t.d_v};
@@ -2497,7 +2510,7 @@ vcm_status vcm_recolor(vcm_ctx *ctx, const vcm_request *req, const uint32_t *d_b
         const Layout L = layout_for(cs, shapes);
         if ((st = ensure_slot(ctx, s, L.bytes, 1, 1, strm)) != VCM_OK)
             return st;
-        if ((st = desc_free(s)) != VCM_OK)
+        if ((st = desc_free(s, strm)) != VCM_OK)
             return st;
         if ((size_t)c.n_vp > ctx->recolor_cap) {
             // earlier work may still read the old list
