@@ -904,7 +904,8 @@ int grid_blocks_for(vcm_ctx *ctx, int box_cap, int total_tiles)
 vcm_status desc_free(Slot &s, cudaStream_t stream)
 {
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    CUDA_TRY(cudaStreamIsCapturing(stream, &cap));
+    if (stream && stream != cudaStreamLegacy)   // (the legacy stream cannot be captured, and asking takes 1 us)
+        CUDA_TRY(cudaStreamIsCapturing(stream, &cap));
     if (s.desc_pending || cap != cudaStreamCaptureStatusNone) {
         const cudaError_t e = cudaEventSynchronize(s.desc_copied);
         if (e != cudaSuccess) {
