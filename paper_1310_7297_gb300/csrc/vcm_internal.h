@@ -32,7 +32,6 @@ constexpr float kBand = 1e-6f;            // FP32 slab margin that is re-decided
 constexpr int kMaxBoxCap = 5000;          // candidate boxes a tile stages in shared memory
 constexpr int kRowCap = 256;              // patch rows a warp stages for the measure
 constexpr int kWarpBoxes = 64;            // boxes of a chunk's list a warp stages
-constexpr int kLongList = 256;            // longer lists are filtered as a viewpoint's passes go over them
 constexpr int kTileBlocks = 8;            // blocks per SM of the tile pass
 constexpr long long kTileWaves = 3;         // waves of resident blocks below which a launch's tiles shrink
 constexpr int kNodeBoxes = 64;             // nearest candidates that the tile's nodes test
@@ -234,7 +233,7 @@ cudaError_t launch_prologue_desc(const void *h_desc, size_t bytes, void *d_desc,
 // Blocks of the tile kernel that fit on one SM for this shared-memory size.
 int tiles_blocks_per_sm(int box_cap, int list_cap = 0);
 
-// One-time per-device setup (constant tables, kernel attributes); must run
+// One-time per-device setup (kernel attributes); must run
 // before any launch is captured into a graph.
 cudaError_t init_device();
 

@@ -708,16 +708,19 @@ __device__ __forceinline__ unsigned bit_run(int start, int n)
 // from the same record: a box that certainly blocks the four extreme patches
 // blocks them all (the one-box check), and the viewpoint is decided.  A
 // viewpoint keeps its records over its column passes when at most 32 boxes
-// are left (nearly always: 1 to 5); otherwise each pass filters the list again.
-// A list of more than kLongList boxes is filtered by the passes only, 32 boxes at
-// a time, nearest first, until no row is open: among thousands of boxes a few near
-// ones usually close a viewpoint, and in strict mode the first blocked row does
-// (512^2 viewpoints in 2D, 100,000 rectangles, lists of 1,900: 0.69 -> 0.31 ms,
-// strict 0.67 -> 0.17; 256^2 x 2, 100,000 posts, strict 0.26 -> 0.13).  The whole
-// list first is better for shorter ones: lists of 240 took 5 % longer with the
-// line at 128 boxes.  It is better too where one box far down the list hides a
-// viewpoint (4.5 M viewpoints, lists of 440, a target of 100 m: 10.0 -> 13.1 ms;
-// 15 viewpoints, lists of 3,000: 0.17 -> 0.29 ms), which a sweep cannot know.
+// are left (nearly always: 1 to 5).  When there are more, the filter ends there and
+// each pass filters the list again, 32 boxes at a time, nearest first, until no
+// row is open: where that many boxes lie before the target a few near ones
+// usually close it, and in strict mode the first blocked row does.  Filtered to its
+// end for the sake of the one-box test, such a list cost more than it saved: 512^2
+// viewpoints in 2D, 100,000 rectangles of 0.3 to 1 m in 1 km, 330 -> 263 us, strict
+// 310 -> 195; as posts, 256^2 x 2 viewpoints, 32 x 16 patches, 404 -> 315, strict
+// 372 -> 195; of 0.5 to 3 m in 10 km 263 -> 292 (2D) and 327 -> 312 (posts).  Long
+// lists without the filter are faster still where no box hides the viewpoint (281
+// and 144 us for the posts), but in cities one further on often does: 100,000
+// rectangles of 5 to 30 m in 10 km 99 us, without 158; with bits, 512^2 x 2
+// viewpoints, 60 m target 306 and 441.  A hiding box behind 32 others is missed: 4.5
+// M viewpoints, 100 m target, one scene 654 -> 680 us, another 1.63 -> 1.38 ms.
 //
 // Measured against the row tests (both passes; 2,048^2 x 8 viewpoints, 100,000
 // boxes, 64 x 32 patches: 10.9 -> 5.4 ms; 512^2 x 5, 5,000 boxes, 32 x 16:
@@ -786,9 +789,9 @@ __device__ __forceinline__ bool record_blocks_rect(float4 r0, float4 r1, float i
     return e0 > x0 * kMore && e1 > x1 * kMore && from < P.w_from * row && to > P.w_to * row;
 }
 
-// The filter of one pass for a viewpoint with a long list or more than 32 kept
-// boxes: lanes over the boxes [base, base + 32); returns the kept ones, records
-// written.  Of boxes that block the whole pass one is enough.
+// The filter of one pass for a viewpoint with more than 32 kept boxes: lanes over
+// the boxes [base, base + 32); returns the kept ones, records written.  Of boxes
+// that block the whole pass one is enough.
 __device__ __noinline__ unsigned pass_records(const DevRequest &R, const float4 *__restrict__ sbox, int n_smem,
                                               Tail spill, int count,
                                               const float4 *__restrict__ gbox, float qu, float qn, float qw, int cp,
@@ -894,15 +897,15 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
     float sum = 0.f, comp = 0.f;
     const int cone = EXTRA && R.cone ? cone_class(R, qu, qn, qw) : kConeIn;
 
-    // the boxes that can block a patch at all, and the one-box test of each; long
-    // lists are left to the passes.  Lists of at most 8 boxes go without the test:
+    // the boxes that can block a patch at all, and the one-box test of each, up to
+    // the 33rd kept one.  Lists of at most 8 boxes go without the test:
     // the tile's checks mostly had these boxes, and a box that blocks every patch
     // closes the rows at its first interval anyway (with the test 73.1 us on
     // 512^2 x 5 viewpoints and 5,000 boxes, 71.9 without)
-    int n_rec = count > kLongList ? 33 : 0;
+    int n_rec = 0;
     {
         const PatchRect P = patch_rect(R.u_min - qu, R.u_max - qu, R.w_min - qw, R.w_max - qw);
-        for (int base = n_rec ? count : 0; base < count; base += 32) {
+        for (int base = 0; base < count; base += 32) {
             bool keep = base + lane < count, full = false;
             float4 r0, r1;
             if (keep) {
@@ -925,6 +928,8 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
                 W.rec_id[at] = base + lane;
             }
             n_rec += __popc(kept);
+            if (n_rec > 32)   // the passes filter the list
+                break;
         }
         __syncwarp();   // the records are written
     }

@@ -83,3 +83,24 @@ def test_long_lists_in_2d(ctx, pu):
         full_parity(ctx, sc, dict(r, flags=flags))
     gv, _, _, st = gpu_run(ctx, r, bits=False)
     assert st["error"] == 0 and st["boxes_listed"] > 0
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 34, 63, 64, 65, 98])
+@pytest.mark.parametrize("wall", [False, True], ids=["posts", "wall"])
+@pytest.mark.parametrize("pu,pw,flags", [(40, 40, 0), (16, 8, 2), (3, 70, 8)])
+def test_kept_boxes_around_the_records_that_a_viewpoint_holds(ctx, n, wall, pu, pw, flags):
+    """Up to n posts in a viewpoint's view (32 records are held; with more the passes
+    filter the list), without and with a box behind them that hides the whole
+    target."""
+    boxes = [((-9 * U + i * 18 * U // n, 8 * U + i * U // 8, 0), (-9 * U + i * 18 * U // n + 60, 8 * U + i * U // 8 + 60, 9 * U))
+             for i in range(n)]
+    if wall:
+        boxes.append(((-30 * U, 2 * U, 0), (30 * U, 3 * U, 40 * U)))
+    sc = scene(3, boxes)
+    ctx.load_scene(sc)
+    ctx.vcm_build(0.0)
+    r = req3((0, 0, 6 * U), width=24 * U, height=9 * U, pu=pu, pw=pw, origin=(-4 * U, 24 * U), step=(U, 2 * U),
+             n=(9, 7), layers=(2 * U, 8 * U), flags=flags)
+    gv, _, st, _, _ = full_parity(ctx, sc, r, bits=False)
+    full_parity(ctx, sc, r)
+    assert st["error"] == 0 and (not wall or not gv.any())
