@@ -423,8 +423,8 @@ vcm_status vcm_get_tune(vcm_ctx *ctx, const vcm_request *req, vcm_tune *out);
  *
  * The work is enqueued on `stream` (a cudaStream_t, NULL = legacy default)
  * of the current device; host inputs are consumed before the call returns.
- * The first call on a device looks up the array's device address and
- * uploads constant tables; make that first call before any stream capture.
+ * The first call on a device looks up the array's device address and sets
+ * kernel attributes; make that first call before any stream capture.
  * Every call on a device reuses that device's array and leaves the last
  * call's contents in it (each call clears what must start at zero).  Calls
  * whose work overlaps on the same GPU, e.g. on two streams, race on the

@@ -233,8 +233,8 @@ cudaError_t launch_prologue_desc(const void *h_desc, size_t bytes, void *d_desc,
 // Blocks of the tile kernel that fit on one SM for this shared-memory size.
 int tiles_blocks_per_sm(int box_cap, int list_cap = 0);
 
-// One-time per-device setup (kernel attributes); must run
-// before any launch is captured into a graph.
+// One-time per-device setup (kernel attributes); must run before any launch is
+// captured into a graph.
 cudaError_t init_device();
 
 // Device address and size of the file-scope scratch array used by
