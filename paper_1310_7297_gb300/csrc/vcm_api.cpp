@@ -364,6 +364,9 @@ void fill_shape(const Canon &c, const vcm_tune &t, DevRequest &d)
     d.groups = 32 / d.nuc;
     d.col_passes = (c.nu + d.nuc - 1) / d.nuc;
     d.rows = (c.nw + d.groups - 1) / d.groups;
+    // with many passes the one filter of the whole list is cheaper than theirs
+    const int passes = d.col_passes * ((d.rows + 31) / 32);
+    d.filter_stop = passes > 2 ? 32 * passes : 32;
     d.inv_row = 1.f / ((float)d.groups * c.row_step);
     d.row_dev = c.row_dev;
     d.tile_x = (int)std::max(1u, t.tile_x);

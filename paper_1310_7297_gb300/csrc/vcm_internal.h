@@ -124,6 +124,7 @@ struct DevRequest {
     int nx, ny, nl;            // viewpoint grid
     int tile_x, tile_y, tiles_x, tiles_y, n_tiles;
     int nuc, groups, col_passes, rows;   // lane mapping: columns and row groups of a pass, column passes, rows per lane
+    int filter_stop;           // kept boxes at which a viewpoint's filter leaves its list to the passes
     float inv_row, row_dev;    // 1 / w step between a lane's rows; how far a row is off an even step
     int blk_base;                // offset of its tile positions in the blocker table, or -1
     const float *u_coord;      // [nu] patch centre coordinate along u

@@ -708,8 +708,9 @@ __device__ __forceinline__ unsigned bit_run(int start, int n)
 // from the same record: a box that certainly blocks the four extreme patches
 // blocks them all (the one-box check), and the viewpoint is decided.  A
 // viewpoint keeps its records over its column passes when at most 32 boxes
-// are left (nearly always: 1 to 5).  When there are more, the filter ends there and
-// each pass filters the list again, 32 boxes at a time, nearest first, until no
+// are left (nearly always: 1 to 5).  When there are more (filter_stop: 32, with
+// more than two passes 32 for each), the filter ends there and each pass filters
+// the list again, 32 boxes at a time, nearest first, until no
 // row is open: where that many boxes lie before the target a few near ones
 // usually close it, and in strict mode the first blocked row does.  Filtered to its
 // end for the sake of the one-box test, such a list cost more than it saved: 512^2
@@ -721,6 +722,9 @@ __device__ __forceinline__ unsigned bit_run(int start, int n)
 // rectangles of 5 to 30 m in 10 km 99 us, without 158; with bits, 512^2 x 2
 // viewpoints, 60 m target 306 and 441.  A hiding box behind 32 others is missed: 4.5
 // M viewpoints, 100 m target, one scene 654 -> 680 us, another 1.63 -> 1.38 ms.
+// The more passes, the more that costs: 16 of them (100 x 100 patches, strict, bits)
+// 2.23 -> 2.97 ms, with 32 boxes per pass 2.32; 3 (31 x 65) 61 -> 84, 61.5 us.  Two
+// (64 patches in 2D) are better with 32: the first of the scenes above 263 and 283 us.
 //
 // Measured against the row tests (both passes; 2,048^2 x 8 viewpoints, 100,000
 // boxes, 64 x 32 patches: 10.9 -> 5.4 ms; 512^2 x 5, 5,000 boxes, 32 x 16:
@@ -897,8 +901,8 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
     float sum = 0.f, comp = 0.f;
     const int cone = EXTRA && R.cone ? cone_class(R, qu, qn, qw) : kConeIn;
 
-    // the boxes that can block a patch at all, and the one-box test of each, up to
-    // the 33rd kept one.  Lists of at most 8 boxes go without the test:
+    // the boxes that can block a patch at all, and the one-box test of each, until
+    // filter_stop are kept.  Lists of at most 8 boxes go without the test:
     // the tile's checks mostly had these boxes, and a box that blocks every patch
     // closes the rows at its first interval anyway (with the test 73.1 us on
     // 512^2 x 5 viewpoints and 5,000 boxes, 71.9 without)
@@ -928,7 +932,7 @@ __device__ __forceinline__ float sweep_viewpoint(const DevRequest &R, const Lane
                 W.rec_id[at] = base + lane;
             }
             n_rec += __popc(kept);
-            if (n_rec > 32)   // the passes filter the list
+            if (n_rec > R.filter_stop)   // the passes filter the list
                 break;
         }
         __syncwarp();   // the records are written
