@@ -72,8 +72,7 @@ def peaks():
 
 
 def hbm_peak():
-    """Copy bandwidth measured on the GB300s, else the recipe's
-    fallback figure."""
+    """The measured copy bandwidth of a GB300, else an earlier measurement."""
     v = peaks().get("hbm_gbs")
     if v:
         return {"value": float(v), "basis": "measured copy bandwidth (MEASURED_PEAKS.json hbm_gbs)"}
